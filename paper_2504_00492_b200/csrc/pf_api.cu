@@ -105,6 +105,7 @@ int check_options(const pf_params* a) {
 Problem as_problem(const pf_params* a) {
     Problem p = as_problem(a->B, a->H, a->L, a->d_k, a->d_v, a->r, a->chunk, a->in_dtype);
     p.mode = a->mode;
+    p.exact = a->step == PF_STEP_EXACT;
     p.wu_builder = a->wu_builder;
     p.ring_depth = a->ring_depth;
     return p;
@@ -146,6 +147,14 @@ int select_impl(Problem& p, int impl) {
 // PF_IMPL_TC: the single launch where it supports the shape; under PF_IMPL_AUTO only where it is also the faster of
 // the two tensor-core forms (an explicit PF_IMPL_TC takes it whenever it can run).
 bool use_fused(const Problem& p) { return fused_supported(p) && (!p.auto_impl || fused_preferred(p)); }
+
+// Calls that the token-by-token kernel takes: those on the fp32 path (unless the Theorem 3.3 builder is asked for), and
+// bf16 calls of so few tokens that a chunk would be mostly padding (one token of 128 sequences: 12 us against 56).
+constexpr int RECUR_MAX_TOKENS = 24;
+bool use_recur(const Problem& p, int impl) {
+    if (impl == PF_IMPL_SIMT) return p.wu_builder == 0;
+    return p.auto_impl && p.L <= RECUR_MAX_TOKENS;
+}
 
 // what the kernels of `impl` carve up (the fp32 step sizes of PF_STEP_EXACT follow it)
 size_t kernel_workspace_need(const Problem& p, int impl) {
@@ -244,7 +253,7 @@ int forward_one(const pf_params* a, bool top) {
     bool own = false;
     if (ws) {
         if (a->workspace_bytes < need || ((uintptr_t)ws & 255u)) return PF_ERR_WORKSPACE;
-    } else if (need > 0) {
+    } else if (need > 0 && !use_recur(p, impl)) {
         PF_CUDA_TRY(cudaMallocAsync(&ws, need, p.stream));
         own = true;
     }
@@ -258,6 +267,11 @@ int forward_one(const pf_params* a, bool top) {
             if (own) cudaFreeAsync(ws, p.stream);
             return st;
         }
+    }
+    if (use_recur(p, impl)) {
+        st = recur_forward(p);
+        if (st == PF_OK && top) end_call();
+        return st;
     }
     if (top) {      // (the passes of a segmented call share the word: the first expired wait of any of them stays)
         cudaError_t e = cudaMemsetAsync(p.status, 0, sizeof(int), p.stream);

@@ -23,6 +23,7 @@ struct Problem {
     float* S_final;
     int in_dtype;
     int mode;           // PF_MODE_SUM (0) or PF_MODE_PRODUCT
+    bool exact;         // PF_STEP_EXACT
     const float* beta32;    // null, or fp32 step sizes [B,H,L,r] (device) that the kernels use in place of beta
     bool auto_impl;         // the caller left the choice of kernels to the library (PF_IMPL_AUTO)
     int wu_builder;         // fp32 SIMT path: 0 = triangular inverse then W = T'K, Uh = T'V; 1 = the wavefront system of
@@ -77,6 +78,9 @@ inline size_t beta32_bytes(const Problem& p) { return align_up((size_t)p.B * p.H
 // fp32 SIMT path (pf_simt.cu)
 size_t simt_workspace_bytes(const Problem& p);
 int simt_forward(const Problem& p, void* workspace);
+
+// the recurrence token by token in fp32 (pf_recur.cu); needs no workspace
+int recur_forward(const Problem& p);
 
 // tcgen05 path (pf_tc.cu)
 bool tc_supported(const Problem& p);
