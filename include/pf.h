@@ -251,6 +251,10 @@ int pf_last_wait_code(void);
  * returns.  For testing the reporting path above; it does not synchronise. */
 int pf_wait_selftest(int* status, int limit_us, void* stream);
 
+/* Calls that bring no workspace take it from a pool of the library's own (one per device), which keeps up to 96 MB of free
+ * pages between calls.  This gives the current device's free pages back; memory of calls still in flight stays. */
+int pf_release_workspaces(void);
+
 /* Number of kernels the last successful call on this host thread enqueued. */
 int pf_last_launch_count(void);
 

@@ -1,4 +1,7 @@
-"""ctypes binding of libpf.so: argument marshalling only -- every step runs in the CUDA kernels.
+"""Binding of libpf.so: argument marshalling only -- every step runs in the CUDA kernels.
+
+Ordinary calls are marshalled by the extension _pf_ext (csrc/pf_ext.cpp); ctypes serves the rest of the ABI, the rarer
+options, and the diagnosis of calls that the extension does not accept.
 
 The function names mirror the C ABI in include/pf.h.  Tensors are torch CUDA tensors (torch is
 used for device memory and streams only).  If the library is missing or cannot be loaded the
@@ -14,6 +17,7 @@ import torch
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_PKG, "libpf.so")
+EXT_PATH = os.path.join(_PKG, "_pf_ext.so")
 
 PF_DTYPE_BF16, PF_DTYPE_F32 = 0, 1
 PF_IMPL_AUTO, PF_IMPL_SIMT, PF_IMPL_TC = 0, 1, 2
@@ -33,6 +37,7 @@ EXPORTS = [
     "pf_profile_enable", "pf_profile_count", "pf_profile_read", "pf_tc_selftest",
     "pf_deltanet_fwd_f32_static", "pf_static_scratch_bytes", "pf_static_scratch_need",
     "pf_workspace_bytes_ex", "pf_select_chunk", "pf_read_status", "pf_last_wait_code", "pf_wait_selftest",
+    "pf_release_workspaces",
 ]
 
 
@@ -114,10 +119,30 @@ def lib() -> ctypes.CDLL:
         L.pf_last_wait_code.argtypes = []
         L.pf_wait_selftest.restype = ci
         L.pf_wait_selftest.argtypes = [vp, ci, vp]
+        L.pf_release_workspaces.restype = ci
+        L.pf_release_workspaces.argtypes = []
         L.pf_tc_selftest.restype = ci
         L.pf_tc_selftest.argtypes = [ci, vp, vp, vp, ci, vp]
         _lib = L
     return _lib
+
+
+_ext = None
+
+
+def _fast(q, k, v, beta, S0, chunk, O, S_final, stream, want_state, f32, impl=0, mode=0, step=0, where=""):
+    """The call through the extension: (O, S_final), or None if it is not an ordinary one."""
+    global _ext
+    if _ext is None:
+        if not os.path.exists(EXT_PATH):
+            raise ImportError(f"{EXT_PATH} not found: build it with `python -m paper_2504_00492_b200.build`")
+        from . import _pf_ext
+        _pf_ext.bind(ctypes.cast(lib().pf_deltanet_fwd_ex, ctypes.c_void_p).value)
+        _ext = _pf_ext.forward
+    out = _ext(q, k, v, beta, S0, chunk, O, S_final, stream, want_state, f32, impl, mode, step)
+    if out.__class__ is int:
+        raise PfError(out, where)
+    return out
 
 
 def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
@@ -160,6 +185,9 @@ def _stream(stream) -> int:
 
 def pf_deltanet_fwd(q, k, v, beta, S0, chunk: int, O=None, S_final=None, stream=None, want_state: bool = True):
     """bf16 q/k/v/beta -> (O fp32 [B,H,L,d_v], S_final fp32 [B,H,d_k,d_v] or None)."""
+    out = _fast(q, k, v, beta, S0, chunk, O, S_final, stream, want_state, False, where="pf_deltanet_fwd")
+    if out is not None:
+        return out
     B, H, L, d_k, d_v, r = _check_inputs(q, k, v, beta, S0, torch.bfloat16)
     O, S_final = _outputs(q, B, H, L, d_k, d_v, O, S_final, want_state)
     with torch.cuda.device(q.device):
@@ -172,6 +200,9 @@ def pf_deltanet_fwd(q, k, v, beta, S0, chunk: int, O=None, S_final=None, stream=
 
 def pf_deltanet_fwd_f32(q, k, v, beta, S0, chunk: int, O=None, S_final=None, stream=None, want_state: bool = True):
     """fp32 q/k/v/beta -> (O, S_final), all arithmetic fp32."""
+    out = _fast(q, k, v, beta, S0, chunk, O, S_final, stream, want_state, True, where="pf_deltanet_fwd_f32")
+    if out is not None:
+        return out
     B, H, L, d_k, d_v, r = _check_inputs(q, k, v, beta, S0, torch.float32)
     O, S_final = _outputs(q, B, H, L, d_k, d_v, O, S_final, want_state)
     with torch.cuda.device(q.device):
@@ -215,6 +246,13 @@ def pf_deltanet_fwd_ex(q, k, v, beta, S0, chunk: int, impl="auto", workspace: Op
     dtype = q.dtype
     if dtype not in (torch.bfloat16, torch.float32):
         raise TypeError("q/k/v/beta must be bf16 or fp32")
+    if workspace is None and status is None and not (segments or wu_builder or ring_depth):
+        out = _fast(q, k, v, beta, S0, chunk, O, S_final, stream, want_state, dtype == torch.float32,
+                    IMPL_BY_NAME[impl] if isinstance(impl, str) else int(impl),
+                    MODE_BY_NAME[mode] if isinstance(mode, str) else int(mode),
+                    STEP_BY_NAME[step] if isinstance(step, str) else int(step), where="pf_deltanet_fwd_ex")
+        if out is not None:
+            return out
     B, H, L, d_k, d_v, r = _check_inputs(q, k, v, beta, S0, dtype)
     O, S_final = _outputs(q, B, H, L, d_k, d_v, O, S_final, want_state)
     p = PfParams()
@@ -285,6 +323,13 @@ def pf_workspace_bytes(B, H, L, d_k, d_v, r, chunk, in_dtype=PF_DTYPE_BF16, impl
 def pf_select_impl(B, H, L, d_k, d_v, r, chunk, in_dtype=PF_DTYPE_BF16, impl="auto") -> int:
     impl = IMPL_BY_NAME[impl] if isinstance(impl, str) else int(impl)
     return int(lib().pf_select_impl(B, H, L, d_k, d_v, r, chunk, in_dtype, impl))
+
+
+def pf_release_workspaces() -> None:
+    """Gives back the free pages of the library's workspace pool on the current device."""
+    st = lib().pf_release_workspaces()
+    if st != 0:
+        raise PfError(st, "pf_release_workspaces")
 
 
 def pf_last_launch_count() -> int:

@@ -1,4 +1,5 @@
-"""Builds the CUDA library in-tree: paper_2504_00492_b200/libpf.so (sm_100a only)."""
+"""Builds in-tree: the CUDA library paper_2504_00492_b200/libpf.so (sm_100a only) and the extension _pf_ext.so through which
+the Python entry points call it."""
 from __future__ import annotations
 
 import glob
@@ -10,6 +11,8 @@ PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libpf.so")
+EXT_SRC = os.path.join(CSRC, "pf_ext.cpp")
+EXT = os.path.join(PKG, "_pf_ext.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -29,11 +32,35 @@ def _stale() -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def build_ext(force: bool = False) -> str:
+    """Compile the call path of the Python entry points against the installed torch's headers."""
+    deps = [EXT_SRC, os.path.join(ROOT, "include", "pf.h")]
+    if not force and os.path.exists(EXT) and all(os.path.getmtime(d) <= os.path.getmtime(EXT) for d in deps):
+        return EXT
+    import sysconfig
+
+    import torch
+    t = os.path.dirname(torch.__file__)
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    tmp = EXT + ".tmp%d" % os.getpid()
+    subprocess.run([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC",
+                    f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+                    "-I", os.path.join(ROOT, "include"), "-isystem", os.path.join(t, "include"),
+                    "-isystem", os.path.join(t, "include", "torch", "csrc", "api", "include"),
+                    "-isystem", sysconfig.get_paths()["include"], "-isystem", os.path.join(cuda, "include"),
+                    EXT_SRC, "-o", tmp, "-L", os.path.join(t, "lib"), "-ltorch_python", "-ltorch_cuda", "-ltorch_cpu",
+                    "-lc10_cuda", "-lc10"], check=True)
+    os.replace(tmp, EXT)
+    return EXT
+
+
 def build(force: bool = False, verbose: bool = False, extra_flags=(), out: str = None) -> str:
     """Compile every .cu under csrc/ and link libpf.so.  Returns the library path.
     extra_flags / out: a diagnostic build (e.g. ("-DPF_ENDS",)) into another file, objects kept apart."""
-    if out is None and not force and not _stale():
-        return LIB
+    if out is None:
+        build_ext(force)
+        if not force and not _stale():
+            return LIB
     nvcc = os.environ.get("NVCC", "nvcc")
     objs = []
     bdir = os.path.join(PKG, "_build" if out is None else "_build_diag")

@@ -72,6 +72,38 @@ int library_status_word(int** out) {
     return PF_OK;
 }
 
+// Workspaces of calls that bring none: a memory pool of the library's own, one per device.  The device's default pool gives
+// its pages back at every synchronisation, and mapping them anew cost the next call 0.4 ms (42 MB) to 4 ms (a two-launch
+// workspace); this one keeps up to WORKSPACE_KEEP bytes of free pages (the rings of the single-launch kernel always fit)
+// until pf_release_workspaces.  Allocation and free stay ordered on the caller's stream.
+constexpr uint64_t WORKSPACE_KEEP = 96ull << 20;
+std::mutex g_pool_mu;
+cudaMemPool_t g_pool[kMaxDevices] = {};
+
+int workspace_alloc(void** ws, size_t bytes, cudaStream_t stream) {
+    int dev = 0;
+    PF_CUDA_TRY(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= kMaxDevices) return PF_ERR_UNSUPPORTED;
+    cudaMemPool_t pool;
+    {
+        std::lock_guard<std::mutex> lock(g_pool_mu);
+        if (!g_pool[dev]) {
+            cudaMemPoolProps props{};
+            props.allocType = cudaMemAllocationTypePinned;
+            props.location.type = cudaMemLocationTypeDevice;
+            props.location.id = dev;
+            cudaMemPool_t made;
+            PF_CUDA_TRY(cudaMemPoolCreate(&made, &props));
+            uint64_t keep = WORKSPACE_KEEP;
+            PF_CUDA_TRY(cudaMemPoolSetAttribute(made, cudaMemPoolAttrReleaseThreshold, &keep));
+            g_pool[dev] = made;
+        }
+        pool = g_pool[dev];
+    }
+    PF_CUDA_TRY(cudaMallocFromPoolAsync(ws, bytes, pool, stream));
+    return PF_OK;
+}
+
 // One warp waits for a flag that nothing sets, with the bounded-wait routine of the kernels and a short limit.
 __global__ void wait_selftest_kernel(int* status, const int* flag, long long limit_cycles) {
     if (threadIdx.x == 0) tc::flag_wait_ge_limit(flag, 1, status, 900, limit_cycles);
@@ -218,11 +250,15 @@ int check_call(const pf_params* a) {
     if (overlaps(a->O, o_bytes, a->q, th * a->d_k * es) || overlaps(a->O, o_bytes, a->k, th * a->r * a->d_k * es) ||
         overlaps(a->O, o_bytes, a->v, th * a->r * a->d_v * es) || overlaps(a->O, o_bytes, a->beta, th * a->r * es))
         return PF_ERR_INVALID;
+    static std::atomic<uint64_t> arch_ok{0};       // (one bit per device ordinal)
     int dev = 0;
     PF_CUDA_TRY(cudaGetDevice(&dev));
+    const uint64_t bit = dev < 64 ? 1ull << dev : 0;
+    if (arch_ok.load(std::memory_order_relaxed) & bit) return PF_OK;
     int major = 0;
     PF_CUDA_TRY(cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev));
     if (major != 10) return PF_ERR_ARCH;
+    arch_ok.fetch_or(bit, std::memory_order_relaxed);
     return PF_OK;
 }
 
@@ -254,7 +290,8 @@ int forward_one(const pf_params* a, bool top) {
     if (ws) {
         if (a->workspace_bytes < need || ((uintptr_t)ws & 255u)) return PF_ERR_WORKSPACE;
     } else if (need > 0 && !use_recur(p, impl)) {
-        PF_CUDA_TRY(cudaMallocAsync(&ws, need, p.stream));
+        st = workspace_alloc(&ws, need, p.stream);
+        if (st != PF_OK) return st;
         own = true;
     }
     if (top) begin_call();
@@ -572,7 +609,8 @@ int forward_segmented(const pf_params* a, int S) {
     if (ws) {
         if (a->workspace_bytes < need || ((uintptr_t)ws & 255u)) return PF_ERR_WORKSPACE;
     } else {
-        PF_CUDA_TRY(cudaMallocAsync(&ws, need, stream));
+        st = workspace_alloc(&ws, need, stream);
+        if (st != PF_OK) return st;
         own = true;
     }
     const size_t ab = seg_array_bytes(a, S);
@@ -781,6 +819,15 @@ int pf_wait_selftest(int* status, int limit_us, void* stream) {
     pf::wait_selftest_kernel<<<1, 32, 0, (cudaStream_t)stream>>>(w, zero_flag[dev], (long long)limit_us * (khz / 1000));
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return pf::record_cuda_error(e, "wait_selftest_kernel");
+    return PF_OK;
+}
+
+int pf_release_workspaces(void) {
+    int dev = 0;
+    PF_CUDA_TRY(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= pf::kMaxDevices) return PF_ERR_UNSUPPORTED;
+    std::lock_guard<std::mutex> lock(pf::g_pool_mu);
+    if (pf::g_pool[dev]) PF_CUDA_TRY(cudaMemPoolTrimTo(pf::g_pool[dev], 0));
     return PF_OK;
 }
 

@@ -7,6 +7,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "pf.h"
 
 namespace pf {
@@ -70,6 +72,17 @@ void end_call();
 // with CUDA events on its stream; otherwise they do nothing.
 void prof_begin(const char* name, cudaStream_t stream);
 void prof_end(cudaStream_t stream);
+
+// Opts a kernel in to `bytes` of dynamic shared memory, once per device (`done`: one bit per device ordinal).
+inline int allow_smem(std::atomic<uint64_t>& done, const void* fn, int bytes) {
+    int dev = 0;
+    PF_CUDA_TRY(cudaGetDevice(&dev));
+    const uint64_t bit = dev < 64 ? 1ull << dev : 0;
+    if (done.load(std::memory_order_acquire) & bit) return PF_OK;
+    PF_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    done.fetch_or(bit, std::memory_order_release);
+    return PF_OK;
+}
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 // room at the end of every workspace for the fp32 step sizes of PF_STEP_EXACT

@@ -312,7 +312,13 @@ int recur_forward(const Problem& p) {
     const void* fn = f32 ? recur_fn<float>(p.d_k, tb, rg, p.r / rg) : recur_fn<__nv_bfloat16>(p.d_k, tb, rg, p.r / rg);
     const long long grid = (long long)p.B * p.H * (p.d_v / RJ);
     if (grid > 0x7fffffffLL) return PF_ERR_UNSUPPORTED;
-    if (smem > 48 * 1024) PF_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    // (opted in once per kernel, to what its longest stages need)
+    static std::atomic<uint64_t> opted_in[2][2][2][16];
+    if (smem > 48 * 1024) {
+        const int st = allow_smem(opted_in[f32][p.d_k == 128][tb == 4][(rg - 1) * 4 + p.r - 1], fn,
+                                  R_STAGES * recur_stage_bytes(16, p.r, p.d_k, f32 ? 4 : 2) + 4 * 128 * 4);
+        if (st != PF_OK) return st;
+    }
     void* args[] = {(void*)&p.q, (void*)&p.k, (void*)&p.v, (void*)&p.beta, (void*)&p.S0, (void*)&p.O, (void*)&p.S_final, (void*)&p.status, (void*)&g};
     prof_begin("recur", p.stream);
     PF_CUDA_TRY(cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(160), args, (size_t)smem, p.stream));
