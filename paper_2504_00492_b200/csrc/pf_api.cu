@@ -176,10 +176,6 @@ int select_impl(Problem& p, int impl) {
     }
 }
 
-// PF_IMPL_TC: the single launch where it supports the shape; under PF_IMPL_AUTO only where it is also the faster of
-// the two tensor-core forms (an explicit PF_IMPL_TC takes it whenever it can run).
-bool use_fused(const Problem& p) { return fused_supported(p) && (!p.auto_impl || fused_preferred(p)); }
-
 // Calls that the token-by-token kernel takes: those on the fp32 path (unless the Theorem 3.3 builder is asked for), and
 // bf16 calls of so few tokens that a chunk would be mostly padding (one token of 128 sequences: 12 us against 56).
 constexpr int RECUR_MAX_TOKENS = 24;
@@ -188,8 +184,24 @@ bool use_recur(const Problem& p, int impl) {
     return p.auto_impl && p.L <= RECUR_MAX_TOKENS;
 }
 
+// Which of the tensor-core kernels.  PF_IMPL_AUTO: the chain kernel, except where the single-launch tcgen05 kernel can run
+// and is the faster one (d = 128, few enough sequences that most SMs build flows, and enough chunks that its first flow's
+// latency does not matter; both estimates are next to their kernels).  An explicit PF_IMPL_TC takes the single launch
+// whenever it can run, and the two-launch form otherwise.
+bool use_fused(const Problem& p) {
+    return fused_supported(p) && (!p.auto_impl || !chain_supported(p) || fused_estimate_us(p) < chain_estimate_us(p));
+}
+bool in_window(const Problem& p) {
+    const long long nseq = (long long)p.B * p.H, sms = sm_count();
+    return p.d_k == 128 && p.d_v == 128 && nseq * 10 > sms * 7 && nseq <= sms - 8;
+}
+bool use_chain(const Problem& p, int impl) {
+    return impl == PF_IMPL_TC && p.auto_impl && !use_recur(p, impl) && chain_supported(p) && !use_fused(p) && !in_window(p);
+}
+
 // what the kernels of `impl` carve up (the fp32 step sizes of PF_STEP_EXACT follow it)
 size_t kernel_workspace_need(const Problem& p, int impl) {
+    if (use_chain(p, impl)) return 1024;       // (word 0 of a caller's workspace is the status word)
     if (impl == PF_IMPL_TC) return use_fused(p) ? fused_workspace_bytes(p) : tc_workspace_bytes(p);
     if (impl == PF_IMPL_TC_SPLIT) return tc_workspace_bytes(p);
     if (impl == PF_IMPL_TC_REFFLOW) return tc_refflow_workspace_bytes(p);
@@ -289,7 +301,7 @@ int forward_one(const pf_params* a, bool top) {
     bool own = false;
     if (ws) {
         if (a->workspace_bytes < need || ((uintptr_t)ws & 255u)) return PF_ERR_WORKSPACE;
-    } else if (need > 0 && !use_recur(p, impl)) {
+    } else if (need > 0 && !use_recur(p, impl) && !use_chain(p, impl)) {
         st = workspace_alloc(&ws, need, p.stream);
         if (st != PF_OK) return st;
         own = true;
@@ -305,8 +317,8 @@ int forward_one(const pf_params* a, bool top) {
             return st;
         }
     }
-    if (use_recur(p, impl)) {
-        st = recur_forward(p);
+    if (use_recur(p, impl) || use_chain(p, impl)) {
+        st = use_recur(p, impl) ? recur_forward(p) : chain_forward(p);
         if (st == PF_OK && top) end_call();
         return st;
     }

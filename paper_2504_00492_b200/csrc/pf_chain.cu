@@ -1,0 +1,724 @@
+// chain: the chunk form in ONE kernel without any hand-off through memory, on warp-level tensor-core products.
+//
+// A sequence is walked in blocks of up to 64 rows (64 / r tokens).  From Theorem 3.2, with rows m, S the state before the block:
+//     T  = (I + Mstrict (.) (diag(beta) K K^T))^{-1} diag(beta)                      (does not depend on S)
+//     P  = (Q K^T) (.) Mincl                                                         (does not depend on S)
+//     U' = T (V - K S^T),       O = Q S^T + P U',       S <- S + U'^T K
+// i.e. W and Uh are never formed: T is applied to V - K S^T instead.  Of the block's operations only three products depend on
+// S one after another, and their operands fit the register layout of mma.sync: with S held as [j][i] accumulators, S K^T,
+// then T applied, then the update are each "registers times shared memory", and the accumulator of one product, packed
+// to fp16, is the A operand of the next.  So a warp carries 16 rows j of S through the whole sequence without exchanging
+// anything with other warps: the serial step has no barrier, no shared-memory round trip and no tensor-memory latency.
+//
+//   chain warps   16 rows j of S each (IS = 2: two warps share the 16 rows, each holds half of the columns i; they add
+//                 their halves of S K^T and Q S^T through shared memory once per block)
+//   prep warps    teams of four: K, Q -> fp16 in place, G = K K^T, the inverse, P; a few blocks ahead
+// A stage of shared memory holds what the chain needs of one block: K, Q (fp16), T, P (fp16), V (bf16 as it came).
+//
+// What bounds it: the mma.sync pipe is busy for about half of the time when every SM has a CTA (d = 128, r = 2: 3.7 k of 7.2 k
+// cycles per block of 32 tokens, 128 columns per CTA), the rest is the latency of the chain's dependent products.  Measured
+// (kernel time, against the tcgen05 kernels in two launches or one): 256 sequences of 1024 tokens, d = 128, r = 2: 0.25 ms
+// against 0.63; 128 sequences of 4096, d = 64, r = 4: 0.38 against 0.93; 48 sequences of 1999, 64 x 128, r = 3: 0.165
+// against 0.33.  Where the tcgen05 kernel in one launch has few sequences and enough SMs to build flows ahead (d = 128), it
+// is the faster one: see chain_preferred.
+//
+// The inverse: warp i of a team owns rows 16 i .. 16 i + 15.  D_i = (I + A_ii)^{-1} by its Neumann product and
+// E_ij = D_i A_ij in registers, then X_ij = -sum_k E_ik X_kj row block by row block (three exchanges through shared memory).
+#include <atomic>
+
+#include "pf_common.cuh"
+#include "pf_tc.cuh"
+#include "pf_tc_prims.cuh"
+
+namespace pf {
+
+using namespace tc;
+
+namespace {
+
+constexpr int NB = 64;               // rows per block
+
+struct ChainMaps {
+    CUtensorMap q, k, v;
+};
+
+struct ChainGeo {
+    int L, d_v, nblk;
+    int rm;             // strict-mask group size (Problem::mask_group)
+    int exact;          // PF_STEP_EXACT
+};
+
+__device__ __forceinline__ uint32_t movmatrix(uint32_t x) {
+    uint32_t y;
+    asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(y) : "r"(x));
+    return y;
+}
+// (a predicated store, not a branch: a branch would keep the compiler from moving anything across it)
+__device__ __forceinline__ void store2_if(float* p, float x, float y, bool pred) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\t@p st.global.v2.f32 [%0], {%1, %2};\n\t}" ::"l"(p), "f"(x), "f"(y),
+                 "r"((unsigned)pred));
+}
+// eight bf16 -> eight fp16 (sign: 0x80008000 to negate them)
+__device__ __forceinline__ uint4 bf16_to_half8(uint4 x, uint32_t sign) {
+    uint32_t* w = (uint32_t*)&x;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) w[i] = pack_h2(__uint_as_float(w[i] << 16), __uint_as_float(w[i] & 0xFFFF0000u)) ^ sign;
+    return x;
+}
+
+template <int DK, int R, int JS>
+struct ChainSmem {
+    static constexpr int C = NB / R;                              // tokens per block
+    static constexpr int CP = (C + 15) / 16 * 16;                 // ... in tiles of 16
+    static constexpr int k_bytes = NB * DK * 2, q_bytes = CP * DK * 2;
+    static constexpr int t_bytes = NB * 128, p_bytes = CP * 128, v_bytes = NB * JS * 2;
+    static constexpr int k_off = 0, q_off = k_off + k_bytes, t_off = q_off + q_bytes, p_off = t_off + t_bytes, v_off = p_off + p_bytes;
+    static constexpr int stage = v_off + v_bytes;
+    static constexpr int tx_bytes = k_bytes + C * DK * 2 + v_bytes;         // what the copies of a block bring
+};
+
+template <int DK, int R, int JS, int IS, int TEAMS, int NS>
+struct ChainCfg {
+    using SM = ChainSmem<DK, R, JS>;
+    static constexpr int NCW = JS / 16 * IS;                      // chain warps
+    static constexpr int threads = 32 * NCW + 128 * TEAMS;
+    static constexpr int xs_off = NS * SM::stage;                 // per team: X (unscaled) while it is being formed
+    static constexpr int beta_off = xs_off + TEAMS * NB * 128;    // per team: 64 step sizes
+    // IS = 2: partial sums on their way to the other warp of the pair, [pair][parity][warp][thread-linear 16-byte pieces]
+    static constexpr int x_piece = 8 + SM::CP / 16;               // 16-byte pieces per thread: 32 of S K^T, 4 per 16 tokens of Q S^T
+    static constexpr int ex_off = beta_off + TEAMS * 256;
+    static constexpr int ex_bytes = IS == 2 ? (JS / 16) * 2 * 2 * x_piece * 512 : 0;
+    static constexpr int total = ex_off + ex_bytes;
+};
+// as many stages as fit, up to six
+template <int DK, int R, int JS, int IS, int TEAMS>
+constexpr int chain_stages() {
+    constexpr int left = 226 * 1024 - ChainCfg<DK, R, JS, IS, TEAMS, 0>::total;
+    constexpr int n = left / ChainSmem<DK, R, JS>::stage;
+    return n < 6 ? n : 6;
+}
+
+// K, Q and V of block b into stage b mod NS (one thread); rows past the sequence arrive as zeros
+template <int DK, int R, int JS, int NS>
+__device__ __forceinline__ void load_block(const ChainMaps& maps, uint8_t* smem, uint64_t* land, int b, int seq, int j0) {
+    using SM = ChainSmem<DK, R, JS>;
+    const int st = b % NS;
+    uint8_t* sg = smem + st * SM::stage;
+    mbar_expect_tx(&land[st], SM::tx_bytes);
+    tma_load_4d(sg + SM::k_off, &maps.k, 0, b * SM::C * R, 0, seq, &land[st]);
+    // (r = 3: a block's 21 tokens sit in slabs of 32 rows, one copy each)
+    constexpr int QS = SM::CP == SM::C ? 1 : DK / 64;
+#pragma unroll
+    for (int h = 0; h < QS; ++h) tma_load_4d(sg + SM::q_off + h * (SM::CP * 128), &maps.q, 0, b * SM::C, h, seq, &land[st]);
+    tma_load_4d(sg + SM::v_off, &maps.v, 0, b * SM::C * R, j0 / (JS < 64 ? JS : 64), seq, &land[st]);
+}
+// offset of the 16-byte piece c8 (= column / 8) of row `row` of the V tile: 128-byte rows (JS >= 64) or 64-byte rows
+template <int JS>
+__device__ __forceinline__ uint32_t v_piece(int row, int c8) {
+    if (JS >= 64) return (uint32_t)((c8 >> 3) * (NB * 128) + row * 128 + (((c8 & 7) ^ (row & 7)) << 4));
+    return (uint32_t)(row * 64 + ((c8 ^ ((row >> 1) & 3)) << 4));
+}
+
+// byte offsets of a lane's row address for ldmatrix.x4 within a slab of 128-byte swizzled rows; the K-step kk of 16 columns
+// is at off ^ (kk << 5), everything else is added
+__device__ __forceinline__ uint32_t lane_off(int row, int half) { return (uint32_t)row * 128u + (uint32_t)((half ^ (row & 7)) << 4); }
+
+// Which warp of a team forms block (16 tokens tt, 16 rows nb) of P: warp w has w + 1 blocks of G, so that all have about as
+// many.  Blocks whose rows are all later than the tile's tokens are nobody's.
+template <int R>
+__host__ __device__ constexpr int p_owner(int tt, int nb) {
+    if (nb >= (tt + 1) * R) return -1;
+    if (R == 1) return 3 - tt;
+    if (R == 2) return tt == 0 ? nb + 1 : nb < 3 ? 0 : 1;
+    if (R == 3) return tt == 0 ? (nb < 2 ? 1 : 2) : nb < 3 ? 0 : 3;
+    return nb < 2 ? 0 : nb - 1;
+}
+// G[rows of block W][row blocks 0 .. W] into ga, and warp W's blocks of -P = (-Q K^T) (.) Mincl, negated back, into shared
+// memory.  All blocks advance together along the contraction, so that eight to ten accumulators are independent and a key
+// fragment serves both.
+template <int DK, int R, int CP, int W>
+__device__ __forceinline__ void gram_blocks(uint32_t k_b, uint32_t q_b, uint8_t* sp, uint32_t offA, uint32_t offN, int gq, int t4,
+                                            float (&ga)[4][2][4]) {
+    constexpr int KT = DK / 16, TT = CP / 16;
+    float pc[TT][4][2][4];
+#pragma unroll
+    for (int kk = 0; kk < KT; ++kk) {
+        uint32_t ka[4], qa[TT][4];
+        ldmatrix_x4(ka, k_b + (offA ^ ((kk & 3) << 5)) + W * 2048 + (kk >> 2) * (NB * 128));
+#pragma unroll
+        for (int tt = 0; tt < TT; ++tt)
+            if (p_owner<R>(tt, 0) == W || p_owner<R>(tt, 1) == W || p_owner<R>(tt, 2) == W || p_owner<R>(tt, 3) == W)
+                ldmatrix_x4(qa[tt], q_b + (offA ^ ((kk & 3) << 5)) + tt * 2048 + (kk >> 2) * (CP * 128));
+#pragma unroll
+        for (int nb = 0; nb < 4; ++nb) {
+            bool used = nb <= W;
+#pragma unroll
+            for (int tt = 0; tt < TT; ++tt) used = used || p_owner<R>(tt, nb) == W;
+            if (!used) continue;
+            uint32_t x[4];
+            ldmatrix_x4(x, k_b + (offN ^ ((kk & 3) << 5)) + nb * 2048 + (kk >> 2) * (NB * 128));
+            if (nb <= W) {
+                mma_acc(ga[nb][0], ka, x[0], x[1], kk > 0);
+                mma_acc(ga[nb][1], ka, x[2], x[3], kk > 0);
+            }
+#pragma unroll
+            for (int tt = 0; tt < TT; ++tt)
+                if (p_owner<R>(tt, nb) == W) {
+                    mma_acc(pc[tt][nb][0], qa[tt], x[0], x[1], kk > 0);
+                    mma_acc(pc[tt][nb][1], qa[tt], x[2], x[3], kk > 0);
+                }
+        }
+    }
+#pragma unroll
+    for (int tt = 0; tt < TT; ++tt)
+#pragma unroll
+        for (int nb = 0; nb < 4; ++nb) {
+            if (p_owner<R>(tt, nb) != W) continue;
+            const int ta = 16 * tt + gq, la = (ta + 1) * R, lb = (ta + 9) * R;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int m = 16 * nb + 8 * h + 2 * t4;
+                const bool all = 16 * nb + 15 < (16 * tt + 1) * R;        // (every row is visible to every token of the block)
+                *(uint32_t*)(sp + chunk_off(ta, 2 * nb + h, CP) + 4 * t4) =
+                    pack_h2(all || m < la ? -pc[tt][nb][h][0] : 0.f, all || m + 1 < la ? -pc[tt][nb][h][1] : 0.f);
+                *(uint32_t*)(sp + chunk_off(ta + 8, 2 * nb + h, CP) + 4 * t4) =
+                    pack_h2(all || m < lb ? -pc[tt][nb][h][2] : 0.f, all || m + 1 < lb ? -pc[tt][nb][h][3] : 0.f);
+            }
+        }
+}
+
+// ---------------------------------------------------------------------------------------------------------------------
+// prep team: blocks b = team, team + TEAMS, ...
+// ---------------------------------------------------------------------------------------------------------------------
+template <int DK, int R, int JS, int IS, int TEAMS, int NS>
+__device__ __forceinline__ void prep_role(const ChainGeo& g, const __nv_bfloat16* __restrict__ beta, int* err, uint8_t* smem,
+                                          uint64_t* land, uint64_t* full, long long seq, int team, int tid) {
+    using CFG = ChainCfg<DK, R, JS, IS, TEAMS, NS>;
+    using SM = ChainSmem<DK, R, JS>;
+    constexpr int C = SM::C, CP = SM::CP;
+    const int w = tid >> 5, lane = tid & 31, gq = lane >> 2, t4 = lane & 3;
+    const int L = g.L;
+    const int bar_id = 1 + team;
+    uint8_t* xs = smem + CFG::xs_off + team * NB * 128;
+    const uint32_t xs_b = smem_u32(xs);
+    float* sBeta = (float*)(smem + CFG::beta_off + team * 256);
+    const uint32_t offA = lane_off(lane & 15, lane >> 4);
+    const uint32_t offN = lane_off((lane & 7) + ((lane >> 4) << 3), (lane >> 3) & 1);
+    const uint32_t offT = lane_off((lane & 7) + (((lane >> 3) & 1) << 3), lane >> 4);
+    const __nv_bfloat16* bs = beta + seq * L * R;
+    auto read_beta = [&](int b) {                                 // rows past the block or the sequence have step size zero
+        return tid < min(C, L - b * C) * R ? __bfloat162float(bs[(long long)b * C * R + tid]) : 0.f;
+    };
+    float breg = team < g.nblk ? read_beta(team) : 0.f;
+#pragma unroll 1
+    for (int b = team; b < g.nblk; b += TEAMS) {
+        const int st = b % NS;
+        uint8_t* sg = smem + st * SM::stage;
+        const uint32_t k_b = smem_u32(sg + SM::k_off), q_b = smem_u32(sg + SM::q_off);
+        // (a failed wait must not strand the others at a barrier: the next one carries the outcome)
+        const bool ok = mbar_wait_clk(&land[st], (uint32_t)(b / NS) & 1, err, 311);
+        // ---- K, Q: bf16 -> fp16 in place (elementwise, so the swizzled layout is untouched), several pieces per round, so that
+        //      their loads are in flight together; Q as -Q: the chain multiplies it with -S
+        {
+            uint4* p = (uint4*)(sg + SM::k_off) + tid;
+            constexpr int PIECES = (SM::k_bytes + SM::q_bytes) / 2048, ROUND = 8;
+#pragma unroll
+            for (int e0 = 0; e0 < PIECES; e0 += ROUND) {
+                uint4 x[ROUND];
+#pragma unroll
+                for (int e = 0; e < ROUND; ++e)
+                    if (e0 + e < PIECES) x[e] = p[(e0 + e) * 128];
+#pragma unroll
+                for (int e = 0; e < ROUND; ++e)
+                    if (e0 + e < PIECES) p[(e0 + e) * 128] = bf16_to_half8(x[e], (e0 + e) * 2048 < SM::k_bytes ? 0u : 0x80008000u);
+            }
+        }
+        fence_async_smem();                                       // (the stage's next copy is ordered after these writes)
+        if (tid < NB) sBeta[tid] = breg;
+        if (b + TEAMS < g.nblk) breg = read_beta(b + TEAMS);
+        if (!named_bar_and(bar_id, 128, ok)) return;
+
+        // ---- G (row block w) and this warp's blocks of P
+        float ga[4][2][4];
+        {
+            uint8_t* sp = sg + SM::p_off;
+            if (w == 0) gram_blocks<DK, R, CP, 0>(k_b, q_b, sp, offA, offN, gq, t4, ga);
+            else if (w == 1) gram_blocks<DK, R, CP, 1>(k_b, q_b, sp, offA, offN, gq, t4, ga);
+            else if (w == 2) gram_blocks<DK, R, CP, 2>(k_b, q_b, sp, offA, offN, gq, t4, ga);
+            else gram_blocks<DK, R, CP, 3>(k_b, q_b, sp, offA, offN, gq, t4, ga);
+        }
+        if (g.exact) {
+            // |k|^2 is the diagonal of G; beta' = (1 - e^{-beta |k|^2}) / |k|^2
+#pragma unroll
+            for (int nb = 0; nb < 4; ++nb)
+                if (nb == w && (gq >> 1) == t4) {
+                    const float n0 = (gq & 1) ? ga[nb][0][1] : ga[nb][0][0], n1 = (gq & 1) ? ga[nb][1][3] : ga[nb][1][2];
+                    const int m = 16 * w + gq;
+                    if (n0 > 0.f) sBeta[m] = -expm1f(-sBeta[m] * n0) / n0;
+                    if (n1 > 0.f) sBeta[m + 8] = -expm1f(-sBeta[m + 8] * n1) / n1;
+                }
+            __syncwarp();
+        }
+        // ---- A = Mstrict (.) (diag(beta) G) as A-operand fragments
+        uint32_t af[4][4];
+        {
+            const int m0 = 16 * w + gq, m1 = m0 + 8;
+            const float b0 = sBeta[m0], b1 = sBeta[m1];
+            const int lim0 = m0 / g.rm * g.rm, lim1 = m1 / g.rm * g.rm;
+#pragma unroll
+            for (int nb = 0; nb < 4; ++nb)
+                if (nb <= w) {
+                    // (with groups of three rows the edge also cuts into the block to the left of the diagonal one)
+                    const bool edge = nb == w || (R == 3 && nb + 1 == w);
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) {
+                            const int c = 16 * nb + 8 * h + 2 * t4 + e;
+                            ga[nb][h][e] = !edge || c < lim0 ? b0 * ga[nb][h][e] : 0.f;
+                            ga[nb][h][2 + e] = !edge || c < lim1 ? b1 * ga[nb][h][2 + e] : 0.f;
+                        }
+                    frag_pack(af[nb], ga[nb]);
+                }
+        }
+        // ---- D = (I + A_ww)^{-1} (Neumann product, A nilpotent), E_j = D A_wj
+        uint32_t df[4], ef[3][4];
+        float dd[2][4];
+        {
+            uint32_t a[4], at[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) a[e] = w == 0 ? af[0][e] : w == 1 ? af[1][e] : w == 2 ? af[2][e] : af[3][e];
+            at[0] = movmatrix(a[0]); at[1] = movmatrix(a[2]); at[2] = movmatrix(a[1]); at[3] = movmatrix(a[3]);
+            neumann16(dd, a, at, lane, g.rm == 1);
+            frag_pack(df, dd);
+        }
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+            if (j < w) {
+                float c[2][4];
+                frag_zero(c);
+                mma_16816(c[0], df, movmatrix(af[j][0]), movmatrix(af[j][1]));
+                mma_16816(c[1], df, movmatrix(af[j][2]), movmatrix(af[j][3]));
+                frag_pack(ef[j], c);
+            }
+        // ---- X_w,j row block by row block; X is left unscaled in the scratch for the row blocks below, T = X diag(beta) in the stage
+        auto put_x = [&](int j, const uint32_t (&f)[4]) {         // (f: packed accumulator fragment)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                *(uint32_t*)(xs + chunk_off(16 * w + gq, 2 * j + h, NB) + 4 * t4) = f[2 * h];
+                *(uint32_t*)(xs + chunk_off(16 * w + gq + 8, 2 * j + h, NB) + 4 * t4) = f[2 * h + 1];
+            }
+        };
+        auto put_t = [&](int j, const float (&x)[2][4]) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float2 bb = *(const float2*)(sBeta + 16 * j + 8 * h + 2 * t4);
+                *(uint32_t*)(sg + SM::t_off + chunk_off(16 * w + gq, 2 * j + h, NB) + 4 * t4) = pack_h2(x[h][0] * bb.x, x[h][1] * bb.y);
+                *(uint32_t*)(sg + SM::t_off + chunk_off(16 * w + gq + 8, 2 * j + h, NB) + 4 * t4) = pack_h2(x[h][2] * bb.x, x[h][3] * bb.y);
+            }
+        };
+        float xa[3][2][4];
+        auto add_ex = [&](int k2, int j) {                        // xa[j] += E_k2 X_k2,j
+            uint32_t x[4];
+            ldmatrix_x4_trans(x, xs_b + (offT ^ (j << 5)) + k2 * 2048);
+            mma_16816(xa[j][0], ef[k2], x[0], x[1]);
+            mma_16816(xa[j][1], ef[k2], x[2], x[3]);
+        };
+        auto finish = [&](int j, bool later) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) xa[j][h][e] = -xa[j][h][e];
+            if (later) {
+                uint32_t f[4];
+                frag_pack(f, xa[j]);
+                put_x(j, f);
+            }
+            put_t(j, xa[j]);
+        };
+#pragma unroll
+        for (int j = 0; j < 3; ++j) frag_zero(xa[j]);
+        put_x(w, df);
+        named_bar(bar_id, 128);
+        put_t(w, dd);                                             // (after the barrier: beta' of the exact step is complete)
+        if (w == 1) {
+            add_ex(0, 0);
+            finish(0, true);
+        } else if (w == 2) {
+            add_ex(1, 1);
+            finish(1, true);
+            add_ex(0, 0);
+        } else if (w == 3) {
+            add_ex(2, 2);
+            finish(2, false);
+            add_ex(1, 1);
+            add_ex(0, 0);
+        }
+        named_bar(bar_id, 128);
+        if (w == 2) {
+            add_ex(1, 0);
+            finish(0, true);
+        } else if (w == 3) {
+            add_ex(1, 0);
+            add_ex(2, 1);
+            finish(1, false);
+        }
+        named_bar(bar_id, 128);
+        if (w == 3) {
+            add_ex(2, 0);
+            finish(0, false);
+        }
+        mbar_arrive(&full[st]);
+    }
+}
+
+// ---------------------------------------------------------------------------------------------------------------------
+// chain warp: rows j of the 16-column group `grp` of the CTA's JS columns, columns i of half `hi` (IS = 2)
+// ---------------------------------------------------------------------------------------------------------------------
+template <int DK, int R, int JS, int IS, int TEAMS, int NS>
+__device__ __forceinline__ void chain_role(const ChainMaps& maps, const ChainGeo& g, const float* __restrict__ S0, float* __restrict__ O,
+                                           float* __restrict__ S_final, int* err, uint8_t* smem, uint64_t* land, uint64_t* full,
+                                           uint64_t* empty, long long seq, int j0, int warp, int lane) {
+    using CFG = ChainCfg<DK, R, JS, IS, TEAMS, NS>;
+    using SM = ChainSmem<DK, R, JS>;
+    constexpr int C = SM::C, CP = SM::CP, TT = CP / 16;
+    constexpr int DI = DK / IS, KT = DI / 16;                     // columns i of this warp, in K-steps of 16
+    const int grp = warp / IS, hi = warp % IS;
+    const int gq = lane >> 2, t4 = lane & 3;
+    const uint32_t offA = lane_off(lane & 15, lane >> 4);
+    const uint32_t offN = lane_off((lane & 7) + ((lane >> 4) << 3), (lane >> 3) & 1);
+    const uint32_t offT = lane_off((lane & 7) + (((lane >> 3) & 1) << 3), lane >> 4);
+    // V, read transposed: matrix id = lane >> 3: rows + 8 (id >> 1), columns 8 (id & 1)
+    const uint32_t offV = v_piece<JS>((lane & 7) + ((lane >> 4) << 3), 2 * grp + ((lane >> 3) & 1));
+    constexpr uint32_t V_STEP = 16 * (JS >= 64 ? 128 : 64);
+    const uint32_t smem_b = smem_u32(smem);
+    // K-step kk of this warp = step hi KT + kk of the row: slab and 32-byte position within it
+    auto kpos = [&](int kk, int slab_bytes) { return (uint32_t)((hi * KT + kk) >> 2) * (uint32_t)slab_bytes; };
+    auto kxor = [&](int kk) { return (uint32_t)(((hi * KT + kk) & 3) << 5); };
+
+    float S[2 * KT][4];                                           // [8 columns i][c]: rows j = gq, gq + 8, columns 2 t4, 2 t4 + 1
+    const int jr = j0 + 16 * grp + gq, i0 = hi * DI + 2 * t4;
+#pragma unroll
+    for (int n = 0; n < 2 * KT; ++n)
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            S[n][e] = S0 ? S0[(seq * DK + i0 + 8 * n + (e & 1)) * g.d_v + jr + 8 * (e >> 1)] : 0.f;
+    float* ob = O + seq * (long long)g.L * g.d_v + j0 + 16 * grp + 2 * t4 + (IS == 2 ? 8 * hi : 0);     // O of the current block
+
+    // IS = 2: what this warp keeps of O of the block before (8 of the 16 columns j), without the other warp's part of Q S^T
+    float ok8[TT][4];
+    int Cv_prev = 0;
+    uint8_t* exw = smem + CFG::ex_off + grp * (4 * CFG::x_piece * 512) + lane * 16;
+    auto store8 = [&](const float4* other) {                      // ob points one block further than what is stored
+#pragma unroll
+        for (int tt = 0; tt < TT; ++tt) {
+            const float4 x = other[(8 + tt) * 32];
+            const int t = 16 * tt + gq;
+            float* o0 = ob + (long long)(t - C) * g.d_v;
+            store2_if(o0, ok8[tt][0] + x.x, ok8[tt][1] + x.y, t < Cv_prev);
+            store2_if(o0 + 8ll * g.d_v, ok8[tt][2] + x.z, ok8[tt][3] + x.w, t + 8 < Cv_prev);
+        }
+    };
+    if (IS == 2)
+#pragma unroll
+        for (int tt = 0; tt < TT; ++tt) {
+            ((float4*)(exw + (2 + hi) * (CFG::x_piece * 512)))[(8 + tt) * 32] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) ok8[tt][e] = 0.f;
+        }
+
+    int st = 0, phase = 0, st_prev = 0, ph_prev = 0;
+#pragma unroll 1
+    for (int b = 0; b < g.nblk; ++b) {
+        const uint32_t sg = smem_b + st * SM::stage;
+        const uint32_t k_b = sg + SM::k_off, q_b = sg + SM::q_off, t_b = sg + SM::t_off, p_b = sg + SM::p_off, v_b = sg + SM::v_off;
+        uint32_t s16[KT][4];                                      // fp16 copy of -S: A operand of -S K^T, B operand of (-Q)(-S)^T
+#pragma unroll
+        for (int kk = 0; kk < KT; ++kk) {
+            s16[kk][0] = pack_h2(-S[2 * kk][0], -S[2 * kk][1]);
+            s16[kk][1] = pack_h2(-S[2 * kk][2], -S[2 * kk][3]);
+            s16[kk][2] = pack_h2(-S[2 * kk + 1][0], -S[2 * kk + 1][1]);
+            s16[kk][3] = pack_h2(-S[2 * kk + 1][2], -S[2 * kk + 1][3]);
+        }
+        // (IS = 2: the pair's barrier below carries the outcome, so that a failed wait never strands the other warp there; V, which
+        //  the team does not touch, had landed before the team arrived: the second wait makes it visible here)
+        const bool ok = mbar_wait_clk(&full[st], (uint32_t)phase, err, 312) && mbar_wait_clk(&land[st], (uint32_t)phase, err, 313);
+        if (IS == 1 && !ok) return;
+        // ---- R = V^T - S K^T: the accumulators start from V (in one warp of a pair)
+        float r[8][4];
+        if (IS == 1 || hi == 0) {
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) {
+                uint32_t x[4];
+                ldmatrix_x4_trans(x, v_b + offV + kk * V_STEP);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    r[2 * kk + (e >> 1)][2 * (e & 1)] = __uint_as_float(x[e] << 16);
+                    r[2 * kk + (e >> 1)][2 * (e & 1) + 1] = __uint_as_float(x[e] & 0xFFFF0000u);
+                }
+            }
+        } else {
+#pragma unroll
+            for (int n = 0; n < 8; ++n)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) r[n][e] = 0.f;
+        }
+#pragma unroll
+        for (int kk = 0; kk < KT; ++kk)
+#pragma unroll
+            for (int np = 0; np < 4; ++np) {
+                uint32_t x[4];
+                ldmatrix_x4(x, k_b + (offN ^ kxor(kk)) + np * 2048 + kpos(kk, NB * 128));
+                mma_16816(r[2 * np], s16[kk], x[0], x[1]);
+                mma_16816(r[2 * np + 1], s16[kk], x[2], x[3]);
+            }
+        if (IS == 2) {
+            // the other warp of the pair has the other half of the sum; with it goes the half of Q S^T of the block before that
+            // the other warp stores
+            float4* mine = (float4*)(exw + ((b & 1) * 2 + hi) * (CFG::x_piece * 512));
+            const float4* other = (const float4*)(exw + ((b & 1) * 2 + (hi ^ 1)) * (CFG::x_piece * 512));
+            const float4* other_o = (const float4*)(exw + (((b & 1) ^ 1) * 2 + (hi ^ 1)) * (CFG::x_piece * 512));
+#pragma unroll
+            for (int n = 0; n < 8; ++n) mine[n * 32] = make_float4(r[n][0], r[n][1], r[n][2], r[n][3]);
+            if (!named_bar_and(1 + TEAMS + grp, 64, ok)) return;
+#pragma unroll
+            for (int n = 0; n < 8; ++n) {
+                const float4 x = other[n * 32];
+                r[n][0] += x.x; r[n][1] += x.y; r[n][2] += x.z; r[n][3] += x.w;
+            }
+            store8(other_o);
+        }
+        // ---- the block NS - 1 further on into the stage that every chain warp has left (a block ago)
+        if (warp == 0 && lane == 0 && b > 0 && b - 1 + NS < g.nblk && mbar_wait_clk(&empty[st_prev], (uint32_t)ph_prev, err, 314))
+            load_block<DK, R, JS, NS>(maps, smem, land, b - 1 + NS, (int)seq, j0);
+        __syncwarp();
+        // ---- U'^T = R T^T (T lower triangular)
+        uint32_t r16[4][4];
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) {
+            r16[kk][0] = pack_h2(r[2 * kk][0], r[2 * kk][1]);
+            r16[kk][1] = pack_h2(r[2 * kk][2], r[2 * kk][3]);
+            r16[kk][2] = pack_h2(r[2 * kk + 1][0], r[2 * kk + 1][1]);
+            r16[kk][3] = pack_h2(r[2 * kk + 1][2], r[2 * kk + 1][3]);
+        }
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk)
+#pragma unroll
+            for (int nb = kk; nb < 4; ++nb) {
+                uint32_t x[4];
+                ldmatrix_x4(x, t_b + (offN ^ (kk << 5)) + nb * 2048);
+                mma_acc(r[2 * nb], r16[kk], x[0], x[1], kk > 0);
+                mma_acc(r[2 * nb + 1], r16[kk], x[2], x[3], kk > 0);
+            }
+        uint32_t u16[4][4];
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) {
+            u16[kk][0] = pack_h2(r[2 * kk][0], r[2 * kk][1]);
+            u16[kk][1] = pack_h2(r[2 * kk][2], r[2 * kk][3]);
+            u16[kk][2] = pack_h2(r[2 * kk + 1][0], r[2 * kk + 1][1]);
+            u16[kk][3] = pack_h2(r[2 * kk + 1][2], r[2 * kk + 1][3]);
+        }
+        // ---- S += U'^T K
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk)
+#pragma unroll
+            for (int ip = 0; ip < KT; ++ip) {
+                uint32_t x[4];
+                ldmatrix_x4_trans(x, k_b + (offT ^ kxor(ip)) + kk * 2048 + kpos(ip, NB * 128));
+                mma_16816(S[2 * ip], u16[kk], x[0], x[1]);
+                mma_16816(S[2 * ip + 1], u16[kk], x[2], x[3]);
+            }
+        // ---- O = Q S^T + P U' with the state before the update, 16 tokens at a time (these products fill the latency of the update)
+        const int Cv = min(C, g.L - b * C);
+#pragma unroll
+        for (int tt = 0; tt < TT; ++tt) {
+            float o[2][4];
+#pragma unroll
+            for (int kk = 0; kk < KT; ++kk) {
+                uint32_t a[4];
+                ldmatrix_x4(a, q_b + (offA ^ kxor(kk)) + tt * 2048 + kpos(kk, CP * 128));
+                mma_acc(o[0], a, s16[kk][0], s16[kk][2], kk > 0);
+                mma_acc(o[1], a, s16[kk][1], s16[kk][3], kk > 0);
+            }
+            float ot[4];
+            if (IS == 2) {
+                float4* mine = (float4*)(exw + ((b & 1) * 2 + hi) * (CFG::x_piece * 512));
+                mine[(8 + tt) * 32] = hi ? make_float4(o[0][0], o[0][1], o[0][2], o[0][3]) : make_float4(o[1][0], o[1][1], o[1][2], o[1][3]);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) ot[e] = hi ? o[1][e] : o[0][e];
+            }
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) {
+                if (kk >= (tt + 1) * R) continue;
+                uint32_t a[4];
+                ldmatrix_x4(a, p_b + (offA ^ (kk << 5)) + tt * 2048);
+                if (IS == 2) {
+                    mma_16816(ot, a, hi ? u16[kk][1] : u16[kk][0], hi ? u16[kk][3] : u16[kk][2]);
+                } else {
+                    mma_16816(o[0], a, u16[kk][0], u16[kk][2]);
+                    mma_16816(o[1], a, u16[kk][1], u16[kk][3]);
+                }
+            }
+            if (IS == 2) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) ok8[tt][e] = ot[e];
+            } else {
+                const int t = 16 * tt + gq;
+                float* o0 = ob + (long long)t * g.d_v;
+                store2_if(o0, o[0][0], o[0][1], t < Cv);
+                store2_if(o0 + 8, o[1][0], o[1][1], t < Cv);
+                store2_if(o0 + 8ll * g.d_v, o[0][2], o[0][3], t + 8 < Cv);
+                store2_if(o0 + 8ll * g.d_v + 8, o[1][2], o[1][3], t + 8 < Cv);
+            }
+        }
+        Cv_prev = Cv;
+        ob += (long long)C * g.d_v;
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&empty[st]);
+        st_prev = st;
+        ph_prev = phase;
+        if (++st == NS) {
+            st = 0;
+            phase ^= 1;
+        }
+    }
+    if (IS == 2) {
+        named_bar(1 + TEAMS + grp, 64);                           // (both warps are here: a failed wait left through the barrier above)
+        store8((const float4*)(exw + (((g.nblk & 1) ^ 1) * 2 + (hi ^ 1)) * (CFG::x_piece * 512)));
+    }
+    if (S_final)
+#pragma unroll
+        for (int n = 0; n < 2 * KT; ++n)
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                S_final[(seq * DK + i0 + 8 * n + (e & 1)) * g.d_v + jr + 8 * (e >> 1)] = S[n][e];
+}
+
+template <int DK, int R, int JS, int IS, int TEAMS, int NS>
+__global__ void __launch_bounds__(ChainCfg<DK, R, JS, IS, TEAMS, NS>::threads, 1)
+chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __restrict__ beta, const float* __restrict__ S0,
+             float* __restrict__ O, float* __restrict__ S_final, int* __restrict__ status, ChainGeo g) {
+    using CFG = ChainCfg<DK, R, JS, IS, TEAMS, NS>;
+    using SM = ChainSmem<DK, R, JS>;
+    extern __shared__ __align__(1024) uint8_t smem[];
+    __shared__ uint64_t land[NS], full[NS], empty[NS];
+    const int tid = threadIdx.x, warp = tid >> 5;
+    const int slices = g.d_v / JS;
+    const long long seq = blockIdx.x / slices;
+    const int j0 = (int)(blockIdx.x % slices) * JS;
+    if ((smem_u32(smem) & 1023u) != 0) {                          // (the swizzled layouts need a 1024-byte aligned base)
+        if (tid == 0) atomicCAS(status, 0, 99);
+        return;
+    }
+    if (tid == 0) {
+        if (blockIdx.x == 0) *status = 0;                         // (the call's status word: a wait expires a second from now at the earliest)
+        for (int x = 0; x < NS; ++x) {
+            mbar_init(&land[x], 1);
+            mbar_init(&full[x], 128);
+            mbar_init(&empty[x], CFG::NCW);
+        }
+        mbar_fence_init();
+        prefetch_tmap(&maps.q);
+        prefetch_tmap(&maps.k);
+        prefetch_tmap(&maps.v);
+    }
+    if (SM::CP > SM::C) {                                         // (r = 3: query rows that no copy writes are read)
+        for (int e = tid; e < NS * SM::stage / 16; e += CFG::threads) ((uint4*)smem)[e] = make_uint4(0, 0, 0, 0);
+        fence_async_smem();
+    }
+    __syncthreads();
+    if (tid == 0)
+        for (int b = 0; b < NS && b < g.nblk; ++b) load_block<DK, R, JS, NS>(maps, smem, land, b, (int)seq, j0);
+    __syncwarp();
+    if (warp < CFG::NCW)
+        chain_role<DK, R, JS, IS, TEAMS, NS>(maps, g, S0, O, S_final, status, smem, land, full, empty, seq, j0, warp, tid & 31);
+    else
+        prep_role<DK, R, JS, IS, TEAMS, NS>(g, beta, status, smem, land, full, seq, (warp - CFG::NCW) >> 2, (tid - 32 * CFG::NCW) & 127);
+}
+
+template <int DK, int R, int JS, int IS, int TEAMS>
+int launch(const Problem& p) {
+    constexpr int NS = chain_stages<DK, R, JS, IS, TEAMS>();
+    using CFG = ChainCfg<DK, R, JS, IS, TEAMS, NS>;
+    static_assert(CFG::total <= 227 * 1024 && NS >= 2, "shared memory budget");
+    const void* fn = (const void*)chain_kernel<DK, R, JS, IS, TEAMS, NS>;
+    constexpr int C = NB / R;
+    ChainGeo g{p.L, p.d_v, (p.L + C - 1) / C, p.mask_group(), p.exact ? 1 : 0};
+    const long long nseq = (long long)p.B * p.H, grid = nseq * (p.d_v / JS);
+    ChainMaps maps;
+    constexpr int VC = JS < 64 ? JS : 64;
+    if (!make_slab_map(&maps.k, p.k, nseq, (uint64_t)p.L * R, DK, 64, NB, DK / 64) || !make_slab_map(&maps.q, p.q, nseq, p.L, DK, 64, C, R == 3 ? 1 : DK / 64) ||
+        !make_slab_map(&maps.v, p.v, nseq, (uint64_t)p.L * R, p.d_v, VC, NB, JS / VC))
+        return record_cuda_error(cudaErrorInvalidValue, "cuTensorMapEncodeTiled");
+    static std::atomic<uint64_t> opted_in{0};
+    const int st = allow_smem(opted_in, fn, CFG::total);
+    if (st != PF_OK) return st;
+    void* args[] = {(void*)&maps, (void*)&p.beta, (void*)&p.S0, (void*)&p.O, (void*)&p.S_final, (void*)&p.status, (void*)&g};
+    prof_begin("chain", p.stream);
+    PF_CUDA_TRY(cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(CFG::threads), args, (size_t)CFG::total, p.stream));
+    prof_end(p.stream);
+    count_launch(1);
+    return PF_OK;
+}
+
+// How a sequence's d_v columns are spread over CTAs.  Fewer columns per CTA make a shorter step but more CTAs; the time is
+// (waves of CTAs) x (time of a step).  Steps relative to each other, measured with one wave at L = 1024 (us for d_k = d_v =
+// 128, r = 2 and r = 4): 32 columns by pairs of warps 67, 117; 64 columns 86, 140; 128 columns 125, 225.  At d_k = 64 a step is
+// short enough that 32 columns gain nothing over 64 (51 against 53 us), and 128 columns cost 1.3 times as much.
+enum { COLS_32, COLS_64, COLS_128 };
+struct Spread {
+    int cols;
+    double waves_x_step;      // in steps of COLS_64
+};
+Spread pick_spread(const Problem& p) {
+    const long long nseq = (long long)p.B * p.H, sms = sm_count();
+    auto waves = [&](int js) { return (double)((nseq * (p.d_v / js) + sms - 1) / sms); };
+    Spread s{COLS_64, waves(64)};
+    if (p.d_k == 128 && 0.8 * waves(32) < s.waves_x_step) s = {COLS_32, 0.8 * waves(32)};
+    if (p.d_v == 128) {
+        const double w = (p.d_k == 128 ? 1.5 : 1.3) * waves(128);
+        if (w < s.waves_x_step) s = {COLS_128, w};
+    }
+    return s;
+}
+
+template <int DK, int R>
+int launch_spread(const Problem& p) {
+    switch (pick_spread(p).cols) {
+        case COLS_32:
+            if constexpr (DK == 128) return launch<DK, R, 32, 2, 2>(p);
+        case COLS_64: return launch<DK, R, 64, 1, 2>(p);
+        default: return launch<DK, R, 128, 1, DK == 64 ? 2 : 1>(p);
+    }
+}
+
+}  // namespace
+
+// An estimate of the kernel's time in us, for the choice between it and the single-launch tcgen05 kernel.
+double chain_estimate_us(const Problem& p) {
+    static const double step[4] = {3.3, 2.6, 2.6, 2.15};     // one block, COLS_64, d_k = 128
+    const int C = NB / p.r;
+    return 6.0 + (double)((p.L + C - 1) / C) * step[p.r - 1] * pick_spread(p).waves_x_step;
+}
+
+bool chain_supported(const Problem& p) {
+    return p.in_dtype == PF_DTYPE_BF16 && p.L >= 1 && (long long)p.B * p.H * (p.d_v / 32) <= 0x7fffffffLL &&
+           (long long)p.L * p.r <= 0x7fffffffLL;
+}
+
+int chain_forward(const Problem& p) {
+    if (p.d_k == 128) switch (p.r) {
+        case 1: return launch_spread<128, 1>(p);
+        case 2: return launch_spread<128, 2>(p);
+        case 3: return launch_spread<128, 3>(p);
+        default: return launch_spread<128, 4>(p);
+    }
+    switch (p.r) {
+        case 1: return launch_spread<64, 1>(p);
+        case 2: return launch_spread<64, 2>(p);
+        case 3: return launch_spread<64, 3>(p);
+        default: return launch_spread<64, 4>(p);
+    }
+}
+
+}  // namespace pf

@@ -95,6 +95,14 @@ int simt_forward(const Problem& p, void* workspace);
 // the recurrence token by token in fp32 (pf_recur.cu); needs no workspace
 int recur_forward(const Problem& p);
 
+// the chunk form in one kernel on warp-level tensor-core products (pf_chain.cu); bf16 inputs, needs no workspace
+bool chain_supported(const Problem& p);
+double chain_estimate_us(const Problem& p);
+int chain_forward(const Problem& p);
+
+// SM count of the current device, 0 if it cannot be found (pf_fused.cu)
+int sm_count();
+
 // tcgen05 path (pf_tc.cu)
 bool tc_supported(const Problem& p);
 bool tc_scan_supported(const Problem& p);

@@ -64,6 +64,23 @@ namespace pf {
 
 using namespace tc;
 
+// SM count of the current device (cached per device ordinal: a process may use several devices)
+int sm_count() {
+    constexpr int MAX_DEV = 64;
+    static std::atomic<int> cache[MAX_DEV];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    if (dev >= 0 && dev < MAX_DEV) {
+        const int have = cache[dev].load(std::memory_order_relaxed);
+        if (have) return have;
+    }
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+    if (dev >= 0 && dev < MAX_DEV) cache[dev].store(sms, std::memory_order_relaxed);
+    return sms;
+}
+
+
 namespace {
 
 constexpr int FT = 512;                 // threads per CTA
@@ -879,51 +896,6 @@ fused_kernel(const __grid_constant__ FusedMaps maps, FusedGeo g, FusedWs ws, con
     if (warp == 0) tmem_dealloc(tb, 512);
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
-                                  const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn encode_fn() {
-    static EncodeTiledFn fn = nullptr;
-    if (!fn) {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult qres;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &qres) == cudaSuccess &&
-            qres == cudaDriverEntryPointSuccess)
-            fn = (EncodeTiledFn)p;
-    }
-    return fn;
-}
-
-// bf16 tensor [seqs][rows][cols], box = 64 cols x box_rows rows x 1, 128B swizzle, zero fill out of bounds
-bool make_map(CUtensorMap* m, const void* base, uint64_t seqs, uint64_t rows, uint64_t cols, uint32_t box_rows) {
-    EncodeTiledFn fn = encode_fn();
-    if (!fn) return false;
-    cuuint64_t dims[3] = {cols, rows, seqs};
-    cuuint64_t strides[2] = {cols * 2, rows * cols * 2};
-    cuuint32_t box[3] = {64, box_rows, 1};
-    cuuint32_t estr[3] = {1, 1, 1};
-    return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// SM count of the current device (cached per device ordinal: a process may use several devices)
-int sm_count() {
-    constexpr int MAX_DEV = 64;
-    static std::atomic<int> cache[MAX_DEV];
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-    if (dev >= 0 && dev < MAX_DEV) {
-        const int have = cache[dev].load(std::memory_order_relaxed);
-        if (have) return have;
-    }
-    int sms = 0;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-    if (dev >= 0 && dev < MAX_DEV) cache[dev].store(sms, std::memory_order_relaxed);
-    return sms;
-}
-
 // Slots per sequence (pf_params.ring_depth, 3..64).  Default 8; 16 for long sequences while all rings together stay
 // well inside the L2: over a thousand chunks the flow CTAs drift apart and a deeper ring absorbs it (measured at
 // 32 sequences of 1024 chunks: 2.29 ms against 2.50 ms; no difference at 128 chunks).
@@ -952,11 +924,13 @@ Carve carve(const Problem& p) {
 
 }  // namespace
 
-// One CTA per sequence scans, the rest build flows.  Measured at d = 128, r = 2: up to about 100 sequences the single
-// launch beats the two-launch form (96: 400 against 477 us at L = 2048), beyond that too few SMs are left for the
-// flows (120: 865 against 600 us; 136: 2194 against 669 us).
-bool fused_preferred(const Problem& p) {
-    return (long long)p.B * p.H * 10 <= (long long)sm_count() * 7;
+// An estimate of the kernel's time in us: the first flow, then per chunk either the scan's step or the time in which the CTAs
+// that do not scan build a chunk of every sequence, whichever is longer.
+double fused_estimate_us(const Problem& p) {
+    const double nseq = (double)p.B * p.H, flows = sm_count() - nseq;
+    const double flow = p.tile_rows() == 128 ? 5.9 : 3.6, step = 1.35;
+    const double build = flow * nseq / flows;
+    return 24.0 + p.chunks_per_seq() * (build > step ? build : step);
 }
 
 bool fused_supported(const Problem& p) {
@@ -993,9 +967,9 @@ int fused_forward(const Problem& p, void* workspace) {
     FusedMaps maps;
     if (NC > 0) {
         const uint64_t seqs = (uint64_t)nseq;
-        if (!make_map(&maps.k, p.k, seqs, (uint64_t)p.L * p.r, p.d_k, p.tile_rows()) ||
-            !make_map(&maps.q, p.q, seqs, (uint64_t)p.L, p.d_k, p.chunk) ||
-            !make_map(&maps.v, p.v, seqs, (uint64_t)p.L * p.r, p.d_v, p.tile_rows()))
+        if (!make_tile_map(&maps.k, p.k, seqs, (uint64_t)p.L * p.r, p.d_k, p.tile_rows()) ||
+            !make_tile_map(&maps.q, p.q, seqs, (uint64_t)p.L, p.d_k, p.chunk) ||
+            !make_tile_map(&maps.v, p.v, seqs, (uint64_t)p.L * p.r, p.d_v, p.tile_rows()))
             return record_cuda_error(cudaErrorInvalidValue, "cuTensorMapEncodeTiled");
     } else {
         memset(&maps, 0, sizeof(maps));

@@ -280,6 +280,40 @@ int pick_dvs(const Problem& p) {
 
 }  // namespace
 
+typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                                  const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+static EncodeTiledFn encode_fn() {
+    static const EncodeTiledFn fn = [] {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult qres;
+        const bool ok = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &qres) == cudaSuccess &&
+                        qres == cudaDriverEntryPointSuccess;
+        return ok ? (EncodeTiledFn)p : nullptr;
+    }();
+    return fn;
+}
+
+static bool encode(CUtensorMap* m, const void* base, int rank, const cuuint64_t* dims, const cuuint64_t* strides, const cuuint32_t* box,
+                   CUtensorMapSwizzle swizzle) {
+    const EncodeTiledFn fn = encode_fn();
+    const cuuint32_t ones[4] = {1, 1, 1, 1};
+    return fn && fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank, const_cast<void*>(base), dims, strides, box, ones,
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+bool make_slab_map(CUtensorMap* m, const void* base, uint64_t seqs, uint64_t rows, uint64_t cols, uint32_t slab_cols, uint32_t box_rows,
+                   uint32_t box_slabs) {
+    const cuuint64_t dims[4] = {slab_cols, rows, cols / slab_cols, seqs}, strides[3] = {cols * 2, slab_cols * 2, rows * cols * 2};
+    const cuuint32_t box[4] = {slab_cols, box_rows, box_slabs, 1};
+    return encode(m, base, 4, dims, strides, box, slab_cols == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B);
+}
+bool make_tile_map(CUtensorMap* m, const void* base, uint64_t seqs, uint64_t rows, uint64_t cols, uint32_t box_rows) {
+    const cuuint64_t dims[3] = {cols, rows, seqs}, strides[2] = {cols * 2, rows * cols * 2};
+    const cuuint32_t box[3] = {64, box_rows, 1};
+    return encode(m, base, 3, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B);
+}
+
 TcGeo tc_geo(const Problem& p) {
     TcGeo g{};
     g.L = p.L; g.d_k = p.d_k; g.d_v = p.d_v; g.r = p.r; g.C = p.chunk; g.n = p.n(); g.NC = p.chunks_per_seq(); g.rm = p.mask_group(); g.b32 = p.beta32;

@@ -1,6 +1,8 @@
 // Internal interfaces of the tensor-core path (shared by pf_tc.cu and pf_tc_flow.cu).
 #pragma once
 
+#include <cuda.h>
+
 #include "pf_common.cuh"
 
 namespace pf {
@@ -19,6 +21,14 @@ struct TcWs {
     uint8_t* Xi;    // [G][xi_bytes]
 };
 
+// Tensor map of a bf16 tensor [seqs][rows][cols], zero fill out of bounds (pf_tc.cu).  The columns are seen as slabs of
+// slab_cols (64 or 32: the swizzle spans a slab's row), so that one copy brings box_slabs slabs of box_rows rows, one slab
+// after another: coordinates (column within the slab, row, slab, sequence).
+bool make_slab_map(CUtensorMap* m, const void* base, uint64_t seqs, uint64_t rows, uint64_t cols, uint32_t slab_cols, uint32_t box_rows,
+                   uint32_t box_slabs);
+// The same as a three-dimensional map with boxes of 64 columns x box_rows rows: coordinates (column, row, sequence).
+bool make_tile_map(CUtensorMap* m, const void* base, uint64_t seqs, uint64_t rows, uint64_t cols, uint32_t box_rows);
+
 TcGeo tc_geo(const Problem& p);
 size_t tc_ws_carve(const Problem& p, void* base, TcWs* out);
 
@@ -33,7 +43,7 @@ size_t tc_refflow_workspace_bytes(const Problem& p);
 
 // pf_fused.cu: flow builders and state scan in one cooperative launch
 bool fused_supported(const Problem& p);
-bool fused_preferred(const Problem& p);     // enough SMs are left for building flows that the single launch wins
+double fused_estimate_us(const Problem& p);
 size_t fused_workspace_bytes(const Problem& p);
 int fused_forward(const Problem& p, void* workspace);
 

@@ -391,35 +391,6 @@ tc_flow(const __grid_constant__ FlowMaps maps, TcGeo g, TcWs ws, const __nv_bflo
     if (warp == 0) tmem_dealloc(tb, SM::tmem_cols);
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
-                                  const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn encode_fn() {
-    static EncodeTiledFn fn = nullptr;
-    if (!fn) {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult qres;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &qres) == cudaSuccess &&
-            qres == cudaDriverEntryPointSuccess)
-            fn = (EncodeTiledFn)p;
-    }
-    return fn;
-}
-
-// bf16 tensor [seqs][rows][cols], box = 64 cols x box_rows rows x 1, 128B swizzle, zero fill out of bounds
-bool make_map(CUtensorMap* m, const void* base, uint64_t seqs, uint64_t rows, uint64_t cols, uint32_t box_rows) {
-    EncodeTiledFn fn = encode_fn();
-    if (!fn) return false;
-    cuuint64_t dims[3] = {cols, rows, seqs};
-    cuuint64_t strides[2] = {cols * 2, rows * cols * 2};
-    cuuint32_t box[3] = {64, box_rows, 1};
-    cuuint32_t estr[3] = {1, 1, 1};
-    return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 template <int N, int DK, int DV>
 int launch(const Problem& p, const TcWs& ws, int dvs, const FlowMaps& maps) {
     using SM = FlowSmem<N, DK, DV>;
@@ -449,9 +420,9 @@ int tc_flow_launch(const Problem& p, const TcWs& ws, int dvs) {
     const int n = p.tile_rows();       // box rows: the whole tile, rows past the chunk's own included (they get beta = 0)
     const uint64_t seqs = (uint64_t)p.B * p.H;
     FlowMaps maps;
-    if (!make_map(&maps.k, p.k, seqs, (uint64_t)p.L * p.r, p.d_k, n) ||
-        !make_map(&maps.q, p.q, seqs, (uint64_t)p.L, p.d_k, p.chunk) ||
-        !make_map(&maps.v, p.v, seqs, (uint64_t)p.L * p.r, p.d_v, n))
+    if (!make_tile_map(&maps.k, p.k, seqs, (uint64_t)p.L * p.r, p.d_k, n) ||
+        !make_tile_map(&maps.q, p.q, seqs, (uint64_t)p.L, p.d_k, p.chunk) ||
+        !make_tile_map(&maps.v, p.v, seqs, (uint64_t)p.L * p.r, p.d_v, n))
         return record_cuda_error(cudaErrorInvalidValue, "cuTensorMapEncodeTiled");
 #define PF_FLOW_CASE(NN, KK, VV) \
     if (n == NN && p.d_k == KK && p.d_v == VV) return launch<NN, KK, VV>(p, ws, dvs, maps);

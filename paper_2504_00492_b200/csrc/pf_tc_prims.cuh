@@ -182,6 +182,12 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, i
         ::"r"(smem_u32(dst)), "l"(map), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar))
         : "memory");
 }
+__device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, int x, int y, int z, int w, uint64_t* bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
+        ::"r"(smem_u32(dst)), "l"(map), "r"(x), "r"(y), "r"(z), "r"(w), "r"(smem_u32(bar))
+        : "memory");
+}
 // 1-D bulk copy global -> shared; both addresses 16-byte aligned, bytes a multiple of 16.
 __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
@@ -397,9 +403,19 @@ __device__ __forceinline__ void commit_uni(uint64_t* bar) {
 
 // ---- warp-level MMA for the small triangular solve -------------------------------------------------
 __device__ __forceinline__ void mma_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
                  : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// c = a b (+ c if acc): without acc the accumulator need not be cleared first
+__device__ __forceinline__ void mma_acc(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1, bool acc) {
+    if (acc) {
+        mma_16816(c, a, b0, b1);
+        return;
+    }
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+        : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
 }
 __device__ __forceinline__ void ldmatrix_x4(uint32_t (&r)[4], uint32_t saddr) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
@@ -444,11 +460,8 @@ __device__ __forceinline__ void frag_zero(float (&c)[2][4]) {
 #pragma unroll
         for (int e = 0; e < 4; ++e) c[h][e] = 0.f;
 }
-__device__ __forceinline__ void diag_inverse16(uint32_t xb, uint8_t* xg, int blk, int lane, int N, bool deep) {
-    const int R0 = 16 * blk, c8 = 2 * blk;
-    uint32_t a[4], at[4];
-    ldmatrix_x4(a, xb + chunk_off(R0 + (lane & 15), c8 + (lane >> 4), N));
-    ldmatrix_x4_trans(at, xb + chunk_off(R0 + (lane & 7) + ((lane >> 4) << 3), c8 + ((lane >> 3) & 1), N));
+// r = (I + A)^{-1} as an accumulator fragment, from the A-operand fragments of A and of A^T
+__device__ __forceinline__ void neumann16(float (&r)[2][4], const uint32_t (&a)[4], const uint32_t (&at)[4], int lane, bool deep) {
     float c[2][4], ct[2][4];
     uint32_t a2[4], a2t[4], a4[4], a4t[4];
     frag_zero(c); frag_zero(ct);
@@ -461,7 +474,6 @@ __device__ __forceinline__ void diag_inverse16(uint32_t xb, uint8_t* xg, int blk
     frag_pack(a4, c); frag_pack(a4t, ct);
     // R = I - A in accumulator layout: thread (g, t) holds rows g, g+8 and columns 8h + 2t, 8h + 2t + 1
     const int gq = lane >> 2, t4 = lane & 3;
-    float r[2][4];
     {
         const __half2 h0 = *reinterpret_cast<const __half2*>(&a[0]), h1 = *reinterpret_cast<const __half2*>(&a[1]);
         const __half2 h2 = *reinterpret_cast<const __half2*>(&a[2]), h3 = *reinterpret_cast<const __half2*>(&a[3]);
@@ -485,6 +497,15 @@ __device__ __forceinline__ void diag_inverse16(uint32_t xb, uint8_t* xg, int blk
         frag_pack(rf, r);
         frag_mul(r, rf, a8t);   // ... (I + A^8)
     }
+}
+__device__ __forceinline__ void diag_inverse16(uint32_t xb, uint8_t* xg, int blk, int lane, int N, bool deep) {
+    const int R0 = 16 * blk, c8 = 2 * blk;
+    uint32_t a[4], at[4];
+    ldmatrix_x4(a, xb + chunk_off(R0 + (lane & 15), c8 + (lane >> 4), N));
+    ldmatrix_x4_trans(at, xb + chunk_off(R0 + (lane & 7) + ((lane >> 4) << 3), c8 + ((lane >> 3) & 1), N));
+    const int gq = lane >> 2, t4 = lane & 3;
+    float r[2][4];
+    neumann16(r, a, at, lane, deep);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         *(uint32_t*)(xg + chunk_off(R0 + gq, c8 + h, N) + 4 * t4) = pack_h2(r[h][0], r[h][1]);
