@@ -47,7 +47,7 @@
 //
 // A scan CTA: warps 0-7 own the state in registers (row j of S per thread, d_k split in two halves of 64 columns).
 // Each chunk they write an fp16 copy of it into TENSOR memory, where it is the A operand of both of the chunk's
-// products (Delta = S E^T issued by warp 0, O^T = S Qt^T issued by warp 13), so the serial step never goes
+// products (Delta = S E^T issued by warp 15, O^T = S Qt^T issued by warp 13), so the serial step never goes
 // through shared memory.  Warps 8-11 add OI and write O, warp 12 streams the E / Xi / Qt images in with bulk
 // copies and is the only poller of the ready flags, warp 14 reports consumed chunks.
 //
@@ -122,10 +122,9 @@ constexpr int F_BAR = F_BETA + 1024;
 constexpr int F_I16 = F_BAR + 512;              // 16 x 16 fp16 identity, unswizzled K-major (512 B)
 constexpr int SMEM_BYTES = F_I16 + 512;         // 231424
 // scan role
-constexpr int S_E = 0;                          // 2 x 32 KB  E images
-constexpr int S_XI = S_E + 2 * 32768;           // 2 x 32 KB  Xi images
-constexpr int S_QT = S_XI + 2 * 32768;          // 2 x 16 KB  Qt images
-constexpr int S_OUT = S_QT + 2 * 16384;         // 2 x 32 KB  fp32 images of S Qt^T, [t][j], on their way into O
+constexpr int S_EQ = 0;                         // 2 x 48 KB  E image, then Qt image (adjacent in the ring slot: one copy)
+constexpr int S_XI = S_EQ + 2 * 49152;          // 2 x 32 KB  Xi images
+constexpr int S_OUT = S_XI + 2 * 32768;         // 2 x 32 KB  fp32 images of S Qt^T, [t][j], on their way into O
 static_assert(S_OUT + 2 * 32768 <= F_BAR, "scan role fits below the barrier block");
 static_assert(SMEM_BYTES <= 227 * 1024, "shared memory budget");
 
@@ -153,15 +152,14 @@ enum {
     B_SLOTOK = 28,    // flag warp: the chunk's ring slot may be written
     B_RADONE = 29,    // mma: [E | Xi^T] complete
     // scan role
-    B_EFULL = 32,     // [2] producer: E image landed
-    B_EEMPTY = 34,    // [2] chain: Delta of that chunk complete
+    B_EQFULL = 32,    // [2] producer: E and Qt images landed
+    B_EQEMPTY = 34,   // [2] mma: Delta and O^T of that chunk complete
     B_XIFULL = 36,    // [2] producer: Xi image landed
     B_XIEMPTY = 38,   // [2] chain: Xi added to the state (one arrival per chain warp)
-    B_QTFULL = 40,    // [2] producer: Qt image landed
-    B_QTEMPTY = 42,   // [2] mma: O^T of that chunk complete
     B_APUB = 44,      // [2 buffers] mma: Delta of the chunk complete (the O^T product may be issued)
     B_S16FREE = 46,   // [2 buffers] mma: the MMAs that read that fp16 copy of the state are complete
     B_DDONE = 48,     // Delta complete
+    B_SPUB = 49,      // chain: fp16 copy of the state in tensor memory (one arrival per chain warp)
     B_ODONE = 50,     // [2] mma: O^T complete
     B_OFREE = 52,     // [2] output warps: O^T drained
     B_COUNT = 54
@@ -656,8 +654,7 @@ __device__ void scan_role(const FusedGeo& g, const FusedWs& ws, const float* __r
         for (int c = 0; c < NC; ++c) {
             const int buf = c & 1;
             // fp16 copy of the state into tensor memory (A operand of Delta and of O^T): 32 packed columns per thread
-            bool ok = true;
-            if (c >= 2) ok = PF_WAIT(B_S16FREE + buf, ((c >> 1) - 1) & 1, 201);
+            if (c >= 2 && !PF_WAIT(B_S16FREE + buf, ((c >> 1) - 1) & 1, 201)) return;
             tc_fence_after();
             {
                 uint32_t pk[32];
@@ -667,36 +664,34 @@ __device__ void scan_role(const FusedGeo& g, const FusedWs& ws, const float* __r
                 tmem_st_wait();
             }
             tc_fence_before();
-            if (!named_bar_and(1, 256, ok)) return;
-            // warp 0 issues Delta[j][i] = sum_i' S[j][i'] E[i][i']; its completion also releases warp 13, which
-            // issues the O^T product of the same copy (so that O^T never sits in front of Delta in the tensor pipe)
-            if (warp == 0) {
-                if (!PF_WAIT(B_EFULL + buf, (c >> 1) & 1, 231)) return;
-                tc_fence_after();
-                gemm_ta<L_NSK, DK, DK, 128>(t_delta, t_a + buf * 64, smem_u32(smem + S_E + buf * 32768));
-                commit_uni(&bar[B_DDONE]);
-                commit_uni(&bar[B_EEMPTY + buf]);
-                commit_uni(&bar[B_APUB + buf]);
-            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bar[B_SPUB]);
+            // (Xi^T is added while the product runs)
             if (!PF_WAIT(B_XIFULL + buf, (c >> 1) & 1, 203)) return;
-            if (!PF_WAIT(B_DDONE, c & 1, 202)) return;
-            tc_fence_after();
-            // S += Delta + Xi^T   (row j, columns 64w..64w+63; Xi^T from its column-group image)
             const uint8_t* xrow = smem + S_XI + buf * 32768 + w * 16384 + j * 16;
 #pragma unroll
-            for (int c0 = 0; c0 < 64; c0 += 32) {
-                uint32_t rr[32];
-                tmem_ld32(t_delta + lane_base + 64 * w + c0, rr);
-                uint4 xi[4];
+            for (int p = 0; p < 8; ++p) {
+                const uint4 xi = *(const uint4*)(xrow + p * 2048);
 #pragma unroll
-                for (int p = 0; p < 4; ++p) xi[p] = *(const uint4*)(xrow + ((c0 >> 3) + p) * 2048);
+                for (int e = 0; e < 8; e += 2) {
+                    const uint32_t wd = ((const uint32_t*)&xi)[e >> 1];
+                    const float2 xv = __half22float2(*reinterpret_cast<const __half2*>(&wd));
+                    S[8 * p + e] += xv.x;
+                    S[8 * p + e + 1] += xv.y;
+                }
+            }
+            if (!PF_WAIT(B_DDONE, c & 1, 202)) return;
+            tc_fence_after();
+            // S += Delta   (row j, columns 64w..64w+63)
+            {
+                uint32_t ra[32], rb[32];
+                tmem_ld32(t_delta + lane_base + 64 * w, ra);
+                tmem_ld32(t_delta + lane_base + 64 * w + 32, rb);
                 tmem_ld_wait();
 #pragma unroll
-                for (int e = 0; e < 32; e += 2) {
-                    const uint32_t wd = ((const uint32_t*)&xi[e >> 3])[(e & 7) >> 1];
-                    const float2 xv = __half22float2(*reinterpret_cast<const __half2*>(&wd));
-                    S[c0 + e] += __uint_as_float(rr[e]) + xv.x;
-                    S[c0 + e + 1] += __uint_as_float(rr[e + 1]) + xv.y;
+                for (int e = 0; e < 32; ++e) {
+                    S[e] += __uint_as_float(ra[e]);
+                    S[32 + e] += __uint_as_float(rb[e]);
                 }
             }
             tc_fence_before();
@@ -749,28 +744,24 @@ __device__ void scan_role(const FusedGeo& g, const FusedWs& ws, const float* __r
     } else if (warp == 12) {
         // ------------------------------------------------ producer: ring -> shared memory ----------------------
         if (lane == 0) {
-            auto load_e = [&](int c) -> bool {
-                const int st = c & 1;
-                if (!smem_wait_ge(vis, c + 1, err, 222)) return false;      // (warp 14 polls the ready flags, ahead of the loads)
-                fence_async_global();
-                if (c >= 2 && !PF_WAIT(B_EEMPTY + st, ((c >> 1) - 1) & 1, 221)) return false;
-                mbar_expect_tx(&bar[B_EFULL + st], DK * DK * 2);
-                bulk_load(smem + S_E + st * 32768, ring + (size_t)(c % g.R) * SLOT_BYTES + SLOT_E, DK * DK * 2, &bar[B_EFULL + st]);
-                return true;
-            };
+            // (two copies per chunk: issuing one costs this thread 400 - 500 cycles whatever its size, and with E, Qt and Xi apart
+            //  and a function call for the count below this thread's 2.4 k cycles per chunk were the whole scan's step)
+            int seen = 0;
 #pragma unroll 1
             for (int c = 0; c < NC; ++c) {
-                if (c == 0 && !load_e(0)) return;
-                // (the flag of chunk c was acquired by load_e(c))
                 const uint8_t* slot = ring + (size_t)(c % g.R) * SLOT_BYTES;
-                const int b = c & 1;
-                if (c >= 2 && !PF_WAIT(B_XIEMPTY + b, ((c >> 1) - 1) & 1, 224)) return;
+                const int b = c & 1, ph = ((c >> 1) - 1) & 1;
+                if (seen <= c) {                       // (warp 14 polls the ready flags, ahead of the loads)
+                    if (!smem_wait_ge(vis, c + 1, err, 222)) return;
+                    seen = *vis;
+                    fence_async_global();
+                }
+                if (c >= 2 && !PF_WAIT(B_EQEMPTY + b, ph, 221)) return;
+                mbar_expect_tx(&bar[B_EQFULL + b], DK * DK * 2 + DK * 128);
+                bulk_load(smem + S_EQ + b * 49152, slot + SLOT_E, DK * DK * 2 + DK * 128, &bar[B_EQFULL + b]);
+                if (c >= 2 && !PF_WAIT(B_XIEMPTY + b, ph, 224)) return;
                 mbar_expect_tx(&bar[B_XIFULL + b], DK * DV * 2);
                 bulk_load(smem + S_XI + b * 32768, slot + SLOT_XI, DK * DV * 2, &bar[B_XIFULL + b]);
-                if (c >= 2 && !PF_WAIT(B_QTEMPTY + b, ((c >> 1) - 1) & 1, 223)) return;
-                mbar_expect_tx(&bar[B_QTFULL + b], DK * 128);
-                bulk_load(smem + S_QT + b * 16384, slot + SLOT_QT, DK * 128, &bar[B_QTFULL + b]);
-                if (c + 1 < NC && !load_e(c + 1)) return;
             }
         }
     } else if (warp == 13) {
@@ -779,52 +770,73 @@ __device__ void scan_role(const FusedGeo& g, const FusedWs& ws, const float* __r
         for (int c = 0; c < NC; ++c) {
             const int buf = c & 1;
             if (!PF_WAIT(B_APUB + buf, (c >> 1) & 1, 235)) return;
-            if (!PF_WAIT(B_QTFULL + buf, (c >> 1) & 1, 234)) return;
             if (c >= 2 && !PF_WAIT(B_OFREE + buf, ((c >> 1) - 1) & 1, 233)) return;
             tc_fence_after();
-            gemm_ta<L_NSMN, 64, DK, 128>(t_o + buf * 64, t_a + buf * 64, smem_u32(smem + S_QT + buf * 16384));
+            gemm_ta<L_NSMN, 64, DK, 128>(t_o + buf * 64, t_a + buf * 64, smem_u32(smem + S_EQ + buf * 49152 + DK * DK * 2));      // (landed with E, which Delta has read)
             commit_uni(&bar[B_ODONE + buf]);
-            commit_uni(&bar[B_QTEMPTY + buf]);
+            commit_uni(&bar[B_EQEMPTY + buf]);
             commit_uni(&bar[B_S16FREE + buf]);
+        }
+    } else if (warp == 15) {
+        // ------------------------------------------------ Delta[j][i] = sum_i' S[j][i'] E[i][i'] (whole warp) ---
+        // (a warp of its own: issuing the product and its commits takes about 900 cycles of a warp, which used to be one of those
+        //  that carry the state.)  Its completion also releases warp 13, which issues the O^T product of the same copy, so that
+        //  O^T never sits in front of Delta in the tensor pipe.
+#pragma unroll 1
+        for (int c = 0; c < NC; ++c) {
+            const int buf = c & 1;
+            if (!PF_WAIT(B_EQFULL + buf, (c >> 1) & 1, 231)) return;
+            if (!PF_WAIT(B_SPUB, c & 1, 236)) return;
+            tc_fence_after();
+            gemm_ta<L_NSK, DK, DK, 128>(t_delta, t_a + buf * 64, smem_u32(smem + S_EQ + buf * 49152));
+            commit_uni(&bar[B_DDONE]);
+            commit_uni(&bar[B_APUB + buf]);
         }
     } else if (warp == 14) {
         // ------------------------------------------------ ready flags in, consumed reports out -----------------
-        // One lane polls the ring's ready flags in chunk order, as far ahead of the loads as the flow CTAs are, and
-        // publishes the count in shared memory (so that no load waits a trip to the L2 for a flag that was set long
-        // ago).  The same loop reports consumption: once the four output warps are done with chunk c, chunks < c
-        // are consumed (the chain finished chunk c-1 before it published the state for chunk c) and their ring
-        // slots may be rewritten.  It polls a shared counter and always reports the latest value, however far it
-        // has fallen behind.
-        if (lane == 0) {
-            int reported = 0, seen = 0;
-            const long long t0 = clock64();
-            long long t_last = t0;
-            while (reported < NC - 1 || seen < NC) {
-                bool progress = false;
-                if (seen < NC && ld_acquire_gpu(&ready[seen % g.R]) >= seen + 1) {
-                    ++seen;
-                    __threadfence_block();
-                    *vis = seen;
-                    progress = true;
-                }
-                const int chunks_done = *odone >> 2;
-                if (chunks_done - 1 > reported) {
-                    reported = chunks_done - 1;
+        // The warp polls the ring's ready flags, as far ahead of the loads as the flow CTAs are, one flag per lane: a flag takes
+        // a trip to the L2 (about 800 cycles), and one after another they held the loads back to one chunk per 2.5 k cycles.  The
+        // count of leading chunks that are ready is published in shared memory.  The same loop reports consumption: once the
+        // four output warps are done with chunk c, chunks < c are consumed (the chain finished chunk c-1 before it published the
+        // state for chunk c) and their ring slots may be rewritten.  It polls a shared counter and always reports the latest
+        // value, however far it has fallen behind.
+        int reported = 0, seen = 0;
+        long long t_last = clock64();
+        while (reported < NC - 1 || seen < NC) {
+            bool progress = false;
+            const int c = seen + lane;
+            const bool up = lane < g.R && c < NC && ld_acquire_gpu(&ready[c % g.R]) >= c + 1;
+            const int n = __ffs(~__ballot_sync(0xffffffffu, up)) - 1;      // (leading chunks that are ready; -1 means all 32)
+            if (n != 0) {
+                seen += n < 0 ? 32 : n;
+                __threadfence();
+                __syncwarp();
+                if (lane == 0) *vis = seen;
+                progress = true;
+            }
+            const int chunks_done = __shfl_sync(0xffffffffu, *odone, 0) >> 2;
+            if (chunks_done - 1 > reported) {
+                reported = chunks_done - 1;
+                if (lane == 0) {
                     __threadfence_block();
                     st_release_gpu(&ws.consumed[seq * 32], reported);
-                    progress = true;
                 }
-                if (progress) {
-                    t_last = clock64();
-                } else if (clock64() - t_last > WAIT_CYCLES) {
+                progress = true;
+            }
+            int stop = 0;
+            if (progress) {
+                t_last = clock64();
+            } else if (lane == 0) {
+                if (clock64() - t_last > WAIT_CYCLES) {
                     atomicCAS(err, 0, 232);
-                    break;
+                    stop = 1;
                 } else if (*(volatile int*)err != 0) {
-                    break;
+                    stop = 1;
                 } else if (seen == NC) {
                     __nanosleep(200);
                 }
             }
+            if (__shfl_sync(0xffffffffu, stop, 0)) break;
         }
     }
 }
@@ -846,11 +858,11 @@ fused_kernel(const __grid_constant__ FusedMaps maps, FusedGeo g, FusedWs ws, con
     if (tid == 0) {
         if (is_scan) {
             for (int x = 0; x < 2; ++x) {
-                mbar_init(&bar[B_EFULL + x], 1); mbar_init(&bar[B_EEMPTY + x], 1);
+                mbar_init(&bar[B_EQFULL + x], 1); mbar_init(&bar[B_EQEMPTY + x], 1);
                 mbar_init(&bar[B_XIFULL + x], 1); mbar_init(&bar[B_XIEMPTY + x], 8);
-                mbar_init(&bar[B_QTFULL + x], 1); mbar_init(&bar[B_QTEMPTY + x], 1);
+                if (x == 0) { mbar_init(&bar[B_DDONE], 1); mbar_init(&bar[B_SPUB], 8); }
                 mbar_init(&bar[B_APUB + x], 1); mbar_init(&bar[B_S16FREE + x], 1);
-                mbar_init(&bar[B_DDONE + x], 1); mbar_init(&bar[B_ODONE + x], 1); mbar_init(&bar[B_OFREE + x], 128);
+                mbar_init(&bar[B_ODONE + x], 1); mbar_init(&bar[B_OFREE + x], 128);
             }
         } else {
             for (int x = 0; x < 2; ++x) {
@@ -896,13 +908,22 @@ fused_kernel(const __grid_constant__ FusedMaps maps, FusedGeo g, FusedWs ws, con
     if (warp == 0) tmem_dealloc(tb, 512);
 }
 
-// Slots per sequence (pf_params.ring_depth, 3..64).  Default 8; 16 for long sequences while all rings together stay
-// well inside the L2: over a thousand chunks the flow CTAs drift apart and a deeper ring absorbs it (measured at
-// 32 sequences of 1024 chunks: 2.29 ms against 2.50 ms; no difference at 128 chunks).
+// Time of a chunk in us, measured: the scan's step, and what the CTAs that do not scan need to build a chunk of every sequence.
+constexpr double SCAN_US = 1.15;
+double build_us(const Problem& p) {
+    const double nseq = (double)p.B * p.H, flows = sm_count() - nseq;
+    return (p.tile_rows() == 128 ? 5.9 : 3.6) * nseq / (flows > 1 ? flows : 1);
+}
+
+// Slots per sequence (pf_params.ring_depth, 3..64).  A slot is busy from the moment a flow CTA may write it until the scan's
+// report of its consumption has come back, 12 - 14 k cycles of latency in all, so that 8 slots hold the scan to one chunk per
+// 1.75 k cycles and more: 16 where the scan is what bounds the kernel (4 sequences of 256 chunks: 423 us with 8 slots, 306 with
+// 16) or where over many chunks the flow CTAs drift apart (32 sequences of 1024 chunks: 2.50 against 2.29 ms), while all rings
+// together stay well inside the L2.  Elsewhere 8: the deeper ring costs L2 (32 sequences of 128 chunks, r = 2: 272 against 281).
 int ring_depth(const Problem& p) {
     const int NC = p.chunks_per_seq();
     int want = p.ring_depth;
-    if (want <= 0) want = (NC > 256 && (size_t)p.B * p.H * 16 * SLOT_BYTES <= ((size_t)48 << 20)) ? 16 : 8;
+    if (want <= 0) want = (NC > 256 || build_us(p) < SCAN_US) && (size_t)p.B * p.H * 16 * SLOT_BYTES <= ((size_t)48 << 20) ? 16 : 8;
     return NC < want ? (NC < 1 ? 1 : NC) : want;
 }
 
@@ -924,13 +945,10 @@ Carve carve(const Problem& p) {
 
 }  // namespace
 
-// An estimate of the kernel's time in us: the first flow, then per chunk either the scan's step or the time in which the CTAs
-// that do not scan build a chunk of every sequence, whichever is longer.
+// An estimate of the kernel's time in us: the first flow, then per chunk whichever is longer of the two above.
 double fused_estimate_us(const Problem& p) {
-    const double nseq = (double)p.B * p.H, flows = sm_count() - nseq;
-    const double flow = p.tile_rows() == 128 ? 5.9 : 3.6, step = 1.35;
-    const double build = flow * nseq / flows;
-    return 24.0 + p.chunks_per_seq() * (build > step ? build : step);
+    const double build = build_us(p);
+    return 22.0 + p.chunks_per_seq() * (build > SCAN_US ? build : SCAN_US);
 }
 
 bool fused_supported(const Problem& p) {
