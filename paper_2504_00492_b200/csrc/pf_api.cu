@@ -201,7 +201,7 @@ bool use_chain(const Problem& p, int impl) {
 
 // what the kernels of `impl` carve up (the fp32 step sizes of PF_STEP_EXACT follow it)
 size_t kernel_workspace_need(const Problem& p, int impl) {
-    if (use_chain(p, impl)) return 1024;       // (word 0 of a caller's workspace is the status word)
+    if (use_chain(p, impl)) return chain_workspace_bytes(p);
     if (impl == PF_IMPL_TC) return use_fused(p) ? fused_workspace_bytes(p) : tc_workspace_bytes(p);
     if (impl == PF_IMPL_TC_SPLIT) return tc_workspace_bytes(p);
     if (impl == PF_IMPL_TC_REFFLOW) return tc_refflow_workspace_bytes(p);
@@ -301,7 +301,7 @@ int forward_one(const pf_params* a, bool top) {
     bool own = false;
     if (ws) {
         if (a->workspace_bytes < need || ((uintptr_t)ws & 255u)) return PF_ERR_WORKSPACE;
-    } else if (need > 0 && !use_recur(p, impl) && !use_chain(p, impl)) {
+    } else if (need > 0 && !use_recur(p, impl) && (!use_chain(p, impl) || chain_needs_workspace(p))) {
         st = workspace_alloc(&ws, need, p.stream);
         if (st != PF_OK) return st;
         own = true;
@@ -318,7 +318,12 @@ int forward_one(const pf_params* a, bool top) {
         }
     }
     if (use_recur(p, impl) || use_chain(p, impl)) {
-        st = use_recur(p, impl) ? recur_forward(p) : chain_forward(p);
+        p.clear_status = top;
+        st = use_recur(p, impl) ? recur_forward(p) : chain_forward(p, ws);
+        if (own) {
+            cudaError_t e = cudaFreeAsync(ws, p.stream);
+            if (e != cudaSuccess && st == PF_OK) st = record_cuda_error(e, "cudaFreeAsync");
+        }
         if (st == PF_OK && top) end_call();
         return st;
     }

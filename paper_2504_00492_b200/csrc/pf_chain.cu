@@ -44,8 +44,10 @@ struct ChainMaps {
 
 struct ChainGeo {
     int L, d_v, nblk;
+    int nseg, seg_blk;  // segments per sequence (1: none) and blocks per segment
     int rm;             // strict-mask group size (Problem::mask_group)
     int exact;          // PF_STEP_EXACT
+    int clear;          // set the status word to 0
 };
 
 __device__ __forceinline__ uint32_t movmatrix(uint32_t x) {
@@ -57,6 +59,9 @@ __device__ __forceinline__ uint32_t movmatrix(uint32_t x) {
 __device__ __forceinline__ void store2_if(float* p, float x, float y, bool pred) {
     asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\t@p st.global.v2.f32 [%0], {%1, %2};\n\t}" ::"l"(p), "f"(x), "f"(y),
                  "r"((unsigned)pred));
+}
+__device__ __forceinline__ void store_h2_if(__half* p, uint32_t x, bool pred) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p st.global.u32 [%0], %1;\n\t}" ::"l"(p), "r"(x), "r"((unsigned)pred));
 }
 // eight bf16 -> eight fp16 (sign: 0x80008000 to negate them)
 __device__ __forceinline__ uint4 bf16_to_half8(uint4 x, uint32_t sign) {
@@ -98,19 +103,31 @@ constexpr int chain_stages() {
     return n < 6 ? n : 6;
 }
 
-// K, Q and V of block b into stage b mod NS (one thread); rows past the sequence arrive as zeros
+// What one CTA of the kernel works on.
+struct ChainPart {
+    int b0, nblk;       // first block of the sequence's, number of blocks
+    int j0;             // first of its JS rows j of the state
+    int width;          // d_v, or d_k for the response to the segment's start state
+    bool response;
+    const float* S0;    // start state of this sequence, or null
+    float* O;           // rows of O of the first block (response: fp16 rows)
+    float* S_end;       // end state [i][j] (response: fp16 [j][i]), or null
+};
+
+// K, Q and V of block b (of this part) into stage b mod NS (one thread); rows past the sequence arrive as zeros
 template <int DK, int R, int JS, int NS>
-__device__ __forceinline__ void load_block(const ChainMaps& maps, uint8_t* smem, uint64_t* land, int b, int seq, int j0) {
+__device__ __forceinline__ void load_block(const ChainMaps& maps, uint8_t* smem, uint64_t* land, int b, int seq, const ChainPart& part) {
     using SM = ChainSmem<DK, R, JS>;
     const int st = b % NS;
     uint8_t* sg = smem + st * SM::stage;
-    mbar_expect_tx(&land[st], SM::tx_bytes);
-    tma_load_4d(sg + SM::k_off, &maps.k, 0, b * SM::C * R, 0, seq, &land[st]);
+    const int bb = part.b0 + b;
+    mbar_expect_tx(&land[st], SM::tx_bytes - (part.response ? SM::v_bytes : 0));
+    tma_load_4d(sg + SM::k_off, &maps.k, 0, bb * SM::C * R, 0, seq, &land[st]);
     // (r = 3: a block's 21 tokens sit in slabs of 32 rows, one copy each)
     constexpr int QS = SM::CP == SM::C ? 1 : DK / 64;
 #pragma unroll
-    for (int h = 0; h < QS; ++h) tma_load_4d(sg + SM::q_off + h * (SM::CP * 128), &maps.q, 0, b * SM::C, h, seq, &land[st]);
-    tma_load_4d(sg + SM::v_off, &maps.v, 0, b * SM::C * R, j0 / (JS < 64 ? JS : 64), seq, &land[st]);
+    for (int h = 0; h < QS; ++h) tma_load_4d(sg + SM::q_off + h * (SM::CP * 128), &maps.q, 0, bb * SM::C, h, seq, &land[st]);
+    if (!part.response) tma_load_4d(sg + SM::v_off, &maps.v, 0, bb * SM::C * R, part.j0 / (JS < 64 ? JS : 64), seq, &land[st]);
 }
 // offset of the 16-byte piece c8 (= column / 8) of row `row` of the V tile: 128-byte rows (JS >= 64) or 64-byte rows
 template <int JS>
@@ -191,7 +208,7 @@ __device__ __forceinline__ void gram_blocks(uint32_t k_b, uint32_t q_b, uint8_t*
 // prep team: blocks b = team, team + TEAMS, ...
 // ---------------------------------------------------------------------------------------------------------------------
 template <int DK, int R, int JS, int IS, int TEAMS, int NS>
-__device__ __forceinline__ void prep_role(const ChainGeo& g, const __nv_bfloat16* __restrict__ beta, int* err, uint8_t* smem,
+__device__ __forceinline__ void prep_role(const ChainGeo& g, const ChainPart& part, const __nv_bfloat16* __restrict__ beta, int* err, uint8_t* smem,
                                           uint64_t* land, uint64_t* full, long long seq, int team, int tid) {
     using CFG = ChainCfg<DK, R, JS, IS, TEAMS, NS>;
     using SM = ChainSmem<DK, R, JS>;
@@ -207,11 +224,11 @@ __device__ __forceinline__ void prep_role(const ChainGeo& g, const __nv_bfloat16
     const uint32_t offT = lane_off((lane & 7) + (((lane >> 3) & 1) << 3), lane >> 4);
     const __nv_bfloat16* bs = beta + seq * L * R;
     auto read_beta = [&](int b) {                                 // rows past the block or the sequence have step size zero
-        return tid < min(C, L - b * C) * R ? __bfloat162float(bs[(long long)b * C * R + tid]) : 0.f;
+        return tid < min(C, L - (part.b0 + b) * C) * R ? __bfloat162float(bs[(long long)(part.b0 + b) * C * R + tid]) : 0.f;
     };
-    float breg = team < g.nblk ? read_beta(team) : 0.f;
+    float breg = team < part.nblk ? read_beta(team) : 0.f;
 #pragma unroll 1
-    for (int b = team; b < g.nblk; b += TEAMS) {
+    for (int b = team; b < part.nblk; b += TEAMS) {
         const int st = b % NS;
         uint8_t* sg = smem + st * SM::stage;
         const uint32_t k_b = smem_u32(sg + SM::k_off), q_b = smem_u32(sg + SM::q_off);
@@ -235,7 +252,7 @@ __device__ __forceinline__ void prep_role(const ChainGeo& g, const __nv_bfloat16
         }
         fence_async_smem();                                       // (the stage's next copy is ordered after these writes)
         if (tid < NB) sBeta[tid] = breg;
-        if (b + TEAMS < g.nblk) breg = read_beta(b + TEAMS);
+        if (b + TEAMS < part.nblk) breg = read_beta(b + TEAMS);
         if (!named_bar_and(bar_id, 128, ok)) return;
 
         // ---- G (row block w) and this warp's blocks of P
@@ -375,10 +392,9 @@ __device__ __forceinline__ void prep_role(const ChainGeo& g, const __nv_bfloat16
 // ---------------------------------------------------------------------------------------------------------------------
 // chain warp: rows j of the 16-column group `grp` of the CTA's JS columns, columns i of half `hi` (IS = 2)
 // ---------------------------------------------------------------------------------------------------------------------
-template <int DK, int R, int JS, int IS, int TEAMS, int NS>
-__device__ __forceinline__ void chain_role(const ChainMaps& maps, const ChainGeo& g, const float* __restrict__ S0, float* __restrict__ O,
-                                           float* __restrict__ S_final, int* err, uint8_t* smem, uint64_t* land, uint64_t* full,
-                                           uint64_t* empty, long long seq, int j0, int warp, int lane) {
+template <int DK, int R, int JS, int IS, int TEAMS, int NS, bool SEG>
+__device__ __forceinline__ void chain_role(const ChainMaps& maps, const ChainGeo& g, const ChainPart& part, int* err, uint8_t* smem,
+                                           uint64_t* land, uint64_t* full, uint64_t* empty, int seq, int warp, int lane) {
     using CFG = ChainCfg<DK, R, JS, IS, TEAMS, NS>;
     using SM = ChainSmem<DK, R, JS>;
     constexpr int C = SM::C, CP = SM::CP, TT = CP / 16;
@@ -397,13 +413,21 @@ __device__ __forceinline__ void chain_role(const ChainMaps& maps, const ChainGeo
     auto kxor = [&](int kk) { return (uint32_t)(((hi * KT + kk) & 3) << 5); };
 
     float S[2 * KT][4];                                           // [8 columns i][c]: rows j = gq, gq + 8, columns 2 t4, 2 t4 + 1
-    const int jr = j0 + 16 * grp + gq, i0 = hi * DI + 2 * t4;
+    const int jr = part.j0 + 16 * grp + gq, i0 = hi * DI + 2 * t4, width = part.width;
 #pragma unroll
     for (int n = 0; n < 2 * KT; ++n)
 #pragma unroll
-        for (int e = 0; e < 4; ++e)
-            S[n][e] = S0 ? S0[(seq * DK + i0 + 8 * n + (e & 1)) * g.d_v + jr + 8 * (e >> 1)] : 0.f;
-    float* ob = O + seq * (long long)g.L * g.d_v + j0 + 16 * grp + 2 * t4 + (IS == 2 ? 8 * hi : 0);     // O of the current block
+        for (int e = 0; e < 4; ++e) {
+            const int i = i0 + 8 * n + (e & 1), j = jr + 8 * (e >> 1);
+            if (SEG && part.response) S[n][e] = i == j ? 1.f : 0.f;
+            else S[n][e] = part.S0 ? part.S0[(long long)i * width + j] : 0.f;
+        }
+    float* ob = part.O + part.j0 + 16 * grp + 2 * t4 + (IS == 2 ? 8 * hi : 0);     // O of the current block (response: in halves)
+    __half* rb = (__half*)part.O + part.j0 + 16 * grp + 2 * t4 + (IS == 2 ? 8 * hi : 0);
+    auto put_o = [&](int t, int dj, float x, float y, bool pred) {     // token t of the current block
+        if (SEG && part.response) store_h2_if(rb + (long long)t * width + dj, pack_h2(x, y), pred);
+        else store2_if(ob + (long long)t * width + dj, x, y, pred);
+    };
 
     // IS = 2: what this warp keeps of O of the block before (8 of the 16 columns j), without the other warp's part of Q S^T
     float ok8[TT][4];
@@ -414,9 +438,8 @@ __device__ __forceinline__ void chain_role(const ChainMaps& maps, const ChainGeo
         for (int tt = 0; tt < TT; ++tt) {
             const float4 x = other[(8 + tt) * 32];
             const int t = 16 * tt + gq;
-            float* o0 = ob + (long long)(t - C) * g.d_v;
-            store2_if(o0, ok8[tt][0] + x.x, ok8[tt][1] + x.y, t < Cv_prev);
-            store2_if(o0 + 8ll * g.d_v, ok8[tt][2] + x.z, ok8[tt][3] + x.w, t + 8 < Cv_prev);
+            put_o(t - C, 0, ok8[tt][0] + x.x, ok8[tt][1] + x.y, t < Cv_prev);
+            put_o(t - C + 8, 0, ok8[tt][2] + x.z, ok8[tt][3] + x.w, t + 8 < Cv_prev);
         }
     };
     if (IS == 2)
@@ -429,7 +452,7 @@ __device__ __forceinline__ void chain_role(const ChainMaps& maps, const ChainGeo
 
     int st = 0, phase = 0, st_prev = 0, ph_prev = 0;
 #pragma unroll 1
-    for (int b = 0; b < g.nblk; ++b) {
+    for (int b = 0; b < part.nblk; ++b) {
         const uint32_t sg = smem_b + st * SM::stage;
         const uint32_t k_b = sg + SM::k_off, q_b = sg + SM::q_off, t_b = sg + SM::t_off, p_b = sg + SM::p_off, v_b = sg + SM::v_off;
         uint32_t s16[KT][4];                                      // fp16 copy of -S: A operand of -S K^T, B operand of (-Q)(-S)^T
@@ -489,8 +512,8 @@ __device__ __forceinline__ void chain_role(const ChainMaps& maps, const ChainGeo
             store8(other_o);
         }
         // ---- the block NS - 1 further on into the stage that every chain warp has left (a block ago)
-        if (warp == 0 && lane == 0 && b > 0 && b - 1 + NS < g.nblk && mbar_wait_clk(&empty[st_prev], (uint32_t)ph_prev, err, 314))
-            load_block<DK, R, JS, NS>(maps, smem, land, b - 1 + NS, (int)seq, j0);
+        if (warp == 0 && lane == 0 && b > 0 && b - 1 + NS < part.nblk && mbar_wait_clk(&empty[st_prev], (uint32_t)ph_prev, err, 314))
+            load_block<DK, R, JS, NS>(maps, smem, land, b - 1 + NS, seq, part);
         __syncwarp();
         // ---- U'^T = R T^T (T lower triangular)
         uint32_t r16[4][4];
@@ -529,7 +552,7 @@ __device__ __forceinline__ void chain_role(const ChainMaps& maps, const ChainGeo
                 mma_16816(S[2 * ip + 1], u16[kk], x[2], x[3]);
             }
         // ---- O = Q S^T + P U' with the state before the update, 16 tokens at a time (these products fill the latency of the update)
-        const int Cv = min(C, g.L - b * C);
+        const int Cv = min(C, g.L - (part.b0 + b) * C);
 #pragma unroll
         for (int tt = 0; tt < TT; ++tt) {
             float o[2][4];
@@ -564,15 +587,15 @@ __device__ __forceinline__ void chain_role(const ChainMaps& maps, const ChainGeo
                 for (int e = 0; e < 4; ++e) ok8[tt][e] = ot[e];
             } else {
                 const int t = 16 * tt + gq;
-                float* o0 = ob + (long long)t * g.d_v;
-                store2_if(o0, o[0][0], o[0][1], t < Cv);
-                store2_if(o0 + 8, o[1][0], o[1][1], t < Cv);
-                store2_if(o0 + 8ll * g.d_v, o[0][2], o[0][3], t + 8 < Cv);
-                store2_if(o0 + 8ll * g.d_v + 8, o[1][2], o[1][3], t + 8 < Cv);
+                put_o(t, 0, o[0][0], o[0][1], t < Cv);
+                put_o(t, 8, o[1][0], o[1][1], t < Cv);
+                put_o(t + 8, 0, o[0][2], o[0][3], t + 8 < Cv);
+                put_o(t + 8, 8, o[1][2], o[1][3], t + 8 < Cv);
             }
         }
         Cv_prev = Cv;
-        ob += (long long)C * g.d_v;
+        ob += (long long)C * width;
+        rb += (long long)C * width;
         __syncwarp();
         if (lane == 0) mbar_arrive(&empty[st]);
         st_prev = st;
@@ -584,34 +607,71 @@ __device__ __forceinline__ void chain_role(const ChainMaps& maps, const ChainGeo
     }
     if (IS == 2) {
         named_bar(1 + TEAMS + grp, 64);                           // (both warps are here: a failed wait left through the barrier above)
-        store8((const float4*)(exw + (((g.nblk & 1) ^ 1) * 2 + (hi ^ 1)) * (CFG::x_piece * 512)));
+        store8((const float4*)(exw + (((part.nblk & 1) ^ 1) * 2 + (hi ^ 1)) * (CFG::x_piece * 512)));
     }
-    if (S_final)
+    if (SEG && part.response) {
+        __half* P = (__half*)part.S_end;
 #pragma unroll
         for (int n = 0; n < 2 * KT; ++n)
 #pragma unroll
-            for (int e = 0; e < 4; ++e)
-                S_final[(seq * DK + i0 + 8 * n + (e & 1)) * g.d_v + jr + 8 * (e >> 1)] = S[n][e];
+            for (int e = 0; e < 4; e += 2) *(uint32_t*)(P + (long long)(jr + 4 * e) * DK + i0 + 8 * n) = pack_h2(S[n][e], S[n][e + 1]);
+    } else if (part.S_end) {
+#pragma unroll
+        for (int n = 0; n < 2 * KT; ++n)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) part.S_end[(long long)(i0 + 8 * n + (e & 1)) * width + jr + 8 * (e >> 1)] = S[n][e];
+    }
 }
 
-template <int DK, int R, int JS, int IS, int TEAMS, int NS>
+// Segments (Section 3, "Scan"; Proposition 2.1): the flow of an interval is the pair (P, Xi) with S_end = S_start P + Xi.  A
+// sequence is cut into segments that are walked side by side: for each the state from zero (S0 for the first segment), whose
+// outputs go to O and whose end is Xi, and, for all but the first, the state from the identity with v = 0, whose "outputs"
+// R_t = P_t q_t are what each token makes of its segment's start state and whose end is P.  Then one kernel composes the
+// segments' start states and another adds start R_t to O.
+struct ChainSeg {
+    __half* R;          // [nseq][L][d_k]
+    __half* P;          // [nseq][nseg][d_k j][d_k i]
+    float* Xi;          // [nseq][nseg][d_k i][d_v j]
+    __half* start;      // [nseq][nseg][d_v j][d_k i]
+};
+
+template <int DK, int R, int JS, int IS, int TEAMS, int NS, bool SEG>
 __global__ void __launch_bounds__(ChainCfg<DK, R, JS, IS, TEAMS, NS>::threads, 1)
 chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __restrict__ beta, const float* __restrict__ S0,
-             float* __restrict__ O, float* __restrict__ S_final, int* __restrict__ status, ChainGeo g) {
+             float* __restrict__ O, float* __restrict__ S_final, int* __restrict__ status, ChainGeo g, ChainSeg sg) {
     using CFG = ChainCfg<DK, R, JS, IS, TEAMS, NS>;
     using SM = ChainSmem<DK, R, JS>;
     extern __shared__ __align__(1024) uint8_t smem[];
     __shared__ uint64_t land[NS], full[NS], empty[NS];
     const int tid = threadIdx.x, warp = tid >> 5;
     const int slices = g.d_v / JS;
-    const long long seq = blockIdx.x / slices;
-    const int j0 = (int)(blockIdx.x % slices) * JS;
+    long long seq;
+    ChainPart part;
+    if (!SEG) {
+        seq = blockIdx.x / slices;
+        part = {0, g.nblk, (int)(blockIdx.x % slices) * JS, g.d_v, false, S0 ? S0 + seq * DK * g.d_v : nullptr,
+                O + seq * g.L * g.d_v, S_final ? S_final + seq * DK * g.d_v : nullptr};
+    } else {
+        constexpr int rs = DK / JS;
+        const int per_seq = g.nseg * slices + (g.nseg - 1) * rs, x = (int)(blockIdx.x % per_seq), y = x - g.nseg * slices;
+        seq = blockIdx.x / per_seq;
+        part.response = y >= 0;
+        const int s = part.response ? 1 + y / rs : x / slices;
+        part.b0 = s * g.seg_blk;
+        part.nblk = min(g.seg_blk, g.nblk - part.b0);
+        part.j0 = (part.response ? y % rs : x % slices) * JS;
+        part.width = part.response ? DK : g.d_v;
+        const long long row0 = seq * g.L + (long long)part.b0 * SM::C, slot = seq * g.nseg + s;
+        part.S0 = s == 0 && S0 ? S0 + seq * DK * g.d_v : nullptr;
+        part.O = part.response ? (float*)(sg.R + row0 * DK) : O + row0 * g.d_v;
+        part.S_end = part.response ? (float*)(sg.P + slot * DK * DK) : sg.Xi + slot * DK * g.d_v;
+    }
     if ((smem_u32(smem) & 1023u) != 0) {                          // (the swizzled layouts need a 1024-byte aligned base)
         if (tid == 0) atomicCAS(status, 0, 99);
         return;
     }
     if (tid == 0) {
-        if (blockIdx.x == 0) *status = 0;                         // (the call's status word: a wait expires a second from now at the earliest)
+        if (blockIdx.x == 0 && g.clear) *status = 0;                      // (the call's status word: a wait expires a second from now at the earliest)
         for (int x = 0; x < NS; ++x) {
             mbar_init(&land[x], 1);
             mbar_init(&full[x], 128);
@@ -622,38 +682,237 @@ chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __rest
         prefetch_tmap(&maps.k);
         prefetch_tmap(&maps.v);
     }
-    if (SM::CP > SM::C) {                                         // (r = 3: query rows that no copy writes are read)
+    if (SM::CP > SM::C || part.response) {                        // (r = 3: query rows that no copy writes are read; a response: v = 0)
         for (int e = tid; e < NS * SM::stage / 16; e += CFG::threads) ((uint4*)smem)[e] = make_uint4(0, 0, 0, 0);
         fence_async_smem();
     }
     __syncthreads();
     if (tid == 0)
-        for (int b = 0; b < NS && b < g.nblk; ++b) load_block<DK, R, JS, NS>(maps, smem, land, b, (int)seq, j0);
+        for (int b = 0; b < NS && b < part.nblk; ++b) load_block<DK, R, JS, NS>(maps, smem, land, b, (int)seq, part);
     __syncwarp();
     if (warp < CFG::NCW)
-        chain_role<DK, R, JS, IS, TEAMS, NS>(maps, g, S0, O, S_final, status, smem, land, full, empty, seq, j0, warp, tid & 31);
+        chain_role<DK, R, JS, IS, TEAMS, NS, SEG>(maps, g, part, status, smem, land, full, empty, (int)seq, warp, tid & 31);
     else
-        prep_role<DK, R, JS, IS, TEAMS, NS>(g, beta, status, smem, land, full, seq, (warp - CFG::NCW) >> 2, (tid - 32 * CFG::NCW) & 127);
+        prep_role<DK, R, JS, IS, TEAMS, NS>(g, part, beta, status, smem, land, full, seq, (warp - CFG::NCW) >> 2, (tid - 32 * CFG::NCW) & 127);
 }
 
-template <int DK, int R, int JS, int IS, int TEAMS>
-int launch(const Problem& p) {
+// Start states of the segments: one CTA per sequence and 16 rows j, serial over the segments; four warps with a quarter of the
+// columns i each.  start(1) = Xi_0, start(s+1) = start(s) P_s + Xi_s; the last one is S_final.  The next P comes while the present
+// one is used.
+template <int DK>
+__global__ void __launch_bounds__(128) chain_compose(ChainSeg sg, float* __restrict__ S_final, int nseg, int d_v) {
+    constexpr int LD = DK + 8, NT = DK / 32, PIECES = DK * DK / 8 / 128;
+    extern __shared__ __align__(16) uint8_t smem[];
+    __half* sP = (__half*)smem;                                   // [2][DK][LD]
+    __half* sA = sP + 2 * DK * LD;                                // [2][16][LD]  fp16 rows of the start state
+    const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31, gq = lane >> 2, t4 = lane & 3;
+    const int groups = d_v / 16;
+    const long long seq = blockIdx.x / groups;
+    const int j = (int)(blockIdx.x % groups) * 16 + gq, i0 = w * (DK / 4) + 2 * t4;
+    auto load_p = [&](int s) {
+        const __half* src = sg.P + (seq * nseg + s) * DK * DK;
+        __half* dst = sP + (s & 1) * DK * LD;
+#pragma unroll
+        for (int e = 0; e < PIECES; ++e) {
+            const int p = e * 128 + tid, row = p / (DK / 8), c = p % (DK / 8);
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst + row * LD + c * 8)), "l"(src + row * DK + c * 8) : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    float S[NT][4];
+    auto xi = [&](int s, float (&x)[NT][4]) {
+        const float* src = sg.Xi + (seq * nseg + s) * DK * d_v;
+#pragma unroll
+        for (int n = 0; n < NT; ++n)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) x[n][e] = src[(long long)(i0 + 8 * n + (e & 1)) * d_v + j + 8 * (e >> 1)];
+    };
+    load_p(1);
+    xi(0, S);
+    for (int s = 1; s < nseg; ++s) {
+        __half* a_s = sA + (s & 1) * 16 * LD;
+        __half* out = sg.start + (seq * nseg + s) * d_v * DK;
+#pragma unroll
+        for (int n = 0; n < NT; ++n)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const uint32_t x = pack_h2(S[n][2 * h], S[n][2 * h + 1]);
+                *(uint32_t*)(a_s + (gq + 8 * h) * LD + i0 + 8 * n) = x;
+                *(uint32_t*)(out + (long long)(j + 8 * h) * DK + i0 + 8 * n) = x;
+            }
+        xi(s, S);
+        if (s + 1 < nseg) {
+            load_p(s + 1);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+        __syncthreads();
+        const __half* P = sP + (s & 1) * DK * LD;
+#pragma unroll
+        for (int kk = 0; kk < DK / 16; ++kk) {
+            uint32_t a[4];
+            ldmatrix_x4(a, smem_u32(a_s + (lane & 15) * LD + 16 * kk + 8 * (lane >> 4)));
+#pragma unroll
+            for (int np = 0; np < NT / 2; ++np) {
+                uint32_t x[4];
+                ldmatrix_x4_trans(x, smem_u32(P + (16 * kk + (lane & 7) + (((lane >> 3) & 1) << 3)) * LD + w * (DK / 4) + 16 * np + 8 * (lane >> 4)));
+                mma_16816(S[2 * np], a, x[0], x[1]);
+                mma_16816(S[2 * np + 1], a, x[2], x[3]);
+            }
+        }
+        __syncthreads();                                          // (P of this step is replaced after the next one's first barrier)
+    }
+    if (S_final) {
+        float* out = S_final + seq * DK * d_v;
+#pragma unroll
+        for (int n = 0; n < NT; ++n)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) out[(long long)(i0 + 8 * n + (e & 1)) * d_v + j + 8 * (e >> 1)] = S[n][e];
+    }
+}
+
+// O[t][j] += sum_i R[t][i] start[j][i] for the tokens of all segments but the first: grid (128-token tiles, nseq (nseg - 1)), a
+// warp per 16 tokens.  Bound by the traffic: per token R once, O read and written.
+template <int DK, int DV>
+__global__ void __launch_bounds__(256) chain_apply(ChainSeg sg, float* __restrict__ O, int L, int seg_tokens, int nseg) {
+    constexpr int LD = DK + 8, KT = DK / 16;
+    extern __shared__ __align__(16) uint8_t smem[];
+    __half* sS = (__half*)smem;                                   // [DV][LD]
+    const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31, gq = lane >> 2, t4 = lane & 3;
+    const long long seq = blockIdx.y / (nseg - 1);
+    const int s = 1 + (int)(blockIdx.y % (nseg - 1));
+    const int t_end = min(L, (s + 1) * seg_tokens), t0 = s * seg_tokens + blockIdx.x * 128 + w * 16 + gq;
+    const __half* src = sg.start + (seq * nseg + s) * DV * DK;
+#pragma unroll
+    for (int e = 0; e < DV * DK / 8 / 256; ++e) {
+        const int p = e * 256 + tid, row = p / (DK / 8), c = p % (DK / 8);
+        *(uint4*)(sS + row * LD + c * 8) = *(const uint4*)(src + row * DK + c * 8);
+    }
+    uint32_t a[KT][4];
+    const bool in0 = t0 < t_end, in1 = t0 + 8 < t_end;
+    const __half* r0 = sg.R + (seq * L + t0) * DK + 2 * t4;
+#pragma unroll
+    for (int kk = 0; kk < KT; ++kk) {
+        a[kk][0] = in0 ? *(const uint32_t*)(r0 + 16 * kk) : 0u;
+        a[kk][1] = in1 ? *(const uint32_t*)(r0 + 8 * DK + 16 * kk) : 0u;
+        a[kk][2] = in0 ? *(const uint32_t*)(r0 + 16 * kk + 8) : 0u;
+        a[kk][3] = in1 ? *(const uint32_t*)(r0 + 8 * DK + 16 * kk + 8) : 0u;
+    }
+    __syncthreads();
+    float* o0 = O + (seq * L + t0) * DV + 2 * t4;
+#pragma unroll
+    for (int np = 0; np < DV / 16; ++np) {
+        float c[2][4];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float2 x = in0 ? *(const float2*)(o0 + 16 * np + 8 * h) : make_float2(0.f, 0.f);
+            const float2 y = in1 ? *(const float2*)(o0 + 8 * DV + 16 * np + 8 * h) : make_float2(0.f, 0.f);
+            c[h][0] = x.x; c[h][1] = x.y; c[h][2] = y.x; c[h][3] = y.y;
+        }
+#pragma unroll
+        for (int kk = 0; kk < KT; ++kk) {
+            uint32_t x[4];
+            ldmatrix_x4(x, smem_u32(sS + (16 * np + (lane & 7) + ((lane >> 4) << 3)) * LD + 16 * kk + 8 * ((lane >> 3) & 1)));
+            mma_16816(c[0], a[kk], x[0], x[1]);
+            mma_16816(c[1], a[kk], x[2], x[3]);
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            if (in0) *(float2*)(o0 + 16 * np + 8 * h) = make_float2(c[h][0], c[h][1]);
+            if (in1) *(float2*)(o0 + 8 * DV + 16 * np + 8 * h) = make_float2(c[h][2], c[h][3]);
+        }
+    }
+}
+
+// How a sequence is spread over CTAs: columns per CTA, and segments.  The time is (waves of CTAs) x (blocks of a segment) x
+// (time of a block), plus what composing segments costs.
+// Columns: fewer per CTA make a shorter step but more CTAs.  Measured with one wave at L = 1024 (us for d_k = d_v = 128, r = 2 and
+// r = 4): 32 columns by pairs of warps 67, 117; 64 columns 86, 140; 128 columns 125, 225.  At d_k = 64 a step is short enough that 32
+// columns gain nothing over 64 (51 against 53 us), and 128 columns cost 1.3 times as much.
+// Segments: as many as one wave of CTAs holds pay for the second walk (the responses) and for two more kernels when few
+// sequences are long: taken where the estimate falls by a quarter at least.
+enum { COLS_32, COLS_64, COLS_128 };
+struct ChainPlan {
+    int cols, nseg, seg_blk;
+    double us;
+};
+ChainPlan make_plan(const Problem& p) {
+    static const double step[2][4] = {{2.25, 1.65, 1.7, 1.46}, {3.3, 2.6, 2.6, 2.15}};      // us per block, 64 columns, d_k = 64 and 128
+    const long long nseq = (long long)p.B * p.H, sms = sm_count();
+    const int C = NB / p.r, nblk = (p.L + C - 1) / C;
+    const double st = step[p.d_k == 128][p.r - 1];
+    auto waves = [&](int js) { return (double)((nseq * (p.d_v / js) + sms - 1) / (sms > 0 ? sms : 1)); };
+    double best = waves(64);
+    ChainPlan plan{COLS_64, 1, nblk, 0.0};
+    if (p.d_k == 128 && 0.8 * waves(32) < best) {
+        best = 0.8 * waves(32);
+        plan.cols = COLS_32;
+    }
+    if (p.d_v == 128) {
+        const double w = (p.d_k == 128 ? 1.5 : 1.3) * waves(128);
+        if (w < best) {
+            best = w;
+            plan.cols = COLS_128;
+        }
+    }
+    plan.us = 6.0 + nblk * st * best;
+    const double limit = 0.75 * plan.us;
+    // (kernels and their gaps, then the traffic of the responses and of O at about 4 TB/s)
+    const double extra = 16.0 + 6.0 + (double)nseq * p.L * (4.0 * p.d_k + 8.0 * p.d_v) / 4e6;
+    for (int cols = p.d_k == 128 ? COLS_32 : COLS_64; cols <= COLS_64; ++cols) {
+        const int js = cols == COLS_32 ? 32 : 64, vs = p.d_v / js, rs = p.d_k / js;
+        const long long most = (sms / nseq + rs) / (vs + rs);
+        for (int want = 2; want <= most && want <= 64 && want <= nblk; ++want) {
+            const int seg_blk = (nblk + want - 1) / want, nseg = (nblk + seg_blk - 1) / seg_blk;
+            const double us = extra + 0.8 * nseg + seg_blk * st * (cols == COLS_32 ? 0.8 : 1.0);
+            if (us < limit && us < plan.us) plan = {cols, nseg, seg_blk, us};
+        }
+    }
+    return plan;
+}
+
+struct ChainCarve {
+    size_t R, P, Xi, start, total;
+};
+ChainCarve carve(const Problem& p, const ChainPlan& plan) {
+    ChainCarve c{};
+    size_t off = 1024;                                            // (word 0 of a caller's workspace is the status word)
+    auto take = [&](size_t bytes) {
+        const size_t at = off;
+        off += align_up(bytes, 256);
+        return at;
+    };
+    if (plan.nseg > 1) {
+        const size_t nseq = (size_t)p.B * p.H, slots = nseq * plan.nseg;
+        c.R = take(nseq * p.L * p.d_k * 2);
+        c.P = take(slots * p.d_k * p.d_k * 2);
+        c.Xi = take(slots * p.d_k * p.d_v * 4);
+        c.start = take(slots * p.d_v * p.d_k * 2);
+    }
+    c.total = off;
+    return c;
+}
+
+template <int DK, int R, int JS, int IS, int TEAMS, bool SEG>
+int launch(const Problem& p, const ChainPlan& plan, const ChainSeg& sg) {
     constexpr int NS = chain_stages<DK, R, JS, IS, TEAMS>();
     using CFG = ChainCfg<DK, R, JS, IS, TEAMS, NS>;
     static_assert(CFG::total <= 227 * 1024 && NS >= 2, "shared memory budget");
-    const void* fn = (const void*)chain_kernel<DK, R, JS, IS, TEAMS, NS>;
+    const void* fn = (const void*)chain_kernel<DK, R, JS, IS, TEAMS, NS, SEG>;
     constexpr int C = NB / R;
-    ChainGeo g{p.L, p.d_v, (p.L + C - 1) / C, p.mask_group(), p.exact ? 1 : 0};
-    const long long nseq = (long long)p.B * p.H, grid = nseq * (p.d_v / JS);
+    ChainGeo g{p.L, p.d_v, (p.L + C - 1) / C, plan.nseg, plan.seg_blk, p.mask_group(), p.exact ? 1 : 0, p.clear_status ? 1 : 0};
+    const long long nseq = (long long)p.B * p.H, grid = nseq * (plan.nseg * (p.d_v / JS) + (plan.nseg - 1) * (DK / JS));
     ChainMaps maps;
     constexpr int VC = JS < 64 ? JS : 64;
-    if (!make_slab_map(&maps.k, p.k, nseq, (uint64_t)p.L * R, DK, 64, NB, DK / 64) || !make_slab_map(&maps.q, p.q, nseq, p.L, DK, 64, C, R == 3 ? 1 : DK / 64) ||
+    if (!make_slab_map(&maps.k, p.k, nseq, (uint64_t)p.L * R, DK, 64, NB, DK / 64) ||
+        !make_slab_map(&maps.q, p.q, nseq, p.L, DK, 64, C, R == 3 ? 1 : DK / 64) ||
         !make_slab_map(&maps.v, p.v, nseq, (uint64_t)p.L * R, p.d_v, VC, NB, JS / VC))
         return record_cuda_error(cudaErrorInvalidValue, "cuTensorMapEncodeTiled");
     static std::atomic<uint64_t> opted_in{0};
     const int st = allow_smem(opted_in, fn, CFG::total);
     if (st != PF_OK) return st;
-    void* args[] = {(void*)&maps, (void*)&p.beta, (void*)&p.S0, (void*)&p.O, (void*)&p.S_final, (void*)&p.status, (void*)&g};
+    void* args[] = {(void*)&maps, (void*)&p.beta, (void*)&p.S0, (void*)&p.O, (void*)&p.S_final, (void*)&p.status, (void*)&g, (void*)&sg};
     prof_begin("chain", p.stream);
     PF_CUDA_TRY(cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(CFG::threads), args, (size_t)CFG::total, p.stream));
     prof_end(p.stream);
@@ -661,64 +920,76 @@ int launch(const Problem& p) {
     return PF_OK;
 }
 
-// How a sequence's d_v columns are spread over CTAs.  Fewer columns per CTA make a shorter step but more CTAs; the time is
-// (waves of CTAs) x (time of a step).  Steps relative to each other, measured with one wave at L = 1024 (us for d_k = d_v =
-// 128, r = 2 and r = 4): 32 columns by pairs of warps 67, 117; 64 columns 86, 140; 128 columns 125, 225.  At d_k = 64 a step is
-// short enough that 32 columns gain nothing over 64 (51 against 53 us), and 128 columns cost 1.3 times as much.
-enum { COLS_32, COLS_64, COLS_128 };
-struct Spread {
-    int cols;
-    double waves_x_step;      // in steps of COLS_64
-};
-Spread pick_spread(const Problem& p) {
-    const long long nseq = (long long)p.B * p.H, sms = sm_count();
-    auto waves = [&](int js) { return (double)((nseq * (p.d_v / js) + sms - 1) / sms); };
-    Spread s{COLS_64, waves(64)};
-    if (p.d_k == 128 && 0.8 * waves(32) < s.waves_x_step) s = {COLS_32, 0.8 * waves(32)};
-    if (p.d_v == 128) {
-        const double w = (p.d_k == 128 ? 1.5 : 1.3) * waves(128);
-        if (w < s.waves_x_step) s = {COLS_128, w};
+template <int DK, int R>
+int launch_plan(const Problem& p, const ChainPlan& plan, const ChainSeg& sg) {
+    if (plan.nseg > 1) {
+        if constexpr (DK == 128)
+            if (plan.cols == COLS_32) return launch<DK, R, 32, 2, 2, true>(p, plan, sg);
+        return launch<DK, R, 64, 1, 2, true>(p, plan, sg);
     }
-    return s;
+    if constexpr (DK == 128)
+        if (plan.cols == COLS_32) return launch<DK, R, 32, 2, 2, false>(p, plan, sg);
+    if (plan.cols == COLS_64) return launch<DK, R, 64, 1, 2, false>(p, plan, sg);
+    return launch<DK, R, 128, 1, DK == 64 ? 2 : 1, false>(p, plan, sg);
+}
+template <int DK>
+int launch_rank(const Problem& p, const ChainPlan& plan, const ChainSeg& sg) {
+    switch (p.r) {
+        case 1: return launch_plan<DK, 1>(p, plan, sg);
+        case 2: return launch_plan<DK, 2>(p, plan, sg);
+        case 3: return launch_plan<DK, 3>(p, plan, sg);
+        default: return launch_plan<DK, 4>(p, plan, sg);
+    }
 }
 
-template <int DK, int R>
-int launch_spread(const Problem& p) {
-    switch (pick_spread(p).cols) {
-        case COLS_32:
-            if constexpr (DK == 128) return launch<DK, R, 32, 2, 2>(p);
-        case COLS_64: return launch<DK, R, 64, 1, 2>(p);
-        default: return launch<DK, R, 128, 1, DK == 64 ? 2 : 1>(p);
+template <int DK, int DV>
+int launch_seg_tail(const Problem& p, const ChainPlan& plan, const ChainSeg& sg) {
+    const int nseq = p.B * p.H, seg_tokens = plan.seg_blk * (NB / p.r);
+    constexpr int LD = DK + 8;
+    {
+        constexpr int smem = (2 * DK + 2 * 16) * LD * 2;
+        static std::atomic<uint64_t> opted_in{0};
+        const int st = allow_smem(opted_in, (const void*)chain_compose<DK>, smem);
+        if (st != PF_OK) return st;
+        prof_begin("chain_compose", p.stream);
+        chain_compose<DK><<<(unsigned)(nseq * (DV / 16)), 128, smem, p.stream>>>(sg, p.S_final, plan.nseg, DV);
+        prof_end(p.stream);
+        PF_CUDA_TRY(cudaGetLastError());
     }
+    constexpr int smem = DV * LD * 2;
+    prof_begin("chain_apply", p.stream);
+    chain_apply<DK, DV><<<dim3((unsigned)((seg_tokens + 127) / 128), (unsigned)(nseq * (plan.nseg - 1))), 256, smem, p.stream>>>(
+        sg, p.O, p.L, seg_tokens, plan.nseg);
+    prof_end(p.stream);
+    PF_CUDA_TRY(cudaGetLastError());
+    count_launch(2);
+    return PF_OK;
 }
 
 }  // namespace
 
-// An estimate of the kernel's time in us, for the choice between it and the single-launch tcgen05 kernel.
-double chain_estimate_us(const Problem& p) {
-    static const double step[4] = {3.3, 2.6, 2.6, 2.15};     // one block, COLS_64, d_k = 128
-    const int C = NB / p.r;
-    return 6.0 + (double)((p.L + C - 1) / C) * step[p.r - 1] * pick_spread(p).waves_x_step;
-}
+double chain_estimate_us(const Problem& p) { return make_plan(p).us; }
+
+size_t chain_workspace_bytes(const Problem& p) { return carve(p, make_plan(p)).total; }
+bool chain_needs_workspace(const Problem& p) { return make_plan(p).nseg > 1; }
 
 bool chain_supported(const Problem& p) {
     return p.in_dtype == PF_DTYPE_BF16 && p.L >= 1 && (long long)p.B * p.H * (p.d_v / 32) <= 0x7fffffffLL &&
            (long long)p.L * p.r <= 0x7fffffffLL;
 }
 
-int chain_forward(const Problem& p) {
-    if (p.d_k == 128) switch (p.r) {
-        case 1: return launch_spread<128, 1>(p);
-        case 2: return launch_spread<128, 2>(p);
-        case 3: return launch_spread<128, 3>(p);
-        default: return launch_spread<128, 4>(p);
+int chain_forward(const Problem& p, void* workspace) {
+    const ChainPlan plan = make_plan(p);
+    ChainSeg sg{};
+    if (plan.nseg > 1) {
+        const ChainCarve c = carve(p, plan);
+        uint8_t* ws = (uint8_t*)workspace;
+        sg = {(__half*)(ws + c.R), (__half*)(ws + c.P), (float*)(ws + c.Xi), (__half*)(ws + c.start)};
     }
-    switch (p.r) {
-        case 1: return launch_spread<64, 1>(p);
-        case 2: return launch_spread<64, 2>(p);
-        case 3: return launch_spread<64, 3>(p);
-        default: return launch_spread<64, 4>(p);
-    }
+    const int st = p.d_k == 128 ? launch_rank<128>(p, plan, sg) : launch_rank<64>(p, plan, sg);
+    if (st != PF_OK || plan.nseg == 1) return st;
+    if (p.d_k == 128) return p.d_v == 128 ? launch_seg_tail<128, 128>(p, plan, sg) : launch_seg_tail<128, 64>(p, plan, sg);
+    return p.d_v == 128 ? launch_seg_tail<64, 128>(p, plan, sg) : launch_seg_tail<64, 64>(p, plan, sg);
 }
 
 }  // namespace pf

@@ -31,6 +31,7 @@ struct Problem {
     int wu_builder;         // fp32 SIMT path: 0 = triangular inverse then W = T'K, Uh = T'V; 1 = the wavefront system of
                             // Theorem 3.3 (pf_params.wu_builder)
     int ring_depth;         // single-launch path: slots per sequence of the hand-off ring, 0 = default (pf_params.ring_depth)
+    bool clear_status;      // the kernels set *status to 0 first (false for the second pass of a segmented call)
     int* status;            // device word that receives the code of the first bounded wait that expires (never null
                             // when a tensor-core kernel is launched)
     cudaStream_t stream;
@@ -95,10 +96,13 @@ int simt_forward(const Problem& p, void* workspace);
 // the recurrence token by token in fp32 (pf_recur.cu); needs no workspace
 int recur_forward(const Problem& p);
 
-// the chunk form in one kernel on warp-level tensor-core products (pf_chain.cu); bf16 inputs, needs no workspace
+// the chunk form on warp-level tensor-core products (pf_chain.cu); bf16 inputs; one kernel and no workspace, or for few long
+// sequences three kernels
 bool chain_supported(const Problem& p);
 double chain_estimate_us(const Problem& p);
-int chain_forward(const Problem& p);
+bool chain_needs_workspace(const Problem& p);
+size_t chain_workspace_bytes(const Problem& p);
+int chain_forward(const Problem& p, void* workspace);
 
 // SM count of the current device, 0 if it cannot be found (pf_fused.cu)
 int sm_count();

@@ -38,6 +38,7 @@ __device__ __forceinline__ void store_if(float* p, float x, bool pred) {
 struct RecurGeo {
     int L, d_v;
     int ts;             // tokens per stage
+    int clear;          // set the status word to 0
     int exact;          // PF_STEP_EXACT
 };
 
@@ -109,7 +110,7 @@ recur_kernel(const Tin* __restrict__ q, const Tin* __restrict__ k, const Tin* __
     auto s_b = [&](int st) { return (float*)(s_v(st) + rows_s * RJ); };
 
     if (tid == 0) {
-        if (blockIdx.x == 0) *status = 0;              // (the call's status word; a wait of this kernel expires a second later at the earliest)
+        if (blockIdx.x == 0 && g.clear) *status = 0;              // (the call's status word; a wait of this kernel expires a second later at the earliest)
         for (int x = 0; x < R_STAGES; ++x) {
             tc::mbar_init(&bar_full[x], 1);
             tc::mbar_init(&bar_empty[x], IG);
@@ -301,7 +302,7 @@ const void* recur_fn(int d_k, int tb, int rg, int gpt) {
 
 int recur_forward(const Problem& p) {
     RecurGeo g{};
-    g.L = p.L; g.d_v = p.d_v; g.exact = p.exact;
+    g.L = p.L; g.d_v = p.d_v; g.exact = p.exact; g.clear = p.clear_status;
     const int rg = p.mask_group();
     const int tb = p.L < 4 ? 1 : 4;
     g.ts = p.L >= 16 ? 16 : (p.L < 1 ? 1 : (p.L + tb - 1) / tb * tb);

@@ -22,3 +22,16 @@ def test_block_edges(mode, step, d_k, d_v, r, L):
 def test_column_spreads(d_k, d_v, r, H):
     w = Workload(f"chain_h{H}", B=1, H=H, L=131, d_k=d_k, d_v=d_v, r=r, chunk=64, s0_std=0.1, seed=300 + r)
     util.check_parity(w)
+
+
+@pytest.mark.parametrize("d_k,d_v,r,H,L,mode", [
+    (128, 128, 1, 1, 3001, "sum"), (128, 128, 2, 3, 2500, "sum"), (64, 64, 1, 2, 4097, "sum"), (64, 128, 3, 1, 2111, "product"),
+    (128, 64, 4, 2, 1500, "sum"), (64, 64, 2, 10, 3000, "product"),
+])
+def test_few_long_sequences_are_walked_in_segments(d_k, d_v, r, H, L, mode):
+    """Told apart by the number of kernels: the walk, the composition of the start states, their contribution to O."""
+    import paper_2504_00492_b200 as pf
+    for s0_std in (0.0, 0.1):
+        w = Workload(f"chain_seg_{L}", B=1, H=H, L=L, d_k=d_k, d_v=d_v, r=r, chunk=64, s0_std=s0_std, seed=400 + r)
+        util.check_parity(w, mode=mode)
+        assert pf.pf_last_launch_count() == 3
