@@ -838,7 +838,7 @@ struct ChainPlan {
     double us;
 };
 ChainPlan make_plan(const Problem& p) {
-    static const double step[2][4] = {{2.25, 1.65, 1.7, 1.46}, {3.3, 2.6, 2.6, 2.15}};      // us per block, 64 columns, d_k = 64 and 128
+    static const double step[2][4] = {{1.95, 1.6, 1.7, 1.48}, {3.3, 2.6, 2.7, 2.2}};      // us per block, 64 columns, d_k = 64 and 128
     const long long nseq = (long long)p.B * p.H, sms = sm_count();
     const int C = NB / p.r, nblk = (p.L + C - 1) / C;
     const double st = step[p.d_k == 128][p.r - 1];

@@ -908,11 +908,12 @@ fused_kernel(const __grid_constant__ FusedMaps maps, FusedGeo g, FusedWs ws, con
     if (warp == 0) tmem_dealloc(tb, 512);
 }
 
-// Time of a chunk in us, measured: the scan's step, and what the CTAs that do not scan need to build a chunk of every sequence.
-constexpr double SCAN_US = 1.15;
+// Time of a chunk in us, measured (8 - 80 sequences, r = 1 .. 4): the scan's step, and what the CTAs that do not scan need to build
+// a chunk of every sequence.
+constexpr double SCAN_US = 1.1;
 double build_us(const Problem& p) {
     const double nseq = (double)p.B * p.H, flows = sm_count() - nseq;
-    return (p.tile_rows() == 128 ? 5.9 : 3.6) * nseq / (flows > 1 ? flows : 1);
+    return (p.tile_rows() == 128 ? 6.6 : 5.1) * nseq / (flows > 1 ? flows : 1);
 }
 
 // Slots per sequence (pf_params.ring_depth, 3..64).  A slot is busy from the moment a flow CTA may write it until the scan's
@@ -923,7 +924,7 @@ double build_us(const Problem& p) {
 int ring_depth(const Problem& p) {
     const int NC = p.chunks_per_seq();
     int want = p.ring_depth;
-    if (want <= 0) want = (NC > 256 || build_us(p) < SCAN_US) && (size_t)p.B * p.H * 16 * SLOT_BYTES <= ((size_t)48 << 20) ? 16 : 8;
+    if (want <= 0) want = (NC > 256 || build_us(p) < 1.5 * SCAN_US) && (size_t)p.B * p.H * 16 * SLOT_BYTES <= ((size_t)48 << 20) ? 16 : 8;
     return NC < want ? (NC < 1 ? 1 : NC) : want;
 }
 
@@ -948,7 +949,7 @@ Carve carve(const Problem& p) {
 // An estimate of the kernel's time in us: the first flow, then per chunk whichever is longer of the two above.
 double fused_estimate_us(const Problem& p) {
     const double build = build_us(p);
-    return 22.0 + p.chunks_per_seq() * (build > SCAN_US ? build : SCAN_US);
+    return 24.0 + p.chunks_per_seq() * (build > SCAN_US ? build : SCAN_US);
 }
 
 bool fused_supported(const Problem& p) {
