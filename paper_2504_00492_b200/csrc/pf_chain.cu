@@ -697,8 +697,8 @@ chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __rest
 }
 
 // Start states of the segments: one CTA per sequence and 16 rows j, serial over the segments; four warps with a quarter of the
-// columns i each.  start(1) = Xi_0, start(s+1) = start(s) P_s + Xi_s; the last one is S_final.  The next P comes while the present
-// one is used.
+// columns i each.  start(1) = Xi_0, start(s+1) = start(s) P_s + Xi_s; the last one is S_final.  The next P and Xi come while the
+// present ones are used.
 template <int DK>
 __global__ void __launch_bounds__(128) chain_compose(ChainSeg sg, float* __restrict__ S_final, int nseg, int d_v) {
     constexpr int LD = DK + 8, NT = DK / 32, PIECES = DK * DK / 8 / 128;
@@ -727,8 +727,10 @@ __global__ void __launch_bounds__(128) chain_compose(ChainSeg sg, float* __restr
 #pragma unroll
             for (int e = 0; e < 4; ++e) x[n][e] = src[(long long)(i0 + 8 * n + (e & 1)) * d_v + j + 8 * (e >> 1)];
     };
+    float X[NT][4];                                               // Xi of the next step
     load_p(1);
     xi(0, S);
+    xi(1, X);
     for (int s = 1; s < nseg; ++s) {
         __half* a_s = sA + (s & 1) * 16 * LD;
         __half* out = sg.start + (seq * nseg + s) * d_v * DK;
@@ -740,8 +742,12 @@ __global__ void __launch_bounds__(128) chain_compose(ChainSeg sg, float* __restr
                 *(uint32_t*)(a_s + (gq + 8 * h) * LD + i0 + 8 * n) = x;
                 *(uint32_t*)(out + (long long)(j + 8 * h) * DK + i0 + 8 * n) = x;
             }
-        xi(s, S);
+#pragma unroll
+        for (int n = 0; n < NT; ++n)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) S[n][e] = X[n][e];
         if (s + 1 < nseg) {
+            xi(s + 1, X);
             load_p(s + 1);
             asm volatile("cp.async.wait_group 1;" ::: "memory");
         } else {
@@ -799,28 +805,29 @@ __global__ void __launch_bounds__(256) chain_apply(ChainSeg sg, float* __restric
         a[kk][2] = in0 ? *(const uint32_t*)(r0 + 16 * kk + 8) : 0u;
         a[kk][3] = in1 ? *(const uint32_t*)(r0 + 8 * DK + 16 * kk + 8) : 0u;
     }
-    __syncthreads();
+    // (every load is requested before the first is used: a store to O between them would hold back those behind it)
     float* o0 = O + (seq * L + t0) * DV + 2 * t4;
+    float c[DV / 8][4];
+#pragma unroll
+    for (int n = 0; n < DV / 8; ++n) {
+        const float2 x = in0 ? *(const float2*)(o0 + 8 * n) : make_float2(0.f, 0.f);
+        const float2 y = in1 ? *(const float2*)(o0 + 8 * DV + 8 * n) : make_float2(0.f, 0.f);
+        c[n][0] = x.x; c[n][1] = x.y; c[n][2] = y.x; c[n][3] = y.y;
+    }
+    __syncthreads();
 #pragma unroll
     for (int np = 0; np < DV / 16; ++np) {
-        float c[2][4];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const float2 x = in0 ? *(const float2*)(o0 + 16 * np + 8 * h) : make_float2(0.f, 0.f);
-            const float2 y = in1 ? *(const float2*)(o0 + 8 * DV + 16 * np + 8 * h) : make_float2(0.f, 0.f);
-            c[h][0] = x.x; c[h][1] = x.y; c[h][2] = y.x; c[h][3] = y.y;
-        }
 #pragma unroll
         for (int kk = 0; kk < KT; ++kk) {
             uint32_t x[4];
             ldmatrix_x4(x, smem_u32(sS + (16 * np + (lane & 7) + ((lane >> 4) << 3)) * LD + 16 * kk + 8 * ((lane >> 3) & 1)));
-            mma_16816(c[0], a[kk], x[0], x[1]);
-            mma_16816(c[1], a[kk], x[2], x[3]);
+            mma_16816(c[2 * np], a[kk], x[0], x[1]);
+            mma_16816(c[2 * np + 1], a[kk], x[2], x[3]);
         }
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            if (in0) *(float2*)(o0 + 16 * np + 8 * h) = make_float2(c[h][0], c[h][1]);
-            if (in1) *(float2*)(o0 + 8 * DV + 16 * np + 8 * h) = make_float2(c[h][2], c[h][3]);
+        for (int n = 2 * np; n < 2 * np + 2; ++n) {
+            if (in0) *(float2*)(o0 + 8 * n) = make_float2(c[n][0], c[n][1]);
+            if (in1) *(float2*)(o0 + 8 * DV + 8 * n) = make_float2(c[n][2], c[n][3]);
         }
     }
 }
