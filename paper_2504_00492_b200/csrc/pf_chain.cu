@@ -223,10 +223,15 @@ __device__ __forceinline__ void prep_role(const ChainGeo& g, const ChainPart& pa
     const uint32_t offN = lane_off((lane & 7) + ((lane >> 4) << 3), (lane >> 3) & 1);
     const uint32_t offT = lane_off((lane & 7) + (((lane >> 3) & 1) << 3), lane >> 4);
     const __nv_bfloat16* bs = beta + seq * L * R;
+    // (the bits as loaded: a conversion next to the load would make every thread wait for it there, a block ahead of its use)
     auto read_beta = [&](int b) {                                 // rows past the block or the sequence have step size zero
-        return tid < min(C, L - (part.b0 + b) * C) * R ? __bfloat162float(bs[(long long)(part.b0 + b) * C * R + tid]) : 0.f;
+        uint16_t x = 0;
+        if (tid < min(C, L - (part.b0 + b) * C) * R)
+            asm volatile("ld.global.nc.b16 %0, [%1];" : "=h"(x) : "l"(bs + (long long)(part.b0 + b) * C * R + tid));
+        return x;
     };
-    float breg = team < part.nblk ? read_beta(team) : 0.f;
+    uint16_t breg = team < part.nblk ? read_beta(team) : 0;
+    const int lim0 = (16 * w + gq) / g.rm * g.rm, lim1 = (16 * w + gq + 8) / g.rm * g.rm;      // (edges of the strict mask)
 #pragma unroll 1
     for (int b = team; b < part.nblk; b += TEAMS) {
         const int st = b % NS;
@@ -251,7 +256,7 @@ __device__ __forceinline__ void prep_role(const ChainGeo& g, const ChainPart& pa
             }
         }
         fence_async_smem();                                       // (the stage's next copy is ordered after these writes)
-        if (tid < NB) sBeta[tid] = breg;
+        if (tid < NB) sBeta[tid] = __uint_as_float((uint32_t)breg << 16);
         if (b + TEAMS < part.nblk) breg = read_beta(b + TEAMS);
         if (!named_bar_and(bar_id, 128, ok)) return;
 
@@ -281,7 +286,6 @@ __device__ __forceinline__ void prep_role(const ChainGeo& g, const ChainPart& pa
         {
             const int m0 = 16 * w + gq, m1 = m0 + 8;
             const float b0 = sBeta[m0], b1 = sBeta[m1];
-            const int lim0 = m0 / g.rm * g.rm, lim1 = m1 / g.rm * g.rm;
 #pragma unroll
             for (int nb = 0; nb < 4; ++nb)
                 if (nb <= w) {
@@ -425,8 +429,9 @@ __device__ __forceinline__ void chain_role(const ChainMaps& maps, const ChainGeo
     float* ob = part.O + part.j0 + 16 * grp + 2 * t4 + (IS == 2 ? 8 * hi : 0);     // O of the current block (response: in halves)
     __half* rb = (__half*)part.O + part.j0 + 16 * grp + 2 * t4 + (IS == 2 ? 8 * hi : 0);
     auto put_o = [&](int t, int dj, float x, float y, bool pred) {     // token t of the current block
-        if (SEG && part.response) store_h2_if(rb + (long long)t * width + dj, pack_h2(x, y), pred);
-        else store2_if(ob + (long long)t * width + dj, x, y, pred);
+        // (both forms, predicated: a branch at every store would keep the products on either side of it apart)
+        if (SEG) store_h2_if(rb + (long long)t * width + dj, pack_h2(x, y), pred && part.response);
+        store2_if(ob + (long long)t * width + dj, x, y, pred && !(SEG && part.response));
     };
 
     // IS = 2: what this warp keeps of O of the block before (8 of the 16 columns j), without the other warp's part of Q S^T
@@ -551,47 +556,69 @@ __device__ __forceinline__ void chain_role(const ChainMaps& maps, const ChainGeo
                 mma_16816(S[2 * ip], u16[kk], x[0], x[1]);
                 mma_16816(S[2 * ip + 1], u16[kk], x[2], x[3]);
             }
-        // ---- O = Q S^T + P U' with the state before the update, 16 tokens at a time (these products fill the latency of the update)
+        // ---- O = Q S^T + P U' with the state before the update (these products fill the latency of the update).  Two tiles of 16
+        //      tokens at a time, or one with its sums in two halves: at least four independent accumulators, the depth of the
+        //      product's pipeline (one tile at a time took 2.8 k cycles of a step of 6.5 k at d_k = 128, r = 1)
         const int Cv = min(C, g.L - (part.b0 + b) * C);
+        constexpr int TG = TT >= 2 ? 2 : 1, SP = 3 - TG;
 #pragma unroll
-        for (int tt = 0; tt < TT; ++tt) {
-            float o[2][4];
+        for (int tg = 0; tg < TT; tg += TG) {
+            float o[TG][SP][2][4];
 #pragma unroll
-            for (int kk = 0; kk < KT; ++kk) {
-                uint32_t a[4];
-                ldmatrix_x4(a, q_b + (offA ^ kxor(kk)) + tt * 2048 + kpos(kk, CP * 128));
-                mma_acc(o[0], a, s16[kk][0], s16[kk][2], kk > 0);
-                mma_acc(o[1], a, s16[kk][1], s16[kk][3], kk > 0);
-            }
-            float ot[4];
+            for (int kk = 0; kk < KT; ++kk)
+#pragma unroll
+                for (int u = 0; u < TG; ++u) {
+                    uint32_t a[4];
+                    ldmatrix_x4(a, q_b + (offA ^ kxor(kk)) + (tg + u) * 2048 + kpos(kk, CP * 128));
+                    mma_acc(o[u][kk % SP][0], a, s16[kk][0], s16[kk][2], kk >= SP);
+                    mma_acc(o[u][kk % SP][1], a, s16[kk][1], s16[kk][3], kk >= SP);
+                }
             if (IS == 2) {
-                float4* mine = (float4*)(exw + ((b & 1) * 2 + hi) * (CFG::x_piece * 512));
-                mine[(8 + tt) * 32] = hi ? make_float4(o[0][0], o[0][1], o[0][2], o[0][3]) : make_float4(o[1][0], o[1][1], o[1][2], o[1][3]);
+                // (the warp keeps 8 of the 16 columns j and hands its half of the sum for the others over)
 #pragma unroll
-                for (int e = 0; e < 4; ++e) ot[e] = hi ? o[1][e] : o[0][e];
-            }
+                for (int u = 0; u < TG; ++u) {
+                    if (SP == 2)
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk) {
-                if (kk >= (tt + 1) * R) continue;
-                uint32_t a[4];
-                ldmatrix_x4(a, p_b + (offA ^ (kk << 5)) + tt * 2048);
-                if (IS == 2) {
-                    mma_16816(ot, a, hi ? u16[kk][1] : u16[kk][0], hi ? u16[kk][3] : u16[kk][2]);
-                } else {
-                    mma_16816(o[0], a, u16[kk][0], u16[kk][2]);
-                    mma_16816(o[1], a, u16[kk][1], u16[kk][3]);
+                        for (int e = 0; e < 4; ++e) {
+                            o[u][0][0][e] += o[u][SP - 1][0][e];
+                            o[u][0][1][e] += o[u][SP - 1][1][e];
+                        }
+                    float4* mine = (float4*)(exw + ((b & 1) * 2 + hi) * (CFG::x_piece * 512));
+                    mine[(8 + tg + u) * 32] = hi ? make_float4(o[u][0][0][0], o[u][0][0][1], o[u][0][0][2], o[u][0][0][3])
+                                                 : make_float4(o[u][0][1][0], o[u][0][1][1], o[u][0][1][2], o[u][0][1][3]);
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) ok8[tg + u][e] = hi ? o[u][0][1][e] : o[u][0][0][e];
                 }
             }
-            if (IS == 2) {
 #pragma unroll
-                for (int e = 0; e < 4; ++e) ok8[tt][e] = ot[e];
-            } else {
-                const int t = 16 * tt + gq;
-                put_o(t, 0, o[0][0], o[0][1], t < Cv);
-                put_o(t, 8, o[1][0], o[1][1], t < Cv);
-                put_o(t + 8, 0, o[0][2], o[0][3], t + 8 < Cv);
-                put_o(t + 8, 8, o[1][2], o[1][3], t + 8 < Cv);
-            }
+            for (int kk = 0; kk < 4; ++kk)
+#pragma unroll
+                for (int u = 0; u < TG; ++u) {
+                    if (kk >= (tg + u + 1) * R) continue;
+                    uint32_t a[4];
+                    ldmatrix_x4(a, p_b + (offA ^ (kk << 5)) + (tg + u) * 2048);
+                    if (IS == 2) {
+                        mma_16816(ok8[tg + u], a, hi ? u16[kk][1] : u16[kk][0], hi ? u16[kk][3] : u16[kk][2]);
+                    } else {
+                        mma_16816(o[u][kk % SP][0], a, u16[kk][0], u16[kk][2]);
+                        mma_16816(o[u][kk % SP][1], a, u16[kk][1], u16[kk][3]);
+                    }
+                }
+            if (IS == 1)
+#pragma unroll
+                for (int u = 0; u < TG; ++u) {
+                    if (SP == 2)
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            o[u][0][0][e] += o[u][SP - 1][0][e];
+                            o[u][0][1][e] += o[u][SP - 1][1][e];
+                        }
+                    const int t = 16 * (tg + u) + gq;
+                    put_o(t, 0, o[u][0][0][0], o[u][0][0][1], t < Cv);
+                    put_o(t, 8, o[u][0][1][0], o[u][0][1][1], t < Cv);
+                    put_o(t + 8, 0, o[u][0][0][2], o[u][0][0][3], t + 8 < Cv);
+                    put_o(t + 8, 8, o[u][0][1][2], o[u][0][1][3], t + 8 < Cv);
+                }
         }
         Cv_prev = Cv;
         ob += (long long)C * width;
