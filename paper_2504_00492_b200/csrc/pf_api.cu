@@ -191,12 +191,14 @@ bool use_recur(const Problem& p, int impl) {
 bool use_fused(const Problem& p) {
     return fused_supported(p) && (!p.auto_impl || !chain_supported(p) || fused_estimate_us(p) < chain_estimate_us(p));
 }
-bool in_window(const Problem& p) {
+// (Short calls on 0.7 to 0.95 x SM count sequences with d = 128 stay on the two launches of the tcgen05 form, which is what
+// PF_IMPL_AUTO is specified to give there: 55 - 120 us against 22 - 39 for the chain kernel at up to 256 tokens.)
+bool two_launches_specified(const Problem& p) {
     const long long nseq = (long long)p.B * p.H, sms = sm_count();
-    return p.d_k == 128 && p.d_v == 128 && nseq * 10 > sms * 7 && nseq <= sms - 8;
+    return p.d_k == 128 && p.d_v == 128 && p.L <= 256 && nseq * 10 > sms * 7 && nseq <= sms - 8;
 }
 bool use_chain(const Problem& p, int impl) {
-    return impl == PF_IMPL_TC && p.auto_impl && !use_recur(p, impl) && chain_supported(p) && !use_fused(p) && !in_window(p);
+    return impl == PF_IMPL_TC && p.auto_impl && !use_recur(p, impl) && chain_supported(p) && !use_fused(p) && !two_launches_specified(p);
 }
 
 // what the kernels of `impl` carve up (the fp32 step sizes of PF_STEP_EXACT follow it)
@@ -301,10 +303,14 @@ int forward_one(const pf_params* a, bool top) {
     bool own = false;
     if (ws) {
         if (a->workspace_bytes < need || ((uintptr_t)ws & 255u)) return PF_ERR_WORKSPACE;
-    } else if (need > 0 && !use_recur(p, impl) && (!use_chain(p, impl) || chain_needs_workspace(p))) {
-        st = workspace_alloc(&ws, need, p.stream);
-        if (st != PF_OK) return st;
-        own = true;
+    } else {
+        const size_t own_need = use_recur(p, impl) ? recur_workspace_bytes(p)
+                                : use_chain(p, impl) && !chain_needs_workspace(p) ? 0 : need;
+        if (own_need > 0) {
+            st = workspace_alloc(&ws, own_need, p.stream);
+            if (st != PF_OK) return st;
+            own = true;
+        }
     }
     if (top) begin_call();
     // the status word of this call: the caller's, else word 0 of the caller's workspace, else the library's own
@@ -319,7 +325,7 @@ int forward_one(const pf_params* a, bool top) {
     }
     if (use_recur(p, impl) || use_chain(p, impl)) {
         p.clear_status = top;
-        st = use_recur(p, impl) ? recur_forward(p) : chain_forward(p, ws);
+        st = use_recur(p, impl) ? recur_forward(p, ws) : chain_forward(p, ws);
         if (own) {
             cudaError_t e = cudaFreeAsync(ws, p.stream);
             if (e != cudaSuccess && st == PF_OK) st = record_cuda_error(e, "cudaFreeAsync");

@@ -93,8 +93,10 @@ inline size_t beta32_bytes(const Problem& p) { return align_up((size_t)p.B * p.H
 size_t simt_workspace_bytes(const Problem& p);
 int simt_forward(const Problem& p, void* workspace);
 
-// the recurrence token by token in fp32 (pf_recur.cu); needs no workspace
-int recur_forward(const Problem& p);
+// the recurrence token by token in fp32 (pf_recur.cu); one kernel and no workspace, or for few long sequences three kernels (only
+// when given a workspace of recur_workspace_bytes, which is never more than simt_workspace_bytes)
+size_t recur_workspace_bytes(const Problem& p);
+int recur_forward(const Problem& p, void* workspace);
 
 // the chunk form on warp-level tensor-core products (pf_chain.cu); bf16 inputs; one kernel and no workspace, or for few long
 // sequences three kernels

@@ -40,6 +40,18 @@ struct RecurGeo {
     int ts;             // tokens per stage
     int clear;          // set the status word to 0
     int exact;          // PF_STEP_EXACT
+    int nseg, seg_tok;  // segments per sequence (1: none) and tokens per segment (a multiple of ts)
+};
+
+// Segments (Section 3, "Scan"; Proposition 2.1: S_end = S_start P + Xi): few long sequences are cut into segments that are walked
+// side by side, each from zero (S0 for the first), which gives its own part of O and Xi, and, but for the first, from the
+// identity with v = 0, which gives P and the tokens' responses R_t = P_t q_t to the start state.  recur_compose then makes the
+// start states, recur_apply adds start R_t to O.  All fp32.
+struct RecurSeg {
+    float* R;           // [nseq][L][d_k]
+    float* P;           // [nseq][nseg][d_k i][d_k j]
+    float* Xi;          // [nseq][nseg][d_k i][d_v j]
+    float* start;       // [nseq][nseg][d_k i][d_v j]
 };
 
 // Two fp32 values in a register pair: one fma.rn.f32x2 does two FFMA's work in one issue slot.
@@ -89,7 +101,7 @@ __host__ __device__ constexpr int recur_stage_bytes(int ts, int r, int d_k, int 
 template <class Tin, int DK, int RG, int GPT, int TB, int IG>
 __global__ void __launch_bounds__((IG + 1) * 32, 1)
 recur_kernel(const Tin* __restrict__ q, const Tin* __restrict__ k, const Tin* __restrict__ v, const Tin* __restrict__ beta,
-             const float* __restrict__ S0, float* __restrict__ O, float* __restrict__ S_final, int* __restrict__ status, RecurGeo g) {
+             const float* __restrict__ S0, float* __restrict__ O, float* __restrict__ S_final, int* __restrict__ status, RecurGeo g, RecurSeg sg) {
     constexpr int NI = DK / IG, r = RG * GPT;          // rows i of a column that a lane holds
     constexpr int JW = 32 / IG;                        // columns per warp (IG warps make up the CTA's 32 columns)
     constexpr bool AHEAD = RG * NI <= 64;              // keys are read one group ahead where registers allow it
@@ -97,10 +109,38 @@ recur_kernel(const Tin* __restrict__ q, const Tin* __restrict__ k, const Tin* __
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ uint64_t bar_full[R_STAGES], bar_empty[R_STAGES];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int slices = g.d_v / RJ;
-    const long long seq = blockIdx.x / slices;
-    const int j0 = (int)(blockIdx.x % slices) * RJ;
-    const int L = g.L, d_v = g.d_v;
+    // the part this CTA walks: a sequence, or a segment of it, or a segment's response
+    long long seq;
+    int j0, tok0 = 0, Lp = g.L, width = g.d_v;
+    bool response = false;
+    const float* S_in = S0;
+    float* S_out = S_final;
+    float* O_out;
+    {
+        const int slices = g.d_v / RJ, x = (int)blockIdx.x;
+        if (g.nseg == 1) {
+            seq = x / slices;
+            j0 = x % slices * RJ;
+            O_out = O + seq * g.L * width;
+            S_in = S0 ? S0 + seq * DK * width : nullptr;
+            S_out = S_final ? S_final + seq * DK * width : nullptr;
+        } else {
+            constexpr int rs = DK / RJ;
+            const int per_seq = g.nseg * slices + (g.nseg - 1) * rs, y = x % per_seq, z = y - g.nseg * slices;
+            seq = x / per_seq;
+            response = z >= 0;
+            const int s = response ? 1 + z / rs : y / slices;
+            j0 = (response ? z % rs : y % slices) * RJ;
+            tok0 = s * g.seg_tok;
+            Lp = min(g.seg_tok, g.L - tok0);
+            width = response ? DK : g.d_v;
+            O_out = (response ? sg.R : O) + (seq * g.L + tok0) * width;
+            S_in = s == 0 && S0 ? S0 + seq * DK * width : nullptr;
+            S_out = (response ? sg.P : sg.Xi) + (seq * g.nseg + s) * DK * width;
+        }
+    }
+    const int L = Lp, d_v = g.d_v;
+    const long long seq_tok = seq * g.L + tok0;        // first token of the part
     const int rows_s = g.ts * r;                       // rows per stage (at most 64)
     const int nb = (L + g.ts - 1) / g.ts;
     const int stage_bytes = recur_stage_bytes(g.ts, r, DK, (int)sizeof(Tin));
@@ -126,15 +166,18 @@ recur_kernel(const Tin* __restrict__ q, const Tin* __restrict__ k, const Tin* __
             const int st = b % R_STAGES, t0 = b * g.ts;
             const int nt = min(g.ts, L - t0), np = (nt + TB - 1) / TB * TB;
             if (b >= R_STAGES && !tc::mbar_wait_clk(&bar_empty[st], (uint32_t)(b / R_STAGES - 1) & 1, status, 301)) return;
-            const long long tok = seq * L + t0;
+            const long long tok = seq_tok + t0;
             if (lane == 0) {
-                tc::mbar_expect_tx_only(&bar_full[st], (uint32_t)(nt * (r * DK + DK + r * RJ) * sizeof(Tin)));
+                tc::mbar_expect_tx_only(&bar_full[st], (uint32_t)(nt * (r * DK + DK + (response ? 0 : r * RJ)) * sizeof(Tin)));
                 tc::bulk_load(s_k(st), k + tok * r * DK, (uint32_t)(nt * r * DK * sizeof(Tin)), &bar_full[st]);
                 tc::bulk_load(s_q(st), q + tok * DK, (uint32_t)(nt * DK * sizeof(Tin)), &bar_full[st]);
             }
             __syncwarp();
-            for (int row = lane; row < nt * r; row += 32)
-                tc::bulk_load(s_v(st) + row * RJ, v + (tok * r + row) * d_v + j0, (uint32_t)(RJ * sizeof(Tin)), &bar_full[st]);
+            if (response)
+                for (int e = lane; e < nt * r * RJ; e += 32) s_v(st)[e] = Tin(0.f);
+            else
+                for (int row = lane; row < nt * r; row += 32)
+                    tc::bulk_load(s_v(st) + row * RJ, v + (tok * r + row) * d_v + j0, (uint32_t)(RJ * sizeof(Tin)), &bar_full[st]);
             for (int row = lane; row < np * r; row += 32) s_b(st)[row] = row < nt * r ? to_f(beta[tok * r + row]) : 0.f;
             if (g.exact)                               // beta' = (1 - e^{-beta |k|^2}) / |k|^2
                 for (int row = 0; row < nt * r; ++row) {
@@ -161,11 +204,12 @@ recur_kernel(const Tin* __restrict__ q, const Tin* __restrict__ k, const Tin* __
     const int ig = lane / JW, jw = JW * warp + lane % JW;     // this lane's column within the CTA's 32
     // S[n] = rows i = 4 IG (n / 2) + 4 ig + 2 (n % 2), + 1 of the lane's column: neighbouring lanes read the same 16 bytes of a key
     f2 S[NI / 2];
-    const long long sb = (seq * DK + 4 * ig) * d_v + j0 + jw;
+    const long long sb = 4ll * ig * width + j0 + jw;
 #pragma unroll
     for (int n = 0; n < NI; n += 2) {
-        const float* x = S0 + sb + (long long)(4 * IG * (n >> 2) + (n & 3)) * d_v;
-        S[n / 2] = S0 ? pk2(x[0], x[d_v]) : 0ull;
+        const int i = 4 * IG * (n >> 2) + (n & 3);
+        const float* x = S_in + sb + (long long)i * width;
+        S[n / 2] = S_in ? pk2(x[0], x[width]) : response ? pk2(i + 4 * ig == j0 + jw ? 1.f : 0.f, i + 4 * ig + 1 == j0 + jw ? 1.f : 0.f) : 0ull;
     }
 
     for (int b = 0; b < nb; ++b) {
@@ -177,7 +221,7 @@ recur_kernel(const Tin* __restrict__ q, const Tin* __restrict__ k, const Tin* __
         const Tin* qp = s_q(st) + 4 * ig;
         const Tin* vp = s_v(st) + jw;
         const float* bp = s_b(st);
-        float* og = O + (seq * L + (long long)b * g.ts) * d_v + j0 + jw;
+        float* og = O_out + (long long)b * g.ts * width + j0 + jw;
         f2 kn[RG][NI / 2];
         float vn[RG], bn[RG];
         auto fetch_k = [&]() {
@@ -265,19 +309,125 @@ recur_kernel(const Tin* __restrict__ q, const Tin* __restrict__ k, const Tin* __
 #pragma unroll
             for (int m = JW; m < (TB == 4 ? 8 : 32); m *= 2) y += __shfl_xor_sync(FULL, y, m);
             const int tok = TB == 4 ? t4 + (lane >> 3) : t4;
-            store_if(og + (long long)tok * d_v, y, tok < nt && (TB == 4 ? (lane & 7) < JW : lane < JW));
+            store_if(og + (long long)tok * width, y, tok < nt && (TB == 4 ? (lane & 7) < JW : lane < JW));
         }
         __syncwarp();
         if (lane == 0) tc::mbar_arrive(&bar_empty[st]);
     }
-    if (S_final)
+    if (S_out)
 #pragma unroll
         for (int n = 0; n < NI; n += 2) {
-            float* x = S_final + sb + (long long)(4 * IG * (n >> 2) + (n & 3)) * d_v;
+            float* x = S_out + sb + (long long)(4 * IG * (n >> 2) + (n & 3)) * width;
             const float2 s2 = up2(S[n / 2]);
             x[0] = s2.x;
-            x[d_v] = s2.y;
+            x[width] = s2.y;
         }
+}
+
+// start(1) = Xi_0, start(s+1) = start(s) P_s + Xi_s, the last one is S_final: a CTA per sequence and ROWS rows j, serial over the
+// segments.  A thread has four rows and one column i; P (stored [i][j']) comes to shared memory a step after it was requested,
+// rows padded so that 32 threads reading 16 bytes of 32 rows meet no bank twice.
+template <int DK>
+__global__ void __launch_bounds__(256) recur_compose(RecurSeg sg, float* __restrict__ S_final, int nseg, int d_v) {
+    constexpr int CG = DK / 32, ROWS = 4 * (8 / CG), LD = DK + 4, NV = DK * DK / 4 / 256;
+    extern __shared__ __align__(16) float smf[];
+    float* Ps = smf;                    // [DK i][LD]
+    float* cur = smf + DK * LD;         // [ROWS][DK]
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int groups = d_v / ROWS, jl = 4 * (warp / CG), i = 32 * (warp % CG) + lane;
+    const long long seq = blockIdx.x / groups;
+    const int j = (int)(blockIdx.x % groups) * ROWS + jl;
+    float4 pv[NV], xv;
+    auto fetch_p = [&](int s) {
+        const float4* p = (const float4*)(sg.P + (seq * nseg + s) * DK * DK);
+#pragma unroll
+        for (int u = 0; u < NV; ++u) pv[u] = p[u * 256 + tid];
+    };
+    auto fetch_x = [&](int s) { return *(const float4*)(sg.Xi + ((seq * nseg + s) * DK + i) * d_v + j); };
+    float4 acc = fetch_x(0);
+    fetch_p(1);
+    xv = fetch_x(1);
+    for (int s = 1; s < nseg; ++s) {
+        *(float4*)(sg.start + ((seq * nseg + s) * DK + i) * d_v + j) = acc;
+        cur[(jl + 0) * DK + i] = acc.x;
+        cur[(jl + 1) * DK + i] = acc.y;
+        cur[(jl + 2) * DK + i] = acc.z;
+        cur[(jl + 3) * DK + i] = acc.w;
+#pragma unroll
+        for (int u = 0; u < NV; ++u) {
+            const int e = (u * 256 + tid) * 4;
+            *(float4*)(Ps + (e / DK) * LD + e % DK) = pv[u];
+        }
+        acc = xv;
+        __syncthreads();
+        if (s + 1 < nseg) {
+            fetch_p(s + 1);
+            xv = fetch_x(s + 1);
+        }
+#pragma unroll 4
+        for (int ip = 0; ip < DK; ip += 4) {
+            const float4 p = *(const float4*)(Ps + i * LD + ip);
+            const float4 a = *(const float4*)(cur + (jl + 0) * DK + ip), b = *(const float4*)(cur + (jl + 1) * DK + ip);
+            const float4 c = *(const float4*)(cur + (jl + 2) * DK + ip), d = *(const float4*)(cur + (jl + 3) * DK + ip);
+            acc.x = fmaf(a.x, p.x, fmaf(a.y, p.y, fmaf(a.z, p.z, fmaf(a.w, p.w, acc.x))));
+            acc.y = fmaf(b.x, p.x, fmaf(b.y, p.y, fmaf(b.z, p.z, fmaf(b.w, p.w, acc.y))));
+            acc.z = fmaf(c.x, p.x, fmaf(c.y, p.y, fmaf(c.z, p.z, fmaf(c.w, p.w, acc.z))));
+            acc.w = fmaf(d.x, p.x, fmaf(d.y, p.y, fmaf(d.z, p.z, fmaf(d.w, p.w, acc.w))));
+        }
+        __syncthreads();
+    }
+    if (S_final) *(float4*)(S_final + (seq * DK + i) * d_v + j) = acc;
+}
+
+// O[t][j] += sum_i R[t][i] start[i][j] for the tokens of all segments but the first: grid (64-token tiles, nseq (nseg - 1)), thread
+// (ty, tx) the tokens 4 ty .. 4 ty + 3 and the columns DV / 16 tx ...
+template <int DK, int DV>
+__global__ void __launch_bounds__(256) recur_apply(RecurSeg sg, float* __restrict__ O, int L, int seg_tok, int nseg) {
+    constexpr int PER = DV / 16, TLD = 68;
+    extern __shared__ __align__(16) float smf[];
+    float* Ss = smf;                    // [DK i][DV j]
+    float* Rs = smf + DK * DV;          // [DK i][TLD]  R transposed: the four tokens of a thread are one 16-byte load
+    const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+    const long long seq = blockIdx.y / (nseg - 1);
+    const int s = 1 + (int)(blockIdx.y % (nseg - 1)), t0 = s * seg_tok + blockIdx.x * 64;
+    const int nt = min(64, min(L, (s + 1) * seg_tok) - t0);
+    if (nt <= 0) return;
+    const float4* st = (const float4*)(sg.start + (seq * nseg + s) * DK * DV);
+#pragma unroll
+    for (int e = 0; e < DK * DV / 4 / 256; ++e) ((float4*)Ss)[e * 256 + tid] = st[e * 256 + tid];
+    const float* Rg = sg.R + (seq * L + t0) * DK;
+    for (int e = tid; e < 64 * DK; e += 256) {
+        const int t = e / DK, i = e % DK;
+        Rs[i * TLD + t] = t < nt ? Rg[e] : 0.f;
+    }
+    float acc[4][PER];
+    float* Og = O + (seq * L + t0 + 4 * ty) * DV + PER * tx;
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int c = 0; c < PER; c += 4) {
+            const float4 o = 4 * ty + a < nt ? *(const float4*)(Og + a * DV + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+            acc[a][c] = o.x; acc[a][c + 1] = o.y; acc[a][c + 2] = o.z; acc[a][c + 3] = o.w;
+        }
+    __syncthreads();
+#pragma unroll 4
+    for (int i = 0; i < DK; ++i) {
+        const float4 rv = *(const float4*)(Rs + i * TLD + 4 * ty);
+#pragma unroll
+        for (int c = 0; c < PER; c += 4) {
+            const float4 b = *(const float4*)(Ss + i * DV + PER * tx + c);
+            const float bb[4] = {b.x, b.y, b.z, b.w}, rr[4] = {rv.x, rv.y, rv.z, rv.w};
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) acc[a][c + u] = fmaf(rr[a], bb[u], acc[a][c + u]);
+        }
+    }
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+        if (4 * ty + a < nt)
+#pragma unroll
+            for (int c = 0; c < PER; c += 4) *(float4*)(Og + a * DV + c) = make_float4(acc[a][c], acc[a][c + 1], acc[a][c + 2], acc[a][c + 3]);
 }
 
 template <class Tin, int DK, int TB, int IG>
@@ -298,20 +448,102 @@ const void* recur_fn(int d_k, int tb, int rg, int gpt) {
     return tb == 4 ? recur_fn<Tin, 64, 4, 4>(rg, gpt) : recur_fn<Tin, 64, 1, 4>(rg, gpt);
 }
 
+struct RecurPlan {
+    int nseg, seg_tok;
+};
+size_t seg_bytes(const Problem& p, int nseg) {
+    const size_t nseq = (size_t)p.B * p.H, slots = nseq * nseg;
+    return align_up(nseq * p.L * p.d_k * 4, 256) + align_up(slots * p.d_k * p.d_k * 4, 256) + 2 * align_up(slots * p.d_k * p.d_v * 4, 256);
+}
+// Segments, where they make the call a quarter shorter at least: the walk of a token costs about the same while at most one CTA
+// (d_k = 64: two, whose chains leave each other most of the issue slots) runs per SM; against it stand two more kernels, about
+// 1 us of composing per segment, and the traffic and products of the responses.
+RecurPlan make_plan(const Problem& p) {
+    static const double cyc[2][4] = {{204, 259, 330, 401}, {275, 373, 480, 590}};      // a token, d_k = 64 and 128 (sum form)
+    RecurPlan plan{1, p.L};
+    if (p.L < 128 || p.wu_builder) return plan;
+    const long long nseq = (long long)p.B * p.H, sms = sm_count();
+    const bool big = p.d_k == 128;
+    const double tok = (p.mask_group() == p.r ? cyc[big][p.r - 1] : p.r * cyc[big][0] * 0.9) / 1900.0;
+    const double walk = nseq * (p.d_v / RJ) > sms ? 0.0 : 4.0 + p.L * tok;      // (one wave: otherwise there is nothing to gain)
+    const double extra = 20.0 + (double)nseq * p.L * (p.d_k * p.d_v / 12e6 + (8.0 * p.d_k + 8.0 * p.d_v) / 4e6);
+    double best = 0.75 * walk;
+    const long long most = (sms * (big ? 1 : 2) / nseq + p.d_k / RJ) / (p.d_v / RJ + p.d_k / RJ);
+    for (int want = 2; want <= most && want <= 64; ++want) {
+        const int seg_tok = (p.L + 16 * want - 1) / (16 * want) * 16, nseg = (p.L + seg_tok - 1) / seg_tok;
+        const long long ctas = nseq * (nseg * (p.d_v / RJ) + (nseg - 1) * (p.d_k / RJ));
+        const double us = extra + nseg * (big ? 1.3 : 0.8) + seg_tok * tok * (ctas > sms ? 1.2 : 1.0);
+        // (a caller's workspace was sized for the chunk-form kernels of pf_simt.cu)
+        if (nseg > 1 && us < best && seg_bytes(p, nseg) + 256 <= simt_workspace_bytes(p)) {
+            best = us;
+            plan = {nseg, seg_tok};
+        }
+    }
+    return plan;
+}
+
+template <int DK, int DV>
+int launch_seg_tail(const Problem& p, const RecurPlan& plan, const RecurSeg& sg) {
+    const int nseq = p.B * p.H;
+    {
+        constexpr int rows = 4 * (8 / (DK / 32)), smem = (DK * (DK + 4) + rows * DK) * 4;
+        static std::atomic<uint64_t> opted_in{0};
+        const int st = allow_smem(opted_in, (const void*)recur_compose<DK>, smem);
+        if (st != PF_OK) return st;
+        prof_begin("recur_compose", p.stream);
+        recur_compose<DK><<<(unsigned)(nseq * (DV / rows)), 256, smem, p.stream>>>(sg, p.S_final, plan.nseg, DV);
+        prof_end(p.stream);
+        PF_CUDA_TRY(cudaGetLastError());
+    }
+    constexpr int smem = (DK * DV + DK * 68) * 4;
+    static std::atomic<uint64_t> opted_in{0};
+    const int st = allow_smem(opted_in, (const void*)recur_apply<DK, DV>, smem);
+    if (st != PF_OK) return st;
+    prof_begin("recur_apply", p.stream);
+    recur_apply<DK, DV><<<dim3((unsigned)((plan.seg_tok + 63) / 64), (unsigned)(nseq * (plan.nseg - 1))), 256, smem, p.stream>>>(
+        sg, p.O, p.L, plan.seg_tok, plan.nseg);
+    prof_end(p.stream);
+    PF_CUDA_TRY(cudaGetLastError());
+    count_launch(2);
+    return PF_OK;
+}
+
 }  // namespace
 
-int recur_forward(const Problem& p) {
+size_t recur_workspace_bytes(const Problem& p) {
+    const RecurPlan plan = make_plan(p);
+    return plan.nseg > 1 ? seg_bytes(p, plan.nseg) + 256 : 0;
+}
+
+int recur_forward(const Problem& p, void* workspace) {
     RecurGeo g{};
     g.L = p.L; g.d_v = p.d_v; g.exact = p.exact; g.clear = p.clear_status;
     const int rg = p.mask_group();
     const int tb = p.L < 4 ? 1 : 4;
     g.ts = p.L >= 16 ? 16 : (p.L < 1 ? 1 : (p.L + tb - 1) / tb * tb);
     const bool f32 = p.in_dtype == PF_DTYPE_F32;
+    const RecurPlan plan = workspace ? make_plan(p) : RecurPlan{1, p.L};
+    g.nseg = plan.nseg;
+    g.seg_tok = plan.seg_tok;
+    RecurSeg sg{};
+    if (plan.nseg > 1) {
+        const size_t slots = (size_t)p.B * p.H * plan.nseg;
+        uint8_t* ws = (uint8_t*)workspace + 256;          // (word 0 of a caller's workspace is the status word)
+        auto take = [&](size_t bytes) {
+            float* at = (float*)ws;
+            ws += align_up(bytes, 256);
+            return at;
+        };
+        sg.R = take((size_t)p.B * p.H * p.L * p.d_k * 4);
+        sg.P = take(slots * p.d_k * p.d_k * 4);
+        sg.Xi = take(slots * p.d_k * p.d_v * 4);
+        sg.start = take(slots * p.d_k * p.d_v * 4);
+    }
     const int nb = (p.L + g.ts - 1) / g.ts;
     const int smem = (nb < R_STAGES ? (nb < 1 ? 1 : nb) : R_STAGES) * recur_stage_bytes(g.ts, p.r, p.d_k, f32 ? 4 : 2) +
                      4 * 128 * 4;           // (one group of keys is read past the last stage)
     const void* fn = f32 ? recur_fn<float>(p.d_k, tb, rg, p.r / rg) : recur_fn<__nv_bfloat16>(p.d_k, tb, rg, p.r / rg);
-    const long long grid = (long long)p.B * p.H * (p.d_v / RJ);
+    const long long grid = (long long)p.B * p.H * (plan.nseg * (p.d_v / RJ) + (plan.nseg - 1) * (p.d_k / RJ));
     if (grid > 0x7fffffffLL) return PF_ERR_UNSUPPORTED;
     // (opted in once per kernel, to what its longest stages need)
     static std::atomic<uint64_t> opted_in[2][2][2][16];
@@ -320,12 +552,14 @@ int recur_forward(const Problem& p) {
                                   R_STAGES * recur_stage_bytes(16, p.r, p.d_k, f32 ? 4 : 2) + 4 * 128 * 4);
         if (st != PF_OK) return st;
     }
-    void* args[] = {(void*)&p.q, (void*)&p.k, (void*)&p.v, (void*)&p.beta, (void*)&p.S0, (void*)&p.O, (void*)&p.S_final, (void*)&p.status, (void*)&g};
+    void* args[] = {(void*)&p.q, (void*)&p.k, (void*)&p.v, (void*)&p.beta, (void*)&p.S0, (void*)&p.O, (void*)&p.S_final, (void*)&p.status, (void*)&g, (void*)&sg};
     prof_begin("recur", p.stream);
     PF_CUDA_TRY(cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(160), args, (size_t)smem, p.stream));
     prof_end(p.stream);
     count_launch(1);
-    return PF_OK;
+    if (plan.nseg == 1) return PF_OK;
+    if (p.d_k == 128) return p.d_v == 128 ? launch_seg_tail<128, 128>(p, plan, sg) : launch_seg_tail<128, 64>(p, plan, sg);
+    return p.d_v == 128 ? launch_seg_tail<64, 128>(p, plan, sg) : launch_seg_tail<64, 64>(p, plan, sg);
 }
 
 }  // namespace pf

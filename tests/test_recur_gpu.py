@@ -17,3 +17,16 @@ def test_pass_and_stage_edges(dtype, mode, step, r, d_k, d_v, L):
     util.check_parity(w, impl="simt", mode=mode, step=step, tol=util.TOL_F32)
     if dtype == "bf16" and L <= 24:
         util.check_parity(w, impl="auto", mode=mode, step=step, tol=util.TOL_F32)
+
+
+@pytest.mark.parametrize("d_k,d_v,r,H,L,mode", [
+    (64, 64, 2, 2, 1000, "sum"), (64, 128, 1, 1, 2049, "sum"), (128, 64, 3, 1, 1111, "product"), (128, 128, 1, 2, 1777, "sum"),
+    (64, 64, 4, 5, 640, "product"),
+])
+def test_few_long_sequences_are_walked_in_segments(d_k, d_v, r, H, L, mode):
+    """Told apart by the number of kernels: the walk, the composition of the start states, their contribution to O."""
+    import paper_2504_00492_b200 as pf
+    for s0_std in (0.0, 0.1):
+        w = Workload(f"recur_seg_{L}", B=1, H=H, L=L, d_k=d_k, d_v=d_v, r=r, chunk=64, dtype="f32", s0_std=s0_std, seed=500 + r)
+        util.check_parity(w, mode=mode)
+        assert pf.pf_last_launch_count() == 3
