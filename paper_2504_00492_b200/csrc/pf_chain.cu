@@ -861,9 +861,9 @@ __global__ void __launch_bounds__(256) chain_apply(ChainSeg sg, float* __restric
 
 // How a sequence is spread over CTAs: columns per CTA, and segments.  The time is (waves of CTAs) x (blocks of a segment) x
 // (time of a block), plus what composing segments costs.
-// Columns: fewer per CTA make a shorter step but more CTAs.  Measured with one wave at L = 1024 (us for d_k = d_v = 128, r = 2 and
-// r = 4): 32 columns by pairs of warps 67, 117; 64 columns 86, 140; 128 columns 125, 225.  At d_k = 64 a step is short enough that 32
-// columns gain nothing over 64 (51 against 53 us), and 128 columns cost 1.3 times as much.
+// Columns: fewer per CTA make a shorter step but more CTAs.  Measured with one wave, us per block for d_k = d_v = 128, r = 1 .. 4: 32
+// columns by pairs of warps 2.35, 1.82, 1.74, 1.70; 64 columns 3.3, 2.5, 2.55, 2.3; 128 columns 4.4, 3.4, 3.4, 3.0.  At d_k = 64 a step
+// is short enough that 32 columns gain nothing over 64, and 128 columns cost 1.53 times as much.
 // Segments: as many as one wave of CTAs holds pay for the second walk (the responses) and for two more kernels when few
 // sequences are long: taken where the estimate falls by a quarter at least.
 enum { COLS_32, COLS_64, COLS_128 };
@@ -872,25 +872,25 @@ struct ChainPlan {
     double us;
 };
 ChainPlan make_plan(const Problem& p) {
-    static const double step[2][4] = {{1.95, 1.6, 1.7, 1.48}, {3.3, 2.6, 2.7, 2.2}};      // us per block, 64 columns, d_k = 64 and 128
+    static const double step[2][4] = {{1.9, 1.45, 1.42, 1.32}, {3.3, 2.5, 2.55, 2.3}};      // us per block, 64 columns, d_k = 64 and 128
     const long long nseq = (long long)p.B * p.H, sms = sm_count();
     const int C = NB / p.r, nblk = (p.L + C - 1) / C;
     const double st = step[p.d_k == 128][p.r - 1];
     auto waves = [&](int js) { return (double)((nseq * (p.d_v / js) + sms - 1) / (sms > 0 ? sms : 1)); };
     double best = waves(64);
     ChainPlan plan{COLS_64, 1, nblk, 0.0};
-    if (p.d_k == 128 && 0.8 * waves(32) < best) {
-        best = 0.8 * waves(32);
+    if (p.d_k == 128 && 0.72 * waves(32) < best) {
+        best = 0.72 * waves(32);
         plan.cols = COLS_32;
     }
     if (p.d_v == 128) {
-        const double w = (p.d_k == 128 ? 1.5 : 1.3) * waves(128);
+        const double w = (p.d_k == 128 ? 1.34 : 1.53) * waves(128);
         if (w < best) {
             best = w;
             plan.cols = COLS_128;
         }
     }
-    plan.us = 6.0 + nblk * st * best;
+    plan.us = 7.0 + nblk * st * best;
     const double limit = 0.75 * plan.us;
     // (kernels and their gaps, then the traffic of the responses and of O at about 4 TB/s)
     const double extra = 16.0 + 6.0 + (double)nseq * p.L * (4.0 * p.d_k + 8.0 * p.d_v) / 4e6;
@@ -899,7 +899,7 @@ ChainPlan make_plan(const Problem& p) {
         const long long most = (sms / nseq + rs) / (vs + rs);
         for (int want = 2; want <= most && want <= 64 && want <= nblk; ++want) {
             const int seg_blk = (nblk + want - 1) / want, nseg = (nblk + seg_blk - 1) / seg_blk;
-            const double us = extra + 0.8 * nseg + seg_blk * st * (cols == COLS_32 ? 0.8 : 1.0);
+            const double us = extra + 0.8 * nseg + seg_blk * st * (cols == COLS_32 ? 0.72 : 1.0);
             if (us < limit && us < plan.us) plan = {cols, nseg, seg_blk, us};
         }
     }
