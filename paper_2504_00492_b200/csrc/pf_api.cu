@@ -177,11 +177,12 @@ int select_impl(Problem& p, int impl) {
 }
 
 // Calls that the token-by-token kernel takes: those on the fp32 path (unless the Theorem 3.3 builder is asked for), and
-// bf16 calls of so few tokens that a chunk would be mostly padding (one token of 128 sequences: 12 us against 56).
-constexpr int RECUR_MAX_TOKENS = 24;
+// bf16 calls of so few tokens that a block of the chunk form would be mostly padding (one token of 128 sequences: 6 us against
+// 13).  The line is where the two kernels' times meet: 30 tokens at r = 1, about 8 at r = 4 or where the sequences are many times
+// the SMs.
 bool use_recur(const Problem& p, int impl) {
     if (impl == PF_IMPL_SIMT) return p.wu_builder == 0;
-    return p.auto_impl && p.L <= RECUR_MAX_TOKENS;
+    return p.auto_impl && p.L <= 64 && (p.L <= 2 || !chain_supported(p) || recur_short_us(p) < chain_short_us(p));
 }
 
 // Which of the tensor-core kernels.  PF_IMPL_AUTO: the chain kernel, except where the single-launch tcgen05 kernel can run
@@ -191,11 +192,11 @@ bool use_recur(const Problem& p, int impl) {
 bool use_fused(const Problem& p) {
     return fused_supported(p) && (!p.auto_impl || !chain_supported(p) || fused_estimate_us(p) < chain_estimate_us(p));
 }
-// (Short calls on 0.7 to 0.95 x SM count sequences with d = 128 stay on the two launches of the tcgen05 form, which is what
-// PF_IMPL_AUTO is specified to give there: 55 - 120 us against 22 - 39 for the chain kernel at up to 256 tokens.)
+// (Calls of 129 to 256 tokens on 0.7 to 0.95 x SM count sequences with d = 128 stay on the two launches of the tcgen05 form, which
+// is what PF_IMPL_AUTO is specified to give there: 75 - 120 us at r = 2 against 23 - 39 for the chain kernel.)
 bool two_launches_specified(const Problem& p) {
     const long long nseq = (long long)p.B * p.H, sms = sm_count();
-    return p.d_k == 128 && p.d_v == 128 && p.L <= 256 && nseq * 10 > sms * 7 && nseq <= sms - 8;
+    return p.d_k == 128 && p.d_v == 128 && p.L > 128 && p.L <= 256 && nseq * 10 > sms * 7 && nseq <= sms - 8;
 }
 bool use_chain(const Problem& p, int impl) {
     return impl == PF_IMPL_TC && p.auto_impl && !use_recur(p, impl) && chain_supported(p) && !use_fused(p) && !two_launches_specified(p);

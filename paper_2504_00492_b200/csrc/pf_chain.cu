@@ -674,7 +674,7 @@ chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __rest
     const int slices = g.d_v / JS;
     long long seq;
     ChainPart part;
-    if (!SEG) {
+    if constexpr (!SEG) {
         seq = blockIdx.x / slices;
         part = {0, g.nblk, (int)(blockIdx.x % slices) * JS, g.d_v, false, S0 ? S0 + seq * DK * g.d_v : nullptr,
                 O + seq * g.L * g.d_v, S_final ? S_final + seq * DK * g.d_v : nullptr};
@@ -729,8 +729,8 @@ chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __rest
 template <int DK>
 __global__ void __launch_bounds__(128) chain_compose(ChainSeg sg, float* __restrict__ S_final, int nseg, int d_v) {
     constexpr int LD = DK + 8, NT = DK / 32, PIECES = DK * DK / 8 / 128;
-    extern __shared__ __align__(16) uint8_t smem[];
-    __half* sP = (__half*)smem;                                   // [2][DK][LD]
+    extern __shared__ __align__(16) uint8_t smem_tail[];
+    __half* sP = (__half*)smem_tail;                                   // [2][DK][LD]
     __half* sA = sP + 2 * DK * LD;                                // [2][16][LD]  fp16 rows of the start state
     const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31, gq = lane >> 2, t4 = lane & 3;
     const int groups = d_v / 16;
@@ -810,8 +810,8 @@ __global__ void __launch_bounds__(128) chain_compose(ChainSeg sg, float* __restr
 template <int DK, int DV>
 __global__ void __launch_bounds__(256) chain_apply(ChainSeg sg, float* __restrict__ O, int L, int seg_tokens, int nseg) {
     constexpr int LD = DK + 8, KT = DK / 16;
-    extern __shared__ __align__(16) uint8_t smem[];
-    __half* sS = (__half*)smem;                                   // [DV][LD]
+    extern __shared__ __align__(16) uint8_t smem_tail[];
+    __half* sS = (__half*)smem_tail;                                   // [DV][LD]
     const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31, gq = lane >> 2, t4 = lane & 3;
     const long long seq = blockIdx.y / (nseg - 1);
     const int s = 1 + (int)(blockIdx.y % (nseg - 1));
@@ -870,6 +870,7 @@ enum { COLS_32, COLS_64, COLS_128 };
 struct ChainPlan {
     int cols, nseg, seg_blk;
     double us;
+    double short_us;          // the kernel alone without segments, the start of each wave counted: what a call of a few blocks takes
 };
 ChainPlan make_plan(const Problem& p) {
     static const double step[2][4] = {{1.9, 1.45, 1.42, 1.32}, {3.3, 2.5, 2.55, 2.3}};      // us per block, 64 columns, d_k = 64 and 128
@@ -878,19 +879,23 @@ ChainPlan make_plan(const Problem& p) {
     const double st = step[p.d_k == 128][p.r - 1];
     auto waves = [&](int js) { return (double)((nseq * (p.d_v / js) + sms - 1) / (sms > 0 ? sms : 1)); };
     double best = waves(64);
-    ChainPlan plan{COLS_64, 1, nblk, 0.0};
+    ChainPlan plan{COLS_64, 1, nblk, 0.0, 0.0};
+    double turns = best;
     if (p.d_k == 128 && 0.72 * waves(32) < best) {
-        best = 0.72 * waves(32);
+        turns = waves(32);
+        best = 0.72 * turns;
         plan.cols = COLS_32;
     }
     if (p.d_v == 128) {
         const double w = (p.d_k == 128 ? 1.34 : 1.53) * waves(128);
         if (w < best) {
             best = w;
+            turns = waves(128);
             plan.cols = COLS_128;
         }
     }
     plan.us = 7.0 + nblk * st * best;
+    plan.short_us = 5.0 * turns + nblk * st * best;
     const double limit = 0.75 * plan.us;
     // (kernels and their gaps, then the traffic of the responses and of O at about 4 TB/s)
     const double extra = 16.0 + 6.0 + (double)nseq * p.L * (4.0 * p.d_k + 8.0 * p.d_v) / 4e6;
@@ -900,7 +905,7 @@ ChainPlan make_plan(const Problem& p) {
         for (int want = 2; want <= most && want <= 64 && want <= nblk; ++want) {
             const int seg_blk = (nblk + want - 1) / want, nseg = (nblk + seg_blk - 1) / seg_blk;
             const double us = extra + 0.8 * nseg + seg_blk * st * (cols == COLS_32 ? 0.72 : 1.0);
-            if (us < limit && us < plan.us) plan = {cols, nseg, seg_blk, us};
+            if (us < limit && us < plan.us) plan = {cols, nseg, seg_blk, us, plan.short_us};
         }
     }
     return plan;
@@ -1003,6 +1008,7 @@ int launch_seg_tail(const Problem& p, const ChainPlan& plan, const ChainSeg& sg)
 }  // namespace
 
 double chain_estimate_us(const Problem& p) { return make_plan(p).us; }
+double chain_short_us(const Problem& p) { return make_plan(p).short_us; }
 
 size_t chain_workspace_bytes(const Problem& p) { return carve(p, make_plan(p)).total; }
 bool chain_needs_workspace(const Problem& p) { return make_plan(p).nseg > 1; }

@@ -96,12 +96,14 @@ int simt_forward(const Problem& p, void* workspace);
 // the recurrence token by token in fp32 (pf_recur.cu); one kernel and no workspace, or for few long sequences three kernels (only
 // when given a workspace of recur_workspace_bytes, which is never more than simt_workspace_bytes)
 size_t recur_workspace_bytes(const Problem& p);
+double recur_short_us(const Problem& p);
 int recur_forward(const Problem& p, void* workspace);
 
 // the chunk form on warp-level tensor-core products (pf_chain.cu); bf16 inputs; one kernel and no workspace, or for few long
 // sequences three kernels
 bool chain_supported(const Problem& p);
 double chain_estimate_us(const Problem& p);
+double chain_short_us(const Problem& p);
 bool chain_needs_workspace(const Problem& p);
 size_t chain_workspace_bytes(const Problem& p);
 int chain_forward(const Problem& p, void* workspace);

@@ -448,6 +448,13 @@ const void* recur_fn(int d_k, int tb, int rg, int gpt) {
     return tb == 4 ? recur_fn<Tin, 64, 4, 4>(rg, gpt) : recur_fn<Tin, 64, 1, 4>(rg, gpt);
 }
 
+// the chain of one token
+double token_us(const Problem& p) {
+    static const double cyc[2][4] = {{204, 259, 330, 401}, {275, 373, 480, 590}};      // d_k = 64 and 128, sum form
+    const bool big = p.d_k == 128;
+    return (p.mask_group() == p.r ? cyc[big][p.r - 1] : p.r * cyc[big][0] * 0.9) / 1900.0;
+}
+
 struct RecurPlan {
     int nseg, seg_tok;
 };
@@ -459,12 +466,11 @@ size_t seg_bytes(const Problem& p, int nseg) {
 // (d_k = 64: two, whose chains leave each other most of the issue slots) runs per SM; against it stand two more kernels, about
 // 1 us of composing per segment, and the traffic and products of the responses.
 RecurPlan make_plan(const Problem& p) {
-    static const double cyc[2][4] = {{204, 259, 330, 401}, {275, 373, 480, 590}};      // a token, d_k = 64 and 128 (sum form)
     RecurPlan plan{1, p.L};
     if (p.L < 128 || p.wu_builder) return plan;
     const long long nseq = (long long)p.B * p.H, sms = sm_count();
     const bool big = p.d_k == 128;
-    const double tok = (p.mask_group() == p.r ? cyc[big][p.r - 1] : p.r * cyc[big][0] * 0.9) / 1900.0;
+    const double tok = token_us(p);
     const double walk = nseq * (p.d_v / RJ) > sms ? 0.0 : 4.0 + p.L * tok;      // (one wave: otherwise there is nothing to gain)
     const double extra = 20.0 + (double)nseq * p.L * (p.d_k * p.d_v / 12e6 + (8.0 * p.d_k + 8.0 * p.d_v) / 4e6);
     double best = 0.75 * walk;
@@ -509,6 +515,14 @@ int launch_seg_tail(const Problem& p, const RecurPlan& plan, const RecurSeg& sg)
 }
 
 }  // namespace
+
+// The kernel's time for a call of a few tokens, without segments (measured up to 64 tokens and 512 sequences): the chain of one
+// token, or where the CTAs are more than the SMs their instructions, which leave little to overlap.
+double recur_short_us(const Problem& p) {
+    const double ctas = (double)p.B * p.H * (p.d_v / RJ), sms = sm_count() > 0 ? sm_count() : 1;
+    const double crowd = (p.d_k == 128 ? 0.9 : 0.72) * ctas / sms;
+    return 3.3 + p.L * 1.1 * token_us(p) * (crowd > 1.0 ? crowd : 1.0);
+}
 
 size_t recur_workspace_bytes(const Problem& p) {
     const RecurPlan plan = make_plan(p);
