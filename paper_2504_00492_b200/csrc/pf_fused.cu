@@ -49,7 +49,7 @@
 // Each chunk they write an fp16 copy of it into TENSOR memory, where it is the A operand of both of the chunk's
 // products (Delta = S E^T issued by warp 15, O^T = S Qt^T issued by warp 13), so the serial step never goes
 // through shared memory.  Warps 8-11 add OI and write O, warp 12 streams the E / Xi / Qt images in with bulk
-// copies and is the only poller of the ready flags, warp 14 reports consumed chunks.
+// copies, warp 14 polls the ready flags and reports consumed chunks.
 //
 // Every wait is bounded (about a second of cycles) and reports a code in the status word.  Outer loops are
 // deliberately kept rolled: the instruction footprint of sixteen differently-specialised warps matters.
@@ -640,7 +640,7 @@ __device__ void scan_role(const FusedGeo& g, const FusedWs& ws, const float* __r
     const uint8_t* ring = ws.ring + (size_t)seq * g.R * SLOT_BYTES;
     const int* ready = ws.ready + seq * 64;
     volatile int* vis = (volatile int*)(smem + F_BAR + B_COUNT * 8 + 8);   // chunks whose ready flag the producer has acquired
-    volatile int* odone = (volatile int*)(smem + F_BAR + B_COUNT * 8 + 12); // output-warp completions (4 per chunk)
+    volatile int* loaded = (volatile int*)(smem + F_BAR + B_COUNT * 8 + 12); // leading chunks whose images are in shared memory
 
     if (warp < 8) {
         // ------------------------------------------------ chain: the state lives here -------------------------
@@ -737,7 +737,6 @@ __device__ void scan_role(const FusedGeo& g, const FusedWs& ws, const float* __r
                 fence_async_global();
                 bulk_reduce_add_f32(O + ((long long)seq * g.L + (long long)c * g.C) * DV, img, (uint32_t)Cv * DV * 4u);
                 bulk_commit();
-                atomicAdd((int*)odone, 4);       // (a counter, not a barrier: the reporter may lag by any amount)
             }
         }
         if (tid == 256) bulk_wait_all();
@@ -791,16 +790,24 @@ __device__ void scan_role(const FusedGeo& g, const FusedWs& ws, const float* __r
             gemm_ta<L_NSK, DK, DK, 128>(t_delta, t_a + buf * 64, smem_u32(smem + S_EQ + buf * 49152));
             commit_uni(&bar[B_DDONE]);
             commit_uni(&bar[B_APUB + buf]);
+            // (with Xi landed too the chunk's ring slot is free; a count, not a barrier: the reporter may lag by any amount)
+            if (!PF_WAIT(B_XIFULL + buf, (c >> 1) & 1, 237)) return;
+            if (lane == 0) {
+                __threadfence_block();
+                *loaded = c + 1;
+            }
         }
     } else if (warp == 14) {
         // ------------------------------------------------ ready flags in, consumed reports out -----------------
         // The warp polls the ring's ready flags, as far ahead of the loads as the flow CTAs are, one flag per lane: a flag takes
         // a trip to the L2 (about 800 cycles), and one after another they held the loads back to one chunk per 2.5 k cycles.  The
-        // count of leading chunks that are ready is published in shared memory.  The same loop reports consumption: once the
-        // four output warps are done with chunk c, chunks < c are consumed (the chain finished chunk c-1 before it published the
-        // state for chunk c) and their ring slots may be rewritten.  It polls a shared counter and always reports the latest
-        // value, however far it has fallen behind.
+        // count of leading chunks that are ready is published in shared memory.  The same loop reports consumption: a ring slot may
+        // be rewritten once its images have been copied into shared memory (reported when the chunk's output was done, the ring was
+        // two steps shorter; with that and a device-wide fence before the count: 32 sequences of 2048 tokens, r = 1: 70.8 us instead
+        // of 69.1; of 8192, r = 2: 277 instead of 269).  It polls a shared counter and always reports the latest value,
+        // however far it has fallen behind.
         int reported = 0, seen = 0;
+        uint32_t idle = 0;
         long long t_last = clock64();
         while (reported < NC - 1 || seen < NC) {
             bool progress = false;
@@ -809,14 +816,16 @@ __device__ void scan_role(const FusedGeo& g, const FusedWs& ws, const float* __r
             const int n = __ffs(~__ballot_sync(0xffffffffu, up)) - 1;      // (leading chunks that are ready; -1 means all 32)
             if (n != 0) {
                 seen += n < 0 ? 32 : n;
-                __threadfence();
                 __syncwarp();
-                if (lane == 0) *vis = seen;
+                if (lane == 0) {
+                    __threadfence_block();
+                    *vis = seen;
+                }
                 progress = true;
             }
-            const int chunks_done = __shfl_sync(0xffffffffu, *odone, 0) >> 2;
-            if (chunks_done - 1 > reported) {
-                reported = chunks_done - 1;
+            const int done = __shfl_sync(0xffffffffu, *loaded, 0);
+            if (done > reported) {
+                reported = done;
                 if (lane == 0) {
                     __threadfence_block();
                     st_release_gpu(&ws.consumed[seq * 32], reported);
@@ -830,7 +839,7 @@ __device__ void scan_role(const FusedGeo& g, const FusedWs& ws, const float* __r
                 if (clock64() - t_last > WAIT_CYCLES) {
                     atomicCAS(err, 0, 232);
                     stop = 1;
-                } else if (*(volatile int*)err != 0) {
+                } else if ((++idle & 31u) == 0 && *(volatile int*)err != 0) {      // (another trip to the L2)
                     stop = 1;
                 } else if (seen == NC) {
                     __nanosleep(200);
