@@ -172,8 +172,9 @@ __device__ __forceinline__ void gram_blocks(uint32_t k_b, uint32_t q_b, uint8_t*
 #pragma unroll
             for (int tt = 0; tt < TT; ++tt) used = used || p_owner<R>(tt, nb) == W;
             if (!used) continue;
-            uint32_t x[4];
-            ldmatrix_x4(x, k_b + (offN ^ ((kk & 3) << 5)) + nb * 2048 + (kk >> 2) * (NB * 128));
+            // (the warp's own rows as columns: the fragment it has, its two middle pieces exchanged)
+            uint32_t x[4] = {ka[0], ka[2], ka[1], ka[3]};
+            if (nb != W) ldmatrix_x4(x, k_b + (offN ^ ((kk & 3) << 5)) + nb * 2048 + (kk >> 2) * (NB * 128));
             if (nb <= W) {
                 mma_acc(ga[nb][0], ka, x[0], x[1], kk > 0);
                 mma_acc(ga[nb][1], ka, x[2], x[3], kk > 0);
