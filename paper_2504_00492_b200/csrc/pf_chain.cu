@@ -15,12 +15,14 @@
 //   prep warps    teams of four: K, Q -> fp16 in place, G = K K^T, the inverse, P; a few blocks ahead
 // A stage of shared memory holds what the chain needs of one block: K, Q (fp16), T, P (fp16), V (bf16 as it came).
 //
-// What bounds it: the mma.sync pipe is busy for about half of the time when every SM has a CTA (d = 128, r = 2: 3.7 k of 7.2 k
-// cycles per block of 32 tokens, 128 columns per CTA), the rest is the latency of the chain's dependent products.  Measured
-// (kernel time, against the tcgen05 kernels in two launches or one): 256 sequences of 1024 tokens, d = 128, r = 2: 0.25 ms
-// against 0.63; 128 sequences of 4096, d = 64, r = 4: 0.38 against 0.93; 48 sequences of 1999, 64 x 128, r = 3: 0.165
-// against 0.33.  Where the tcgen05 kernel in one launch has few sequences and enough SMs to build flows ahead (d = 128), it
-// is the faster one: see chain_preferred.
+// What bounds it: where every SM has a CTA (d = 128, r = 2, 128 columns per CTA) a block of 32 tokens takes 6.5 k cycles, of
+// which the shared-memory pipe is busy for 80 % and the mma.sync pipe for 58 %; with few CTAs it is the latency of the chain's
+// dependent products (1.8 us a block at d = 128, 1.3 at 64).  Measured (kernel time, against the tcgen05 kernels in two
+// launches or one): 256 sequences of 1024 tokens, d = 128, r = 2: 0.23 ms against 0.63; 128 sequences of 4096, d = 64, r = 4: 0.35
+// against 0.93; 48 sequences of 1999, 64 x 128, r = 3: 0.149 against 0.33.  Measured and not taken: chain warps of 32 rows (half the
+// shared-memory reads, but one such warp per scheduler does not hide its own latencies: 0.31 ms at the first size), fragments
+// requested two to six ahead by hand (0.243), G from the bf16 tiles with the conversion after it (0.27).  Where the tcgen05 kernel
+// in one launch has few sequences and enough SMs to build flows ahead (d = 128), it is the faster one: see the estimates.
 //
 // The inverse: warp i of a team owns rows 16 i .. 16 i + 15.  D_i = (I + A_ii)^{-1} by its Neumann product and
 // E_ij = D_i A_ij in registers, then X_ij = -sum_k E_ik X_kj row block by row block (three exchanges through shared memory).
@@ -88,10 +90,10 @@ struct ChainCfg {
     static constexpr int NCW = JS / 16 * IS;                      // chain warps
     static constexpr int threads = 32 * NCW + 128 * TEAMS;
     static constexpr int xs_off = NS * SM::stage;                 // per team: X (unscaled) while it is being formed
-    static constexpr int beta_off = xs_off + TEAMS * NB * 128;    // per team: 64 step sizes
+    static constexpr int beta_off = xs_off + TEAMS * NB * 128;    // per team: 64 step sizes, of two blocks in turn
     // IS = 2: partial sums on their way to the other warp of the pair, [pair][parity][warp][thread-linear 16-byte pieces]
     static constexpr int x_piece = 8 + SM::CP / 16;               // 16-byte pieces per thread: 32 of S K^T, 4 per 16 tokens of Q S^T
-    static constexpr int ex_off = beta_off + TEAMS * 256;
+    static constexpr int ex_off = beta_off + TEAMS * 512;
     static constexpr int ex_bytes = IS == 2 ? (JS / 16) * 2 * 2 * x_piece * 512 : 0;
     static constexpr int total = ex_off + ex_bytes;
 };
@@ -172,9 +174,10 @@ __device__ __forceinline__ void gram_blocks(uint32_t k_b, uint32_t q_b, uint8_t*
 #pragma unroll
             for (int tt = 0; tt < TT; ++tt) used = used || p_owner<R>(tt, nb) == W;
             if (!used) continue;
-            // (the warp's own rows as columns: the fragment it has, its two middle pieces exchanged)
+            // (the warp's own rows as columns: the fragment it has, its two middle pieces exchanged; at d_k = 128 holding it that
+            //  long pays at r = 2 only: 231 us instead of 234 for 256 sequences of 1024 tokens, but 365 instead of 350 at r = 3)
             uint32_t x[4] = {ka[0], ka[2], ka[1], ka[3]};
-            if (nb != W) ldmatrix_x4(x, k_b + (offN ^ ((kk & 3) << 5)) + nb * 2048 + (kk >> 2) * (NB * 128));
+            if (nb != W || (DK == 128 && R != 2)) ldmatrix_x4(x, k_b + (offN ^ ((kk & 3) << 5)) + nb * 2048 + (kk >> 2) * (NB * 128));
             if (nb <= W) {
                 mma_acc(ga[nb][0], ka, x[0], x[1], kk > 0);
                 mma_acc(ga[nb][1], ka, x[2], x[3], kk > 0);
@@ -219,7 +222,6 @@ __device__ __forceinline__ void prep_role(const ChainGeo& g, const ChainPart& pa
     const int bar_id = 1 + team;
     uint8_t* xs = smem + CFG::xs_off + team * NB * 128;
     const uint32_t xs_b = smem_u32(xs);
-    float* sBeta = (float*)(smem + CFG::beta_off + team * 256);
     const uint32_t offA = lane_off(lane & 15, lane >> 4);
     const uint32_t offN = lane_off((lane & 7) + ((lane >> 4) << 3), (lane >> 3) & 1);
     const uint32_t offT = lane_off((lane & 7) + (((lane >> 3) & 1) << 3), lane >> 4);
@@ -238,6 +240,8 @@ __device__ __forceinline__ void prep_role(const ChainGeo& g, const ChainPart& pa
         const int st = b % NS;
         uint8_t* sg = smem + st * SM::stage;
         const uint32_t k_b = smem_u32(sg + SM::k_off), q_b = smem_u32(sg + SM::q_off);
+        // (two in turn: another warp may still be scaling T of the block before)
+        float* sBeta = (float*)(smem + CFG::beta_off + team * 512 + (b / TEAMS & 1) * 256);
         // (a failed wait must not strand the others at a barrier: the next one carries the outcome)
         const bool ok = mbar_wait_clk(&land[st], (uint32_t)(b / NS) & 1, err, 311);
         // ---- K, Q: bf16 -> fp16 in place (elementwise, so the swizzled layout is untouched), several pieces per round, so that
