@@ -699,11 +699,11 @@ chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __rest
         part.S_end = part.response ? (float*)(sg.P + slot * DK * DK) : sg.Xi + slot * DK * g.d_v;
     }
     if ((smem_u32(smem) & 1023u) != 0) {                          // (the swizzled layouts need a 1024-byte aligned base)
+        wait_for_previous_kernel();
         if (tid == 0) atomicCAS(status, 0, 99);
         return;
     }
     if (tid == 0) {
-        if (blockIdx.x == 0 && g.clear) *status = 0;                      // (the call's status word: a wait expires a second from now at the earliest)
         for (int x = 0; x < NS; ++x) {
             mbar_init(&land[x], 1);
             mbar_init(&full[x], 128);
@@ -718,6 +718,9 @@ chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __rest
         for (int e = tid; e < NS * SM::stage / 16; e += CFG::threads) ((uint4*)smem)[e] = make_uint4(0, 0, 0, 0);
         fence_async_smem();
     }
+    wait_for_previous_kernel();
+    if (!SEG) let_next_kernel_start();      // (chain_compose's blocks would crowd on what few multiprocessors have room: 144 us instead of 140)
+    if (tid == 0 && blockIdx.x == 0 && g.clear) *status = 0;      // (the call's status word: a wait expires a second from now at the earliest)
     __syncthreads();
     if (tid == 0)
         for (int b = 0; b < NS && b < part.nblk; ++b) load_block<DK, R, JS, NS>(maps, smem, land, b, (int)seq, part);
@@ -760,6 +763,7 @@ __global__ void __launch_bounds__(128) chain_compose(ChainSeg sg, float* __restr
             for (int e = 0; e < 4; ++e) x[n][e] = src[(long long)(i0 + 8 * n + (e & 1)) * d_v + j + 8 * (e >> 1)];
     };
     float X[NT][4];                                               // Xi of the next step
+    wait_for_previous_kernel();
     load_p(1);
     xi(0, S);
     xi(1, X);
@@ -822,6 +826,7 @@ __global__ void __launch_bounds__(256) chain_apply(ChainSeg sg, float* __restric
     const int s = 1 + (int)(blockIdx.y % (nseg - 1));
     const int t_end = min(L, (s + 1) * seg_tokens), t0 = s * seg_tokens + blockIdx.x * 128 + w * 16 + gq;
     const __half* src = sg.start + (seq * nseg + s) * DV * DK;
+    wait_for_previous_kernel();
 #pragma unroll
     for (int e = 0; e < DV * DK / 8 / 256; ++e) {
         const int p = e * 256 + tid, row = p / (DK / 8), c = p % (DK / 8);
@@ -847,6 +852,9 @@ __global__ void __launch_bounds__(256) chain_apply(ChainSeg sg, float* __restric
         c[n][0] = x.x; c[n][1] = x.y; c[n][2] = y.x; c[n][3] = y.y;
     }
     __syncthreads();
+    // (where the blocks are many, those of the next kernel would come to multiprocessors in the order in which these leave, apart
+    //  from their neighbours with the same inputs: calls of 4 sequences of 16384 tokens one after another 139 us instead of 133)
+    if (gridDim.x * gridDim.y <= 128) let_next_kernel_start();
 #pragma unroll
     for (int np = 0; np < DV / 16; ++np) {
 #pragma unroll
@@ -958,7 +966,7 @@ int launch(const Problem& p, const ChainPlan& plan, const ChainSeg& sg) {
     if (st != PF_OK) return st;
     void* args[] = {(void*)&maps, (void*)&p.beta, (void*)&p.S0, (void*)&p.O, (void*)&p.S_final, (void*)&p.status, (void*)&g, (void*)&sg};
     prof_begin("chain", p.stream);
-    PF_CUDA_TRY(cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(CFG::threads), args, (size_t)CFG::total, p.stream));
+    PF_CUDA_TRY(launch_early(fn, dim3((unsigned)grid), CFG::threads, args, (size_t)CFG::total, p.stream));
     prof_end(p.stream);
     count_launch(1);
     return PF_OK;
@@ -988,7 +996,7 @@ int launch_rank(const Problem& p, const ChainPlan& plan, const ChainSeg& sg) {
 
 template <int DK, int DV>
 int launch_seg_tail(const Problem& p, const ChainPlan& plan, const ChainSeg& sg) {
-    const int nseq = p.B * p.H, seg_tokens = plan.seg_blk * (NB / p.r);
+    const int nseq = p.B * p.H, dv = DV, seg_tokens = plan.seg_blk * (NB / p.r);
     constexpr int LD = DK + 8;
     {
         constexpr int smem = (2 * DK + 2 * 16) * LD * 2;
@@ -996,16 +1004,16 @@ int launch_seg_tail(const Problem& p, const ChainPlan& plan, const ChainSeg& sg)
         const int st = allow_smem(opted_in, (const void*)chain_compose<DK>, smem);
         if (st != PF_OK) return st;
         prof_begin("chain_compose", p.stream);
-        chain_compose<DK><<<(unsigned)(nseq * (DV / 16)), 128, smem, p.stream>>>(sg, p.S_final, plan.nseg, DV);
+        void* args[] = {(void*)&sg, (void*)&p.S_final, (void*)&plan.nseg, (void*)&dv};
+        PF_CUDA_TRY(launch_early((const void*)chain_compose<DK>, dim3((unsigned)(nseq * (DV / 16))), 128, args, smem, p.stream));
         prof_end(p.stream);
-        PF_CUDA_TRY(cudaGetLastError());
     }
     constexpr int smem = DV * LD * 2;
     prof_begin("chain_apply", p.stream);
-    chain_apply<DK, DV><<<dim3((unsigned)((seg_tokens + 127) / 128), (unsigned)(nseq * (plan.nseg - 1))), 256, smem, p.stream>>>(
-        sg, p.O, p.L, seg_tokens, plan.nseg);
+    void* args[] = {(void*)&sg, (void*)&p.O, (void*)&p.L, (void*)&seg_tokens, (void*)&plan.nseg};
+    PF_CUDA_TRY(launch_early((const void*)chain_apply<DK, DV>, dim3((unsigned)((seg_tokens + 127) / 128), (unsigned)(nseq * (plan.nseg - 1))), 256,
+                             args, smem, p.stream));
     prof_end(p.stream);
-    PF_CUDA_TRY(cudaGetLastError());
     count_launch(2);
     return PF_OK;
 }

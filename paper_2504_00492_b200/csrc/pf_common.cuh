@@ -85,6 +85,30 @@ inline int allow_smem(std::atomic<uint64_t>& done, const void* fn, int bytes) {
     return PF_OK;
 }
 
+// Launches a kernel that calls wait_for_previous_kernel() before it touches global memory, so that its launch and its set-up
+// (barriers, tensor maps) overlap the end of the kernel before it on the stream, or more of it if that one calls
+// let_next_kernel_start().  Calls one after another: 2 - 3 us less each (a decoded token 8.2 -> 5.5 us, 333 tokens of 16 sequences
+// 25.4 -> 23.4), and as much again for the two tail kernels of a call in segments (70 -> 62 us at 16 fp32 sequences of 1000).
+inline cudaError_t launch_early(const void* fn, dim3 grid, unsigned threads, void** args, size_t smem, cudaStream_t stream) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelExC(&cfg, fn, args);
+}
+#ifdef __CUDACC__
+// All threads: the kernel before this one on the stream is complete and its writes are visible.
+__device__ __forceinline__ void wait_for_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// The next kernel's blocks may take the multiprocessors that this one leaves free.
+__device__ __forceinline__ void let_next_kernel_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+#endif
+
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 // room at the end of every workspace for the fp32 step sizes of PF_STEP_EXACT
 inline size_t beta32_bytes(const Problem& p) { return align_up((size_t)p.B * p.H * p.L * p.r * 4, 256); }

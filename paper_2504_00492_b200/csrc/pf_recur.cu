@@ -150,13 +150,15 @@ recur_kernel(const Tin* __restrict__ q, const Tin* __restrict__ k, const Tin* __
     auto s_b = [&](int st) { return (float*)(s_v(st) + rows_s * RJ); };
 
     if (tid == 0) {
-        if (blockIdx.x == 0 && g.clear) *status = 0;              // (the call's status word; a wait of this kernel expires a second later at the earliest)
         for (int x = 0; x < R_STAGES; ++x) {
             tc::mbar_init(&bar_full[x], 1);
             tc::mbar_init(&bar_empty[x], IG);
         }
         tc::mbar_fence_init();
     }
+    wait_for_previous_kernel();
+    if (g.nseg == 1) let_next_kernel_start();      // (recur_compose's blocks would crowd on what few multiprocessors have room: 75 us instead of 70)
+    if (tid == 0 && blockIdx.x == 0 && g.clear) *status = 0;      // (the call's status word; a wait of this kernel expires a second later at the earliest)
     __syncthreads();
 
     if (warp == IG) {
@@ -344,6 +346,7 @@ __global__ void __launch_bounds__(256) recur_compose(RecurSeg sg, float* __restr
         for (int u = 0; u < NV; ++u) pv[u] = p[u * 256 + tid];
     };
     auto fetch_x = [&](int s) { return *(const float4*)(sg.Xi + ((seq * nseg + s) * DK + i) * d_v + j); };
+    wait_for_previous_kernel();
     float4 acc = fetch_x(0);
     fetch_p(1);
     xv = fetch_x(1);
@@ -391,6 +394,8 @@ __global__ void __launch_bounds__(256) recur_apply(RecurSeg sg, float* __restric
     const long long seq = blockIdx.y / (nseg - 1);
     const int s = 1 + (int)(blockIdx.y % (nseg - 1)), t0 = s * seg_tok + blockIdx.x * 64;
     const int nt = min(64, min(L, (s + 1) * seg_tok) - t0);
+    wait_for_previous_kernel();
+    let_next_kernel_start();
     if (nt <= 0) return;
     const float4* st = (const float4*)(sg.start + (seq * nseg + s) * DK * DV);
 #pragma unroll
@@ -490,26 +495,26 @@ RecurPlan make_plan(const Problem& p) {
 
 template <int DK, int DV>
 int launch_seg_tail(const Problem& p, const RecurPlan& plan, const RecurSeg& sg) {
-    const int nseq = p.B * p.H;
+    const int nseq = p.B * p.H, dv = DV;
     {
         constexpr int rows = 4 * (8 / (DK / 32)), smem = (DK * (DK + 4) + rows * DK) * 4;
         static std::atomic<uint64_t> opted_in{0};
         const int st = allow_smem(opted_in, (const void*)recur_compose<DK>, smem);
         if (st != PF_OK) return st;
         prof_begin("recur_compose", p.stream);
-        recur_compose<DK><<<(unsigned)(nseq * (DV / rows)), 256, smem, p.stream>>>(sg, p.S_final, plan.nseg, DV);
+        void* args[] = {(void*)&sg, (void*)&p.S_final, (void*)&plan.nseg, (void*)&dv};
+        PF_CUDA_TRY(launch_early((const void*)recur_compose<DK>, dim3((unsigned)(nseq * (DV / rows))), 256, args, smem, p.stream));
         prof_end(p.stream);
-        PF_CUDA_TRY(cudaGetLastError());
     }
     constexpr int smem = (DK * DV + DK * 68) * 4;
     static std::atomic<uint64_t> opted_in{0};
     const int st = allow_smem(opted_in, (const void*)recur_apply<DK, DV>, smem);
     if (st != PF_OK) return st;
     prof_begin("recur_apply", p.stream);
-    recur_apply<DK, DV><<<dim3((unsigned)((plan.seg_tok + 63) / 64), (unsigned)(nseq * (plan.nseg - 1))), 256, smem, p.stream>>>(
-        sg, p.O, p.L, plan.seg_tok, plan.nseg);
+    void* args[] = {(void*)&sg, (void*)&p.O, (void*)&p.L, (void*)&plan.seg_tok, (void*)&plan.nseg};
+    PF_CUDA_TRY(launch_early((const void*)recur_apply<DK, DV>, dim3((unsigned)((plan.seg_tok + 63) / 64), (unsigned)(nseq * (plan.nseg - 1))),
+                             256, args, smem, p.stream));
     prof_end(p.stream);
-    PF_CUDA_TRY(cudaGetLastError());
     count_launch(2);
     return PF_OK;
 }
@@ -568,7 +573,7 @@ int recur_forward(const Problem& p, void* workspace) {
     }
     void* args[] = {(void*)&p.q, (void*)&p.k, (void*)&p.v, (void*)&p.beta, (void*)&p.S0, (void*)&p.O, (void*)&p.S_final, (void*)&p.status, (void*)&g, (void*)&sg};
     prof_begin("recur", p.stream);
-    PF_CUDA_TRY(cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(160), args, (size_t)smem, p.stream));
+    PF_CUDA_TRY(launch_early(fn, dim3((unsigned)grid), 160, args, (size_t)smem, p.stream));
     prof_end(p.stream);
     count_launch(1);
     if (plan.nseg == 1) return PF_OK;
