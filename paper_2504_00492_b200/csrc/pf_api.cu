@@ -334,7 +334,9 @@ int forward_one(const pf_params* a, bool top) {
         if (st == PF_OK && top) end_call();
         return st;
     }
-    if (top) {      // (the passes of a segmented call share the word: the first expired wait of any of them stays)
+    // (the passes of a segmented call share the word: the first expired wait of any of them stays)
+    p.clear_status = top && impl == PF_IMPL_TC && use_fused(p);      // the single launch clears it itself
+    if (top && !p.clear_status) {
         cudaError_t e = cudaMemsetAsync(p.status, 0, sizeof(int), p.stream);
         if (e != cudaSuccess) {
             if (own) cudaFreeAsync(ws, p.stream);

@@ -101,7 +101,9 @@ struct FusedGeo {
 };
 
 struct FusedWs {
-    int* status;        // word 0: first expired wait (0 = none)
+    int* status;        // in the workspace, cleared with the flags: first expired wait of this launch (0 = none)
+    int* report;        // the call's status word
+    int clear;          // set the call's status word to 0
     int* ready;         // [nseq][64] (R <= 64 used): chunk index + 1 once the slot holds that chunk; 256 B per sequence
     int* consumed;      // [nseq][32]: word 0 = number of leading chunks the scan no longer needs; 128 B per sequence
     uint8_t* ring;      // [nseq][R][SLOT_BYTES]
@@ -861,9 +863,11 @@ fused_kernel(const __grid_constant__ FusedMaps maps, FusedGeo g, FusedWs ws, con
     const bool is_scan = (int)blockIdx.x < g.n_scan;
 
     if ((smem_u32(smem) & 1023u) != 0) {       // the swizzled layouts need a 1024-byte aligned base
-        if (tid == 0) atomicCAS(ws.status, 0, 99);
+        if (tid == 0) atomicCAS(ws.report, 0, 99);
         return;     // uniform: every thread of the CTA leaves
     }
+    // (a wait expires a second from now at the earliest; a memset of its own in front of the kernel cost the call 2.5 us)
+    if (tid == 0 && blockIdx.x == 0 && ws.clear) *ws.report = 0;
     if (tid == 0) {
         if (is_scan) {
             for (int x = 0; x < 2; ++x) {
@@ -911,9 +915,12 @@ fused_kernel(const __grid_constant__ FusedMaps maps, FusedGeo g, FusedWs ws, con
     if (is_scan) scan_role(g, ws, S0, O, S_final, smem, bar, tb, (int)blockIdx.x);
     else flow_role<N>(maps, g, ws, beta, O, smem, bar, tb, (int)blockIdx.x - g.n_scan);
 
-
     tc_fence_before();
     __syncthreads();
+    if (tid == FT - 32 && ws.report != ws.status) {
+        const int code = *(volatile int*)ws.status;
+        if (code != 0) atomicCAS(ws.report, 0, code);
+    }
     if (warp == 0) tmem_dealloc(tb, 512);
 }
 
@@ -980,7 +987,9 @@ int fused_forward(const Problem& p, void* workspace) {
     const Carve cv = carve(p);
     uint8_t* base = (uint8_t*)workspace;
     FusedWs ws;
-    ws.status = p.status;
+    ws.status = (int*)base;
+    ws.report = p.status;
+    ws.clear = p.clear_status && p.status != (int*)base;
     ws.ready = (int*)(base + cv.ready);
     ws.consumed = (int*)(base + cv.consumed);
     ws.ring = base + cv.ring;
