@@ -25,8 +25,8 @@
  *   - Tensor pointers are DEVICE pointers owned by the caller, dense row-major in the shapes given;
  *     the library neither frees nor keeps them.  q/k/v/beta/O must be 16-byte aligned.
  *   - `stream` is a cudaStream_t (NULL = the default stream).  Work is enqueued; the calls do not
- *     synchronise (pf_read_status and pf_profile_read do).  Unless a workspace is passed through pf_deltanet_fwd_ex, scratch memory is
- *     taken and returned with stream-ordered allocation on `stream`.
+ *     synchronise (pf_read_status and pf_profile_read do).  Unless a workspace is passed through pf_deltanet_fwd_ex, scratch
+ *     memory is taken from and returned to a pool of the library's own, ordered on `stream` (see pf_release_workspaces).
  *   - O must not alias an input.  S_final may alias S0.
  *   - Return value: PF_OK (0) or a negative pf_status.  Nothing is launched when an argument check
  *     fails.  No exceptions, no exit().
@@ -82,22 +82,24 @@ enum { PF_MODE_SUM = 0, PF_MODE_PRODUCT = 1 };
  *                   form with r > 1 returns PF_ERR_UNSUPPORTED.  beta' < 1/|k|^2, so every factor contracts. */
 enum { PF_STEP_EULER = 0, PF_STEP_EXACT = 1 };
 
-/* Which kernels evaluate the chunk form.
- *   PF_IMPL_AUTO : tensor-core path where it supports the shape/dtype, else the fp32 SIMT path.  The result does
- *                  not depend on the chunk length beyond rounding, so AUTO may evaluate with another chunk length
- *                  than the one passed when that puts the problem on the tensor-core kernels, which take up to 128
+/* Which kernels evaluate the operation.
+ *   PF_IMPL_AUTO : bf16: whichever is expected to be faster of the chunk form on warp-level tensor-core products (one
+ *                  kernel, blocks of 64 / r tokens; few long sequences in segments side by side, three kernels), the
+ *                  tcgen05 kernels, and, for a few tokens, the recurrence token by token.  fp32: the recurrence token by
+ *                  token.  The result does not depend on the chunk length beyond rounding, so AUTO may evaluate with
+ *                  another chunk length than the one passed.  The tcgen05 kernels take up to 128
  *                  rows (chunk * r) per chunk: a chunk with more rows is evaluated as consecutive blocks of whole
  *                  tokens (r = 4 with chunk 64 as blocks of 32 tokens, r = 3 with chunk 64 as blocks of 42), the
  *                  block forward substitution of the chunk's triangular system with the coupling between blocks
  *                  carried by the state; a chunk with fewer than 64 rows is lengthened.  pf_select_chunk tells which
  *                  length is used.  PF_IMPL_TC and PF_IMPL_TC_SPLIT split long chunks into blocks the same way but
  *                  never lengthen a chunk; PF_IMPL_SIMT and PF_IMPL_TC_REFFLOW use `chunk` as given.
- *   PF_IMPL_SIMT : fp32 FFMA kernels (any supported shape; the only path for PF_DTYPE_F32).
+ *   PF_IMPL_SIMT : fp32 FFMA kernels (any supported shape; the only path for PF_DTYPE_F32): the recurrence token by token, or
+ *                  with wu_builder = 1 the chunk form.
  *   PF_IMPL_TC   : tcgen05 tensor-core kernels (bf16 inputs); PF_ERR_UNSUPPORTED otherwise.  For
  *                  d_k = d_v = 128 with at most (SM count - 8) sequences this is ONE cooperative launch in
  *                  which flow-building CTAs and state-scanning CTAs run side by side; other shapes take
- *                  the two-launch form below.  (PF_IMPL_AUTO takes the single launch only up to 0.7 x SM count
- *                  sequences: beyond that too few SMs are left for building flows and two launches are faster.)   */
+ *                  the two-launch form below.  (PF_IMPL_AUTO takes the single launch only where most SMs can build flows.)   */
 enum { PF_IMPL_AUTO = 0, PF_IMPL_SIMT = 1, PF_IMPL_TC = 2,
        /* diagnostic: per-chunk flows built by the fp32 SIMT kernels, state scan on tensor cores */
        PF_IMPL_TC_REFFLOW = 3,
@@ -173,7 +175,7 @@ typedef struct pf_params {
     int in_dtype;             /* PF_DTYPE_BF16 or PF_DTYPE_F32 */
     int impl;                 /* PF_IMPL_* */
     void* workspace;          /* device scratch of >= pf_workspace_bytes(...) bytes, 256-byte aligned,
-                                 or NULL: stream-ordered allocation inside the call */
+                                 or NULL: taken from the library's pool */
     size_t workspace_bytes;
     void* stream;
     int mode;                 /* PF_MODE_SUM (0) or PF_MODE_PRODUCT; anything else: PF_ERR_INVALID */
@@ -220,7 +222,7 @@ size_t pf_workspace_bytes_ex(const pf_params* p);
 /* Which PF_IMPL_* pf_deltanet_fwd_ex would run for this problem (negative pf_status if none). */
 int pf_select_impl(int B, int H, int L, int d_k, int d_v, int r, int chunk, int in_dtype, int impl);
 /* The chunk length the kernels would be run with: `chunk` itself for an explicit implementation; under PF_IMPL_AUTO
- * possibly another supported length (see PF_IMPL_AUTO).  Negative pf_status if the problem is not supported. */
+ * possibly another supported length (see PF_IMPL_AUTO; that of the tcgen05 kernels: the others have their own blocks).  Negative pf_status if the problem is not supported. */
 int pf_select_chunk(int B, int H, int L, int d_k, int d_v, int r, int chunk, int in_dtype, int impl);
 
 /*
@@ -240,8 +242,9 @@ int pf_select_chunk(int B, int H, int L, int d_k, int d_v, int r, int chunk, int
  * word on the current device.  pf_last_wait_code() then gives the code that was read (host thread local):
  *     1xx  flow-building role of the single-launch path (101-103 solve warps, 11x-12x bulk warps, 14x-15x MMA-issuing
  *          warps, 16x flag warp),   2xx  its scanning role (20x chain, 21x output, 22x loads, 23x MMA issue),
+ *     30x  the token-by-token kernel,   31x  the warp-level chunk kernel,
  *     1-99 the two-launch path (tc_flow, tc_scan),   99  shared memory not 1024-byte aligned,   900  pf_wait_selftest.
- * The fp32 SIMT kernels have no such waits.
+ * The chunk-form fp32 kernels have no such waits.
  */
 int pf_read_status(const void* word, void* stream);
 int pf_last_wait_code(void);
