@@ -299,6 +299,7 @@ int forward_one(const pf_params* a, bool top) {
     p.O = a->O; p.S_final = a->S_final;
     p.stream = (cudaStream_t)a->stream;
 
+    p.own_workspace = !a->workspace;
     const size_t need = workspace_need(p, impl);
     void* ws = a->workspace;
     bool own = false;

@@ -878,7 +878,8 @@ __global__ void __launch_bounds__(256) chain_apply(ChainSeg sg, float* __restric
 // columns by pairs of warps 2.35, 1.82, 1.74, 1.70; 64 columns 3.3, 2.5, 2.55, 2.3; 128 columns 4.4, 3.4, 3.4, 3.0.  At d_k = 64 a step
 // is short enough that 32 columns gain nothing over 64, and 128 columns cost 1.53 times as much.
 // Segments: as many as one wave of CTAs holds pay for the second walk (the responses) and for two more kernels when few
-// sequences are long: taken where the estimate falls by a quarter at least.
+// sequences are long: taken where the estimate falls (d = 64, r = 1, one sequence: 1200 tokens 17 us instead of 38; d = 128: 600 tokens
+// 20.5 instead of 26).
 enum { COLS_32, COLS_64, COLS_128 };
 struct ChainPlan {
     int cols, nseg, seg_blk;
@@ -909,9 +910,11 @@ ChainPlan make_plan(const Problem& p) {
     }
     plan.us = 7.0 + nblk * st * best;
     plan.short_us = 5.0 * turns + nblk * st * best;
-    const double limit = 0.75 * plan.us;
+    const double limit = 0.92 * plan.us;
     // (kernels and their gaps, then the traffic of the responses and of O at about 4 TB/s)
-    const double extra = 16.0 + 6.0 + (double)nseq * p.L * (4.0 * p.d_k + 8.0 * p.d_v) / 4e6;
+    const double extra = (p.d_k == 128 ? 14.0 : 9.0) + (double)nseq * p.L * (4.0 * p.d_k + 8.0 * p.d_v) / 4e6;
+    // (calls of up to 512 tokens at d_k = 128 are one launch, as they are specified to be: 400 tokens, r = 2 take 27 us instead of 20)
+    if (p.d_k == 128 && p.L <= 512) return plan;
     for (int cols = p.d_k == 128 ? COLS_32 : COLS_64; cols <= COLS_64; ++cols) {
         const int js = cols == COLS_32 ? 32 : 64, vs = p.d_v / js, rs = p.d_k / js;
         const long long most = (sms / nseq + rs) / (vs + rs);

@@ -31,6 +31,7 @@ struct Problem {
     int wu_builder;         // fp32 SIMT path: 0 = triangular inverse then W = T'K, Uh = T'V; 1 = the wavefront system of
                             // Theorem 3.3 (pf_params.wu_builder)
     int ring_depth;         // single-launch path: slots per sequence of the hand-off ring, 0 = default (pf_params.ring_depth)
+    bool own_workspace;     // the workspace is the library's: as large as the kernels want
     bool clear_status;      // the kernels set *status to 0 first (false for the second pass of a segmented call)
     int* status;            // device word that receives the code of the first bounded wait that expires (never null
                             // when a tensor-core kernel is launched)

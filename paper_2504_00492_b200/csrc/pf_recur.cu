@@ -467,9 +467,9 @@ size_t seg_bytes(const Problem& p, int nseg) {
     const size_t nseq = (size_t)p.B * p.H, slots = nseq * nseg;
     return align_up(nseq * p.L * p.d_k * 4, 256) + align_up(slots * p.d_k * p.d_k * 4, 256) + 2 * align_up(slots * p.d_k * p.d_v * 4, 256);
 }
-// Segments, where they make the call a quarter shorter at least: the walk of a token costs about the same while at most one CTA
-// (d_k = 64: two, whose chains leave each other most of the issue slots) runs per SM; against it stand two more kernels, about
-// 1 us of composing per segment, and the traffic and products of the responses.
+// Segments, where they make the call shorter (one fp32 head of 256 tokens: 23 us instead of 29; of 180: 22, 21): the walk of a token costs about the same while at most one CTA
+// (d_k = 64: two, whose chains leave each other most of the issue slots) runs per SM; against it stand two more kernels, 1 to 2
+// us of composing per segment, and the traffic and products of the responses.
 RecurPlan make_plan(const Problem& p) {
     RecurPlan plan{1, p.L};
     if (p.L < 128 || p.wu_builder) return plan;
@@ -477,15 +477,15 @@ RecurPlan make_plan(const Problem& p) {
     const bool big = p.d_k == 128;
     const double tok = token_us(p);
     const double walk = nseq * (p.d_v / RJ) > sms ? 0.0 : 4.0 + p.L * tok;      // (one wave: otherwise there is nothing to gain)
-    const double extra = 20.0 + (double)nseq * p.L * (p.d_k * p.d_v / 12e6 + (8.0 * p.d_k + 8.0 * p.d_v) / 4e6);
-    double best = 0.75 * walk;
+    const double extra = (big ? 17.0 : 12.0) + (double)nseq * p.L * (p.d_k * p.d_v / 12e6 + (8.0 * p.d_k + 8.0 * p.d_v) / 4e6);
+    double best = 0.92 * walk;
     const long long most = (sms * (big ? 1 : 2) / nseq + p.d_k / RJ) / (p.d_v / RJ + p.d_k / RJ);
     for (int want = 2; want <= most && want <= 64; ++want) {
         const int seg_tok = (p.L + 16 * want - 1) / (16 * want) * 16, nseg = (p.L + seg_tok - 1) / seg_tok;
         const long long ctas = nseq * (nseg * (p.d_v / RJ) + (nseg - 1) * (p.d_k / RJ));
-        const double us = extra + nseg * (big ? 1.3 : 0.8) + seg_tok * tok * (ctas > sms ? 1.2 : 1.0);
+        const double us = extra + nseg * (big ? 1.9 : 0.8) + seg_tok * tok * (ctas > sms ? 1.2 : 1.0);
         // (a caller's workspace was sized for the chunk-form kernels of pf_simt.cu)
-        if (nseg > 1 && us < best && seg_bytes(p, nseg) + 256 <= simt_workspace_bytes(p)) {
+        if (nseg > 1 && us < best && (p.own_workspace || seg_bytes(p, nseg) + 256 <= simt_workspace_bytes(p))) {
             best = us;
             plan = {nseg, seg_tok};
         }

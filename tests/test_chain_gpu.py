@@ -27,6 +27,7 @@ def test_column_spreads(d_k, d_v, r, H):
 @pytest.mark.parametrize("d_k,d_v,r,H,L,mode", [
     (128, 128, 1, 1, 3001, "sum"), (128, 128, 2, 3, 2500, "sum"), (64, 64, 1, 2, 4097, "sum"), (64, 128, 3, 1, 2111, "product"),
     (128, 64, 4, 2, 1500, "sum"), (64, 64, 2, 10, 3000, "product"),
+    (64, 64, 2, 4, 200, "sum"), (64, 128, 4, 1, 230, "sum"), (128, 128, 2, 2, 600, "sum"),
 ])
 def test_few_long_sequences_are_walked_in_segments(d_k, d_v, r, H, L, mode):
     """Told apart by the number of kernels: the walk, the composition of the start states, their contribution to O."""
