@@ -2,6 +2,7 @@
 with each way of spreading a sequence's columns over CTAs (2, 40 and 160 sequences)."""
 import pytest
 
+import pf_synth
 from pf_synth import Workload
 from tests import util
 
@@ -36,3 +37,18 @@ def test_few_long_sequences_are_walked_in_segments(d_k, d_v, r, H, L, mode):
         w = Workload(f"chain_seg_{L}", B=1, H=H, L=L, d_k=d_k, d_v=d_v, r=r, chunk=64, s0_std=s0_std, seed=400 + r)
         util.check_parity(w, mode=mode)
         assert pf.pf_last_launch_count() == 3
+
+
+@pytest.mark.parametrize("d_k,d_v,r,H,L,mode", [(128, 128, 1, 4, 8000, "sum"), (64, 64, 1, 2, 4097, "sum"), (128, 128, 2, 3, 2500, "product"),
+                                                (64, 128, 3, 1, 2111, "sum")])
+def test_segments_of_a_state_that_changes_slowly(d_k, d_v, r, H, L, mode):
+    """Step sizes of about 0.01: a segment changes little of its start state, and only the change may be rounded to fp16 (2^-11 of
+    it; the whole sequence changes less than half of the state here), not the state once per segment."""
+    import paper_2504_00492_b200 as pf
+    w = Workload(f"slow_{L}", B=1, H=H, L=L, d_k=d_k, d_v=d_v, r=r, chunk=64, s0_std=0.1, beta_scale=0.02, seed=500 + r)
+    inp = pf_synth.make_inputs(w)
+    O, S = util.run_gpu(w, inp, mode=mode)
+    assert pf.pf_last_launch_count() == 3
+    O_ref, S_ref = util.run_oracle(inp, mode=mode)
+    util.check_per_sequence(O, O_ref, util.TOL_BF16, "O")
+    assert util.rel_l2(S, S_ref) <= 2 ** -12, util.rel_l2(S, S_ref)
