@@ -120,8 +120,11 @@ enum { PF_IMPL_AUTO = 0, PF_IMPL_SIMT = 1, PF_IMPL_TC = 2,
  * Value range: the tensor-core kernels round q, k, v, the per-chunk operands derived from them and, once per chunk,
  * the state S to fp16 before each product (fp32 accumulation).  fp16 has the 8 significant bits of bf16 and more, but
  * only the exponent range 6.1e-5 .. 65504: an element of v, S0 or of the running state beyond 65504 in magnitude becomes
- * infinite without an error code, and elements below 6.1e-5 lose precision gradually.  The stated tolerance (2e-3 of
- * max|O|) is tested for |v|, |S| up to the order of 1e3.  The operation is linear in (v, S0): scale them by a power
+ * infinite without an error code, and elements below 6.1e-5 lose precision gradually.  Products of the state with keys may
+ * exceed 65504 (with keys of length 1, S k reaches sqrt(d_k) times the largest entry of S): they stay in fp32 in the tcgen05
+ * kernels, and the warp-level kernel, where they are operands, computes the columns of O and S_final that lost them once more
+ * in fp32 (slowly, 1.3 to 3 us a token; columns that are infinite or NaN for other reasons pay this too).  The stated tolerance
+ * (2e-3 of max|O|) is tested for |v|, |S| up to the order of 1e3, and for states of 2e4 aligned with a key.  The operation is linear in (v, S0): scale them by a power
  * of two and O, S_final back for data outside that range, or ask for PF_IMPL_SIMT (fp32 throughout, no such limit).
  */
 int pf_deltanet_fwd(const void* q, const void* k, const void* v, const void* beta, const float* S0,

@@ -24,8 +24,15 @@
 // requested two to six ahead by hand (0.243), G from the bf16 tiles with the conversion after it (0.27).  Where the tcgen05 kernel
 // in one launch has few sequences and enough SMs to build flows ahead (d = 128), it is the faster one: see the estimates.
 //
+// Range: V - K S^T and U' are packed to fp16 like every other operand, and K S^T reaches sqrt(d_k) times the largest entry of S, so
+// that a state well inside fp16's 65504 can overflow them.  What overflows leaves its row of S infinite or NaN to the end of the walk
+// (infinity times anything is infinite or NaN), so one look at each row when the walk is over finds it and the blocks pay nothing:
+// the warp then walks its 16 rows once more, token by token in fp32 (walk_fp32).
+//
 // The inverse: warp i of a team owns rows 16 i .. 16 i + 15.  D_i = (I + A_ii)^{-1} by its Neumann product and
 // E_ij = D_i A_ij in registers, then X_ij = -sum_k E_ik X_kj row block by row block (three exchanges through shared memory).
+#include <float.h>
+
 #include <atomic>
 
 #include "pf_common.cuh"
@@ -50,6 +57,9 @@ struct ChainGeo {
     int rm;             // strict-mask group size (Problem::mask_group)
     int exact;          // PF_STEP_EXACT
     int clear;          // set the status word to 0
+    const __nv_bfloat16 *q, *k, *v, *beta;      // the inputs once more, for walk_fp32
+    const float* S0;
+    float *O, *S_final;
 };
 
 __device__ __forceinline__ uint32_t movmatrix(uint32_t x) {
@@ -116,6 +126,132 @@ struct ChainPart {
     float* S_end;       // end state [i][j] (response: fp16 [j][i] without its diagonal), or null
     float* D;           // response: the end state's diagonal
 };
+
+// Segments (Section 3, "Scan"; Proposition 2.1): the flow of an interval is the pair (P, Xi) with S_end = S_start P + Xi.  A
+// sequence is cut into segments that are walked side by side: for each the state from zero (S0 for the first segment), whose
+// outputs go to O and whose end is Xi, and, for all but the first, the state from the identity with v = 0, whose "outputs"
+// R_t = P_t q_t are what each token makes of its segment's start state and whose end is P.  Then one kernel composes the
+// segments' start states and another adds start R_t to O.
+// The diagonal of P is kept apart, in fp32, and fp16 is for the rest: where the step sizes are small P is close to the identity, and
+// rounding all of it (and the start state before it) would round the whole state once per segment (step sizes of 0.01, 8000
+// tokens in 9 segments: relative error of S_final 7.2e-4, this way 6.1e-5, 4.6e-5 in the tcgen05 kernels; at step sizes around 0.5
+// 3.49e-4 and 3.44e-4).
+struct ChainSeg {
+    __half* R;          // [nseq][L][d_k]
+    __half* P;          // [nseq][nseg][d_k j][d_k i], zeros on the diagonal
+    float* D;           // [nseq][nseg][d_k]: the diagonal
+    float* Xi;          // [nseq][nseg][d_k i][d_v j]
+    __half* start;      // [nseq][nseg][d_v j][d_k i]
+};
+
+// The kernel's arguments, for walk_fp32.
+struct ChainArgs {
+    ChainGeo g;
+    ChainSeg seg;
+};
+
+// What this CTA works on; seq: its sequence.
+template <int DK, int JS, int C, bool SEG>
+__device__ __forceinline__ ChainPart chain_part(const ChainGeo& g, const ChainSeg& sg, const float* S0, float* O, float* S_final, long long& seq) {
+    ChainPart part;
+    const int slices = g.d_v / JS;
+    if constexpr (!SEG) {
+        seq = blockIdx.x / slices;
+        part = {0, g.nblk, (int)(blockIdx.x % slices) * JS, g.d_v, false, S0 ? S0 + seq * DK * g.d_v : nullptr, O + seq * g.L * g.d_v,
+                S_final ? S_final + seq * DK * g.d_v : nullptr, nullptr};
+    } else {
+        constexpr int rs = DK / JS;
+        const int per_seq = g.nseg * slices + (g.nseg - 1) * rs, x = (int)(blockIdx.x % per_seq), y = x - g.nseg * slices;
+        seq = blockIdx.x / per_seq;
+        part.response = y >= 0;
+        const int s = part.response ? 1 + y / rs : x / slices;
+        part.b0 = s * g.seg_blk;
+        part.nblk = min(g.seg_blk, g.nblk - part.b0);
+        part.j0 = (part.response ? y % rs : x % slices) * JS;
+        part.width = part.response ? DK : g.d_v;
+        const long long row0 = seq * g.L + (long long)part.b0 * C, slot = seq * g.nseg + s;
+        part.S0 = s == 0 && S0 ? S0 + seq * DK * g.d_v : nullptr;
+        part.O = part.response ? (float*)(sg.R + row0 * DK) : O + row0 * g.d_v;
+        part.S_end = part.response ? (float*)(sg.P + slot * DK * DK) : sg.Xi + slot * DK * g.d_v;
+        part.D = sg.D + slot * DK;
+    }
+    return part;
+}
+
+// How they reach it.  The call is never made in ordinary use, but how it is written decides which registers the chain has: by value
+// cost the kernels that have none to spare 4 - 8 % (250 sequences of 1000, d = 128, r = 2: 243 us; from shared memory 227; without the
+// call 226), from shared memory the others up to 5 % (64 x 128, r = 4: 246 us; by value 235; without 236).
+template <int DK, int JS, bool SEG>
+constexpr bool WALK_BY_REF = DK == 128 && (JS == 128 || (SEG && JS == 64));
+
+// 16 rows of S from row `row0` of the CTA's on, once more: the recurrence token by token in fp32, by one warp, two lanes to a row.  Not
+// a fast path (1.3 us a token at d_k = 128, r = 1, 3.0 at 64, r = 4): it is there so that every state that fp16 can hold gives a finite
+// result, whatever the products with it reach.
+template <int DK, int R, int JS, bool SEG, class Args>
+__device__ __noinline__ void walk_fp32(Args args, int row0) {
+    constexpr int C = NB / R, NI = DK / 2;                        // columns i per lane
+    const ChainGeo g = args.g;
+    const ChainSeg sg = args.seg;
+    long long seq;
+    const ChainPart part = chain_part<DK, JS, C, SEG>(g, sg, g.S0, g.O, g.S_final, seq);
+    const int lane = threadIdx.x & 31, i0 = (lane & 1) * NI, j = part.j0 + row0 + (lane >> 1);
+    const long long tok0 = seq * g.L + (long long)part.b0 * C;
+    const int tokens = min(part.nblk * C, g.L - part.b0 * C), group = g.rm == 1 ? 1 : R;      // (group: factors that read the same state)
+    auto dot = [&](const float (&S)[NI], const __nv_bfloat16* x, bool self) {
+        float d = 0.f;
+#pragma unroll
+        for (int n = 0; n < NI; n += 8) {
+            const uint4 y = *(const uint4*)(x + i0 + n);
+            const uint32_t* w = (const uint32_t*)&y;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const float z = __uint_as_float(e & 1 ? w[e / 2] & 0xFFFF0000u : w[e / 2] << 16);
+                d = fmaf(self ? z : S[n + e], z, d);
+            }
+        }
+        return d + __shfl_xor_sync(0xffffffffu, d, 1);
+    };
+    float S[NI];
+#pragma unroll
+    for (int n = 0; n < NI; ++n) S[n] = part.S0 ? part.S0[(long long)(i0 + n) * g.d_v + j] : 0.f;
+#pragma unroll 1
+    for (int t = 0; t < tokens; ++t) {
+#pragma unroll 1
+        for (int f = 0; f < R; f += group) {
+            const long long m0 = (tok0 + t) * R + f;
+            float u[R];
+#pragma unroll
+            for (int x = 0; x < R; ++x) {
+                if (x >= group) break;
+                const __nv_bfloat16* kr = g.k + (m0 + x) * DK;
+                float b = __bfloat162float(g.beta[m0 + x]);
+                if (g.exact) {
+                    const float n2 = dot(S, kr, true);
+                    if (n2 > 0.f) b = -expm1f(-b * n2) / n2;
+                }
+                u[x] = b * (__bfloat162float(g.v[(m0 + x) * g.d_v + j]) - dot(S, kr, false));
+            }
+#pragma unroll
+            for (int x = 0; x < R; ++x) {
+                if (x >= group) break;
+                const __nv_bfloat16* kr = g.k + (m0 + x) * DK + i0;
+#pragma unroll
+                for (int n = 0; n < NI; n += 8) {
+                    const uint4 y = *(const uint4*)(kr + n);
+                    const uint32_t* w = (const uint32_t*)&y;
+#pragma unroll
+                    for (int e = 0; e < 8; ++e)
+                        S[n + e] = fmaf(u[x], __uint_as_float(e & 1 ? w[e / 2] & 0xFFFF0000u : w[e / 2] << 16), S[n + e]);
+                }
+            }
+        }
+        const float o = dot(S, g.q + (tok0 + t) * DK, false);
+        if ((lane & 1) == 0) part.O[(long long)t * g.d_v + j] = o;
+    }
+    if (part.S_end)
+#pragma unroll
+        for (int n = 0; n < NI; ++n) part.S_end[(long long)(i0 + n) * g.d_v + j] = S[n];
+}
 
 // K, Q and V of block b (of this part) into stage b mod NS (one thread); rows past the sequence arrive as zeros
 template <int DK, int R, int JS, int NS>
@@ -404,7 +540,8 @@ __device__ __forceinline__ void prep_role(const ChainGeo& g, const ChainPart& pa
 // ---------------------------------------------------------------------------------------------------------------------
 template <int DK, int R, int JS, int IS, int TEAMS, int NS, bool SEG>
 __device__ __forceinline__ void chain_role(const ChainMaps& maps, const ChainGeo& g, const ChainPart& part, int* err, uint8_t* smem,
-                                           uint64_t* land, uint64_t* full, uint64_t* empty, int seq, int warp, int lane) {
+                                           uint64_t* land, uint64_t* full, uint64_t* empty, const ChainSeg& seg, ChainArgs& args, int seq, int warp,
+                                           int lane) {
     using CFG = ChainCfg<DK, R, JS, IS, TEAMS, NS>;
     using SM = ChainSmem<DK, R, JS>;
     constexpr int C = SM::C, CP = SM::CP, TT = CP / 16;
@@ -653,6 +790,16 @@ __device__ __forceinline__ void chain_role(const ChainMaps& maps, const ChainGeo
                 if (i == j) part.D[j] = S[n][e];
                 if (i + 1 == j) part.D[j] = S[n][e + 1];
             }
+        return;
+    }
+    // (one entry tells for its row.  The end state may replace the start state, which is still needed where rows are lost)
+    bool lost = __any_sync(0xffffffffu, !(fabsf(S[0][0]) <= FLT_MAX) || !(fabsf(S[0][2]) <= FLT_MAX));
+    if (IS == 2) lost = !named_bar_and(1 + TEAMS + grp, 64, !lost);   // (both warps of a pair have written their last O)
+    if (lost) {
+        if (hi == 0) {
+            if constexpr (WALK_BY_REF<DK, JS, SEG>) walk_fp32<DK, R, JS, SEG, const ChainArgs&>(args, 16 * grp);
+            else walk_fp32<DK, R, JS, SEG, ChainArgs>(ChainArgs{g, seg}, 16 * grp);
+        }
     } else if (part.S_end) {
 #pragma unroll
         for (int n = 0; n < 2 * KT; ++n)
@@ -660,23 +807,6 @@ __device__ __forceinline__ void chain_role(const ChainMaps& maps, const ChainGeo
             for (int e = 0; e < 4; ++e) part.S_end[(long long)(i0 + 8 * n + (e & 1)) * width + jr + 8 * (e >> 1)] = S[n][e];
     }
 }
-
-// Segments (Section 3, "Scan"; Proposition 2.1): the flow of an interval is the pair (P, Xi) with S_end = S_start P + Xi.  A
-// sequence is cut into segments that are walked side by side: for each the state from zero (S0 for the first segment), whose
-// outputs go to O and whose end is Xi, and, for all but the first, the state from the identity with v = 0, whose "outputs"
-// R_t = P_t q_t are what each token makes of its segment's start state and whose end is P.  Then one kernel composes the
-// segments' start states and another adds start R_t to O.
-// The diagonal of P is kept apart, in fp32, and fp16 is for the rest: where the step sizes are small P is close to the identity, and
-// rounding all of it (and the start state before it) would round the whole state once per segment (step sizes of 0.01, 8000
-// tokens in 9 segments: relative error of S_final 7.2e-4, this way 6.1e-5, 4.6e-5 in the tcgen05 kernels; at step sizes around 0.5
-// 3.49e-4 and 3.44e-4).
-struct ChainSeg {
-    __half* R;          // [nseq][L][d_k]
-    __half* P;          // [nseq][nseg][d_k j][d_k i], zeros on the diagonal
-    float* D;           // [nseq][nseg][d_k]: the diagonal
-    float* Xi;          // [nseq][nseg][d_k i][d_v j]
-    __half* start;      // [nseq][nseg][d_v j][d_k i]
-};
 
 template <int DK, int R, int JS, int IS, int TEAMS, int NS, bool SEG>
 __global__ void __launch_bounds__(ChainCfg<DK, R, JS, IS, TEAMS, NS>::threads, 1)
@@ -686,35 +816,16 @@ chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __rest
     using SM = ChainSmem<DK, R, JS>;
     extern __shared__ __align__(1024) uint8_t smem[];
     __shared__ uint64_t land[NS], full[NS], empty[NS];
+    __shared__ ChainArgs args;
     const int tid = threadIdx.x, warp = tid >> 5;
-    const int slices = g.d_v / JS;
     long long seq;
-    ChainPart part;
-    if constexpr (!SEG) {
-        seq = blockIdx.x / slices;
-        part = {0, g.nblk, (int)(blockIdx.x % slices) * JS, g.d_v, false, S0 ? S0 + seq * DK * g.d_v : nullptr,
-                O + seq * g.L * g.d_v, S_final ? S_final + seq * DK * g.d_v : nullptr, nullptr};
-    } else {
-        constexpr int rs = DK / JS;
-        const int per_seq = g.nseg * slices + (g.nseg - 1) * rs, x = (int)(blockIdx.x % per_seq), y = x - g.nseg * slices;
-        seq = blockIdx.x / per_seq;
-        part.response = y >= 0;
-        const int s = part.response ? 1 + y / rs : x / slices;
-        part.b0 = s * g.seg_blk;
-        part.nblk = min(g.seg_blk, g.nblk - part.b0);
-        part.j0 = (part.response ? y % rs : x % slices) * JS;
-        part.width = part.response ? DK : g.d_v;
-        const long long row0 = seq * g.L + (long long)part.b0 * SM::C, slot = seq * g.nseg + s;
-        part.S0 = s == 0 && S0 ? S0 + seq * DK * g.d_v : nullptr;
-        part.O = part.response ? (float*)(sg.R + row0 * DK) : O + row0 * g.d_v;
-        part.S_end = part.response ? (float*)(sg.P + slot * DK * DK) : sg.Xi + slot * DK * g.d_v;
-        part.D = sg.D + slot * DK;
-    }
+    const ChainPart part = chain_part<DK, JS, SM::C, SEG>(g, sg, S0, O, S_final, seq);
     if ((smem_u32(smem) & 1023u) != 0) {                          // (the swizzled layouts need a 1024-byte aligned base)
         wait_for_previous_kernel();
         if (tid == 0) atomicCAS(status, 0, 99);
         return;
     }
+    if (WALK_BY_REF<DK, JS, SEG> && tid == 32) args = {g, sg};
     if (tid == 0) {
         for (int x = 0; x < NS; ++x) {
             mbar_init(&land[x], 1);
@@ -738,7 +849,7 @@ chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __rest
         for (int b = 0; b < NS && b < part.nblk; ++b) load_block<DK, R, JS, NS>(maps, smem, land, b, (int)seq, part);
     __syncwarp();
     if (warp < CFG::NCW)
-        chain_role<DK, R, JS, IS, TEAMS, NS, SEG>(maps, g, part, status, smem, land, full, empty, (int)seq, warp, tid & 31);
+        chain_role<DK, R, JS, IS, TEAMS, NS, SEG>(maps, g, part, status, smem, land, full, empty, sg, args, (int)seq, warp, tid & 31);
     else
         prep_role<DK, R, JS, IS, TEAMS, NS>(g, part, beta, status, smem, land, full, seq, (warp - CFG::NCW) >> 2, (tid - 32 * CFG::NCW) & 127);
 }
@@ -976,7 +1087,9 @@ int launch(const Problem& p, const ChainPlan& plan, const ChainSeg& sg) {
     static_assert(CFG::total <= 227 * 1024 && NS >= 2, "shared memory budget");
     const void* fn = (const void*)chain_kernel<DK, R, JS, IS, TEAMS, NS, SEG>;
     constexpr int C = NB / R;
-    ChainGeo g{p.L, p.d_v, (p.L + C - 1) / C, plan.nseg, plan.seg_blk, p.mask_group(), p.exact ? 1 : 0, p.clear_status ? 1 : 0};
+    ChainGeo g{p.L, p.d_v, (p.L + C - 1) / C, plan.nseg, plan.seg_blk, p.mask_group(), p.exact ? 1 : 0, p.clear_status ? 1 : 0,
+               (const __nv_bfloat16*)p.q, (const __nv_bfloat16*)p.k, (const __nv_bfloat16*)p.v, (const __nv_bfloat16*)p.beta,
+               p.S0, p.O, p.S_final};
     const long long nseq = (long long)p.B * p.H, grid = nseq * (plan.nseg * (p.d_v / JS) + (plan.nseg - 1) * (DK / JS));
     ChainMaps maps;
     constexpr int VC = JS < 64 ? JS : 64;

@@ -1,6 +1,8 @@
 """The one-kernel chunk form (bf16 calls that the library chooses the kernels for) at the edges of its blocks of 64 rows and
 with each way of spreading a sequence's columns over CTAs (2, 40 and 160 sequences)."""
+import numpy as np
 import pytest
+import torch
 
 import pf_synth
 from pf_synth import Workload
@@ -37,6 +39,66 @@ def test_few_long_sequences_are_walked_in_segments(d_k, d_v, r, H, L, mode):
         w = Workload(f"chain_seg_{L}", B=1, H=H, L=L, d_k=d_k, d_v=d_v, r=r, chunk=64, s0_std=s0_std, seed=400 + r)
         util.check_parity(w, mode=mode)
         assert pf.pf_last_launch_count() == 3
+
+
+# (sequences, lengths and head dimensions that reach every spread of the columns, the segments and, with 32 x 2048 at d = 128, the
+#  single launch)
+RANGE_CASES = [
+    (128, 128, 1, 2, 225, "sum", "chain"), (128, 128, 2, 2, 200, "product", "chain"), (128, 64, 3, 2, 148, "sum", "chain"),
+    (128, 128, 4, 2, 113, "sum", "chain"), (64, 64, 2, 40, 131, "sum", "chain"), (64, 128, 3, 160, 131, "product", "chain"),
+    (128, 128, 2, 160, 131, "sum", "chain"), (64, 64, 4, 160, 70, "sum", "chain"), (128, 128, 1, 70, 300, "sum", "chain"),
+    (128, 128, 2, 3, 2500, "sum", "chain"), (64, 64, 1, 2, 4097, "sum", "chain"), (128, 128, 2, 32, 2048, "sum", "fused"),
+]
+
+
+@pytest.mark.parametrize("token", [0, 60])
+@pytest.mark.parametrize("d_k,d_v,r,H,L,mode,kernel", RANGE_CASES)
+def test_a_state_that_fp16_holds_but_its_products_with_keys_exceed(d_k, d_v, r, H, L, mode, kernel, token):
+    """Two columns of the start state have entries of 2e4, all aligned with the key of one token, so that the product S k there is
+    2e4 sqrt(d_k) = 1.6e5 or 2.3e5, past what fp16 holds; beta is 2 there (the state is reflected, its size stays) or 1/4 (U'
+    stays below, V - K S^T does not).  In those columns everything else is small beside the state, and the other columns
+    must not notice."""
+    import paper_2504_00492_b200 as pf
+    w = Workload("range_keys", B=1, H=H, L=L, d_k=d_k, d_v=d_v, r=r, chunk=64, s0_std=0.1, seed=600 + r)
+    inp = pf_synth.make_inputs(w)
+    sign = torch.where(torch.randn(d_k, generator=torch.Generator().manual_seed(7)) < 0, -1.0, 1.0)
+    big = [5, d_v - 1]
+    # the tokens before it leave these columns alone: their keys are orthogonal to the state (neighbouring entries cancel)
+    for t in range(token):
+        x = inp.k[:, :, t].float() * sign
+        x = (x[..., 0::2] - x[..., 1::2]).repeat_interleave(2, -1) * torch.tensor([1.0, -1.0]).repeat(d_k // 2)
+        inp.k[:, :, t] = (x / x.norm(dim=-1, keepdim=True) * sign).to(inp.k.dtype)
+    inp.k[:, :, token, 0] = (sign / d_k ** 0.5).to(inp.k.dtype)
+    # (each factor takes about beta / d_k of the state away: step sizes with which what S_final keeps of the start state is still large)
+    inp.beta *= min(1.0, 2.0 * d_k / (L * r))
+    inp.beta[:, 0::2, token, 0], inp.beta[:, 1::2, token, 0] = 2.0, 0.25
+    inp.S0[:, :, :, big] = (2e4 * sign)[:, None]
+    d = inp.to("cuda")
+    out = []
+    assert kernel in util.kernels_of(lambda: out.append(pf.pf_deltanet_fwd_ex(d.q, d.k, d.v, d.beta, d.S0, w.chunk, mode=mode)))
+    assert pf.pf_read_status() == 0
+    rest = [j for j in range(d_v) if j not in big]
+    for x, ref, what in zip(out[0], util.run_oracle(inp, mode=mode), ("O", "S_final")):
+        x = x.cpu().numpy()
+        assert np.isfinite(x).all(), what
+        # (a step's rounding error is relative to the state at that step, so the bound is TOL_BF16 of the largest entries there have been)
+        err, top = np.abs(x - ref)[..., big].max(axis=(-1, -2)), np.abs(ref[..., big]).max(axis=(-1, -2))
+        assert (err <= util.TOL_BF16 * np.maximum(top, 2e4)).all(), (what, (err / np.maximum(top, 2e4)).max())
+        util.check_per_sequence(x[..., rest], ref[..., rest], util.TOL_BF16, what + ", other columns")
+
+
+def test_a_call_whose_end_state_replaces_its_start_state():
+    """S_final written over S0, also where rows of the state have to be walked a second time."""
+    import paper_2504_00492_b200 as pf
+    w = Workload("in_place", B=1, H=2, L=96, d_k=128, d_v=128, r=2, chunk=64, s0_std=0.1, seed=611)
+    inp = pf_synth.make_inputs(w)
+    inp.S0[:, 1, :, 3] = 2e4
+    inp.k[:, :, 0, 0] = 128 ** -0.5
+    d = inp.to("cuda")
+    O, S = pf.pf_deltanet_fwd(d.q, d.k, d.v, d.beta, d.S0, w.chunk)
+    O2, S2 = pf.pf_deltanet_fwd(d.q, d.k, d.v, d.beta, d.S0, w.chunk, S_final=d.S0)
+    assert torch.isfinite(O).all() and torch.isfinite(S).all()
+    assert torch.equal(O, O2) and torch.equal(S, S2) and S2.data_ptr() == d.S0.data_ptr()
 
 
 @pytest.mark.parametrize("d_k,d_v,r,H,L,mode", [(128, 128, 1, 4, 8000, "sum"), (64, 64, 1, 2, 4097, "sum"), (128, 128, 2, 3, 2500, "product"),

@@ -57,6 +57,26 @@ def run_gpu(w: pf_synth.Workload, inp: pf_synth.Inputs, impl="auto", chunk=None,
     return O.cpu().numpy(), Sf.cpu().numpy()
 
 
+def kernels_of(call):
+    """The names of the kernels that `call` (one call of the library) launched, in order."""
+    import ctypes
+
+    from paper_2504_00492_b200 import binding
+    lib = binding.lib()
+    lib.pf_profile_enable(1)
+    try:
+        call()
+        torch.cuda.synchronize()
+        names = []
+        for i in range(lib.pf_profile_count()):
+            name, ms = ctypes.create_string_buffer(64), ctypes.c_float(0)
+            assert lib.pf_profile_read(i, name, 64, ctypes.byref(ms)) == 0
+            names.append(name.value.decode())
+    finally:
+        lib.pf_profile_enable(0)
+    return names
+
+
 def run_oracle(inp: pf_synth.Inputs, mode="sum", step="euler"):
     return oracle.deltanet_fwd(inp.q, inp.k, inp.v, inp.beta, inp.S0, mode=mode, exact=(step == "exact"))
 
