@@ -8,6 +8,7 @@
 #include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
 #include <limits.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include "pf.h"
@@ -28,7 +29,10 @@ bool get_tensor(PyObject* o, const at::Tensor** out) {
 
 // forward(q, k, v, beta, S0, chunk, O, S_final, stream, want_state, f32, impl, mode, step)
 //   -> (O, S_final), or the library's status (int) if it is not 0, or None: not the ordinary case
+// What torch throws on the way (no memory for the outputs, no device, a tensor without storage such as a traced one) becomes the
+// Python exception that torch gives it.
 PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    HANDLE_TH_ERRORS
     if (n != 14 || !g_forward) Py_RETURN_NONE;
     const at::Tensor *q, *k, *v, *beta, *s0 = nullptr;
     if (!get_tensor(a[0], &q) || !get_tensor(a[1], &k) || !get_tensor(a[2], &v) || !get_tensor(a[3], &beta)) Py_RETURN_NONE;
@@ -94,6 +98,7 @@ PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t n) {
     put(0, a[6], O);
     put(1, a[7], S);
     return out;
+    END_HANDLE_TH_ERRORS
 }
 
 // bind(address of pf_deltanet_fwd_ex)
