@@ -263,7 +263,6 @@ def pf_deltanet_fwd_ex(q, k, v, beta, S0, chunk: int, impl="auto", workspace: Op
     p.impl = IMPL_BY_NAME[impl] if isinstance(impl, str) else int(impl)
     if workspace is not None:
         p.workspace, p.workspace_bytes = workspace.data_ptr(), workspace.numel() * workspace.element_size()
-    p.stream = _stream(stream)
     p.mode = MODE_BY_NAME[mode] if isinstance(mode, str) else int(mode)
     p.step = STEP_BY_NAME[step] if isinstance(step, str) else int(step)
     p.segments, p.wu_builder, p.ring_depth = int(segments), int(wu_builder), int(ring_depth)
@@ -272,6 +271,7 @@ def pf_deltanet_fwd_ex(q, k, v, beta, S0, chunk: int, impl="auto", workspace: Op
             raise ValueError("status must be an int32 CUDA tensor")
         p.status = status.data_ptr()
     with torch.cuda.device(q.device):
+        p.stream = _stream(stream)
         st = lib().pf_deltanet_fwd_ex(ctypes.byref(p))
     if st != 0:
         raise PfError(st, "pf_deltanet_fwd_ex")

@@ -60,11 +60,10 @@ PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (a[6] != Py_None && !get_tensor(a[6], &o_in)) Py_RETURN_NONE;
     if (a[7] != Py_None && !get_tensor(a[7], &s_in)) Py_RETURN_NONE;
 
-    // (the stream is the current one of the caller's current device, as in the Python code)
-    const c10::DeviceIndex cur = c10::cuda::current_device();
-    const cudaStream_t stream = c10::cuda::getCurrentCUDAStream(cur).stream();
+    // (the stream is the current one of the tensors' device, whatever device is current)
     c10::cuda::OptionalCUDAGuard guard;
-    if (cur != dev.index()) guard.set_device(dev);
+    if (c10::cuda::current_device() != dev.index()) guard.set_device(dev);
+    const cudaStream_t stream = c10::cuda::getCurrentCUDAStream(dev.index()).stream();
     at::Tensor O, S;
     if (!o_in) O = at::Tensor(at::detail::empty_cuda({B, H, L, dv}, at::kFloat, dev, std::nullopt));
     if (!s_in && want_state) S = at::Tensor(at::detail::empty_cuda({B, H, dk, dv}, at::kFloat, dev, std::nullopt));
