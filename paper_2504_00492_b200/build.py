@@ -13,6 +13,7 @@ CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libpf.so")
 EXT_SRC = os.path.join(CSRC, "pf_ext.cpp")
 EXT = os.path.join(PKG, "_pf_ext.so")
+EXT_TAG = os.path.join(PKG, "_build", "_pf_ext.tag")      # what EXT was built against
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -32,14 +33,26 @@ def _stale() -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
-def build_ext(force: bool = False) -> str:
-    """Compile the call path of the Python entry points against the installed torch's headers."""
+def _ext_stale(tag: str) -> bool:
     deps = [EXT_SRC, os.path.join(ROOT, "include", "pf.h")]
-    if not force and os.path.exists(EXT) and all(os.path.getmtime(d) <= os.path.getmtime(EXT) for d in deps):
-        return EXT
+    if not os.path.exists(EXT) or any(os.path.getmtime(d) > os.path.getmtime(EXT) for d in deps):
+        return True
+    try:
+        with open(EXT_TAG) as f:
+            return f.read() != tag
+    except OSError:
+        return True
+
+
+def build_ext(force: bool = False) -> str:
+    """Compile the call path of the Python entry points against the installed torch's headers (and again when another torch or
+    Python is installed: the extension is tied to their ABI)."""
     import sysconfig
 
     import torch
+    tag = f"torch {torch.__version__} abi {int(torch._C._GLIBCXX_USE_CXX11_ABI)} python {sysconfig.get_config_var('SOABI')}"
+    if not force and not _ext_stale(tag):
+        return EXT
     t = os.path.dirname(torch.__file__)
     cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
     tmp = EXT + ".tmp%d" % os.getpid()
@@ -51,6 +64,9 @@ def build_ext(force: bool = False) -> str:
                     EXT_SRC, "-o", tmp, "-L", os.path.join(t, "lib"), "-ltorch_python", "-ltorch_cuda", "-ltorch_cpu",
                     "-lc10_cuda", "-lc10"], check=True)
     os.replace(tmp, EXT)
+    os.makedirs(os.path.dirname(EXT_TAG), exist_ok=True)
+    with open(EXT_TAG, "w") as f:
+        f.write(tag)
     return EXT
 
 
