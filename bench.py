@@ -63,6 +63,88 @@ def flops_per_chunk(w, tri: bool) -> dict:
     }
 
 
+def flops_per_block(w, tri: bool) -> dict:
+    """FLOPs of the chain kernel for one block of 64 / r tokens: T' is applied to V - K S^T, W and Uh are never formed."""
+    C, r, dk, dv = 64 // w.r, w.r, w.d_k, w.d_v
+    n = C * r
+    h = 0.5 if tri else 1.0
+    return {
+        "gram": 2 * n * n * dk * h, "solve": n ** 3 / 3.0, "attn": 2 * C * n * dk * h, "ks": 2 * n * dk * dv,
+        "t": 2 * n * n * dv * h, "state": 2 * n * dk * dv, "out": 2 * C * dk * dv + 2 * C * n * dv * h,
+    }
+
+
+def chunk_of(kernel: str, w, chunk_selected: int) -> int:
+    """Tokens per chunk that `kernel` evaluates with: `chunk_selected` (pf_select_chunk) in the tcgen05 and the fp32 chunk-form
+    kernels, 64 / r in the chain kernel, one in the token-by-token kernel."""
+    return {"chain": 64 // w.r, "recur": 1}.get(kernel, chunk_selected)
+
+
+def pass_flops(kernel: str, w, chunk_selected: int, tri: bool, solve: bool = True) -> float:
+    """FLOPs of one whole pass in the form that `kernel` (a kernel that does all of it, or a part of the chunk form) evaluates."""
+    if kernel == "recur":
+        return w.token_heads * (4 * w.r + 2) * w.d_k * w.d_v
+    chunk = chunk_of(kernel, w, chunk_selected)
+    fl = flops_per_block(w, tri) if kernel == "chain" else flops_per_chunk(w.with_(chunk=chunk), tri)
+    return w.B * w.H * ((w.L + chunk - 1) // chunk) * sum(v for k, v in fl.items() if solve or k != "solve")
+
+
+def math_peak(kernel: str, peaks: dict):
+    """What bounds the arithmetic of `kernel`, and its rate in TFLOP/s: tensor cores, or FFMA (148 SMs x 128 lanes x 2 at the
+    maximum clock) in the fp32 kernels."""
+    if kernel.startswith("simt") or kernel.startswith("recur"):
+        return "alu", 148 * 128 * 2 * peaks.get("sm_max_mhz", 1965.0) * 1e6 / 1e12
+    return "tensor", peaks["bf16_tflops"]
+
+
+# which algorithmic steps of the chunk form each kernel covers that does not do the whole pass
+KERNEL_STEPS = {
+    "simt_gram": ["gram", "attn"], "simt_solve": ["solve"], "simt_wu": ["wu"], "simt_scan": ["corr", "out", "state"],
+    "tc_flow": ["gram", "solve", "wu", "attn"], "tc_scan": ["corr", "out", "state"],
+}
+
+
+WHOLE_PASS = ("fused", "chain", "recur")      # each followed by two small kernels where it walks in segments
+
+
+def main_kernel(prof: dict) -> str:
+    """The kernel that does the whole pass, else the one that takes most of the time (`prof`: ms per kernel of one call)."""
+    return next((k for k in WHOLE_PASS if k in prof), None) or max(prof, key=prof.get)
+
+
+def kernel_roofline(prof: dict, w, chunk_selected: int, peaks: dict, peak_kind: str):
+    """The roofline entry of the call's main kernel."""
+    if not prof:
+        return None
+    top = main_kernel(prof)
+    seconds = prof[top] * 1e-3
+    kind, rate = math_peak(top, peaks)
+    common = {"kernel": top, "ms_per_launch": prof[top], "peaks": peak_kind, "kernel_ms": prof}
+    if top not in WHOLE_PASS:
+        fl_tri = flops_per_chunk(w.with_(chunk=chunk_selected), tri=True)
+        fl = w.B * w.H * ((w.L + chunk_selected - 1) // chunk_selected) * sum(fl_tri[s] for s in KERNEL_STEPS.get(top, list(fl_tri)))
+        achieved = fl / seconds / 1e12
+        return {"bound": kind, "achieved": achieved, "peak": rate, "unit": "TFLOP/s", "frac": achieved / rate, "traffic": None,
+                "flops_per_launch": fl, "flop_count": "triangular-aware", **common}
+    # The kernel does everything: its algorithmic traffic is one read of q, k, v, beta and one write of O.  What binds is
+    # the longer of that and the arithmetic of its own form (dense FLOPs), each at the measured peak; both are printed.
+    nbytes = w.token_heads * alg_bytes_per_token_head(w)
+    fl = pass_flops(top, w, chunk_selected, tri=False, solve=False)
+    gbs, tflops = nbytes / seconds / 1e9, fl / seconds / 1e12
+    math = {"tflops_dense": tflops, "peak": rate, "frac": tflops / rate}
+    if kind == "tensor":
+        math["pipe_active_pct"], math["pipe_active_from"] = ncu_tensor_pipe(w) if top == "fused" else (None, None)
+    out = {"bound": "hbm", "achieved": gbs, "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": gbs / peaks["hbm_gbs"]}
+    if fl / rate / 1e3 > nbytes / peaks["hbm_gbs"]:
+        out = {"bound": kind, "achieved": tflops, "peak": rate, "unit": "TFLOP/s", "frac": tflops / rate}
+    return {**out, "traffic": ncu_traffic(w) if top == "fused" else None, "bytes_per_launch": nbytes, kind: math, **common}
+
+
+def l2_note(nbytes: int) -> str:
+    """How the timed steps meet the L2 (126 MB): every step reads and writes the same resident tensors."""
+    return "inputs+outputs (%.1f MB) %s" % (nbytes / 1e6, "larger than L2" if nbytes > 126e6 else "fit the L2 and may stay there between steps")
+
+
 # Figures from ncu captures of the single-launch kernel, valid only for the kernel sources they were taken on (the
 # hash of those sources is stored with them; the commands are in profiles/fused_kernel_c2.md):
 #   NCU_TRAFFIC      DRAM bytes (read + write) of one full-size launch: {workload: (hash, bytes)}
@@ -394,10 +476,9 @@ def main():
     if args.wu_builder:
         options["wu_builder"] = args.wu_builder
     in_dtype = pf.PF_DTYPE_F32 if w.dtype == "f32" else pf.PF_DTYPE_BF16
-    # PF_IMPL_AUTO may evaluate with a shorter chunk than the one asked for (the recurrence's result does not depend
-    # on it); the work counts below use the chunk length the kernels ran with.
+    # PF_IMPL_AUTO may evaluate with another chunk than the one asked for (the recurrence's result does not depend
+    # on it); the work counts below use the form and the chunk length of the kernel that ran.
     chunk_used = pf.pf_select_chunk(w.B, w.H, w.L, w.d_k, w.d_v, w.r, w.chunk, in_dtype, args.path)
-    w_eval = w.with_(chunk=chunk_used)
 
     def forward(q, k, v, beta, S0, O=None, S_final=None, stream=None):
         if options:
@@ -481,49 +562,17 @@ def main():
 
     # ---- per-kernel times and the roofline of the dominant kernel -----------------------------------------
     prof = kernel_profile(forward, d, steps=min(args.steps, 10))
-    G = w.B * w.H * ((w.L + chunk_used - 1) // chunk_used)
+    top = main_kernel(prof) if prof else "fused"
+    chunk_evaluated = chunk_of(top, w, chunk_used)
     th = w.token_heads
-    fl_tri = flops_per_chunk(w_eval, tri=True)
-    fl_dense = flops_per_chunk(w_eval, tri=False)
     ms_step = total_ms / args.steps
+    fl_dense, fl_tri = (pass_flops(top, w, chunk_used, tri) for tri in (False, True))
     t_hbm_us = th * alg_bytes_per_token_head(w) / (peaks["hbm_gbs"] * 1e9) * 1e6
-    t_flop_us = G * sum(fl_dense[k] for k in fl_dense if k != "solve") / (peaks["bf16_tflops"] * 1e12) * 1e6
+    t_flop_us = pass_flops(top, w, chunk_used, tri=False, solve=False) / (math_peak(top, peaks)[1] * 1e12) * 1e6
     path = {"t_hbm_us": t_hbm_us, "t_flop_dense_us": t_flop_us, "frac": max(t_hbm_us, t_flop_us) / (ms_step * 1e3),
-            "peaks": peak_kind, "tflops_dense": G * sum(fl_dense.values()) / (ms_step * 1e-3) / 1e12,
-            "tflops_tri": G * sum(fl_tri.values()) / (ms_step * 1e-3) / 1e12,
+            "peaks": peak_kind, "tflops_dense": fl_dense / (ms_step * 1e-3) / 1e12, "tflops_tri": fl_tri / (ms_step * 1e-3) / 1e12,
             "hbm_gbs_algorithmic": th * alg_bytes_per_token_head(w) / (ms_step * 1e-3) / 1e9}
-    # which algorithmic steps each kernel covers (triangular-aware FLOPs: the conservative count)
-    kernel_steps = {
-        "simt_gram": ["gram", "attn"], "simt_solve": ["solve"], "simt_wu": ["wu"], "simt_scan": ["corr", "out", "state"],
-        "tc_flow": ["gram", "solve", "wu", "attn"], "tc_scan": ["corr", "out", "state"],
-    }
-    roofline = None
-    if prof:
-        top = max(prof, key=prof.get)
-        if top == "fused":
-            # The single-launch path does everything: its algorithmic traffic is one read of q, k, v, beta and one
-            # write of O; at the measured peaks that HBM time exceeds the tensor time of the dense FLOPs, so HBM is
-            # the roofline that binds (the tensor figure is printed beside it).
-            nbytes = th * alg_bytes_per_token_head(w)
-            achieved = nbytes / (prof[top] * 1e-3) / 1e9
-            fl_d = G * sum(fl_dense[k] for k in fl_dense if k != "solve")
-            roofline = {"bound": "hbm", "kernel": top, "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
-                        "frac": achieved / peaks["hbm_gbs"], "traffic": ncu_traffic(w), "ms_per_launch": prof[top],
-                        "peaks": peak_kind, "bytes_per_launch": nbytes,
-                        "tensor": {"tflops_dense": fl_d / (prof[top] * 1e-3) / 1e12, "peak": peaks["bf16_tflops"],
-                                   "frac": fl_d / (prof[top] * 1e-3) / 1e12 / peaks["bf16_tflops"],
-                                   "pipe_active_pct": ncu_tensor_pipe(w)[0], "pipe_active_from": ncu_tensor_pipe(w)[1]},
-                        "kernel_ms": prof}
-        else:
-            steps_of = kernel_steps.get(top, list(fl_tri))
-            fl = G * sum(fl_tri[s] for s in steps_of)
-            achieved = fl / (prof[top] * 1e-3) / 1e12
-            bound = "alu" if top.startswith("simt") else "tensor"
-            # fp32 FFMA peak: 148 SMs x 128 lanes x 2 FLOP x max SM clock
-            peak = 148 * 128 * 2 * peaks.get("sm_max_mhz", 1965.0) * 1e6 / 1e12 if bound == "alu" else peaks["bf16_tflops"]
-            roofline = {"bound": bound, "kernel": top, "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-                        "frac": achieved / peak, "traffic": None, "ms_per_launch": prof[top], "peaks": peak_kind,
-                        "flops_per_launch": fl, "flop_count": "triangular-aware", "kernel_ms": prof}
+    roofline = kernel_roofline(prof, w, chunk_used, peaks, peak_kind)
 
     if rank == 0:
         cpu = None
@@ -539,8 +588,8 @@ def main():
                 w.B, w.H, w.L, w.d_k, w.d_v, w.r, w.chunk, in_dtype, args.path) in (2, 4) else "f32",      # PF_IMPL_TC, PF_IMPL_TC_SPLIT
             "data": "synthetic",
             "config": {"workload": w.name, "B": w.B, "H": w.H, "L": w.L, "d_k": w.d_k, "d_v": w.d_v, "r": w.r,
-                       "chunk": w.chunk, "chunk_evaluated": chunk_used, "path": args.path, "l2": "inputs+outputs (%.0f MB) larger than L2" % (
-                           (host.nbytes() + O.numel() * 4) / 1e6), "parallelism": "replicas" if world > 1 else "1 GPU"},
+                       "chunk": w.chunk, "chunk_evaluated": chunk_evaluated, "path": args.path,
+                       "l2": l2_note(host.nbytes() + O.numel() * 4), "parallelism": "replicas" if world > 1 else "1 GPU"},
             "ms_per_step_median": statistics.median(per_step), "ms_per_step_min": min(per_step), "ms_per_step_max": max(per_step),
             "token_heads_per_s": value * w.H,
             "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
