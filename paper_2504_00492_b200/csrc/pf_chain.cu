@@ -885,17 +885,18 @@ __global__ void __launch_bounds__(128) chain_compose(ChainSeg sg, float* __restr
 #pragma unroll
             for (int e = 0; e < 4; ++e) x[n][e] = src[(long long)(i0 + 8 * n + (e & 1)) * d_v + j + 8 * (e >> 1)];
     };
-    float2 D[NT];                                                 // diagonal of P of the next step
-    auto diagonal = [&](int s) {
+    auto diagonal = [&](int s, float2 (&x)[NT]) {
 #pragma unroll
-        for (int n = 0; n < NT; ++n) D[n] = *(const float2*)(sg.D + (seq * nseg + s) * DK + i0 + 8 * n);
+        for (int n = 0; n < NT; ++n) x[n] = *(const float2*)(sg.D + (seq * nseg + s) * DK + i0 + 8 * n);
     };
-    float X[NT][4];                                               // Xi of the next step
+    float X[NT][4], Xn[NT][4];                                    // Xi of this step and of the next
+    float2 D[NT], Dn[NT];                                         // the diagonal of P likewise
     wait_for_previous_kernel();
     load_p(1);
     xi(0, S);
     xi(1, X);
-    diagonal(1);
+    diagonal(1, D);
+#pragma unroll 1
     for (int s = 1; s < nseg; ++s) {
         __half* a_s = sA + (s & 1) * 16 * LD;
         __half* out = sg.start + (seq * nseg + s) * d_v * DK;
@@ -907,13 +908,9 @@ __global__ void __launch_bounds__(128) chain_compose(ChainSeg sg, float* __restr
                 *(uint32_t*)(a_s + (gq + 8 * h) * LD + i0 + 8 * n) = x;
                 *(uint32_t*)(out + (long long)(j + 8 * h) * DK + i0 + 8 * n) = x;
             }
-#pragma unroll
-        for (int n = 0; n < NT; ++n)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) S[n][e] = fmaf(S[n][e], e & 1 ? D[n].y : D[n].x, X[n][e]);
         if (s + 1 < nseg) {
-            xi(s + 1, X);
-            diagonal(s + 1);
+            xi(s + 1, Xn);
+            diagonal(s + 1, Dn);
             load_p(s + 1);
             asm volatile("cp.async.wait_group 1;" ::: "memory");
         } else {
@@ -929,9 +926,19 @@ __global__ void __launch_bounds__(128) chain_compose(ChainSeg sg, float* __restr
             for (int np = 0; np < NT / 2; ++np) {
                 uint32_t x[4];
                 ldmatrix_x4_trans(x, smem_u32(P + (16 * kk + (lane & 7) + (((lane >> 3) & 1) << 3)) * LD + w * (DK / 4) + 16 * np + 8 * (lane >> 4)));
-                mma_16816(S[2 * np], a, x[0], x[1]);
-                mma_16816(S[2 * np + 1], a, x[2], x[3]);
+                mma_acc(M[2 * np], a, x[0], x[1], kk > 0);
+                mma_acc(M[2 * np + 1], a, x[2], x[3], kk > 0);
             }
+        }
+        // (Xi and the diagonal last: their loads have had the whole step)
+#pragma unroll
+        for (int n = 0; n < NT; ++n) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                S[n][e] = fmaf(S[n][e], e & 1 ? D[n].y : D[n].x, X[n][e]) + M[n][e];
+                if (s + 1 < nseg) X[n][e] = Xn[n][e];
+            }
+            if (s + 1 < nseg) D[n] = Dn[n];
         }
         __syncthreads();                                          // (P of this step is replaced after the next one's first barrier)
     }
