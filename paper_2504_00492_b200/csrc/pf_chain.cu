@@ -18,8 +18,8 @@
 // What bounds it: where every SM has a CTA (d = 128, r = 2, 128 columns per CTA) a block of 32 tokens takes 6.5 k cycles, of
 // which the shared-memory pipe is busy for 80 % and the mma.sync pipe for 58 %; with few CTAs it is the latency of the chain's
 // dependent products (1.8 us a block at d = 128, 1.3 at 64).  Measured (kernel time, against the tcgen05 kernels in two
-// launches or one): 256 sequences of 1024 tokens, d = 128, r = 2: 0.23 ms against 0.63; 128 sequences of 4096, d = 64, r = 4: 0.35
-// against 0.93; 48 sequences of 1999, 64 x 128, r = 3: 0.149 against 0.33.  Measured and not taken: chain warps of 32 rows (half the
+// launches or one): 256 sequences of 1024 tokens, d = 128, r = 2: 0.23 ms against 0.63; 128 sequences of 4096, d = 64, r = 4: 0.34
+// against 0.93; 48 sequences of 1999, 64 x 128, r = 3: 0.145 against 0.33.  Measured and not taken: chain warps of 32 rows (half the
 // shared-memory reads, but one such warp per scheduler does not hide its own latencies: 0.31 ms at the first size), fragments
 // requested two to six ahead by hand (0.243), G from the bf16 tiles with the conversion after it (0.27).  Where the tcgen05 kernel
 // in one launch has few sequences and enough SMs to build flows ahead (d = 128), it is the faster one: see the estimates.
@@ -311,8 +311,10 @@ __device__ __forceinline__ void gram_blocks(uint32_t k_b, uint32_t q_b, uint8_t*
 #pragma unroll
             for (int tt = 0; tt < TT; ++tt) used = used || p_owner<R>(tt, nb) == W;
             if (!used) continue;
-            // (the warp's own rows as columns: the fragment it has, its two middle pieces exchanged; at d_k = 128 holding it that
-            //  long pays at r = 2 only: 231 us instead of 234 for 256 sequences of 1024 tokens, but 365 instead of 350 at r = 3)
+            // (the warp's own rows as columns: the fragment it has, its two middle pieces exchanged, where holding it that long costs
+            //  no other register.  us with it and with a second load, 250 sequences of 1000 and 3 of 8192 tokens: d_k = 64, r = 2: 145
+            //  and 147, r = 4: 236 and 238.5; d_k = 128: r = 1 154 and 155, but 128 x 64 119 and 108; r = 2 228 and 227, 128 x 64 157 and
+            //  160; r = 3 348 and 339, 136 and 114; r = 4 410 and 388, 121 and 123)
             uint32_t x[4] = {ka[0], ka[2], ka[1], ka[3]};
             if (nb != W || (DK == 128 && R != 2)) ldmatrix_x4(x, k_b + (offN ^ ((kk & 3) << 5)) + nb * 2048 + (kk >> 2) * (NB * 128));
             if (nb <= W) {
@@ -918,6 +920,7 @@ __global__ void __launch_bounds__(128) chain_compose(ChainSeg sg, float* __restr
         }
         __syncthreads();
         const __half* P = sP + (s & 1) * DK * LD;
+        float M[NT][4];
 #pragma unroll
         for (int kk = 0; kk < DK / 16; ++kk) {
             uint32_t a[4];
@@ -989,8 +992,10 @@ __global__ void __launch_bounds__(256) chain_apply(ChainSeg sg, float* __restric
         c[n][0] = x.x; c[n][1] = x.y; c[n][2] = y.x; c[n][3] = y.y;
     }
     __syncthreads();
-    // (where the blocks are many, those of the next kernel would come to multiprocessors in the order in which these leave, apart
-    //  from their neighbours with the same inputs: calls of 4 sequences of 16384 tokens one after another 139 us instead of 133)
+    // (calls one after another, us with an early start of the next and without: 15 blocks 30.6 and 31.3, 62: 43.2 and 43.7 (d = 128,
+    //  r = 1), 26.2 and 27.1 (d = 64).  Where the blocks are many the next kernel's come to multiprocessors in the order in which
+    //  these leave, apart from their neighbours with the same inputs: at d = 128 1 - 4 % slower, 256 blocks 101.2 and 99.5, 1024: 350 and
+    //  337 (r = 2); at d = 64 1 - 2 % faster, 256 blocks 37.3 and 38.0.  The line is below the first shape that loses)
     if (gridDim.x * gridDim.y <= 128) let_next_kernel_start();
 #pragma unroll
     for (int np = 0; np < DV / 16; ++np) {

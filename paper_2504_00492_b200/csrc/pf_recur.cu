@@ -5,8 +5,8 @@
 // Gram product, no inverse, no W / Uh), and no intermediate ever leaves the SM: q, k, v, beta are read once per 32 columns
 // of the state, O is written once.  What bounds it is the serial chain of one token (dot products, two shuffle stages, the
 // update): 204 cycles at d_k = 64, r = 1 and 373 at d_k = 128, r = 2, of which the FFMA pipe is busy for 160.
-// Measured (fp32): B*H = 32, L = 2048, d = 128, r = 2: 0.397 ms against 4.9 ms for the four chunk-form kernels in
-// pf_simt.cu; one head, L = 256, d = 64, r = 1: 32 us against 209.
+// Measured (fp32): B*H = 32, L = 2048, d = 128, r = 2: 0.389 ms against 4.9 ms for the four chunk-form kernels in
+// pf_simt.cu; one head, L = 256, d = 64, r = 1: 32 us walked as a whole, 23 in segments, against 209.
 //
 // A CTA takes one sequence and 32 columns j of the state S[j][i] (API layout X[i][j]); each of its four computing warps 8
 // columns, without any exchange between warps.  Lane (ig, j) of a warp holds S[j][i] for a quarter of the rows i, so a dot
