@@ -178,11 +178,12 @@ __device__ __forceinline__ ChainPart chain_part(const ChainGeo& g, const ChainSe
     return part;
 }
 
-// How they reach it.  The call is never made in ordinary use, but how it is written decides which registers the chain has: by value
-// cost the kernels that have none to spare 4 - 8 % (250 sequences of 1000, d = 128, r = 2: 243 us; from shared memory 227; without the
-// call 226), from shared memory the others up to 5 % (64 x 128, r = 4: 246 us; by value 235; without 236).
-template <int DK, int JS, bool SEG>
-constexpr bool WALK_BY_REF = DK == 128 && (JS == 128 || (SEG && JS == 64));
+// How they reach it.  The call is never made in ordinary use, but how it is written decides which registers the chain has.  us by value, from
+// shared memory, and without the call: 250 sequences of 1000, d = 128, r = 2 (128 columns per CTA): 243, 227, 226; 64 x 128, r = 4: 235, 246,
+// 236; 19 of 6950 in segments, 64 x 128: r = 1 139, 144, 130, r = 2 193, 183, 181, r = 3 278, 263, 269; 64 x 64, r = 2 108, 103, 102; at d_k = 128
+// in segments both alike.
+template <int DK, int R, int JS, bool SEG>
+constexpr bool WALK_BY_REF = SEG ? !(DK == 64 && R == 1) : DK == 128 && JS == 128;
 
 // 16 rows of S from row `row0` of the CTA's on, once more: the recurrence token by token in fp32, by one warp, two lanes to a row.  Not
 // a fast path (1.3 us a token at d_k = 128, r = 1, 3.0 at 64, r = 4): it is there so that every state that fp16 can hold gives a finite
@@ -799,7 +800,7 @@ __device__ __forceinline__ void chain_role(const ChainMaps& maps, const ChainGeo
     if (IS == 2) lost = !named_bar_and(1 + TEAMS + grp, 64, !lost);   // (both warps of a pair have written their last O)
     if (lost) {
         if (hi == 0) {
-            if constexpr (WALK_BY_REF<DK, JS, SEG>) walk_fp32<DK, R, JS, SEG, const ChainArgs&>(args, 16 * grp);
+            if constexpr (WALK_BY_REF<DK, R, JS, SEG>) walk_fp32<DK, R, JS, SEG, const ChainArgs&>(args, 16 * grp);
             else walk_fp32<DK, R, JS, SEG, ChainArgs>(ChainArgs{g, seg}, 16 * grp);
         }
     } else if (part.S_end) {
@@ -827,7 +828,7 @@ chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __rest
         if (tid == 0) atomicCAS(status, 0, 99);
         return;
     }
-    if (WALK_BY_REF<DK, JS, SEG> && tid == 32) args = {g, sg};
+    if (WALK_BY_REF<DK, R, JS, SEG> && tid == 32) args = {g, sg};
     if (tid == 0) {
         for (int x = 0; x < NS; ++x) {
             mbar_init(&land[x], 1);
