@@ -1,36 +1,44 @@
-// chain: the chunk form in ONE kernel without any hand-off through memory, on warp-level tensor-core products.
+// chain: the chunk form in ONE kernel without any hand-off through memory; a CTA walks a sequence (or a segment of one).
 //
 // A sequence is walked in blocks of up to 64 rows (64 / r tokens).  From Theorem 3.2, with rows m, S the state before the block:
 //     T  = (I + Mstrict (.) (diag(beta) K K^T))^{-1} diag(beta)                      (does not depend on S)
 //     P  = (Q K^T) (.) Mincl                                                         (does not depend on S)
 //     U' = T (V - K S^T),       O = Q S^T + P U',       S <- S + U'^T K
-// i.e. W and Uh are never formed: T is applied to V - K S^T instead.  Of the block's operations only three products depend on
-// S one after another, and their operands fit the register layout of mma.sync: with S held as [j][i] accumulators, S K^T,
-// then T applied, then the update are each "registers times shared memory", and the accumulator of one product, packed
-// to fp16, is the A operand of the next.  So a warp carries 16 rows j of S through the whole sequence without exchanging
-// anything with other warps: the serial step has no barrier, no shared-memory round trip and no tensor-memory latency.
+// i.e. W and Uh are never formed: T is applied to V - K S^T instead.  Only three products of a block depend on S one after another:
+// R = V - K S^T, U' = T R and the update.  All are tcgen05 products of 128 rows j (d_v = 64: half of them nobody's) whose A operand lies
+// in tensor memory and whose B operand is a tile of shared memory as TMA or the preparing warps left it.  S stays in tensor memory as the
+// fp32 accumulator of its update; between two products the chain warps convert an accumulator to the next one's fp16 operand.
 //
-//   chain warps   16 rows j of S each (IS = 2: two warps share the 16 rows, each holds half of the columns i; they add
-//                 their halves of S K^T and Q S^T through shared memory once per block)
-//   prep warps    teams of four: K, Q -> fp16 in place, G = K K^T, the inverse, P; a few blocks ahead
-// A stage of shared memory holds what the chain needs of one block: K, Q (fp16), T, P (fp16), V (bf16 as it came).
+// Warps (their registers moved to where they are needed):
+//   chain (8)     fp32 accumulators -> fp16 operands: -S, R, U' in turn, 32 rows j and half of the columns each
+//   products (3)  one warp each for the chain's, the output's (O^T = S Q^T + U'^T P^T) and the Gram products (G = K K^T and K Q^T, 64 rows,
+//                 from the bf16 tiles as they land)
+//   solve (2 x 4) T of every other block: G from tensor memory, the inverse on mma.sync
+//   convert (4)   K, Q -> fp16 in place, P out of tensor memory into shared memory
+//   output (4)    O^T out of tensor memory into the rows of O;  and one warp issues the copies
+// A stage of shared memory holds what the chain needs of one block: K, Q (fp16), T, P (fp16), V (bf16 as it came, added to R's
+// accumulator as V^T times an identity).
 //
-// What bounds it: where every SM has a CTA (d = 128, r = 2, 128 columns per CTA) a block of 32 tokens takes 6.5 k cycles, of
-// which the shared-memory pipe is busy for 80 % and the mma.sync pipe for 58 %; with few CTAs it is the latency of the chain's
-// dependent products (1.8 us a block at d = 128, 1.3 at 64).  Measured (kernel time, against the tcgen05 kernels in two
-// launches or one): 256 sequences of 1024 tokens, d = 128, r = 2: 0.23 ms against 0.63; 128 sequences of 4096, d = 64, r = 4: 0.34
-// against 0.93; 48 sequences of 1999, 64 x 128, r = 3: 0.145 against 0.33.  Measured and not taken: chain warps of 32 rows (half the
-// shared-memory reads, but one such warp per scheduler does not hide its own latencies: 0.31 ms at the first size), fragments
-// requested two to six ahead by hand (0.243), G from the bf16 tiles with the conversion after it (0.27).  Where the tcgen05 kernel
-// in one launch has few sequences and enough SMs to build flows ahead (d = 128), it is the faster one: see the estimates.
+// What bounds it: the three trips of a block (product, tensor memory to registers and back: 1.6 k cycles when nothing else runs on the
+// SM), drawn out to 2.9 k at d = 128, r = 2 by the other warps' work and, above all, by instruction fetch: the dozen programs together do not
+// fit the instruction cache, and where two neighbouring SMs are busy a miss costs more (3.4 k cycles with 148 CTAs).  So what is not on the
+// chain's path is written small (loops kept rolled, one election per group of products, waits that sleep): 256 sequences of 1024
+// tokens, d = 128, r = 2: 119 us, with the inverse unrolled 146, with waits that poll 220.  Measured (us, before: the same blocks on
+// warp-level products, a warp carrying 16 rows j in registers; a shared-memory read of every tile by every such warp): 256 sequences of
+// 1024, d = 128, r = 2: 227 -> 133 (calls one after another); 128 of 4096, d = 64, r = 4: 340 -> 307; 48 of 1999, 64 x 128, r = 3: 146 -> 85 (2 segments);
+// 4 of 16384, d = 128, r = 1: 135 -> 81 (segments); 32 of 2048, d = 128, r = 1: 68 -> 55 (the tcgen05 kernel in one launch before).
+// Measured and not taken: the update's and V - K S^T's products in halves, so that one half is converted while the other is being multiplied (the
+// probe's 1.6 k cycles have it; here 412 us against 389 at 32 sequences of 8192: more instructions); the output's products issued by the chain's
+// warp (462); one election per product instead of per group (427 against 420 then, 179 against 146 with all SMs busy); products in loops on
+// the chain's path too (489).
 //
 // Range: V - K S^T and U' are packed to fp16 like every other operand, and K S^T reaches sqrt(d_k) times the largest entry of S, so
 // that a state well inside fp16's 65504 can overflow them.  What overflows leaves its row of S infinite or NaN to the end of the walk
 // (infinity times anything is infinite or NaN), so one look at each row when the walk is over finds it and the blocks pay nothing:
-// the warp then walks its 16 rows once more, token by token in fp32 (walk_fp32).
+// its rows are then walked once more, token by token in fp32 (walk_fp32).
 //
-// The inverse: warp i of a team owns rows 16 i .. 16 i + 15.  D_i = (I + A_ii)^{-1} by its Neumann product and
-// E_ij = D_i A_ij in registers, then X_ij = -sum_k E_ik X_kj row block by row block (three exchanges through shared memory).
+// The inverse: warp w of a team owns rows 16 w .. 16 w + 15 of G, forms A's blocks there and D_w = (I + A_ww)^{-1} by its Neumann product,
+// and after one exchange through shared memory column block w of X: X_ww = D_w, X_iw = -D_i sum_k A_ik X_kw.
 #include <float.h>
 
 #include <atomic>
@@ -67,20 +75,41 @@ __device__ __forceinline__ uint32_t movmatrix(uint32_t x) {
     asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(y) : "r"(x));
     return y;
 }
-// (a predicated store, not a branch: a branch would keep the compiler from moving anything across it)
-__device__ __forceinline__ void store2_if(float* p, float x, float y, bool pred) {
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\t@p st.global.v2.f32 [%0], {%1, %2};\n\t}" ::"l"(p), "f"(x), "f"(y),
-                 "r"((unsigned)pred));
-}
-__device__ __forceinline__ void store_h2_if(__half* p, uint32_t x, bool pred) {
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p st.global.u32 [%0], %1;\n\t}" ::"l"(p), "r"(x), "r"((unsigned)pred));
-}
 // eight bf16 -> eight fp16 (sign: 0x80008000 to negate them)
 __device__ __forceinline__ uint4 bf16_to_half8(uint4 x, uint32_t sign) {
     uint32_t* w = (uint32_t*)&x;
 #pragma unroll
     for (int i = 0; i < 4; ++i) w[i] = pack_h2(__uint_as_float(w[i] << 16), __uint_as_float(w[i] & 0xFFFF0000u)) ^ sign;
     return x;
+}
+
+// Waits in few instructions and without a call: the kernel's warps have half a dozen programs, and what they execute together has to stay
+// in the instruction cache; and a kernel that calls functions cannot move registers between its warps.  LAZY: an unsuccessful try
+// suspends the warp for up to a millisecond, so that the many warps with time to spare do not take the others' issue slots by polling
+// (256 sequences of 1024: 136 us against 220); without it a warp wakes up sooner, and the chain's own waits do (32 sequences of 8192: 455
+// against 462).  Both give up after about a second.
+template <bool LAZY>
+__device__ __forceinline__ bool wait_inline(uint64_t* bar, uint32_t parity, int* err, int code) {
+    const uint32_t addr = smem_u32(bar);
+#pragma unroll 1
+    for (int it = 0; it < (LAZY ? 1000 : 1 << 24); ++it) {
+        uint32_t ok;
+        if (LAZY)
+            asm volatile(
+                "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 1000000;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                : "=r"(ok)
+                : "r"(addr), "r"(parity)
+                : "memory");
+        else
+            asm volatile(
+                "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                : "=r"(ok)
+                : "r"(addr), "r"(parity)
+                : "memory");
+        if (ok) return true;
+    }
+    atomicCAS(err, 0, code);
+    return false;
 }
 
 template <int DK, int R, int JS>
@@ -94,32 +123,52 @@ struct ChainSmem {
     static constexpr int tx_bytes = k_bytes + C * DK * 2 + v_bytes;         // what the copies of a block bring
 };
 
-template <int DK, int R, int JS, int IS, int TEAMS, int NS>
+constexpr int TEAMS = 2;             // solve teams
+// warps: 0-7 chain, 8-11 output, 12-15 conversion, then the solve teams, then products of the chain, products of the output, Gram
+// products, copies
+constexpr int W_OUT = 8, W_CONV = 12, W_SOLVE = 16, W_MMA = W_SOLVE + 4 * TEAMS, W_MMA_OUT = W_MMA + 1, W_GRAM = W_MMA + 2, W_LOAD = W_MMA + 3,
+              CHAIN_THREADS = 32 * (W_MMA + 4);
+
+// Registers per thread: the launch's, and what each warpgroup makes of them (the sum is the launch's)
+constexpr int REGS = 72, REGS_CHAIN = 80, REGS_OUT = 48, REGS_CONV = 56, REGS_ISSUE = 56, REGS_SOLVE = 88;
+static_assert(2 * REGS_CHAIN + REGS_OUT + REGS_CONV + REGS_ISSUE + TEAMS * REGS_SOLVE <= REGS * CHAIN_THREADS / 128, "registers of the launch");
+template <int N>
+__device__ __forceinline__ void set_registers() {
+    if (N > REGS) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
+    else asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N));
+}
+
+template <int DK, int R, int DV, int NS>
 struct ChainCfg {
-    using SM = ChainSmem<DK, R, JS>;
-    static constexpr int NCW = JS / 16 * IS;                      // chain warps
-    static constexpr int threads = 32 * NCW + 128 * TEAMS;
+    using SM = ChainSmem<DK, R, DV>;
     static constexpr int xs_off = NS * SM::stage;                 // per team: X (unscaled) while it is being formed
     static constexpr int beta_off = xs_off + TEAMS * NB * 128;    // per team: 64 step sizes, of two blocks in turn
-    // IS = 2: partial sums on their way to the other warp of the pair, [pair][parity][warp][thread-linear 16-byte pieces]
-    static constexpr int x_piece = 8 + SM::CP / 16;               // 16-byte pieces per thread: 32 of S K^T, 4 per 16 tokens of Q S^T
-    static constexpr int ex_off = beta_off + TEAMS * 512;
-    static constexpr int ex_bytes = IS == 2 ? (JS / 16) * 2 * 2 * x_piece * 512 : 0;
-    static constexpr int total = ex_off + ex_bytes;
+    static constexpr int i16_off = beta_off + TEAMS * 512;        // a 16 x 16 identity in bf16, unswizzled K-major
+    static constexpr int total = i16_off + 512;
 };
 // as many stages as fit, up to six
-template <int DK, int R, int JS, int IS, int TEAMS>
+template <int DK, int R, int DV>
 constexpr int chain_stages() {
-    constexpr int left = 226 * 1024 - ChainCfg<DK, R, JS, IS, TEAMS, 0>::total;
-    constexpr int n = left / ChainSmem<DK, R, JS>::stage;
+    constexpr int left = 226 * 1024 - ChainCfg<DK, R, DV, 0>::total;
+    constexpr int n = left / ChainSmem<DK, R, DV>::stage;
     return n < 6 ? n : 6;
 }
+
+// Tensor memory: columns
+constexpr uint32_t T_S = 0;          // S, fp32 [j][i]
+constexpr uint32_t T_S16 = 128;      // -S, fp16 pairs
+constexpr uint32_t T_R = 192;        // V^T - S K^T, then U'^T over it, fp32 [j][m]
+constexpr uint32_t T_R16 = 256;      // V^T - S K^T and
+constexpr uint32_t T_U16 = 288;      // U'^T in fp16 pairs
+constexpr uint32_t T_G = 320;        // G, fp32 [m][m'] (16 rows in each quarter of the lanes, as products of 64 rows are laid out)
+constexpr uint32_t T_P = 384;        // P^T before its mask, fp32 [m][t], likewise
+template <int CP> constexpr int O_BUFS = CP > 32 ? 1 : 2;         // O^T, fp32 [j][t]: of two blocks in turn where there is room
+template <int CP> __device__ __forceinline__ uint32_t o_cols(int b) { return CP > 32 ? 448u : 416u + 32u * (b & 1); }
 
 // What one CTA of the kernel works on.
 struct ChainPart {
     int b0, nblk;       // first block of the sequence's, number of blocks
-    int j0;             // first of its JS rows j of the state
-    int width;          // d_v, or d_k for the response to the segment's start state
+    int width;          // rows j of the state: d_v, or d_k for the response to the segment's start state
     bool response;
     const float* S0;    // start state of this sequence, or null
     float* O;           // rows of O of the first block (response: fp16 rows)
@@ -151,23 +200,20 @@ struct ChainArgs {
 };
 
 // What this CTA works on; seq: its sequence.
-template <int DK, int JS, int C, bool SEG>
+template <int DK, int C, bool SEG>
 __device__ __forceinline__ ChainPart chain_part(const ChainGeo& g, const ChainSeg& sg, const float* S0, float* O, float* S_final, long long& seq) {
     ChainPart part;
-    const int slices = g.d_v / JS;
     if constexpr (!SEG) {
-        seq = blockIdx.x / slices;
-        part = {0, g.nblk, (int)(blockIdx.x % slices) * JS, g.d_v, false, S0 ? S0 + seq * DK * g.d_v : nullptr, O + seq * g.L * g.d_v,
+        seq = blockIdx.x;
+        part = {0, g.nblk, g.d_v, false, S0 ? S0 + seq * DK * g.d_v : nullptr, O + seq * g.L * g.d_v,
                 S_final ? S_final + seq * DK * g.d_v : nullptr, nullptr};
     } else {
-        constexpr int rs = DK / JS;
-        const int per_seq = g.nseg * slices + (g.nseg - 1) * rs, x = (int)(blockIdx.x % per_seq), y = x - g.nseg * slices;
+        const int per_seq = 2 * g.nseg - 1, x = (int)(blockIdx.x % per_seq);
         seq = blockIdx.x / per_seq;
-        part.response = y >= 0;
-        const int s = part.response ? 1 + y / rs : x / slices;
+        part.response = x >= g.nseg;
+        const int s = part.response ? 1 + x - g.nseg : x;
         part.b0 = s * g.seg_blk;
         part.nblk = min(g.seg_blk, g.nblk - part.b0);
-        part.j0 = (part.response ? y % rs : x % slices) * JS;
         part.width = part.response ? DK : g.d_v;
         const long long row0 = seq * g.L + (long long)part.b0 * C, slot = seq * g.nseg + s;
         part.S0 = s == 0 && S0 ? S0 + seq * DK * g.d_v : nullptr;
@@ -178,24 +224,13 @@ __device__ __forceinline__ ChainPart chain_part(const ChainGeo& g, const ChainSe
     return part;
 }
 
-// How they reach it.  The call is never made in ordinary use, but how it is written decides which registers the chain has.  us by value, from
-// shared memory, and without the call: 250 sequences of 1000, d = 128, r = 2 (128 columns per CTA): 243, 227, 226; 64 x 128, r = 4: 235, 246,
-// 236; 19 of 6950 in segments, 64 x 128: r = 1 139, 144, 130, r = 2 193, 183, 181, r = 3 278, 263, 269; 64 x 64, r = 2 108, 103, 102; at d_k = 128
-// in segments both alike.
-template <int DK, int R, int JS, bool SEG>
-constexpr bool WALK_BY_REF = SEG ? !(DK == 64 && R == 1) : DK == 128 && JS == 128;
-
-// 16 rows of S from row `row0` of the CTA's on, once more: the recurrence token by token in fp32, by one warp, two lanes to a row.  Not
-// a fast path (1.3 us a token at d_k = 128, r = 1, 3.0 at 64, r = 4): it is there so that every state that fp16 can hold gives a finite
-// result, whatever the products with it reach.
-template <int DK, int R, int JS, bool SEG, class Args>
-__device__ __noinline__ void walk_fp32(Args args, int row0) {
-    constexpr int C = NB / R, NI = DK / 2;                        // columns i per lane
-    const ChainGeo g = args.g;
-    const ChainSeg sg = args.seg;
-    long long seq;
-    const ChainPart part = chain_part<DK, JS, C, SEG>(g, sg, g.S0, g.O, g.S_final, seq);
-    const int lane = threadIdx.x & 31, i0 = (lane & 1) * NI, j = part.j0 + row0 + (lane >> 1);
+// Eight rows of S from row `row0` on, once more: the recurrence token by token in fp32, by one warp, four lanes to a row.  Not a fast
+// path: it is there so that every state that fp16 can hold gives a finite result, whatever the products with it reach.
+template <int DK, int R, bool SEG>
+__device__ __forceinline__ void walk_fp32(const ChainArgs& args, const ChainPart& part, long long seq, int row0) {
+    constexpr int C = NB / R, NI = DK / 4;                        // columns i per lane
+    const ChainGeo& g = args.g;
+    const int lane = threadIdx.x & 31, i0 = (lane & 3) * NI, j = row0 + (lane >> 2);
     const long long tok0 = seq * g.L + (long long)part.b0 * C;
     const int tokens = min(part.nblk * C, g.L - part.b0 * C), group = g.rm == 1 ? 1 : R;      // (group: factors that read the same state)
     auto dot = [&](const float (&S)[NI], const __nv_bfloat16* x, bool self) {
@@ -210,7 +245,8 @@ __device__ __noinline__ void walk_fp32(Args args, int row0) {
                 d = fmaf(self ? z : S[n + e], z, d);
             }
         }
-        return d + __shfl_xor_sync(0xffffffffu, d, 1);
+        d += __shfl_xor_sync(0xffffffffu, d, 1);
+        return d + __shfl_xor_sync(0xffffffffu, d, 2);
     };
     float S[NI];
 #pragma unroll
@@ -247,7 +283,7 @@ __device__ __noinline__ void walk_fp32(Args args, int row0) {
             }
         }
         const float o = dot(S, g.q + (tok0 + t) * DK, false);
-        if ((lane & 1) == 0) part.O[(long long)t * g.d_v + j] = o;
+        if ((lane & 3) == 0) part.O[(long long)t * g.d_v + j] = o;
     }
     if (part.S_end)
 #pragma unroll
@@ -267,104 +303,78 @@ __device__ __forceinline__ void load_block(const ChainMaps& maps, uint8_t* smem,
     constexpr int QS = SM::CP == SM::C ? 1 : DK / 64;
 #pragma unroll
     for (int h = 0; h < QS; ++h) tma_load_4d(sg + SM::q_off + h * (SM::CP * 128), &maps.q, 0, bb * SM::C, h, seq, &land[st]);
-    if (!part.response) tma_load_4d(sg + SM::v_off, &maps.v, 0, bb * SM::C * R, part.j0 / (JS < 64 ? JS : 64), seq, &land[st]);
+    if (!part.response) tma_load_4d(sg + SM::v_off, &maps.v, 0, bb * SM::C * R, 0, seq, &land[st]);
 }
-// offset of the 16-byte piece c8 (= column / 8) of row `row` of the V tile: 128-byte rows (JS >= 64) or 64-byte rows
-template <int JS>
-__device__ __forceinline__ uint32_t v_piece(int row, int c8) {
-    if (JS >= 64) return (uint32_t)((c8 >> 3) * (NB * 128) + row * 128 + (((c8 & 7) ^ (row & 7)) << 4));
-    return (uint32_t)(row * 64 + ((c8 ^ ((row >> 1) & 3)) << 4));
-}
-
 // byte offsets of a lane's row address for ldmatrix.x4 within a slab of 128-byte swizzled rows; the K-step kk of 16 columns
 // is at off ^ (kk << 5), everything else is added
 __device__ __forceinline__ uint32_t lane_off(int row, int half) { return (uint32_t)row * 128u + (uint32_t)((half ^ (row & 7)) << 4); }
 
-// Which warp of a team forms block (16 tokens tt, 16 rows nb) of P: warp w has w + 1 blocks of G, so that all have about as
-// many.  Blocks whose rows are all later than the tile's tokens are nobody's.
-template <int R>
-__host__ __device__ constexpr int p_owner(int tt, int nb) {
-    if (nb >= (tt + 1) * R) return -1;
-    if (R == 1) return 3 - tt;
-    if (R == 2) return tt == 0 ? nb + 1 : nb < 3 ? 0 : 1;
-    if (R == 3) return tt == 0 ? (nb < 2 ? 1 : 2) : nb < 3 ? 0 : 3;
-    return nb < 2 ? 0 : nb - 1;
+enum {
+    B_SP = 0,       // chain: fp16 copy of S published
+    B_RD = 1,       // products: V^T - S K^T complete
+    B_RP = 2,       // chain: its fp16 copy published
+    B_UD = 3,       // products: U' complete
+    B_UP = 4,       // chain: its fp16 copy published
+    B_SD = 5,       // products: S complete
+    B_QD = 6,       // output products: Q S^T complete
+    B_OD = 7,       // [2] output products: O^T complete
+    B_OFREE = 9,    // [2] output: O^T read
+    B_GD = 11,      // [team] Gram products: G complete
+    B_GFREE = 13,   // solve: G read
+    B_PD = 14,      // Gram products: P^T complete (and nothing reads the block's K and Q as bf16 any more)
+    B_PFREE = 15,   // conversion: P^T read
+    B_LAND = 16     // then [NS] each: a block's tiles landed, a block prepared, a block's stage free
+};
+
+// Products over several K-steps, descriptors by their low words (a stage's address changes nothing else); whole warp, converged, and one
+// election for all of them (an election each is half as many instructions again).
+constexpr uint32_t DESC_HI = (1024u >> 4) | (1u << 14) | (2u << 29);          // SBO 1024 bytes, version, 128-byte swizzle
+__device__ __forceinline__ uint64_t desc_lo(uint32_t lo) { return ((uint64_t)DESC_HI << 32) | lo; }
+__device__ __forceinline__ uint32_t lo_of(uint32_t saddr, uint32_t slab_bytes = 16) { return (saddr >> 4) | (slab_bytes >> 4 << 16); }
+// D [128 x N] (+)= A (tensor memory) B^T: B K-major (MN false) or MN-major, KSTEPS K-steps, slabs of B_ROWS rows
+template <bool MN, int N, int KSTEPS, int B_ROWS>
+__device__ __forceinline__ void products_ta(uint32_t d, uint32_t a, uint32_t b_lo, bool acc) {
+    if (elect_one())
+#pragma unroll
+    for (int kk = 0; kk < KSTEPS; ++kk)
+            mma_f16_ta(d, a + 8 * kk, desc_lo(b_lo + (kstep_off<MN ? L_SWMN : L_SWK, B_ROWS>(kk) >> 4)), make_idesc(N, false, MN, false), acc || kk > 0);
 }
-// G[rows of block W][row blocks 0 .. W] into ga, and warp W's blocks of -P = (-Q K^T) (.) Mincl, negated back, into shared
-// memory.  All blocks advance together along the contraction, so that eight to ten accumulators are independent and a key
-// fragment serves both.
-template <int DK, int R, int CP, int W>
-__device__ __forceinline__ void gram_blocks(uint32_t k_b, uint32_t q_b, uint8_t* sp, uint32_t offA, uint32_t offN, int gq, int t4,
-                                            float (&ga)[4][2][4]) {
-    constexpr int KT = DK / 16, TT = CP / 16;
-    float pc[TT][4][2][4];
+// The same for K = 64 and one slab B [N rows][64 columns], K-major, whose columns from 16 kk on are zero (and need not have been
+// written) in the rows before 16 (kk / GROUP): a K-step leaves those columns of D alone.
+template <int N, int GROUP>
+__device__ __forceinline__ void products_lower(uint32_t d, uint32_t a, uint32_t b_lo, bool acc) {
 #pragma unroll
-    for (int kk = 0; kk < KT; ++kk) {
-        uint32_t ka[4], qa[TT][4];
-        ldmatrix_x4(ka, k_b + (offA ^ ((kk & 3) << 5)) + W * 2048 + (kk >> 2) * (NB * 128));
-#pragma unroll
-        for (int tt = 0; tt < TT; ++tt)
-            if (p_owner<R>(tt, 0) == W || p_owner<R>(tt, 1) == W || p_owner<R>(tt, 2) == W || p_owner<R>(tt, 3) == W)
-                ldmatrix_x4(qa[tt], q_b + (offA ^ ((kk & 3) << 5)) + tt * 2048 + (kk >> 2) * (CP * 128));
-#pragma unroll
-        for (int nb = 0; nb < 4; ++nb) {
-            bool used = nb <= W;
-#pragma unroll
-            for (int tt = 0; tt < TT; ++tt) used = used || p_owner<R>(tt, nb) == W;
-            if (!used) continue;
-            // (the warp's own rows as columns: the fragment it has, its two middle pieces exchanged, where holding it that long costs
-            //  no other register.  us with it and with a second load, 250 sequences of 1000 and 3 of 8192 tokens: d_k = 64, r = 2: 145
-            //  and 147, r = 4: 236 and 238.5; d_k = 128: r = 1 154 and 155, but 128 x 64 119 and 108; r = 2 228 and 227, 128 x 64 157 and
-            //  160; r = 3 348 and 339, 136 and 114; r = 4 410 and 388, 121 and 123)
-            uint32_t x[4] = {ka[0], ka[2], ka[1], ka[3]};
-            if (nb != W || (DK == 128 && R != 2)) ldmatrix_x4(x, k_b + (offN ^ ((kk & 3) << 5)) + nb * 2048 + (kk >> 2) * (NB * 128));
-            if (nb <= W) {
-                mma_acc(ga[nb][0], ka, x[0], x[1], kk > 0);
-                mma_acc(ga[nb][1], ka, x[2], x[3], kk > 0);
-            }
-#pragma unroll
-            for (int tt = 0; tt < TT; ++tt)
-                if (p_owner<R>(tt, nb) == W) {
-                    mma_acc(pc[tt][nb][0], qa[tt], x[0], x[1], kk > 0);
-                    mma_acc(pc[tt][nb][1], qa[tt], x[2], x[3], kk > 0);
-                }
-        }
+    for (int kk = 0; kk < 4; ++kk) {
+        const int n0 = 16 * (kk / GROUP);
+        if (n0 < N && elect_one()) mma_f16_ta(d + n0, a + 8 * kk, desc_lo(b_lo + ((n0 * 128 + kk * 32) >> 4)), make_idesc(N - n0, false, false, false), acc || kk > 0);
     }
+}
+// D [64 x N] = A B^T, both K-major bf16 in shared memory
+template <int N, int K, int A_ROWS, int B_ROWS>
+__device__ __forceinline__ void products_ss(uint32_t d, uint32_t a_base, uint32_t b_base) {
+    constexpr uint32_t idesc = (make_idesc(N, false, false, false) & ~(31u << 24)) | (4u << 24) | (1u << 7) | (1u << 10);     // (64 rows, bf16)
+    const uint32_t a = lo_of(a_base), b = lo_of(b_base);
+    if (elect_one())
 #pragma unroll
-    for (int tt = 0; tt < TT; ++tt)
-#pragma unroll
-        for (int nb = 0; nb < 4; ++nb) {
-            if (p_owner<R>(tt, nb) != W) continue;
-            const int ta = 16 * tt + gq, la = (ta + 1) * R, lb = (ta + 9) * R;
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int m = 16 * nb + 8 * h + 2 * t4;
-                const bool all = 16 * nb + 15 < (16 * tt + 1) * R;        // (every row is visible to every token of the block)
-                *(uint32_t*)(sp + chunk_off(ta, 2 * nb + h, CP) + 4 * t4) =
-                    pack_h2(all || m < la ? -pc[tt][nb][h][0] : 0.f, all || m + 1 < la ? -pc[tt][nb][h][1] : 0.f);
-                *(uint32_t*)(sp + chunk_off(ta + 8, 2 * nb + h, CP) + 4 * t4) =
-                    pack_h2(all || m < lb ? -pc[tt][nb][h][2] : 0.f, all || m + 1 < lb ? -pc[tt][nb][h][3] : 0.f);
-            }
-        }
+    for (int kk = 0; kk < K / 16; ++kk)
+            mma_f16(d, desc_lo(a + (kstep_off<L_SWK, A_ROWS>(kk) >> 4)), desc_lo(b + (kstep_off<L_SWK, B_ROWS>(kk) >> 4)), idesc, kk > 0);
 }
 
 // ---------------------------------------------------------------------------------------------------------------------
-// prep team: blocks b = team, team + TEAMS, ...
+// solve team: T of blocks b = team, team + TEAMS, ...
 // ---------------------------------------------------------------------------------------------------------------------
-template <int DK, int R, int JS, int IS, int TEAMS, int NS>
-__device__ __forceinline__ void prep_role(const ChainGeo& g, const ChainPart& part, const __nv_bfloat16* __restrict__ beta, int* err, uint8_t* smem,
-                                          uint64_t* land, uint64_t* full, long long seq, int team, int tid) {
-    using CFG = ChainCfg<DK, R, JS, IS, TEAMS, NS>;
+template <int DK, int R, int JS, int NS>
+__device__ __forceinline__ void solve_role(const ChainGeo& g, const ChainPart& part, const __nv_bfloat16* __restrict__ beta, int* err, uint8_t* smem,
+                                           uint64_t* bar, uint64_t* full, uint32_t tb, long long seq, int team, int tid) {
+    using CFG = ChainCfg<DK, R, JS, NS>;
     using SM = ChainSmem<DK, R, JS>;
-    constexpr int C = SM::C, CP = SM::CP;
+    constexpr int C = SM::C;
     const int w = tid >> 5, lane = tid & 31, gq = lane >> 2, t4 = lane & 3;
     const int L = g.L;
     const int bar_id = 1 + team;
     uint8_t* xs = smem + CFG::xs_off + team * NB * 128;
     const uint32_t xs_b = smem_u32(xs);
-    const uint32_t offA = lane_off(lane & 15, lane >> 4);
-    const uint32_t offN = lane_off((lane & 7) + ((lane >> 4) << 3), (lane >> 3) & 1);
-    const uint32_t offT = lane_off((lane & 7) + (((lane >> 3) & 1) << 3), lane >> 4);
+    const uint32_t offA = lane_off(lane & 15, lane >> 4), offN = lane_off((lane & 7) + ((lane >> 4) << 3), (lane >> 3) & 1);
     const __nv_bfloat16* bs = beta + seq * L * R;
     // (the bits as loaded: a conversion next to the load would make every thread wait for it there, a block ahead of its use)
     auto read_beta = [&](int b) {                                 // rows past the block or the sequence have step size zero
@@ -379,482 +389,533 @@ __device__ __forceinline__ void prep_role(const ChainGeo& g, const ChainPart& pa
     for (int b = team; b < part.nblk; b += TEAMS) {
         const int st = b % NS;
         uint8_t* sg = smem + st * SM::stage;
-        const uint32_t k_b = smem_u32(sg + SM::k_off), q_b = smem_u32(sg + SM::q_off);
         // (two in turn: another warp may still be scaling T of the block before)
         float* sBeta = (float*)(smem + CFG::beta_off + team * 512 + (b / TEAMS & 1) * 256);
-        // (a failed wait must not strand the others at a barrier: the next one carries the outcome)
-        const bool ok = mbar_wait_clk(&land[st], (uint32_t)(b / NS) & 1, err, 311);
-        // ---- K, Q: bf16 -> fp16 in place (elementwise, so the swizzled layout is untouched), several pieces per round, so that
-        //      their loads are in flight together; Q as -Q: the chain multiplies it with -S
-        {
-            uint4* p = (uint4*)(sg + SM::k_off) + tid;
-            constexpr int PIECES = (SM::k_bytes + SM::q_bytes) / 2048, ROUND = 8;
-#pragma unroll
-            for (int e0 = 0; e0 < PIECES; e0 += ROUND) {
-                uint4 x[ROUND];
-#pragma unroll
-                for (int e = 0; e < ROUND; ++e)
-                    if (e0 + e < PIECES) x[e] = p[(e0 + e) * 128];
-#pragma unroll
-                for (int e = 0; e < ROUND; ++e)
-                    if (e0 + e < PIECES) p[(e0 + e) * 128] = bf16_to_half8(x[e], (e0 + e) * 2048 < SM::k_bytes ? 0u : 0x80008000u);
-            }
-        }
-        fence_async_smem();                                       // (the stage's next copy is ordered after these writes)
         if (tid < NB) sBeta[tid] = __uint_as_float((uint32_t)breg << 16);
         if (b + TEAMS < part.nblk) breg = read_beta(b + TEAMS);
-        if (!named_bar_and(bar_id, 128, ok)) return;
-
-        // ---- G (row block w) and this warp's blocks of P
-        float ga[4][2][4];
-        {
-            uint8_t* sp = sg + SM::p_off;
-            if (w == 0) gram_blocks<DK, R, CP, 0>(k_b, q_b, sp, offA, offN, gq, t4, ga);
-            else if (w == 1) gram_blocks<DK, R, CP, 1>(k_b, q_b, sp, offA, offN, gq, t4, ga);
-            else if (w == 2) gram_blocks<DK, R, CP, 2>(k_b, q_b, sp, offA, offN, gq, t4, ga);
-            else gram_blocks<DK, R, CP, 3>(k_b, q_b, sp, offA, offN, gq, t4, ga);
-        }
+        // (a failed wait must not strand the others at a barrier: the next one carries the outcome)
+        const bool ok = wait_inline<true>(&bar[B_GD + team], (uint32_t)(b / TEAMS) & 1, err, 311);
+        tc_fence_after();
+        if (!named_bar_and(bar_id, 128, ok)) return;              // (step sizes)
+        const uint32_t t_g = tb + T_G + ((uint32_t)(32 * w) << 16);
+        uint32_t x[8];                                            // 16 columns of G, rows 16 w .. 16 w + 15, as mma.sync's accumulators
+        const int m0 = 16 * w + gq, m1 = m0 + 8;
         if (g.exact) {
             // |k|^2 is the diagonal of G; beta' = (1 - e^{-beta |k|^2}) / |k|^2
-#pragma unroll
-            for (int nb = 0; nb < 4; ++nb)
-                if (nb == w && (gq >> 1) == t4) {
-                    const float n0 = (gq & 1) ? ga[nb][0][1] : ga[nb][0][0], n1 = (gq & 1) ? ga[nb][1][3] : ga[nb][1][2];
-                    const int m = 16 * w + gq;
-                    if (n0 > 0.f) sBeta[m] = -expm1f(-sBeta[m] * n0) / n0;
-                    if (n1 > 0.f) sBeta[m + 8] = -expm1f(-sBeta[m + 8] * n1) / n1;
+            tmem_ld_frag<16>(t_g + 16 * w, x);
+            tmem_ld_wait();
+            if ((gq >> 1) == t4)
+#pragma unroll 1
+                for (int h = 0; h < 2; ++h) {
+                    const float n = __uint_as_float(h == 0 ? (gq & 1 ? x[1] : x[0]) : (gq & 1 ? x[7] : x[6]));
+                    if (n > 0.f) sBeta[m0 + 8 * h] = -expm1f(-sBeta[m0 + 8 * h] * n) / n;
                 }
             __syncwarp();
         }
-        // ---- A = Mstrict (.) (diag(beta) G) as A-operand fragments
-        uint32_t af[4][4];
-        {
-            const int m0 = 16 * w + gq, m1 = m0 + 8;
-            const float b0 = sBeta[m0], b1 = sBeta[m1];
-#pragma unroll
-            for (int nb = 0; nb < 4; ++nb)
-                if (nb <= w) {
-                    // (with groups of three rows the edge also cuts into the block to the left of the diagonal one)
-                    const bool edge = nb == w || (R == 3 && nb + 1 == w);
-#pragma unroll
-                    for (int h = 0; h < 2; ++h)
-#pragma unroll
-                        for (int e = 0; e < 2; ++e) {
-                            const int c = 16 * nb + 8 * h + 2 * t4 + e;
-                            ga[nb][h][e] = !edge || c < lim0 ? b0 * ga[nb][h][e] : 0.f;
-                            ga[nb][h][2 + e] = !edge || c < lim1 ? b1 * ga[nb][h][2 + e] : 0.f;
-                        }
-                    frag_pack(af[nb], ga[nb]);
-                }
-        }
-        // ---- D = (I + A_ww)^{-1} (Neumann product, A nilpotent), E_j = D A_wj
-        uint32_t df[4], ef[3][4];
-        float dd[2][4];
-        {
-            uint32_t a[4], at[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) a[e] = w == 0 ? af[0][e] : w == 1 ? af[1][e] : w == 2 ? af[2][e] : af[3][e];
-            at[0] = movmatrix(a[0]); at[1] = movmatrix(a[2]); at[2] = movmatrix(a[1]); at[3] = movmatrix(a[3]);
-            neumann16(dd, a, at, lane, g.rm == 1);
-            frag_pack(df, dd);
-        }
-#pragma unroll
-        for (int j = 0; j < 3; ++j)
-            if (j < w) {
-                float c[2][4];
-                frag_zero(c);
-                mma_16816(c[0], df, movmatrix(af[j][0]), movmatrix(af[j][1]));
-                mma_16816(c[1], df, movmatrix(af[j][2]), movmatrix(af[j][3]));
-                frag_pack(ef[j], c);
-            }
-        // ---- X_w,j row block by row block; X is left unscaled in the scratch for the row blocks below, T = X diag(beta) in the stage
-        auto put_x = [&](int j, const uint32_t (&f)[4]) {         // (f: packed accumulator fragment)
+        // ---- A = Mstrict (.) (diag(beta) G): its blocks left of the diagonal go to the other warps, the diagonal one stays as an A operand
+        const float b0 = sBeta[m0], b1 = sBeta[m1];
+        auto put = [&](int j, const uint32_t (&f)[4]) {           // (f: packed accumulator fragment)
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                *(uint32_t*)(xs + chunk_off(16 * w + gq, 2 * j + h, NB) + 4 * t4) = f[2 * h];
-                *(uint32_t*)(xs + chunk_off(16 * w + gq + 8, 2 * j + h, NB) + 4 * t4) = f[2 * h + 1];
+                uint8_t* at = xs + m0 * 128 + 4 * t4 + (((2 * j + h) ^ gq) << 4);
+                *(uint32_t*)at = f[2 * h];
+                *(uint32_t*)(at + 8 * 128) = f[2 * h + 1];
             }
         };
-        auto put_t = [&](int j, const float (&x)[2][4]) {
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const float2 bb = *(const float2*)(sBeta + 16 * j + 8 * h + 2 * t4);
-                *(uint32_t*)(sg + SM::t_off + chunk_off(16 * w + gq, 2 * j + h, NB) + 4 * t4) = pack_h2(x[h][0] * bb.x, x[h][1] * bb.y);
-                *(uint32_t*)(sg + SM::t_off + chunk_off(16 * w + gq + 8, 2 * j + h, NB) + 4 * t4) = pack_h2(x[h][2] * bb.x, x[h][3] * bb.y);
-            }
-        };
-        float xa[3][2][4];
-        auto add_ex = [&](int k2, int j) {                        // xa[j] += E_k2 X_k2,j
-            uint32_t x[4];
-            ldmatrix_x4_trans(x, xs_b + (offT ^ (j << 5)) + k2 * 2048);
-            mma_16816(xa[j][0], ef[k2], x[0], x[1]);
-            mma_16816(xa[j][1], ef[k2], x[2], x[3]);
-        };
-        auto finish = [&](int j, bool later) {
+        uint32_t af[4];
+#pragma unroll 1
+        for (int nb = 0;; ++nb) {
+            tmem_ld_frag<16>(t_g + 16 * nb, x);
+            tmem_ld_wait();
+            float v[2][4];
+            const int c0 = 16 * nb + 2 * t4;
 #pragma unroll
             for (int h = 0; h < 2; ++h)
 #pragma unroll
-                for (int e = 0; e < 4; ++e) xa[j][h][e] = -xa[j][h][e];
-            if (later) {
-                uint32_t f[4];
-                frag_pack(f, xa[j]);
-                put_x(j, f);
-            }
-            put_t(j, xa[j]);
-        };
+                for (int e = 0; e < 2; ++e) {
+                    v[h][e] = c0 + 8 * h + e < lim0 ? b0 * __uint_as_float(x[4 * h + e]) : 0.f;
+                    v[h][2 + e] = c0 + 8 * h + e < lim1 ? b1 * __uint_as_float(x[4 * h + 2 + e]) : 0.f;
+                }
+            frag_pack(af, v);
+            if (nb == w) break;
+            put(nb, af);
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bar[B_GFREE]);
+        // ---- D_w = (I + A_ww)^{-1} (Neumann product, A nilpotent) for the other warps
+        uint32_t y0[4];                                           // X_ww^T as an A operand
+        {
+            uint32_t at[4], df[4];
+            float dd[2][4];
+            at[0] = movmatrix(af[0]); at[1] = movmatrix(af[2]); at[2] = movmatrix(af[1]); at[3] = movmatrix(af[3]);
+            neumann16(dd, af, at, lane, g.rm == 1);
+            frag_pack(df, dd);
+            put(w, df);
+            y0[0] = movmatrix(df[0]); y0[1] = movmatrix(df[2]); y0[2] = movmatrix(df[1]); y0[3] = movmatrix(df[3]);
 #pragma unroll
-        for (int j = 0; j < 3; ++j) frag_zero(xa[j]);
-        put_x(w, df);
-        named_bar(bar_id, 128);
-        put_t(w, dd);                                             // (after the barrier: beta' of the exact step is complete)
-        if (w == 1) {
-            add_ex(0, 0);
-            finish(0, true);
-        } else if (w == 2) {
-            add_ex(1, 1);
-            finish(1, true);
-            add_ex(0, 0);
-        } else if (w == 3) {
-            add_ex(2, 2);
-            finish(2, false);
-            add_ex(1, 1);
-            add_ex(0, 0);
+            for (int h = 0; h < 2; ++h) {
+                const float2 bb = *(const float2*)(sBeta + 16 * w + 8 * h + 2 * t4);
+                uint8_t* at_ = sg + SM::t_off + m0 * 128 + 4 * t4 + (((2 * w + h) ^ gq) << 4);
+                *(uint32_t*)at_ = pack_h2(dd[h][0] * bb.x, dd[h][1] * bb.y);
+                *(uint32_t*)(at_ + 8 * 128) = pack_h2(dd[h][2] * bb.x, dd[h][3] * bb.y);
+            }
         }
         named_bar(bar_id, 128);
-        if (w == 2) {
-            add_ex(1, 0);
-            finish(0, true);
-        } else if (w == 3) {
-            add_ex(1, 0);
-            add_ex(2, 1);
-            finish(1, false);
+        // ---- down the column: X_iw = -D_i sum_k A_ik X_kw, transposed; T = X diag(beta).  X_iw^T goes above the diagonal, where A has
+        //      nothing
+#pragma unroll 1
+        for (int i = w + 1; i < 4; ++i) {
+            float c[2][4], z[2][4];
+            uint32_t f[4], y[4], a[4];
+            ldmatrix_x4(a, xs_b + (offN ^ (uint32_t)(w << 5)) + i * 2048);
+            mma_acc(c[0], y0, a[0], a[1], false);
+            mma_acc(c[1], y0, a[2], a[3], false);
+#pragma unroll 1
+            for (int k = w + 1; k < i; ++k) {
+                ldmatrix_x4(y, xs_b + (offA ^ (uint32_t)(k << 5)) + w * 2048);
+                ldmatrix_x4(a, xs_b + (offN ^ (uint32_t)(k << 5)) + i * 2048);
+                mma_16816(c[0], y, a[0], a[1]);
+                mma_16816(c[1], y, a[2], a[3]);
+            }
+            frag_pack(f, c);
+            ldmatrix_x4(a, xs_b + (offN ^ (uint32_t)(i << 5)) + i * 2048);
+            mma_acc(z[0], f, a[0], a[1], false);
+            mma_acc(z[1], f, a[2], a[3], false);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) z[h][e] = -z[h][e];
+                uint8_t* row = sg + SM::t_off + (16 * i + 8 * h + gq) * 128 + 4 * t4;
+                *(uint32_t*)(row + (((2 * w) ^ gq) << 4)) = movmatrix(pack_h2(z[h][0] * b0, z[h][1] * b0));
+                *(uint32_t*)(row + (((2 * w + 1) ^ gq) << 4)) = movmatrix(pack_h2(z[h][2] * b1, z[h][3] * b1));
+                uint8_t* at = xs + m0 * 128 + 4 * t4 + (((2 * i + h) ^ gq) << 4);
+                *(uint32_t*)at = pack_h2(z[h][0], z[h][1]);
+                *(uint32_t*)(at + 8 * 128) = pack_h2(z[h][2], z[h][3]);
+            }
+            __syncwarp();
         }
-        named_bar(bar_id, 128);
-        if (w == 3) {
-            add_ex(2, 0);
-            finish(0, false);
-        }
+        fence_async_smem();
         mbar_arrive(&full[st]);
     }
 }
 
-// ---------------------------------------------------------------------------------------------------------------------
-// chain warp: rows j of the 16-column group `grp` of the CTA's JS columns, columns i of half `hi` (IS = 2)
-// ---------------------------------------------------------------------------------------------------------------------
-template <int DK, int R, int JS, int IS, int TEAMS, int NS, bool SEG>
-__device__ __forceinline__ void chain_role(const ChainMaps& maps, const ChainGeo& g, const ChainPart& part, int* err, uint8_t* smem,
-                                           uint64_t* land, uint64_t* full, uint64_t* empty, const ChainSeg& seg, ChainArgs& args, int seq, int warp,
-                                           int lane) {
-    using CFG = ChainCfg<DK, R, JS, IS, TEAMS, NS>;
+// Conversion: K and Q of every block to fp16 in place, once the Gram products have read them as they came (Q as -Q: the chain
+// multiplies it with -S), and P.  Four warps.
+template <int DK, int R, int JS, int NS>
+__device__ __forceinline__ void convert_role(const ChainPart& part, int* err, uint8_t* smem, uint64_t* bar, uint64_t* full, uint32_t tb, int tid) {
     using SM = ChainSmem<DK, R, JS>;
-    constexpr int C = SM::C, CP = SM::CP, TT = CP / 16;
-    constexpr int DI = DK / IS, KT = DI / 16;                     // columns i of this warp, in K-steps of 16
-    const int grp = warp / IS, hi = warp % IS;
-    const int gq = lane >> 2, t4 = lane & 3;
-    const uint32_t offA = lane_off(lane & 15, lane >> 4);
-    const uint32_t offN = lane_off((lane & 7) + ((lane >> 4) << 3), (lane >> 3) & 1);
-    const uint32_t offT = lane_off((lane & 7) + (((lane >> 3) & 1) << 3), lane >> 4);
-    // V, read transposed: matrix id = lane >> 3: rows + 8 (id >> 1), columns 8 (id & 1)
-    const uint32_t offV = v_piece<JS>((lane & 7) + ((lane >> 4) << 3), 2 * grp + ((lane >> 3) & 1));
-    constexpr uint32_t V_STEP = 16 * (JS >= 64 ? 128 : 64);
-    const uint32_t smem_b = smem_u32(smem);
-    // K-step kk of this warp = step hi KT + kk of the row: slab and 32-byte position within it
-    auto kpos = [&](int kk, int slab_bytes) { return (uint32_t)((hi * KT + kk) >> 2) * (uint32_t)slab_bytes; };
-    auto kxor = [&](int kk) { return (uint32_t)(((hi * KT + kk) & 3) << 5); };
-
-    float S[2 * KT][4];                                           // [8 columns i][c]: rows j = gq, gq + 8, columns 2 t4, 2 t4 + 1
-    const int jr = part.j0 + 16 * grp + gq, i0 = hi * DI + 2 * t4, width = part.width;
-#pragma unroll
-    for (int n = 0; n < 2 * KT; ++n)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int i = i0 + 8 * n + (e & 1), j = jr + 8 * (e >> 1);
-            if (SEG && part.response) S[n][e] = i == j ? 1.f : 0.f;
-            else S[n][e] = part.S0 ? part.S0[(long long)i * width + j] : 0.f;
-        }
-    float* ob = part.O + part.j0 + 16 * grp + 2 * t4 + (IS == 2 ? 8 * hi : 0);     // O of the current block (response: in halves)
-    __half* rb = (__half*)part.O + part.j0 + 16 * grp + 2 * t4 + (IS == 2 ? 8 * hi : 0);
-    auto put_o = [&](int t, int dj, float x, float y, bool pred) {     // token t of the current block
-        // (both forms, predicated: a branch at every store would keep the products on either side of it apart)
-        if (SEG) store_h2_if(rb + (long long)t * width + dj, pack_h2(x, y), pred && part.response);
-        store2_if(ob + (long long)t * width + dj, x, y, pred && !(SEG && part.response));
-    };
-
-    // IS = 2: what this warp keeps of O of the block before (8 of the 16 columns j), without the other warp's part of Q S^T
-    float ok8[TT][4];
-    int Cv_prev = 0;
-    uint8_t* exw = smem + CFG::ex_off + grp * (4 * CFG::x_piece * 512) + lane * 16;
-    auto store8 = [&](const float4* other) {                      // ob points one block further than what is stored
-#pragma unroll
-        for (int tt = 0; tt < TT; ++tt) {
-            const float4 x = other[(8 + tt) * 32];
-            const int t = 16 * tt + gq;
-            put_o(t - C, 0, ok8[tt][0] + x.x, ok8[tt][1] + x.y, t < Cv_prev);
-            put_o(t - C + 8, 0, ok8[tt][2] + x.z, ok8[tt][3] + x.w, t + 8 < Cv_prev);
-        }
-    };
-    if (IS == 2)
-#pragma unroll
-        for (int tt = 0; tt < TT; ++tt) {
-            ((float4*)(exw + (2 + hi) * (CFG::x_piece * 512)))[(8 + tt) * 32] = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-            for (int e = 0; e < 4; ++e) ok8[tt][e] = 0.f;
-        }
-
-    int st = 0, phase = 0, st_prev = 0, ph_prev = 0;
+    constexpr int CP = SM::CP;
+    const int w = tid >> 5, lane = tid & 31, gq = lane >> 2, t4 = lane & 3;
 #pragma unroll 1
     for (int b = 0; b < part.nblk; ++b) {
-        const uint32_t sg = smem_b + st * SM::stage;
-        const uint32_t k_b = sg + SM::k_off, q_b = sg + SM::q_off, t_b = sg + SM::t_off, p_b = sg + SM::p_off, v_b = sg + SM::v_off;
-        uint32_t s16[KT][4];                                      // fp16 copy of -S: A operand of -S K^T, B operand of (-Q)(-S)^T
-#pragma unroll
-        for (int kk = 0; kk < KT; ++kk) {
-            s16[kk][0] = pack_h2(-S[2 * kk][0], -S[2 * kk][1]);
-            s16[kk][1] = pack_h2(-S[2 * kk][2], -S[2 * kk][3]);
-            s16[kk][2] = pack_h2(-S[2 * kk + 1][0], -S[2 * kk + 1][1]);
-            s16[kk][3] = pack_h2(-S[2 * kk + 1][2], -S[2 * kk + 1][3]);
-        }
-        // (IS = 2: the pair's barrier below carries the outcome, so that a failed wait never strands the other warp there; V, which
-        //  the team does not touch, had landed before the team arrived: the second wait makes it visible here)
-        const bool ok = mbar_wait_clk(&full[st], (uint32_t)phase, err, 312) && mbar_wait_clk(&land[st], (uint32_t)phase, err, 313);
-        if (IS == 1 && !ok) return;
-        // ---- R = V^T - S K^T: the accumulators start from V (in one warp of a pair)
-        float r[8][4];
-        if (IS == 1 || hi == 0) {
-#pragma unroll
-            for (int kk = 0; kk < 4; ++kk) {
-                uint32_t x[4];
-                ldmatrix_x4_trans(x, v_b + offV + kk * V_STEP);
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    r[2 * kk + (e >> 1)][2 * (e & 1)] = __uint_as_float(x[e] << 16);
-                    r[2 * kk + (e >> 1)][2 * (e & 1) + 1] = __uint_as_float(x[e] & 0xFFFF0000u);
-                }
-            }
-        } else {
-#pragma unroll
-            for (int n = 0; n < 8; ++n)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) r[n][e] = 0.f;
-        }
-#pragma unroll
-        for (int kk = 0; kk < KT; ++kk)
-#pragma unroll
-            for (int np = 0; np < 4; ++np) {
-                uint32_t x[4];
-                ldmatrix_x4(x, k_b + (offN ^ kxor(kk)) + np * 2048 + kpos(kk, NB * 128));
-                mma_16816(r[2 * np], s16[kk], x[0], x[1]);
-                mma_16816(r[2 * np + 1], s16[kk], x[2], x[3]);
-            }
-        if (IS == 2) {
-            // the other warp of the pair has the other half of the sum; with it goes the half of Q S^T of the block before that
-            // the other warp stores
-            float4* mine = (float4*)(exw + ((b & 1) * 2 + hi) * (CFG::x_piece * 512));
-            const float4* other = (const float4*)(exw + ((b & 1) * 2 + (hi ^ 1)) * (CFG::x_piece * 512));
-            const float4* other_o = (const float4*)(exw + (((b & 1) ^ 1) * 2 + (hi ^ 1)) * (CFG::x_piece * 512));
-#pragma unroll
-            for (int n = 0; n < 8; ++n) mine[n * 32] = make_float4(r[n][0], r[n][1], r[n][2], r[n][3]);
-            if (!named_bar_and(1 + TEAMS + grp, 64, ok)) return;
-#pragma unroll
-            for (int n = 0; n < 8; ++n) {
-                const float4 x = other[n * 32];
-                r[n][0] += x.x; r[n][1] += x.y; r[n][2] += x.z; r[n][3] += x.w;
-            }
-            store8(other_o);
-        }
-        // ---- the block NS - 1 further on into the stage that every chain warp has left (a block ago)
-        if (warp == 0 && lane == 0 && b > 0 && b - 1 + NS < part.nblk && mbar_wait_clk(&empty[st_prev], (uint32_t)ph_prev, err, 314))
-            load_block<DK, R, JS, NS>(maps, smem, land, b - 1 + NS, seq, part);
+        uint8_t* sg = smem + (b % NS) * SM::stage;
+        if (!wait_inline<true>(&bar[B_PD], b & 1, err, 315)) return;
+        tc_fence_after();
+        // ---- P^T rows m = 16 w .. 16 w + 15, columns t; P = its transpose (.) Mincl: row m is seen by tokens t with m < (t + 1) R
+        uint32_t x[CP / 2];
+        tmem_ld_frag<CP>(tb + T_P + ((uint32_t)(32 * w) << 16), x);
+        tmem_ld_wait();
+        tc_fence_before();
         __syncwarp();
-        // ---- U'^T = R T^T (T lower triangular)
-        uint32_t r16[4][4];
+        if (lane == 0) mbar_arrive(&bar[B_PFREE]);
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk) {
-            r16[kk][0] = pack_h2(r[2 * kk][0], r[2 * kk][1]);
-            r16[kk][1] = pack_h2(r[2 * kk][2], r[2 * kk][3]);
-            r16[kk][2] = pack_h2(r[2 * kk + 1][0], r[2 * kk + 1][1]);
-            r16[kk][3] = pack_h2(r[2 * kk + 1][2], r[2 * kk + 1][3]);
-        }
+        for (int n = 0; n < CP / 8; ++n) {
+            if (CP >= 16 && 16 * w >= (n / 2 * 16 + 16) * R) continue;       // (nothing of the block of 16 tokens sees these rows)
+            const int t = 8 * n + 2 * t4;
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk)
-#pragma unroll
-            for (int nb = kk; nb < 4; ++nb) {
-                uint32_t x[4];
-                ldmatrix_x4(x, t_b + (offN ^ (kk << 5)) + nb * 2048);
-                mma_acc(r[2 * nb], r16[kk], x[0], x[1], kk > 0);
-                mma_acc(r[2 * nb + 1], r16[kk], x[2], x[3], kk > 0);
+            for (int h = 0; h < 2; ++h) {
+                const int m = 16 * w + 8 * h + gq;
+                const uint32_t y = movmatrix(pack_h2(m < (t + 1) * R ? __uint_as_float(x[4 * n + 2 * h]) : 0.f,
+                                                     m < (t + 2) * R ? __uint_as_float(x[4 * n + 2 * h + 1]) : 0.f));
+                *(uint32_t*)(sg + SM::p_off + chunk_off(8 * n + gq, 2 * w + h, CP) + 4 * t4) = y;
             }
-        uint32_t u16[4][4];
-#pragma unroll
-        for (int kk = 0; kk < 4; ++kk) {
-            u16[kk][0] = pack_h2(r[2 * kk][0], r[2 * kk][1]);
-            u16[kk][1] = pack_h2(r[2 * kk][2], r[2 * kk][3]);
-            u16[kk][2] = pack_h2(r[2 * kk + 1][0], r[2 * kk + 1][1]);
-            u16[kk][3] = pack_h2(r[2 * kk + 1][2], r[2 * kk + 1][3]);
         }
-        // ---- S += U'^T K
+        // ---- bf16 -> fp16 (elementwise, so the swizzled layout is untouched), several pieces per round, so that their loads are in flight together
+        uint4* p = (uint4*)(sg + SM::k_off) + tid;
+        constexpr int PIECES = (SM::k_bytes + SM::q_bytes) / 2048, ROUND = PIECES % 4 == 0 ? 4 : PIECES % 3 == 0 ? 3 : 5;
+        static_assert(PIECES % ROUND == 0, "pieces per round");
+#pragma unroll 1
+        for (int e0 = 0; e0 < PIECES; e0 += ROUND) {
+            uint4 y[ROUND];
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk)
+            for (int e = 0; e < ROUND; ++e) y[e] = p[(e0 + e) * 128];
 #pragma unroll
-            for (int ip = 0; ip < KT; ++ip) {
-                uint32_t x[4];
-                ldmatrix_x4_trans(x, k_b + (offT ^ kxor(ip)) + kk * 2048 + kpos(ip, NB * 128));
-                mma_16816(S[2 * ip], u16[kk], x[0], x[1]);
-                mma_16816(S[2 * ip + 1], u16[kk], x[2], x[3]);
-            }
-        // ---- O = Q S^T + P U' with the state before the update (these products fill the latency of the update).  Two tiles of 16
-        //      tokens at a time, or one with its sums in two halves: at least four independent accumulators, the depth of the
-        //      product's pipeline (one tile at a time took 2.8 k cycles of a step of 6.5 k at d_k = 128, r = 1)
-        const int Cv = min(C, g.L - (part.b0 + b) * C);
-        constexpr int TG = TT >= 2 ? 2 : 1, SP = 3 - TG;
-#pragma unroll
-        for (int tg = 0; tg < TT; tg += TG) {
-            float o[TG][SP][2][4];
-#pragma unroll
-            for (int kk = 0; kk < KT; ++kk)
-#pragma unroll
-                for (int u = 0; u < TG; ++u) {
-                    uint32_t a[4];
-                    ldmatrix_x4(a, q_b + (offA ^ kxor(kk)) + (tg + u) * 2048 + kpos(kk, CP * 128));
-                    mma_acc(o[u][kk % SP][0], a, s16[kk][0], s16[kk][2], kk >= SP);
-                    mma_acc(o[u][kk % SP][1], a, s16[kk][1], s16[kk][3], kk >= SP);
-                }
-            if (IS == 2) {
-                // (the warp keeps 8 of the 16 columns j and hands its half of the sum for the others over)
-#pragma unroll
-                for (int u = 0; u < TG; ++u) {
-                    if (SP == 2)
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            o[u][0][0][e] += o[u][SP - 1][0][e];
-                            o[u][0][1][e] += o[u][SP - 1][1][e];
-                        }
-                    float4* mine = (float4*)(exw + ((b & 1) * 2 + hi) * (CFG::x_piece * 512));
-                    mine[(8 + tg + u) * 32] = hi ? make_float4(o[u][0][0][0], o[u][0][0][1], o[u][0][0][2], o[u][0][0][3])
-                                                 : make_float4(o[u][0][1][0], o[u][0][1][1], o[u][0][1][2], o[u][0][1][3]);
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) ok8[tg + u][e] = hi ? o[u][0][1][e] : o[u][0][0][e];
-                }
-            }
-#pragma unroll
-            for (int kk = 0; kk < 4; ++kk)
-#pragma unroll
-                for (int u = 0; u < TG; ++u) {
-                    if (kk >= (tg + u + 1) * R) continue;
-                    uint32_t a[4];
-                    ldmatrix_x4(a, p_b + (offA ^ (kk << 5)) + (tg + u) * 2048);
-                    if (IS == 2) {
-                        mma_16816(ok8[tg + u], a, hi ? u16[kk][1] : u16[kk][0], hi ? u16[kk][3] : u16[kk][2]);
-                    } else {
-                        mma_16816(o[u][kk % SP][0], a, u16[kk][0], u16[kk][2]);
-                        mma_16816(o[u][kk % SP][1], a, u16[kk][1], u16[kk][3]);
-                    }
-                }
-            if (IS == 1)
-#pragma unroll
-                for (int u = 0; u < TG; ++u) {
-                    if (SP == 2)
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            o[u][0][0][e] += o[u][SP - 1][0][e];
-                            o[u][0][1][e] += o[u][SP - 1][1][e];
-                        }
-                    const int t = 16 * (tg + u) + gq;
-                    put_o(t, 0, o[u][0][0][0], o[u][0][0][1], t < Cv);
-                    put_o(t, 8, o[u][0][1][0], o[u][0][1][1], t < Cv);
-                    put_o(t + 8, 0, o[u][0][0][2], o[u][0][0][3], t + 8 < Cv);
-                    put_o(t + 8, 8, o[u][0][1][2], o[u][0][1][3], t + 8 < Cv);
-                }
+            for (int e = 0; e < ROUND; ++e) p[(e0 + e) * 128] = bf16_to_half8(y[e], (e0 + e) * 2048 < SM::k_bytes ? 0u : 0x80008000u);
         }
-        Cv_prev = Cv;
-        ob += (long long)C * width;
-        rb += (long long)C * width;
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&empty[st]);
-        st_prev = st;
-        ph_prev = phase;
+        fence_async_smem();
+        mbar_arrive(&full[b % NS]);
+    }
+}
+
+// Gram products (one warp): G = K K^T and K Q^T from the bf16 tiles as they landed, in products of 64 rows.
+template <int DK, int R, int JS, int NS>
+__device__ __forceinline__ void gram_role(const ChainPart& part, int* err, uint8_t* smem, uint64_t* bar, uint64_t* land, uint32_t tb) {
+    using SM = ChainSmem<DK, R, JS>;
+    int st = 0, phase = 0;
+#pragma unroll 1
+    for (int b = 0; b < part.nblk; ++b) {
+        const uint32_t k_b = smem_u32(smem + st * SM::stage + SM::k_off), q_b = k_b + SM::q_off - SM::k_off;
+        if (!wait_inline<true>(&land[st], phase, err, 316)) return;
+        if (b > 0 && !wait_inline<true>(&bar[B_GFREE], (b - 1) & 1, err, 317)) return;
+        tc_fence_after();
+        products_ss<NB, DK, NB, NB>(tb + T_G, k_b, k_b);
+        commit_uni(&bar[B_GD + b % TEAMS]);
+        if (b > 0 && !wait_inline<true>(&bar[B_PFREE], (b - 1) & 1, err, 318)) return;
+        tc_fence_after();
+        products_ss<SM::CP, DK, NB, SM::CP>(tb + T_P, k_b, q_b);
+        commit_uni(&bar[B_PD]);
         if (++st == NS) {
             st = 0;
             phase ^= 1;
         }
     }
-    if (IS == 2) {
-        named_bar(1 + TEAMS + grp, 64);                           // (both warps are here: a failed wait left through the barrier above)
-        store8((const float4*)(exw + (((part.nblk & 1) ^ 1) * 2 + (hi ^ 1)) * (CFG::x_piece * 512)));
-    }
-    if (SEG && part.response) {
-        __half* P = (__half*)part.S_end;
+}
+
+// ---------------------------------------------------------------------------------------------------------------------
+// The serial part: S in tensor memory, row j = lane j.
+// ---------------------------------------------------------------------------------------------------------------------
+// N columns of an fp32 accumulator, in fp16 pairs (negated) as the A operand of the next product.  (A load and its wait cost about the
+// same whatever the width.)
+template <int N, bool NEG>
+__device__ __forceinline__ void to_operand(uint32_t src, uint32_t dst) {
+    uint32_t x[N / 32][32], h[16];
 #pragma unroll
-        for (int n = 0; n < 2 * KT; ++n)
+    for (int c = 0; c < N / 32; ++c) tmem_ld32(src + 32 * c, x[c]);
+    tmem_ld_wait();
 #pragma unroll
-            for (int e = 0; e < 4; e += 2) {
-                const int j = jr + 4 * e, i = i0 + 8 * n;
-                *(uint32_t*)(P + (long long)j * DK + i) = pack_h2(i == j ? 0.f : S[n][e], i + 1 == j ? 0.f : S[n][e + 1]);
-                if (i == j) part.D[j] = S[n][e];
-                if (i + 1 == j) part.D[j] = S[n][e + 1];
-            }
-        return;
-    }
-    // (one entry tells for its row.  The end state may replace the start state, which is still needed where rows are lost)
-    bool lost = __any_sync(0xffffffffu, !(fabsf(S[0][0]) <= FLT_MAX) || !(fabsf(S[0][2]) <= FLT_MAX));
-    if (IS == 2) lost = !named_bar_and(1 + TEAMS + grp, 64, !lost);   // (both warps of a pair have written their last O)
-    if (lost) {
-        if (hi == 0) {
-            if constexpr (WALK_BY_REF<DK, R, JS, SEG>) walk_fp32<DK, R, JS, SEG, const ChainArgs&>(args, 16 * grp);
-            else walk_fp32<DK, R, JS, SEG, ChainArgs>(ChainArgs{g, seg}, 16 * grp);
+    for (int c = 0; c < N / 32; ++c) {
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+            const float lo = __uint_as_float(x[c][2 * e]), hi = __uint_as_float(x[c][2 * e + 1]);
+            h[e] = NEG ? pack_h2(-lo, -hi) : pack_h2(lo, hi);
         }
-    } else if (part.S_end) {
-#pragma unroll
-        for (int n = 0; n < 2 * KT; ++n)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) part.S_end[(long long)(i0 + 8 * n + (e & 1)) * width + jr + 8 * (e >> 1)] = S[n][e];
+        tmem_st16(dst + 16 * c, h);
     }
 }
 
-template <int DK, int R, int JS, int IS, int TEAMS, int NS, bool SEG>
-__global__ void __launch_bounds__(ChainCfg<DK, R, JS, IS, TEAMS, NS>::threads, 1)
+// warp `warp` of eight: rows j = 32 (warp & 3) + lane, half warp >> 2 of the columns of everything
+template <int DK>
+__device__ __forceinline__ void chain_role(const ChainPart& part, int* err, uint64_t* bar, uint32_t tb, int warp, int lane) {
+    constexpr int HC = DK / 2;                                    // columns i of this warp
+    const int h = warp >> 2, j = 32 * (warp & 3) + lane;
+    const uint32_t lanes = (uint32_t)(32 * (warp & 3)) << 16;
+    const uint32_t t_s = tb + T_S + h * HC + lanes, t_s16 = tb + T_S16 + h * HC / 2 + lanes, t_u16 = tb + T_U16 + 16 * h + lanes;
+#pragma unroll 1
+    for (int c = 0; c < HC; c += 16) {
+        uint32_t x[16], y[8];
+        const float* s0 = part.S0 + (long long)(h * HC + c) * part.width + j;
+#pragma unroll
+        for (int e = 0; e < 16; ++e) x[e] = __float_as_uint(part.S0 ? s0[e * part.width] : part.response && h * HC + c + e == j ? 1.f : 0.f);
+        tmem_st16(t_s + c, x);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) y[e] = pack_h2(-__uint_as_float(x[2 * e]), -__uint_as_float(x[2 * e + 1]));
+        tmem_st8(t_s16 + c / 2, y);
+    }
+    auto publish = [&](int b) {
+        tmem_st_wait();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bar[b]);
+    };
+    const uint32_t t_r = tb + T_R + 32 * h + lanes, t_r16 = tb + T_R16 + 16 * h + lanes;
+#pragma unroll 1
+    for (int b = 0; b < part.nblk; ++b) {
+        publish(B_SP);
+        if (!wait_inline<false>(&bar[B_RD], b & 1, err, 312)) return;
+        tc_fence_after();
+        to_operand<32, false>(t_r, t_r16);
+        publish(B_RP);
+        if (!wait_inline<false>(&bar[B_UD], b & 1, err, 313)) return;
+        tc_fence_after();
+        to_operand<32, false>(t_r, t_u16);
+        publish(B_UP);
+        if (!wait_inline<false>(&bar[B_SD], b & 1, err, 314)) return;
+        tc_fence_after();
+        to_operand<HC, true>(t_s, t_s16);
+    }
+    tmem_st_wait();
+}
+
+// The products of the chain (one warp).
+template <int DK, int R, int DV, int NS>
+__device__ __forceinline__ void mma_role(const ChainPart& part, int* err, uint8_t* smem, uint64_t* bar, uint32_t tb) {
+    using CFG = ChainCfg<DK, R, DV, NS>;
+    using SM = ChainSmem<DK, R, DV>;
+    constexpr int K_SLAB = NB * 128, OB = O_BUFS<SM::CP>;
+    uint64_t *land = bar + B_LAND, *full = land + NS, *empty = full + NS;
+    const uint32_t smem_b = smem_u32(smem), i16_b = smem_b + CFG::i16_off;
+    const uint32_t t_r = tb + T_R;
+    // V^T of a block into the accumulator: 16 columns m at a time, as V^T times a 16 x 16 identity, both bf16 (V as it came).  At
+    // d_v = 64 the tile's 64 columns are read twice: rows j past d_v are nobody's.
+    auto put_v = [&](int st) {
+        const uint32_t v_lo = lo_of(smem_b + st * SM::stage + SM::v_off, DV == 128 ? K_SLAB : 0);
+        const uint64_t i16 = desc_ns_kmajor(i16_b, 16);
+        constexpr uint32_t idesc = make_idesc(16, true, false, false) | (1u << 7) | (1u << 10);
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            if (elect_one()) mma_f16(t_r + 16 * c, desc_lo(v_lo + c * (2048 >> 4)), i16, idesc, false);
+    };
+    int st = 0, phase = 0;
+#pragma unroll 1
+    for (int b = 0; b < part.nblk; ++b) {
+        const uint32_t sg = smem_b + st * SM::stage, k_lo = lo_of(sg + SM::k_off), kt_lo = lo_of(sg + SM::k_off, K_SLAB), t_lo = lo_of(sg + SM::t_off);
+        // ---- V^T (the accumulator's last reader, the chain warps' conversion of U' of the block before, is done)
+        if (!part.response) {
+            if (!wait_inline<false>(&land[st], phase, err, 327)) return;
+            tc_fence_after();
+            put_v(st);
+        }
+        if (!wait_inline<false>(&full[st], phase, err, 322) || !wait_inline<false>(&bar[B_SP], b & 1, err, 323)) return;
+        tc_fence_after();
+        // ---- R = V^T - S K^T
+        products_ta<false, NB, DK / 16, NB>(t_r, tb + T_S16, k_lo, !part.response);
+        commit_uni(&bar[B_RD]);
+        // ---- U'^T = R T^T (T lower triangular: rows m' = 16 kk .. of the contraction reach columns m >= 16 kk only)
+        // (U' completes only after the last reader of the block before's, P U', so that the chain warps need not wait for that)
+        if (b > 0 && !wait_inline<false>(&bar[B_OD + (b - 1) % OB], ((b - 1) / OB) & 1, err, 319)) return;
+        if (!wait_inline<false>(&bar[B_RP], b & 1, err, 326)) return;
+        tc_fence_after();
+        products_lower<NB, 1>(t_r, tb + T_R16, t_lo, false);
+        commit_uni(&bar[B_UD]);
+        // ---- S += U'^T K
+        // (and S only after Q S^T)
+        if (!wait_inline<false>(&bar[B_QD], b & 1, err, 320) || !wait_inline<false>(&bar[B_UP], b & 1, err, 328)) return;
+        tc_fence_after();
+        products_ta<true, DK, NB / 16, NB>(tb + T_S, tb + T_U16, kt_lo, true);
+        commit_uni(&bar[B_SD]);
+        commit_uni(&empty[st]);
+        if (++st == NS) {
+            st = 0;
+            phase ^= 1;
+        }
+    }
+}
+
+// The products of the output (one warp): O^T = S Q^T + U'^T P^T with the state before the update.
+template <int DK, int R, int DV, int NS>
+__device__ __forceinline__ void mma_out_role(const ChainPart& part, int* err, uint8_t* smem, uint64_t* bar, uint32_t tb) {
+    using SM = ChainSmem<DK, R, DV>;
+    constexpr int CP = SM::CP, OB = O_BUFS<CP>;
+    uint64_t *full = bar + B_LAND + NS, *empty = full + NS;
+    const uint32_t smem_b = smem_u32(smem);
+    int st = 0, phase = 0;
+#pragma unroll 1
+    for (int b = 0; b < part.nblk; ++b) {
+        const uint32_t sg = smem_b + st * SM::stage, t_o = tb + o_cols<CP>(b);
+        if (!wait_inline<true>(&full[st], phase, err, 351) || !wait_inline<true>(&bar[B_SP], b & 1, err, 352)) return;
+        if (b >= OB && !wait_inline<true>(&bar[B_OFREE + b % OB], (b / OB - 1) & 1, err, 325)) return;
+        tc_fence_after();
+        products_ta<false, CP, DK / 16, CP>(t_o, tb + T_S16, lo_of(sg + SM::q_off), false);
+        commit_uni(&bar[B_QD]);
+        if (!wait_inline<true>(&bar[B_UP], b & 1, err, 354)) return;
+        tc_fence_after();
+        // (rows 16 kk .. of the contraction are seen from tile kk / R of 16 tokens on)
+        products_lower<CP, R>(t_o, tb + T_U16, lo_of(sg + SM::p_off), true);
+        commit_uni(&bar[B_OD + b % OB]);
+        commit_uni(&empty[st]);
+        if (++st == NS) {
+            st = 0;
+            phase ^= 1;
+        }
+    }
+}
+
+// O of each block from tensor memory to global memory: warp `warp` of four has rows j = 32 warp + lane, and one store of a warp is
+// 128 contiguous bytes of a token's row (64 of a response's).
+template <int C, int CP, int DK, int DV>
+__device__ __forceinline__ void out_role(const ChainGeo& g, const ChainPart& part, int* err, uint64_t* bar, uint32_t tb, int warp, int lane) {
+    constexpr int OB = O_BUFS<CP>;
+    const int j = 32 * warp + lane;
+    const uint32_t lanes = (uint32_t)(32 * warp) << 16;
+    float* o = part.O + j;
+    __half* oh = (__half*)part.O + j;
+#pragma unroll 1
+    for (int b = 0; b < part.nblk; ++b) {
+        if (!wait_inline<true>(&bar[B_OD + b % OB], (b / OB) & 1, err, 331)) return;
+        tc_fence_after();
+        const int Cv = min(C, g.L - (part.b0 + b) * C);
+#pragma unroll 1
+        for (int c = 0; c < CP; c += 16) {
+            uint32_t x[16];
+            tmem_ld16(tb + o_cols<CP>(b) + lanes + c, x);
+            tmem_ld_wait();
+            if (c + 16 == CP) {
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&bar[B_OFREE + b % OB]);
+            }
+            if (part.response) {
+#pragma unroll
+                for (int t = 0; t < 16; ++t)
+                    if (c + t < Cv) oh[(c + t) * DK] = __float2half_rn(__uint_as_float(x[t]));
+            } else if (c + 16 <= Cv) {
+#pragma unroll
+                for (int t = 0; t < 16; ++t) o[(c + t) * DV] = __uint_as_float(x[t]);
+            } else {
+#pragma unroll
+                for (int t = 0; t < 16; ++t)
+                    if (c + t < Cv) o[(c + t) * DV] = __uint_as_float(x[t]);
+            }
+        }
+        o += C * DV;
+        oh += C * DK;
+    }
+}
+
+// The end state, once every role is done.
+template <int DK, int R, bool SEG>
+__device__ __forceinline__ void end_state(const ChainPart& part, const ChainArgs& args, long long seq, uint32_t tb, int warp, int lane) {
+    constexpr int HC = DK / 2;
+    const int h = warp >> 2, quarter = warp & 3, j = 32 * quarter + lane;
+    const uint32_t t_s = tb + T_S + h * HC + ((uint32_t)(32 * quarter) << 16);
+    if (part.response) {
+        __half* P = (__half*)part.S_end + (long long)j * DK + h * HC;
+#pragma unroll 1
+        for (int c = 0; c < HC; c += 32) {
+            uint32_t x[32];
+            tmem_ld32(t_s + c, x);
+            tmem_ld_wait();
+#pragma unroll
+            for (int e = 0; e < 32; ++e)
+                if (h * HC + c + e == j) {
+                    part.D[j] = __uint_as_float(x[e]);
+                    x[e] = 0;
+                }
+#pragma unroll
+            for (int e = 0; e < 32; e += 8)
+                *(uint4*)(P + c + e) = make_uint4(pack_h2(__uint_as_float(x[e]), __uint_as_float(x[e + 1])), pack_h2(__uint_as_float(x[e + 2]), __uint_as_float(x[e + 3])),
+                                                  pack_h2(__uint_as_float(x[e + 4]), __uint_as_float(x[e + 5])), pack_h2(__uint_as_float(x[e + 6]), __uint_as_float(x[e + 7])));
+        }
+        return;
+    }
+    // (one entry tells for its row.  The end state may replace the start state, which is still needed where rows are lost)
+    uint32_t x[32];
+    tmem_ld32(t_s, x);
+    tmem_ld_wait();
+    const bool lost = !named_bar_and(1 + quarter, 64, fabsf(__uint_as_float(x[0])) <= FLT_MAX);
+    if (lost) {
+#pragma unroll 1
+        for (int r0 = 0; r0 < 16; r0 += 8) walk_fp32<DK, R, SEG>(args, part, seq, 32 * quarter + 16 * h + r0);
+    } else if (part.S_end) {
+#pragma unroll 1
+        for (int c = 0; c < HC; c += 32) {
+            tmem_ld32(t_s + c, x);
+            tmem_ld_wait();
+#pragma unroll
+            for (int e = 0; e < 32; ++e) part.S_end[(long long)(h * HC + c + e) * part.width + j] = __uint_as_float(x[e]);
+        }
+    }
+}
+
+template <int DK, int R, int DV, int NS, bool SEG>
+__global__ void __launch_bounds__(CHAIN_THREADS, 1)
 chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __restrict__ beta, const float* __restrict__ S0,
              float* __restrict__ O, float* __restrict__ S_final, int* __restrict__ status, ChainGeo g, ChainSeg sg) {
-    using CFG = ChainCfg<DK, R, JS, IS, TEAMS, NS>;
-    using SM = ChainSmem<DK, R, JS>;
+    using CFG = ChainCfg<DK, R, DV, NS>;
+    using SM = ChainSmem<DK, R, DV>;
     extern __shared__ __align__(1024) uint8_t smem[];
-    __shared__ uint64_t land[NS], full[NS], empty[NS];
+    __shared__ uint64_t bar[B_LAND + 3 * NS];
+    __shared__ uint32_t tmem_base;
     __shared__ ChainArgs args;
-    const int tid = threadIdx.x, warp = tid >> 5;
+    uint64_t *land = bar + B_LAND, *full = land + NS, *empty = full + NS;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     long long seq;
-    const ChainPart part = chain_part<DK, JS, SM::C, SEG>(g, sg, S0, O, S_final, seq);
+    const ChainPart part = chain_part<DK, SM::C, SEG>(g, sg, S0, O, S_final, seq);
+    const int quarters = part.width / 32;                         // lane quarters that hold rows of the state
     if ((smem_u32(smem) & 1023u) != 0) {                          // (the swizzled layouts need a 1024-byte aligned base)
         wait_for_previous_kernel();
         if (tid == 0) atomicCAS(status, 0, 99);
         return;
     }
-    if (WALK_BY_REF<DK, R, JS, SEG> && tid == 32) args = {g, sg};
+    if (tid == 32) args = {g, sg};
     if (tid == 0) {
+        mbar_init(&bar[B_SP], 2 * quarters);
+        mbar_init(&bar[B_RP], 2 * quarters);
+        mbar_init(&bar[B_UP], 2 * quarters);
+        mbar_init(&bar[B_RD], 1);
+        mbar_init(&bar[B_SD], 1);
+        mbar_init(&bar[B_UD], 1);
+        mbar_init(&bar[B_QD], 1);
+        mbar_init(&bar[B_PD], 1);
+        mbar_init(&bar[B_GFREE], 4);
+        mbar_init(&bar[B_PFREE], 4);
+        for (int x = 0; x < 2; ++x) {
+            mbar_init(&bar[B_OD + x], 1);
+            mbar_init(&bar[B_OFREE + x], quarters);
+            mbar_init(&bar[B_GD + x], 1);
+        }
         for (int x = 0; x < NS; ++x) {
             mbar_init(&land[x], 1);
-            mbar_init(&full[x], 128);
-            mbar_init(&empty[x], CFG::NCW);
+            mbar_init(&full[x], 256);
+            mbar_init(&empty[x], 2);
         }
         mbar_fence_init();
         prefetch_tmap(&maps.q);
         prefetch_tmap(&maps.k);
         prefetch_tmap(&maps.v);
     }
-    if (SM::CP > SM::C || part.response) {                        // (r = 3: query rows that no copy writes are read; a response: v = 0)
-        for (int e = tid; e < NS * SM::stage / 16; e += CFG::threads) ((uint4*)smem)[e] = make_uint4(0, 0, 0, 0);
-        fence_async_smem();
-    }
+    if (warp == W_MMA) tmem_alloc(&tmem_base, 512);
+    if (SM::CP > SM::C)                                           // (r = 3: query rows that no copy writes are read)
+        for (int e = tid; e < NS * SM::stage / 16; e += CHAIN_THREADS) ((uint4*)smem)[e] = make_uint4(0, 0, 0, 0);
+    if (tid < 256) *(uint16_t*)(smem + CFG::i16_off + ns_off(tid >> 4, tid & 15, 16)) = (tid >> 4) == (tid & 15) ? 0x3F80 : 0;
+    fence_async_smem();
     wait_for_previous_kernel();
     if (!SEG) let_next_kernel_start();      // (chain_compose's blocks would crowd on what few multiprocessors have room: 144 us instead of 140)
     if (tid == 0 && blockIdx.x == 0 && g.clear) *status = 0;      // (the call's status word: a wait expires a second from now at the earliest)
+    tc_fence_before();
     __syncthreads();
-    if (tid == 0)
-        for (int b = 0; b < NS && b < part.nblk; ++b) load_block<DK, R, JS, NS>(maps, smem, land, b, (int)seq, part);
-    __syncwarp();
-    if (warp < CFG::NCW)
-        chain_role<DK, R, JS, IS, TEAMS, NS, SEG>(maps, g, part, status, smem, land, full, empty, sg, args, (int)seq, warp, tid & 31);
-    else
-        prep_role<DK, R, JS, IS, TEAMS, NS>(g, part, beta, status, smem, land, full, seq, (warp - CFG::NCW) >> 2, (tid - 32 * CFG::NCW) & 127);
+    tc_fence_after();
+    const uint32_t tb = tmem_base;
+    // (each warpgroup sets its registers once, and no code is shared after that: its end is in its own branch)
+    auto all_done = [&]() {
+        __syncwarp();
+        tc_fence_before();
+        named_bar(0, CHAIN_THREADS);
+        tc_fence_after();
+    };
+    if (warp < W_OUT) {
+        set_registers<REGS_CHAIN>();
+        const bool holds_state = (warp & 3) < quarters;
+        if (holds_state) chain_role<DK>(part, status, bar, tb, warp, lane);
+        all_done();                                               // (every output is written, all products are complete)
+        if (holds_state) end_state<DK, R, SEG>(part, args, seq, tb, warp, lane);
+        all_done();
+    } else if (warp < W_CONV) {
+        set_registers<REGS_OUT>();
+        if (warp - W_OUT < quarters) out_role<SM::C, SM::CP, DK, DV>(g, part, status, bar, tb, warp - W_OUT, lane);
+        all_done();
+        all_done();
+    } else if (warp < W_SOLVE) {
+        set_registers<REGS_CONV>();
+        convert_role<DK, R, DV, NS>(part, status, smem, bar, full, tb, tid - 32 * W_CONV);
+        all_done();
+        all_done();
+    } else if (warp < W_MMA) {
+        set_registers<REGS_SOLVE>();
+        solve_role<DK, R, DV, NS>(g, part, beta, status, smem, bar, full, tb, seq, (warp - W_SOLVE) >> 2, (tid - 32 * W_SOLVE) & 127);
+        all_done();
+        all_done();
+    } else {
+        set_registers<REGS_ISSUE>();
+        if (warp == W_MMA) {
+            mma_role<DK, R, DV, NS>(part, status, smem, bar, tb);
+        } else if (warp == W_MMA_OUT) {
+            mma_out_role<DK, R, DV, NS>(part, status, smem, bar, tb);
+        } else if (warp == W_GRAM) {
+            gram_role<DK, R, DV, NS>(part, status, smem, bar, land, tb);
+        } else if (warp == W_LOAD) {
+            bool ok = true;
+#pragma unroll 1
+            for (int b = 0; ok && b < part.nblk; ++b) {
+                if (b >= NS) ok = wait_inline<true>(&empty[b % NS], (b / NS - 1) & 1, status, 341);
+                if (ok && lane == 0) load_block<DK, R, DV, NS>(maps, smem, land, b, (int)seq, part);
+            }
+        }
+        all_done();
+        all_done();
+        if (warp == W_MMA) tmem_dealloc(tb, 512);
+    }
 }
 
 // Start states of the segments: one CTA per sequence and 16 rows j, serial over the segments; four warps with a quarter of the
@@ -1015,57 +1076,37 @@ __global__ void __launch_bounds__(256) chain_apply(ChainSeg sg, float* __restric
     }
 }
 
-// How a sequence is spread over CTAs: columns per CTA, and segments.  The time is (waves of CTAs) x (blocks of a segment) x
-// (time of a block), plus what composing segments costs.
-// Columns: fewer per CTA make a shorter step but more CTAs.  Measured with one wave, us per block for d_k = d_v = 128, r = 1 .. 4: 32
-// columns by pairs of warps 2.35, 1.82, 1.74, 1.70; 64 columns 3.3, 2.5, 2.55, 2.3; 128 columns 4.4, 3.4, 3.4, 3.0.  At d_k = 64 a step
-// is short enough that 32 columns gain nothing over 64, and 128 columns cost 1.53 times as much.
-// Segments: as many as one wave of CTAs holds pay for the second walk (the responses) and for two more kernels when few
-// sequences are long: taken where the estimate falls (d = 64, r = 1, one sequence: 1200 tokens 17 us instead of 38; d = 128: 600 tokens
-// 20.5 instead of 26).
-enum { COLS_32, COLS_64, COLS_128 };
+// A sequence has one CTA, or where few sequences are long, segments walked side by side: as many as one wave of CTAs holds pay for
+// the second walk (the responses) and for two more kernels.  The time is 7 us, (waves of CTAs) x (blocks of a segment) x (time of a
+// block) and what composing segments costs.  Measured, us per block for r = 1 .. 4 with 32 CTAs (d_k = 64 and 128), and with 148, when
+// two multiprocessors share what they fetch instructions through; and 8192 tokens of 4 sequences, d = 128, r = 1, in 1, 2, 4, 8, 16
+// segments: 259, 136, 85, 60, 55 us; of 2, d = 64, r = 2, in 2, 4, 8, 16: 163, 88, 53, 40.
 struct ChainPlan {
-    int cols, nseg, seg_blk;
+    int nseg, seg_blk;
     double us;
     double short_us;          // the kernel alone without segments, the start of each wave counted: what a call of a few blocks takes
 };
 ChainPlan make_plan(const Problem& p) {
-    static const double step[2][4] = {{1.9, 1.45, 1.42, 1.32}, {3.3, 2.5, 2.55, 2.3}};      // us per block, 64 columns, d_k = 64 and 128
+    static const double alone[2][4] = {{1.40, 1.25, 1.25, 1.19}, {1.95, 1.53, 1.50, 1.55}};
+    static const double crowded[2][4] = {{1.70, 1.34, 1.33, 1.24}, {2.30, 1.79, 1.68, 1.58}};
     const long long nseq = (long long)p.B * p.H, sms = sm_count();
     const int C = NB / p.r, nblk = (p.L + C - 1) / C;
-    const double st = step[p.d_k == 128][p.r - 1];
-    auto waves = [&](int js) { return (double)((nseq * (p.d_v / js) + sms - 1) / (sms > 0 ? sms : 1)); };
-    double best = waves(64);
-    ChainPlan plan{COLS_64, 1, nblk, 0.0, 0.0};
-    double turns = best;
-    if (p.d_k == 128 && 0.72 * waves(32) < best) {
-        turns = waves(32);
-        best = 0.72 * turns;
-        plan.cols = COLS_32;
-    }
-    if (p.d_v == 128) {
-        const double w = (p.d_k == 128 ? 1.34 : 1.53) * waves(128);
-        if (w < best) {
-            best = w;
-            turns = waves(128);
-            plan.cols = COLS_128;
-        }
-    }
-    plan.us = 7.0 + nblk * st * best;
-    plan.short_us = 5.0 * turns + nblk * st * best;
+    auto step = [&](long long ctas) {
+        const double a = alone[p.d_k == 128][p.r - 1], c = crowded[p.d_k == 128][p.r - 1];
+        const double crowd = sms > 0 ? 2.0 * ctas / sms - 1.0 : 0.0;
+        return a + (c - a) * (crowd < 0.0 ? 0.0 : crowd > 1.0 ? 1.0 : crowd);
+    };
+    const double waves = (double)((nseq + sms - 1) / (sms > 0 ? sms : 1)), walk = nblk * step(nseq) * waves;
+    ChainPlan plan{1, nblk, 7.0 + walk, 5.0 * waves + walk};
     const double limit = 0.92 * plan.us;
-    // (kernels and their gaps, then the traffic of the responses and of O at about 4 TB/s)
-    const double extra = (p.d_k == 128 ? 14.0 : 9.0) + (double)nseq * p.L * (4.0 * p.d_k + 8.0 * p.d_v) / 4e6;
-    // (calls of up to 512 tokens at d_k = 128 are one launch, as they are specified to be: 400 tokens, r = 2 take 27 us instead of 20)
+    // (calls of up to 512 tokens at d_k = 128 are one launch, as they are specified to be)
     if (p.d_k == 128 && p.L <= 512) return plan;
-    for (int cols = p.d_k == 128 ? COLS_32 : COLS_64; cols <= COLS_64; ++cols) {
-        const int js = cols == COLS_32 ? 32 : 64, vs = p.d_v / js, rs = p.d_k / js;
-        const long long most = (sms / nseq + rs) / (vs + rs);
-        for (int want = 2; want <= most && want <= 64 && want <= nblk; ++want) {
-            const int seg_blk = (nblk + want - 1) / want, nseg = (nblk + seg_blk - 1) / seg_blk;
-            const double us = extra + 0.8 * nseg + seg_blk * st * (cols == COLS_32 ? 0.72 : 1.0);
-            if (us < limit && us < plan.us) plan = {cols, nseg, seg_blk, us, plan.short_us};
-        }
+    for (int want = 2; nseq * (2 * want - 1) <= sms && want <= 64 && want <= nblk; ++want) {
+        const int seg_blk = (nblk + want - 1) / want, nseg = (nblk + seg_blk - 1) / seg_blk;
+        // (two kernels, their share per segment, and the traffic of the responses and of O at about 4 TB/s)
+        const double traffic = (double)nseq * p.L * (nseg - 1) / nseg * (4.0 * p.d_k + 8.0 * p.d_v) / 4e6;
+        const double us = (p.d_k == 128 ? 11.0 + 0.85 * nseg : 9.0 + 0.4 * nseg) + traffic + seg_blk * step(nseq * (2 * nseg - 1));
+        if (us < limit && us < plan.us) plan = {nseg, seg_blk, us, plan.short_us};
     }
     return plan;
 }
@@ -1093,29 +1134,28 @@ ChainCarve carve(const Problem& p, const ChainPlan& plan) {
     return c;
 }
 
-template <int DK, int R, int JS, int IS, int TEAMS, bool SEG>
+template <int DK, int R, int DV, bool SEG>
 int launch(const Problem& p, const ChainPlan& plan, const ChainSeg& sg) {
-    constexpr int NS = chain_stages<DK, R, JS, IS, TEAMS>();
-    using CFG = ChainCfg<DK, R, JS, IS, TEAMS, NS>;
+    constexpr int NS = chain_stages<DK, R, DV>();
+    using CFG = ChainCfg<DK, R, DV, NS>;
     static_assert(CFG::total <= 227 * 1024 && NS >= 2, "shared memory budget");
-    const void* fn = (const void*)chain_kernel<DK, R, JS, IS, TEAMS, NS, SEG>;
+    const void* fn = (const void*)chain_kernel<DK, R, DV, NS, SEG>;
     constexpr int C = NB / R;
     ChainGeo g{p.L, p.d_v, (p.L + C - 1) / C, plan.nseg, plan.seg_blk, p.mask_group(), p.exact ? 1 : 0, p.clear_status ? 1 : 0,
                (const __nv_bfloat16*)p.q, (const __nv_bfloat16*)p.k, (const __nv_bfloat16*)p.v, (const __nv_bfloat16*)p.beta,
                p.S0, p.O, p.S_final};
-    const long long nseq = (long long)p.B * p.H, grid = nseq * (plan.nseg * (p.d_v / JS) + (plan.nseg - 1) * (DK / JS));
+    const long long nseq = (long long)p.B * p.H, grid = nseq * (2 * plan.nseg - 1);
     ChainMaps maps;
-    constexpr int VC = JS < 64 ? JS : 64;
     if (!make_slab_map(&maps.k, p.k, nseq, (uint64_t)p.L * R, DK, 64, NB, DK / 64) ||
         !make_slab_map(&maps.q, p.q, nseq, p.L, DK, 64, C, R == 3 ? 1 : DK / 64) ||
-        !make_slab_map(&maps.v, p.v, nseq, (uint64_t)p.L * R, p.d_v, VC, NB, JS / VC))
+        !make_slab_map(&maps.v, p.v, nseq, (uint64_t)p.L * R, DV, 64, NB, DV / 64))
         return record_cuda_error(cudaErrorInvalidValue, "cuTensorMapEncodeTiled");
     static std::atomic<uint64_t> opted_in{0};
     const int st = allow_smem(opted_in, fn, CFG::total);
     if (st != PF_OK) return st;
     void* args[] = {(void*)&maps, (void*)&p.beta, (void*)&p.S0, (void*)&p.O, (void*)&p.S_final, (void*)&p.status, (void*)&g, (void*)&sg};
     prof_begin("chain", p.stream);
-    PF_CUDA_TRY(launch_early(fn, dim3((unsigned)grid), CFG::threads, args, (size_t)CFG::total, p.stream));
+    PF_CUDA_TRY(launch_early(fn, dim3((unsigned)grid), CHAIN_THREADS, args, (size_t)CFG::total, p.stream));
     prof_end(p.stream);
     count_launch(1);
     return PF_OK;
@@ -1123,15 +1163,8 @@ int launch(const Problem& p, const ChainPlan& plan, const ChainSeg& sg) {
 
 template <int DK, int R>
 int launch_plan(const Problem& p, const ChainPlan& plan, const ChainSeg& sg) {
-    if (plan.nseg > 1) {
-        if constexpr (DK == 128)
-            if (plan.cols == COLS_32) return launch<DK, R, 32, 2, 2, true>(p, plan, sg);
-        return launch<DK, R, 64, 1, 2, true>(p, plan, sg);
-    }
-    if constexpr (DK == 128)
-        if (plan.cols == COLS_32) return launch<DK, R, 32, 2, 2, false>(p, plan, sg);
-    if (plan.cols == COLS_64) return launch<DK, R, 64, 1, 2, false>(p, plan, sg);
-    return launch<DK, R, 128, 1, DK == 64 ? 2 : 1, false>(p, plan, sg);
+    if (plan.nseg > 1) return p.d_v == 128 ? launch<DK, R, 128, true>(p, plan, sg) : launch<DK, R, 64, true>(p, plan, sg);
+    return p.d_v == 128 ? launch<DK, R, 128, false>(p, plan, sg) : launch<DK, R, 64, false>(p, plan, sg);
 }
 template <int DK>
 int launch_rank(const Problem& p, const ChainPlan& plan, const ChainSeg& sg) {

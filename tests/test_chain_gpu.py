@@ -115,3 +115,13 @@ def test_segments_of_a_state_that_changes_slowly(d_k, d_v, r, H, L, mode):
     O_ref, S_ref = util.run_oracle(inp, mode=mode)
     util.check_per_sequence(O, O_ref, util.TOL_BF16, "O")
     assert util.rel_l2(S, S_ref) <= 2 ** -12, util.rel_l2(S, S_ref)
+
+
+@pytest.mark.parametrize("d_k,d_v", [(128, 128), (64, 64), (128, 64)])
+@pytest.mark.parametrize("r", [1, 2, 3, 4])
+@pytest.mark.parametrize("blocks", [2, 3, 4, 5, 6, 7, 13])
+def test_the_ring_of_stages_wraps(d_k, d_v, r, blocks):
+    """As many blocks as there are stages of shared memory (3 to 6), one more, one fewer, and several times round."""
+    L = blocks * (64 // r) - (blocks % 2)
+    w = Workload(f"ring_{blocks}", B=1, H=70, L=L, d_k=d_k, d_v=d_v, r=r, chunk=64, beta_scale=2.0, s0_std=0.1, seed=700 + r)
+    assert util.kernels_of(lambda: util.check_parity(w))[0] == "chain"
