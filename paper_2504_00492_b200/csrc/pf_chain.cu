@@ -11,26 +11,30 @@
 //
 // Warps (their registers moved to where they are needed):
 //   chain (8)     fp32 accumulators -> fp16 operands: -S, R, U' in turn, 32 rows j and half of the columns each
-//   products (3)  one warp each for the chain's, the output's (O^T = S Q^T + U'^T P^T) and the Gram products (G = K K^T and K Q^T, 64 rows,
-//                 from the bf16 tiles as they land)
+//   products (3)  one warp each for the chain's, the output's (O^T = S Q^T + U'^T P^T) and the Gram products ([G | P^T] = K [K^T | Q^T], 64
+//                 rows, from the bf16 tiles as they land)
 //   solve (2 x 4) T of every other block: G from tensor memory, the inverse on mma.sync
 //   convert (4)   K, Q -> fp16 in place, P out of tensor memory into shared memory
 //   output (4)    O^T out of tensor memory into the rows of O;  and one warp issues the copies
-// A stage of shared memory holds what the chain needs of one block: K, Q (fp16), T, P (fp16), V (bf16 as it came, added to R's
-// accumulator as V^T times an identity).
+// A stage of shared memory holds what the chain needs of one block: K, Q (fp16, the rows of Q behind those of K), T, P (fp16), V (bf16 as
+// it came, added to R's accumulator as V^T times an identity).
 //
-// What bounds it: the three trips of a block (product, tensor memory to registers and back: 1.6 k cycles when nothing else runs on the
-// SM), drawn out to 2.9 k at d = 128, r = 2 by the other warps' work and, above all, by instruction fetch: the dozen programs together do not
-// fit the instruction cache, and where two neighbouring SMs are busy a miss costs more (3.4 k cycles with 148 CTAs).  So what is not on the
-// chain's path is written small (loops kept rolled, one election per group of products, waits that sleep): 256 sequences of 1024
-// tokens, d = 128, r = 2: 119 us, with the inverse unrolled 146, with waits that poll 220.  Measured (us, before: the same blocks on
+// What bounds it: the three trips of a block (issue 4 to 8 products at 30 cycles each, tensor memory to registers and back), 2.2 k cycles at
+// d = 128 with everything but the chain's own warps switched off, drawn out to 2.6 - 3 k by the others: all products go through one
+// queue, in which those of 64 rows or few columns take as long as large ones (26 - 32 cycles; so G and P^T are one product: 16 products less
+// a block, 133.8 -> 131.3 us at the first size below), and the warps share issue slots (so whoever waits off the chain's path does it at
+// named barriers) and the instruction cache (so what is off the chain's path is written small).  148 CTAs at r = 1 move 5.5 TB/s, 84 % of
+// what a copy reaches.  Measured (us, before: the same blocks on
 // warp-level products, a warp carrying 16 rows j in registers; a shared-memory read of every tile by every such warp): 256 sequences of
-// 1024, d = 128, r = 2: 227 -> 133 (calls one after another); 128 of 4096, d = 64, r = 4: 340 -> 307; 48 of 1999, 64 x 128, r = 3: 146 -> 85 (2 segments);
-// 4 of 16384, d = 128, r = 1: 135 -> 81 (segments); 32 of 2048, d = 128, r = 1: 68 -> 55 (the tcgen05 kernel in one launch before).
+// 1024, d = 128, r = 2: 227 -> 131 (calls one after another); 128 of 4096, d = 64, r = 4: 340 -> 285; 48 of 1999, 64 x 128, r = 3: 146 -> 80 (2 segments);
+// 4 of 16384, d = 128, r = 1: 135 -> 80 (segments); 32 of 2048, d = 128, r = 1: 68 -> 54 (the tcgen05 kernel in one launch before).
 // Measured and not taken: the update's and V - K S^T's products in halves, so that one half is converted while the other is being multiplied (the
 // probe's 1.6 k cycles have it; here 412 us against 389 at 32 sequences of 8192: more instructions); the output's products issued by the chain's
 // warp (462); one election per product instead of per group (427 against 420 then, 179 against 146 with all SMs busy); products in loops on
-// the chain's path too (489).
+// the chain's path too (489).  S K^T and S Q^T as one product (8 products less a block, but the larger one on the chain's path: 131 -> 136 at 256
+// sequences, 290 -> 322 at d = 64, r = 4).  The chain's warps at named barriers too, one warp watching the products' ends for them (293 -> 328).
+// V in one buffer apart from the stages, which makes room for one more (142.6 -> 152.4, 128 sequences of 2048, d = 64, r = 4).  The
+// state before the last block's update in V - K S^T, with U'^T K K^T of the two blocks in its place (172 us at 256 sequences: 20 products more).
 //
 // Range: V - K S^T and U' are packed to fp16 like every other operand, and K S^T reaches sqrt(d_k) times the largest entry of S, so
 // that a state well inside fp16's 65504 can overflow them.  What overflows leaves its row of S infinite or NaN to the end of the walk
@@ -38,7 +42,8 @@
 // its rows are then walked once more, token by token in fp32 (walk_fp32).
 //
 // The inverse: warp w of a team owns rows 16 w .. 16 w + 15 of G, forms A's blocks there and D_w = (I + A_ww)^{-1} by its Neumann product,
-// and after one exchange through shared memory column block w of X: X_ww = D_w, X_iw = -D_i sum_k A_ik X_kw.
+// and after one exchange through shared memory column block w of X: X_ww = D_w, X_iw = -D_i sum_k A_ik X_kw, each X_iw^T left in
+// registers as the operand of the next (through shared memory and in loops: 58.1 us instead of 56.5, 148 sequences of 1024, r = 2).
 #include <float.h>
 
 #include <atomic>
@@ -70,16 +75,23 @@ struct ChainGeo {
     float *O, *S_final;
 };
 
+// four 8 x 8 matrices to shared memory (transposed): lane l has the address of row l % 8 of matrix l / 8
+__device__ __forceinline__ void stmatrix_x4(uint32_t saddr, const uint32_t (&r)[4]) {
+    asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1,%2,%3,%4};" ::"r"(saddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
+}
+__device__ __forceinline__ void stmatrix_x4_trans(uint32_t saddr, const uint32_t (&r)[4]) {
+    asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1,%2,%3,%4};" ::"r"(saddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
+}
 __device__ __forceinline__ uint32_t movmatrix(uint32_t x) {
     uint32_t y;
     asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(y) : "r"(x));
     return y;
 }
-// eight bf16 -> eight fp16 (sign: 0x80008000 to negate them)
-__device__ __forceinline__ uint4 bf16_to_half8(uint4 x, uint32_t sign) {
+// eight bf16 -> eight fp16
+__device__ __forceinline__ uint4 bf16_to_half8(uint4 x) {
     uint32_t* w = (uint32_t*)&x;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) w[i] = pack_h2(__uint_as_float(w[i] << 16), __uint_as_float(w[i] & 0xFFFF0000u)) ^ sign;
+    for (int i = 0; i < 4; ++i) w[i] = pack_h2(__uint_as_float(w[i] << 16), __uint_as_float(w[i] & 0xFFFF0000u));
     return x;
 }
 
@@ -118,7 +130,8 @@ struct ChainSmem {
     static constexpr int CP = (C + 15) / 16 * 16;                 // ... in tiles of 16
     static constexpr int k_bytes = NB * DK * 2, q_bytes = CP * DK * 2;
     static constexpr int t_bytes = NB * 128, p_bytes = CP * 128, v_bytes = NB * JS * 2;
-    static constexpr int k_off = 0, q_off = k_off + k_bytes, t_off = q_off + q_bytes, p_off = t_off + t_bytes, v_off = p_off + p_bytes;
+    // slabs of 64 columns, in each the rows of K and then those of Q: one operand of NB + CP rows
+    static constexpr int rows = NB + CP, k_off = 0, q_off = NB * 128, t_off = k_bytes + q_bytes, p_off = t_off + t_bytes, v_off = p_off + p_bytes;
     static constexpr int stage = v_off + v_bytes;
     static constexpr int tx_bytes = k_bytes + C * DK * 2 + v_bytes;         // what the copies of a block bring
 };
@@ -154,14 +167,15 @@ constexpr int chain_stages() {
     return n < 6 ? n : 6;
 }
 
-// Tensor memory: columns
+// Tensor memory: columns.  All 512 are this CTA's, so that they are these very addresses: constants, where a base read from shared memory
+// would go through a register to each product.
 constexpr uint32_t T_S = 0;          // S, fp32 [j][i]
 constexpr uint32_t T_S16 = 128;      // -S, fp16 pairs
 constexpr uint32_t T_R = 192;        // V^T - S K^T, then U'^T over it, fp32 [j][m]
 constexpr uint32_t T_R16 = 256;      // V^T - S K^T and
 constexpr uint32_t T_U16 = 288;      // U'^T in fp16 pairs
 constexpr uint32_t T_G = 320;        // G, fp32 [m][m'] (16 rows in each quarter of the lanes, as products of 64 rows are laid out)
-constexpr uint32_t T_P = 384;        // P^T before its mask, fp32 [m][t], likewise
+constexpr uint32_t T_P = 384;        // P^T before its mask, fp32 [m][t], likewise: behind T_G, one product
 template <int CP> constexpr int O_BUFS = CP > 32 ? 1 : 2;         // O^T, fp32 [j][t]: of two blocks in turn where there is room
 template <int CP> __device__ __forceinline__ uint32_t o_cols(int b) { return CP > 32 ? 448u : 416u + 32u * (b & 1); }
 
@@ -298,32 +312,47 @@ __device__ __forceinline__ void load_block(const ChainMaps& maps, uint8_t* smem,
     uint8_t* sg = smem + st * SM::stage;
     const int bb = part.b0 + b;
     mbar_expect_tx(&land[st], SM::tx_bytes - (part.response ? SM::v_bytes : 0));
-    tma_load_4d(sg + SM::k_off, &maps.k, 0, bb * SM::C * R, 0, seq, &land[st]);
-    // (r = 3: a block's 21 tokens sit in slabs of 32 rows, one copy each)
-    constexpr int QS = SM::CP == SM::C ? 1 : DK / 64;
 #pragma unroll
-    for (int h = 0; h < QS; ++h) tma_load_4d(sg + SM::q_off + h * (SM::CP * 128), &maps.q, 0, bb * SM::C, h, seq, &land[st]);
+    for (int h = 0; h < DK / 64; ++h) {
+        tma_load_4d(sg + SM::k_off + h * (SM::rows * 128), &maps.k, 0, bb * SM::C * R, h, seq, &land[st]);
+        tma_load_4d(sg + SM::q_off + h * (SM::rows * 128), &maps.q, 0, bb * SM::C, h, seq, &land[st]);
+    }
     if (!part.response) tma_load_4d(sg + SM::v_off, &maps.v, 0, bb * SM::C * R, 0, seq, &land[st]);
 }
 // byte offsets of a lane's row address for ldmatrix.x4 within a slab of 128-byte swizzled rows; the K-step kk of 16 columns
 // is at off ^ (kk << 5), everything else is added
 __device__ __forceinline__ uint32_t lane_off(int row, int half) { return (uint32_t)row * 128u + (uint32_t)((half ^ (row & 7)) << 4); }
 
+// Most warps wait at named barriers, which take no issue slots: of all that watch mbarriers (which has to be done in a loop) for the end of
+// a product there is one warp, the one that issued it, and it passes the news on.  Those that wait at named barriers never give up, so
+// whoever watches an mbarrier takes part in them to the end, also when it has given up (`ok`).
+enum {
+    N_TEAM = 1,     // [2] solve teams
+    N_GD = 5,       // [team] Gram products -> solve: G complete
+    N_GFREE = 7,    // solve -> Gram products: G read
+    N_PD = 8,       // Gram products -> conversion: P^T complete (and nothing reads the block's K and Q as bf16 any more)
+    N_PFREE = 9,    // conversion -> Gram products: P^T read
+    N_OD = 10       // [2] output products -> output: O^T complete
+};
+__device__ __forceinline__ void named_arrive(int id, int nthreads) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(nthreads) : "memory"); }
+// (after a wait for a product's mbarrier, by a whole warp)
+__device__ __forceinline__ void pass_on(int id, int nthreads) {
+    tc_fence_after();
+    tc_fence_before();
+    named_arrive(id, nthreads);
+}
 enum {
     B_SP = 0,       // chain: fp16 copy of S published
     B_RD = 1,       // products: V^T - S K^T complete
-    B_RP = 2,       // chain: its fp16 copy published
-    B_UD = 3,       // products: U' complete
-    B_UP = 4,       // chain: its fp16 copy published
-    B_SD = 5,       // products: S complete
-    B_QD = 6,       // output products: Q S^T complete
-    B_OD = 7,       // [2] output products: O^T complete
-    B_OFREE = 9,    // [2] output: O^T read
-    B_GD = 11,      // [team] Gram products: G complete
-    B_GFREE = 13,   // solve: G read
-    B_PD = 14,      // Gram products: P^T complete (and nothing reads the block's K and Q as bf16 any more)
-    B_PFREE = 15,   // conversion: P^T read
-    B_LAND = 16     // then [NS] each: a block's tiles landed, a block prepared, a block's stage free
+    B_UD = 2,       // products: U' complete
+    B_UP = 3,       // chain: its fp16 copy published
+    B_SD = 4,       // products: S complete
+    B_QD = 5,       // output products: Q S^T complete
+    B_OD = 6,       // [2] output products: O^T complete
+    B_OFREE = 8,    // [2] output: O^T read
+    B_GD = 10,      // Gram products: G and P^T complete
+    B_RP = 11,      // chain: the fp16 copy of R published
+    B_LAND = 12     // then [NS] each: a block's tiles landed, a block prepared, a block's stage free
 };
 
 // Products over several K-steps, descriptors by their low words (a stage's address changes nothing else); whole warp, converged, and one
@@ -331,49 +360,48 @@ enum {
 constexpr uint32_t DESC_HI = (1024u >> 4) | (1u << 14) | (2u << 29);          // SBO 1024 bytes, version, 128-byte swizzle
 __device__ __forceinline__ uint64_t desc_lo(uint32_t lo) { return ((uint64_t)DESC_HI << 32) | lo; }
 __device__ __forceinline__ uint32_t lo_of(uint32_t saddr, uint32_t slab_bytes = 16) { return (saddr >> 4) | (slab_bytes >> 4 << 16); }
-// D [128 x N] (+)= A (tensor memory) B^T: B K-major (MN false) or MN-major, KSTEPS K-steps, slabs of B_ROWS rows
-template <bool MN, int N, int KSTEPS, int B_ROWS>
+// D [128 x N] (+)= A (tensor memory; NEG: -A) B^T: B K-major (MN false) or MN-major, KSTEPS K-steps, slabs of B_ROWS rows
+template <bool MN, int N, int KSTEPS, int B_ROWS, bool NEG = false>
 __device__ __forceinline__ void products_ta(uint32_t d, uint32_t a, uint32_t b_lo, bool acc) {
     if (elect_one())
 #pragma unroll
     for (int kk = 0; kk < KSTEPS; ++kk)
-            mma_f16_ta(d, a + 8 * kk, desc_lo(b_lo + (kstep_off<MN ? L_SWMN : L_SWK, B_ROWS>(kk) >> 4)), make_idesc(N, false, MN, false), acc || kk > 0);
+            mma_f16_ta(d, a + 8 * kk, desc_lo(b_lo + (kstep_off<MN ? L_SWMN : L_SWK, B_ROWS>(kk) >> 4)), make_idesc(N, false, MN, NEG), acc || kk > 0);
 }
 // The same for K = 64 and one slab B [N rows][64 columns], K-major, whose columns from 16 kk on are zero (and need not have been
 // written) in the rows before 16 (kk / GROUP): a K-step leaves those columns of D alone.
 template <int N, int GROUP>
 __device__ __forceinline__ void products_lower(uint32_t d, uint32_t a, uint32_t b_lo, bool acc) {
+    if (elect_one())
 #pragma unroll
     for (int kk = 0; kk < 4; ++kk) {
         const int n0 = 16 * (kk / GROUP);
-        if (n0 < N && elect_one()) mma_f16_ta(d + n0, a + 8 * kk, desc_lo(b_lo + ((n0 * 128 + kk * 32) >> 4)), make_idesc(N - n0, false, false, false), acc || kk > 0);
+        if (n0 < N) mma_f16_ta(d + n0, a + 8 * kk, desc_lo(b_lo + ((n0 * 128 + kk * 32) >> 4)), make_idesc(N - n0, false, false, false), acc || kk > 0);
     }
 }
-// D [64 x N] = A B^T, both K-major bf16 in shared memory
-template <int N, int K, int A_ROWS, int B_ROWS>
-__device__ __forceinline__ void products_ss(uint32_t d, uint32_t a_base, uint32_t b_base) {
+// D [64 x N] = A B^T, B [N rows] K-major bf16 in shared memory, in slabs of ROWS rows, A its first 64 rows
+template <int N, int K, int ROWS>
+__device__ __forceinline__ void products_ss(uint32_t d, uint32_t b_base) {
     constexpr uint32_t idesc = (make_idesc(N, false, false, false) & ~(31u << 24)) | (4u << 24) | (1u << 7) | (1u << 10);     // (64 rows, bf16)
-    const uint32_t a = lo_of(a_base), b = lo_of(b_base);
+    const uint32_t b = lo_of(b_base);
     if (elect_one())
 #pragma unroll
     for (int kk = 0; kk < K / 16; ++kk)
-            mma_f16(d, desc_lo(a + (kstep_off<L_SWK, A_ROWS>(kk) >> 4)), desc_lo(b + (kstep_off<L_SWK, B_ROWS>(kk) >> 4)), idesc, kk > 0);
+            mma_f16(d, desc_lo(b + (kstep_off<L_SWK, ROWS>(kk) >> 4)), desc_lo(b + (kstep_off<L_SWK, ROWS>(kk) >> 4)), idesc, kk > 0);
 }
 
 // ---------------------------------------------------------------------------------------------------------------------
 // solve team: T of blocks b = team, team + TEAMS, ...
 // ---------------------------------------------------------------------------------------------------------------------
 template <int DK, int R, int JS, int NS>
-__device__ __forceinline__ void solve_role(const ChainGeo& g, const ChainPart& part, const __nv_bfloat16* __restrict__ beta, int* err, uint8_t* smem,
-                                           uint64_t* bar, uint64_t* full, uint32_t tb, long long seq, int team, int tid) {
+__device__ __forceinline__ void solve_role(const ChainGeo& g, const ChainPart& part, const __nv_bfloat16* __restrict__ beta, uint8_t* smem,
+                                           uint64_t* full, long long seq, int team, int tid) {
     using CFG = ChainCfg<DK, R, JS, NS>;
     using SM = ChainSmem<DK, R, JS>;
     constexpr int C = SM::C;
     const int w = tid >> 5, lane = tid & 31, gq = lane >> 2, t4 = lane & 3;
     const int L = g.L;
-    const int bar_id = 1 + team;
-    uint8_t* xs = smem + CFG::xs_off + team * NB * 128;
-    const uint32_t xs_b = smem_u32(xs);
+    const uint32_t xs_b = smem_u32(smem) + CFG::xs_off + team * NB * 128, xs_w = xs_b + w * 2048;
     const uint32_t offA = lane_off(lane & 15, lane >> 4), offN = lane_off((lane & 7) + ((lane >> 4) << 3), (lane >> 3) & 1);
     const __nv_bfloat16* bs = beta + seq * L * R;
     // (the bits as loaded: a conversion next to the load would make every thread wait for it there, a block ahead of its use)
@@ -388,16 +416,14 @@ __device__ __forceinline__ void solve_role(const ChainGeo& g, const ChainPart& p
 #pragma unroll 1
     for (int b = team; b < part.nblk; b += TEAMS) {
         const int st = b % NS;
-        uint8_t* sg = smem + st * SM::stage;
+        const uint32_t t_b = smem_u32(smem) + st * SM::stage + SM::t_off;
         // (two in turn: another warp may still be scaling T of the block before)
         float* sBeta = (float*)(smem + CFG::beta_off + team * 512 + (b / TEAMS & 1) * 256);
         if (tid < NB) sBeta[tid] = __uint_as_float((uint32_t)breg << 16);
         if (b + TEAMS < part.nblk) breg = read_beta(b + TEAMS);
-        // (a failed wait must not strand the others at a barrier: the next one carries the outcome)
-        const bool ok = wait_inline<true>(&bar[B_GD + team], (uint32_t)(b / TEAMS) & 1, err, 311);
+        named_bar(N_GD + team, 160);                              // (and the step sizes)
         tc_fence_after();
-        if (!named_bar_and(bar_id, 128, ok)) return;              // (step sizes)
-        const uint32_t t_g = tb + T_G + ((uint32_t)(32 * w) << 16);
+        const uint32_t t_g = T_G + ((uint32_t)(32 * w) << 16);
         uint32_t x[8];                                            // 16 columns of G, rows 16 w .. 16 w + 15, as mma.sync's accumulators
         const int m0 = 16 * w + gq, m1 = m0 + 8;
         if (g.exact) {
@@ -414,14 +440,6 @@ __device__ __forceinline__ void solve_role(const ChainGeo& g, const ChainPart& p
         }
         // ---- A = Mstrict (.) (diag(beta) G): its blocks left of the diagonal go to the other warps, the diagonal one stays as an A operand
         const float b0 = sBeta[m0], b1 = sBeta[m1];
-        auto put = [&](int j, const uint32_t (&f)[4]) {           // (f: packed accumulator fragment)
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                uint8_t* at = xs + m0 * 128 + 4 * t4 + (((2 * j + h) ^ gq) << 4);
-                *(uint32_t*)at = f[2 * h];
-                *(uint32_t*)(at + 8 * 128) = f[2 * h + 1];
-            }
-        };
         uint32_t af[4];
 #pragma unroll 1
         for (int nb = 0;; ++nb) {
@@ -433,16 +451,23 @@ __device__ __forceinline__ void solve_role(const ChainGeo& g, const ChainPart& p
             for (int h = 0; h < 2; ++h)
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
-                    v[h][e] = c0 + 8 * h + e < lim0 ? b0 * __uint_as_float(x[4 * h + e]) : 0.f;
-                    v[h][2 + e] = c0 + 8 * h + e < lim1 ? b1 * __uint_as_float(x[4 * h + 2 + e]) : 0.f;
+                    v[h][e] = b0 * __uint_as_float(x[4 * h + e]);
+                    v[h][2 + e] = b1 * __uint_as_float(x[4 * h + 2 + e]);
                 }
+            if (nb == w || R == 3)                                // (groups of three rows reach across the edge of a tile)
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        if (c0 + 8 * h + e >= lim0) v[h][e] = 0.f;
+                        if (c0 + 8 * h + e >= lim1) v[h][2 + e] = 0.f;
+                    }
             frag_pack(af, v);
             if (nb == w) break;
-            put(nb, af);
+            stmatrix_x4(xs_w + (offA ^ (uint32_t)(nb << 5)), af);
         }
         tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&bar[B_GFREE]);
+        if (b + 1 < part.nblk) named_arrive(N_GFREE, 160);
         // ---- D_w = (I + A_ww)^{-1} (Neumann product, A nilpotent) for the other warps
         uint32_t y0[4];                                           // X_ww^T as an A operand
         {
@@ -451,84 +476,82 @@ __device__ __forceinline__ void solve_role(const ChainGeo& g, const ChainPart& p
             at[0] = movmatrix(af[0]); at[1] = movmatrix(af[2]); at[2] = movmatrix(af[1]); at[3] = movmatrix(af[3]);
             neumann16(dd, af, at, lane, g.rm == 1);
             frag_pack(df, dd);
-            put(w, df);
+            stmatrix_x4(xs_w + (offA ^ (uint32_t)(w << 5)), df);
             y0[0] = movmatrix(df[0]); y0[1] = movmatrix(df[2]); y0[2] = movmatrix(df[1]); y0[3] = movmatrix(df[3]);
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const float2 bb = *(const float2*)(sBeta + 16 * w + 8 * h + 2 * t4);
-                uint8_t* at_ = sg + SM::t_off + m0 * 128 + 4 * t4 + (((2 * w + h) ^ gq) << 4);
-                *(uint32_t*)at_ = pack_h2(dd[h][0] * bb.x, dd[h][1] * bb.y);
-                *(uint32_t*)(at_ + 8 * 128) = pack_h2(dd[h][2] * bb.x, dd[h][3] * bb.y);
+                dd[h][0] *= bb.x; dd[h][1] *= bb.y; dd[h][2] *= bb.x; dd[h][3] *= bb.y;
             }
+            frag_pack(df, dd);
+            stmatrix_x4(t_b + w * 2048 + (offA ^ (uint32_t)(w << 5)), df);
         }
-        named_bar(bar_id, 128);
-        // ---- down the column: X_iw = -D_i sum_k A_ik X_kw, transposed; T = X diag(beta).  X_iw^T goes above the diagonal, where A has
-        //      nothing
-#pragma unroll 1
-        for (int i = w + 1; i < 4; ++i) {
+        named_bar(N_TEAM + team, 128);
+        // ---- down the column: X_iw = -D_i sum_k A_ik X_kw, transposed, in registers; T = X diag(beta)
+        uint32_t y[3][4];                                         // X_kw^T of k = w, w + 1, w + 2
+#pragma unroll
+        for (int e = 0; e < 4; ++e) y[0][e] = y0[e];
+#pragma unroll
+        for (int n = 1; n < 4; ++n) {
+            const int i = w + n;
+            if (i > 3) break;
             float c[2][4], z[2][4];
-            uint32_t f[4], y[4], a[4];
-            ldmatrix_x4(a, xs_b + (offN ^ (uint32_t)(w << 5)) + i * 2048);
-            mma_acc(c[0], y0, a[0], a[1], false);
-            mma_acc(c[1], y0, a[2], a[3], false);
-#pragma unroll 1
-            for (int k = w + 1; k < i; ++k) {
-                ldmatrix_x4(y, xs_b + (offA ^ (uint32_t)(k << 5)) + w * 2048);
-                ldmatrix_x4(a, xs_b + (offN ^ (uint32_t)(k << 5)) + i * 2048);
-                mma_16816(c[0], y, a[0], a[1]);
-                mma_16816(c[1], y, a[2], a[3]);
+            uint32_t f[4], a[4];
+#pragma unroll
+            for (int k = 0; k < n; ++k) {
+                ldmatrix_x4(a, xs_b + (offN ^ (uint32_t)((w + k) << 5)) + i * 2048);
+                mma_acc(c[0], y[k], a[0], a[1], k > 0);
+                mma_acc(c[1], y[k], a[2], a[3], k > 0);
             }
-            frag_pack(f, c);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) f[e] = pack_h2(-c[e / 2][e % 2 * 2], -c[e / 2][e % 2 * 2 + 1]);
             ldmatrix_x4(a, xs_b + (offN ^ (uint32_t)(i << 5)) + i * 2048);
             mma_acc(z[0], f, a[0], a[1], false);
             mma_acc(z[1], f, a[2], a[3], false);
+            if (n < 3) frag_pack(y[n < 3 ? n : 0], z);
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-#pragma unroll
-                for (int e = 0; e < 4; ++e) z[h][e] = -z[h][e];
-                uint8_t* row = sg + SM::t_off + (16 * i + 8 * h + gq) * 128 + 4 * t4;
-                *(uint32_t*)(row + (((2 * w) ^ gq) << 4)) = movmatrix(pack_h2(z[h][0] * b0, z[h][1] * b0));
-                *(uint32_t*)(row + (((2 * w + 1) ^ gq) << 4)) = movmatrix(pack_h2(z[h][2] * b1, z[h][3] * b1));
-                uint8_t* at = xs + m0 * 128 + 4 * t4 + (((2 * i + h) ^ gq) << 4);
-                *(uint32_t*)at = pack_h2(z[h][0], z[h][1]);
-                *(uint32_t*)(at + 8 * 128) = pack_h2(z[h][2], z[h][3]);
-            }
-            __syncwarp();
+            for (int e = 0; e < 4; ++e) f[e] = pack_h2(z[e / 2][e % 2 * 2] * (e % 2 ? b1 : b0), z[e / 2][e % 2 * 2 + 1] * (e % 2 ? b1 : b0));
+            stmatrix_x4_trans(t_b + i * 2048 + (offN ^ (uint32_t)(w << 5)), f);
         }
         fence_async_smem();
         mbar_arrive(&full[st]);
     }
 }
 
-// Conversion: K and Q of every block to fp16 in place, once the Gram products have read them as they came (Q as -Q: the chain
-// multiplies it with -S), and P.  Four warps.
+// Conversion: K and Q of every block to fp16 in place, once the Gram products have read them as they came, and P.  Four warps.
 template <int DK, int R, int JS, int NS>
-__device__ __forceinline__ void convert_role(const ChainPart& part, int* err, uint8_t* smem, uint64_t* bar, uint64_t* full, uint32_t tb, int tid) {
+__device__ __forceinline__ void convert_role(const ChainPart& part, uint8_t* smem, uint64_t* full, int tid) {
     using SM = ChainSmem<DK, R, JS>;
     constexpr int CP = SM::CP;
     const int w = tid >> 5, lane = tid & 31, gq = lane >> 2, t4 = lane & 3;
+    const uint32_t p_at = smem_u32(smem) + SM::p_off + (lane_off((lane & 7) + ((lane >> 4) << 3), (lane >> 3) & 1) ^ (uint32_t)(w << 5));
 #pragma unroll 1
     for (int b = 0; b < part.nblk; ++b) {
-        uint8_t* sg = smem + (b % NS) * SM::stage;
-        if (!wait_inline<true>(&bar[B_PD], b & 1, err, 315)) return;
+        const int st = b % NS;
+        uint8_t* sg = smem + st * SM::stage;
+        named_bar(N_PD, 160);
         tc_fence_after();
         // ---- P^T rows m = 16 w .. 16 w + 15, columns t; P = its transpose (.) Mincl: row m is seen by tokens t with m < (t + 1) R
-        uint32_t x[CP / 2];
-        tmem_ld_frag<CP>(tb + T_P + ((uint32_t)(32 * w) << 16), x);
-        tmem_ld_wait();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&bar[B_PFREE]);
+        constexpr int PC = CP < 32 ? CP : 32;                     // (columns at a time)
+#pragma unroll 1
+        for (int t0 = 0; t0 < CP; t0 += PC) {
+            uint32_t x[PC / 2];
+            tmem_ld_frag<PC>(T_P + t0 + ((uint32_t)(32 * w) << 16), x);
+            tmem_ld_wait();
+            if (t0 + PC == CP) {
+                tc_fence_before();
+                if (b + 1 < part.nblk) named_arrive(N_PFREE, 160);
+            }
 #pragma unroll
-        for (int n = 0; n < CP / 8; ++n) {
-            if (CP >= 16 && 16 * w >= (n / 2 * 16 + 16) * R) continue;       // (nothing of the block of 16 tokens sees these rows)
-            const int t = 8 * n + 2 * t4;
+            for (int n = 0; n < PC / 8; n += 2) {
+                if (16 * w >= (t0 + 8 * n + 16) * R) continue;    // (nothing of the block of 16 tokens sees these rows)
+                uint32_t y[4];
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int m = 16 * w + 8 * h + gq;
-                const uint32_t y = movmatrix(pack_h2(m < (t + 1) * R ? __uint_as_float(x[4 * n + 2 * h]) : 0.f,
-                                                     m < (t + 2) * R ? __uint_as_float(x[4 * n + 2 * h + 1]) : 0.f));
-                *(uint32_t*)(sg + SM::p_off + chunk_off(8 * n + gq, 2 * w + h, CP) + 4 * t4) = y;
+                for (int e = 0; e < 4; ++e) {
+                    const int t = t0 + 8 * (n + e / 2) + 2 * t4, m = 16 * w + 8 * (e % 2) + gq, at = 4 * n + 2 * e;
+                    y[e] = pack_h2(m < (t + 1) * R ? __uint_as_float(x[at]) : 0.f, m < (t + 2) * R ? __uint_as_float(x[at + 1]) : 0.f);
+                }
+                stmatrix_x4_trans(p_at + st * SM::stage + t0 * 128 + n * 1024, y);
             }
         }
         // ---- bf16 -> fp16 (elementwise, so the swizzled layout is untouched), several pieces per round, so that their loads are in flight together
@@ -541,30 +564,34 @@ __device__ __forceinline__ void convert_role(const ChainPart& part, int* err, ui
 #pragma unroll
             for (int e = 0; e < ROUND; ++e) y[e] = p[(e0 + e) * 128];
 #pragma unroll
-            for (int e = 0; e < ROUND; ++e) p[(e0 + e) * 128] = bf16_to_half8(y[e], (e0 + e) * 2048 < SM::k_bytes ? 0u : 0x80008000u);
+            for (int e = 0; e < ROUND; ++e) p[(e0 + e) * 128] = bf16_to_half8(y[e]);
         }
         fence_async_smem();
-        mbar_arrive(&full[b % NS]);
+        mbar_arrive(&full[st]);
     }
 }
 
-// Gram products (one warp): G = K K^T and K Q^T from the bf16 tiles as they landed, in products of 64 rows.
+// Gram products (one warp): G = K K^T and K Q^T from the bf16 tiles as they landed, in products of 64 rows and NB + CP columns.
 template <int DK, int R, int JS, int NS>
-__device__ __forceinline__ void gram_role(const ChainPart& part, int* err, uint8_t* smem, uint64_t* bar, uint64_t* land, uint32_t tb) {
+__device__ __forceinline__ void gram_role(const ChainPart& part, int* err, uint8_t* smem, uint64_t* bar, uint64_t* land) {
     using SM = ChainSmem<DK, R, JS>;
     int st = 0, phase = 0;
+    bool ok = true;
 #pragma unroll 1
     for (int b = 0; b < part.nblk; ++b) {
-        const uint32_t k_b = smem_u32(smem + st * SM::stage + SM::k_off), q_b = k_b + SM::q_off - SM::k_off;
-        if (!wait_inline<true>(&land[st], phase, err, 316)) return;
-        if (b > 0 && !wait_inline<true>(&bar[B_GFREE], (b - 1) & 1, err, 317)) return;
+        ok = ok && wait_inline<true>(&land[st], phase, err, 316);
+        if (b > 0) {
+            named_bar(N_GFREE, 160);
+            named_bar(N_PFREE, 160);
+        }
         tc_fence_after();
-        products_ss<NB, DK, NB, NB>(tb + T_G, k_b, k_b);
-        commit_uni(&bar[B_GD + b % TEAMS]);
-        if (b > 0 && !wait_inline<true>(&bar[B_PFREE], (b - 1) & 1, err, 318)) return;
-        tc_fence_after();
-        products_ss<SM::CP, DK, NB, SM::CP>(tb + T_P, k_b, q_b);
-        commit_uni(&bar[B_PD]);
+        if (ok) {
+            products_ss<SM::rows, DK, SM::rows>(T_G, smem_u32(smem + st * SM::stage));
+            commit_uni(&bar[B_GD]);
+        }
+        ok = ok && wait_inline<true>(&bar[B_GD], b & 1, err, 311);
+        pass_on(N_GD + b % TEAMS, 160);
+        named_arrive(N_PD, 160);
         if (++st == NS) {
             st = 0;
             phase ^= 1;
@@ -596,11 +623,11 @@ __device__ __forceinline__ void to_operand(uint32_t src, uint32_t dst) {
 
 // warp `warp` of eight: rows j = 32 (warp & 3) + lane, half warp >> 2 of the columns of everything
 template <int DK>
-__device__ __forceinline__ void chain_role(const ChainPart& part, int* err, uint64_t* bar, uint32_t tb, int warp, int lane) {
+__device__ __forceinline__ void chain_role(const ChainPart& part, int* err, uint64_t* bar, int warp, int lane) {
     constexpr int HC = DK / 2;                                    // columns i of this warp
     const int h = warp >> 2, j = 32 * (warp & 3) + lane;
     const uint32_t lanes = (uint32_t)(32 * (warp & 3)) << 16;
-    const uint32_t t_s = tb + T_S + h * HC + lanes, t_s16 = tb + T_S16 + h * HC / 2 + lanes, t_u16 = tb + T_U16 + 16 * h + lanes;
+    const uint32_t t_s = T_S + h * HC + lanes, t_s16 = T_S16 + h * HC / 2 + lanes, t_u16 = T_U16 + 16 * h + lanes;
 #pragma unroll 1
     for (int c = 0; c < HC; c += 16) {
         uint32_t x[16], y[8];
@@ -618,7 +645,7 @@ __device__ __forceinline__ void chain_role(const ChainPart& part, int* err, uint
         __syncwarp();
         if (lane == 0) mbar_arrive(&bar[b]);
     };
-    const uint32_t t_r = tb + T_R + 32 * h + lanes, t_r16 = tb + T_R16 + 16 * h + lanes;
+    const uint32_t t_r = T_R + 32 * h + lanes, t_r16 = T_R16 + 16 * h + lanes;
 #pragma unroll 1
     for (int b = 0; b < part.nblk; ++b) {
         publish(B_SP);
@@ -639,22 +666,23 @@ __device__ __forceinline__ void chain_role(const ChainPart& part, int* err, uint
 
 // The products of the chain (one warp).
 template <int DK, int R, int DV, int NS>
-__device__ __forceinline__ void mma_role(const ChainPart& part, int* err, uint8_t* smem, uint64_t* bar, uint32_t tb) {
+__device__ __forceinline__ void mma_role(const ChainPart& part, int* err, uint8_t* smem, uint64_t* bar) {
     using CFG = ChainCfg<DK, R, DV, NS>;
     using SM = ChainSmem<DK, R, DV>;
-    constexpr int K_SLAB = NB * 128, OB = O_BUFS<SM::CP>;
+    constexpr int V_SLAB = NB * 128, K_SLAB = SM::rows * 128, OB = O_BUFS<SM::CP>;
     uint64_t *land = bar + B_LAND, *full = land + NS, *empty = full + NS;
     const uint32_t smem_b = smem_u32(smem), i16_b = smem_b + CFG::i16_off;
-    const uint32_t t_r = tb + T_R;
+    const uint32_t t_r = T_R;
     // V^T of a block into the accumulator: 16 columns m at a time, as V^T times a 16 x 16 identity, both bf16 (V as it came).  At
     // d_v = 64 the tile's 64 columns are read twice: rows j past d_v are nobody's.
     auto put_v = [&](int st) {
-        const uint32_t v_lo = lo_of(smem_b + st * SM::stage + SM::v_off, DV == 128 ? K_SLAB : 0);
+        const uint32_t v_lo = lo_of(smem_b + st * SM::stage + SM::v_off, DV == 128 ? V_SLAB : 0);
         const uint64_t i16 = desc_ns_kmajor(i16_b, 16);
         constexpr uint32_t idesc = make_idesc(16, true, false, false) | (1u << 7) | (1u << 10);
+        if (elect_one())
 #pragma unroll
         for (int c = 0; c < 4; ++c)
-            if (elect_one()) mma_f16(t_r + 16 * c, desc_lo(v_lo + c * (2048 >> 4)), i16, idesc, false);
+            mma_f16(t_r + 16 * c, desc_lo(v_lo + c * (2048 >> 4)), i16, idesc, false);
     };
     int st = 0, phase = 0;
 #pragma unroll 1
@@ -669,20 +697,20 @@ __device__ __forceinline__ void mma_role(const ChainPart& part, int* err, uint8_
         if (!wait_inline<false>(&full[st], phase, err, 322) || !wait_inline<false>(&bar[B_SP], b & 1, err, 323)) return;
         tc_fence_after();
         // ---- R = V^T - S K^T
-        products_ta<false, NB, DK / 16, NB>(t_r, tb + T_S16, k_lo, !part.response);
+        products_ta<false, NB, DK / 16, SM::rows>(t_r, T_S16, k_lo, !part.response);
         commit_uni(&bar[B_RD]);
         // ---- U'^T = R T^T (T lower triangular: rows m' = 16 kk .. of the contraction reach columns m >= 16 kk only)
         // (U' completes only after the last reader of the block before's, P U', so that the chain warps need not wait for that)
         if (b > 0 && !wait_inline<false>(&bar[B_OD + (b - 1) % OB], ((b - 1) / OB) & 1, err, 319)) return;
         if (!wait_inline<false>(&bar[B_RP], b & 1, err, 326)) return;
         tc_fence_after();
-        products_lower<NB, 1>(t_r, tb + T_R16, t_lo, false);
+        products_lower<NB, 1>(t_r, T_R16, t_lo, false);
         commit_uni(&bar[B_UD]);
         // ---- S += U'^T K
         // (and S only after Q S^T)
         if (!wait_inline<false>(&bar[B_QD], b & 1, err, 320) || !wait_inline<false>(&bar[B_UP], b & 1, err, 328)) return;
         tc_fence_after();
-        products_ta<true, DK, NB / 16, NB>(tb + T_S, tb + T_U16, kt_lo, true);
+        products_ta<true, DK, NB / 16, SM::rows>(T_S, T_U16, kt_lo, true);
         commit_uni(&bar[B_SD]);
         commit_uni(&empty[st]);
         if (++st == NS) {
@@ -694,26 +722,36 @@ __device__ __forceinline__ void mma_role(const ChainPart& part, int* err, uint8_
 
 // The products of the output (one warp): O^T = S Q^T + U'^T P^T with the state before the update.
 template <int DK, int R, int DV, int NS>
-__device__ __forceinline__ void mma_out_role(const ChainPart& part, int* err, uint8_t* smem, uint64_t* bar, uint32_t tb) {
+__device__ __forceinline__ void mma_out_role(const ChainPart& part, int* err, uint8_t* smem, uint64_t* bar) {
     using SM = ChainSmem<DK, R, DV>;
     constexpr int CP = SM::CP, OB = O_BUFS<CP>;
     uint64_t *full = bar + B_LAND + NS, *empty = full + NS;
     const uint32_t smem_b = smem_u32(smem);
+    const int parties = part.width + 32;
     int st = 0, phase = 0;
+    bool ok = true;
 #pragma unroll 1
     for (int b = 0; b < part.nblk; ++b) {
-        const uint32_t sg = smem_b + st * SM::stage, t_o = tb + o_cols<CP>(b);
-        if (!wait_inline<true>(&full[st], phase, err, 351) || !wait_inline<true>(&bar[B_SP], b & 1, err, 352)) return;
-        if (b >= OB && !wait_inline<true>(&bar[B_OFREE + b % OB], (b / OB - 1) & 1, err, 325)) return;
+        const uint32_t sg = smem_b + st * SM::stage, t_o = o_cols<CP>(b);
+        ok = ok && wait_inline<true>(&full[st], phase, err, 351) && wait_inline<true>(&bar[B_SP], b & 1, err, 352);
+        if (b >= OB) ok = ok && wait_inline<true>(&bar[B_OFREE + b % OB], (b / OB - 1) & 1, err, 325);
         tc_fence_after();
-        products_ta<false, CP, DK / 16, CP>(t_o, tb + T_S16, lo_of(sg + SM::q_off), false);
-        commit_uni(&bar[B_QD]);
-        if (!wait_inline<true>(&bar[B_UP], b & 1, err, 354)) return;
+        if (ok) {
+            products_ta<false, CP, DK / 16, SM::rows, true>(t_o, T_S16, lo_of(sg + SM::q_off), false);
+            commit_uni(&bar[B_QD]);
+        }
+        ok = ok && wait_inline<true>(&bar[B_UP], b & 1, err, 354);
         tc_fence_after();
-        // (rows 16 kk .. of the contraction are seen from tile kk / R of 16 tokens on)
-        products_lower<CP, R>(t_o, tb + T_U16, lo_of(sg + SM::p_off), true);
-        commit_uni(&bar[B_OD + b % OB]);
-        commit_uni(&empty[st]);
+        if (ok) {
+            // (rows 16 kk .. of the contraction are seen from tile kk / R of 16 tokens on)
+            products_lower<CP, R>(t_o, T_U16, lo_of(sg + SM::p_off), true);
+            commit_uni(&bar[B_OD + b % OB]);
+            commit_uni(&empty[st]);
+        }
+        ok = ok && wait_inline<true>(&bar[B_OD + b % OB], (b / OB) & 1, err, 331);
+        // (also when it has given up: the output's warps must have passed this barrier before it is arrived at again)
+        if (b >= OB) ok = wait_inline<true>(&bar[B_OFREE + b % OB], (b / OB - 1) & 1, err, 332) && ok;
+        pass_on(N_OD + b % OB, parties);
         if (++st == NS) {
             st = 0;
             phase ^= 1;
@@ -724,21 +762,21 @@ __device__ __forceinline__ void mma_out_role(const ChainPart& part, int* err, ui
 // O of each block from tensor memory to global memory: warp `warp` of four has rows j = 32 warp + lane, and one store of a warp is
 // 128 contiguous bytes of a token's row (64 of a response's).
 template <int C, int CP, int DK, int DV>
-__device__ __forceinline__ void out_role(const ChainGeo& g, const ChainPart& part, int* err, uint64_t* bar, uint32_t tb, int warp, int lane) {
+__device__ __forceinline__ void out_role(const ChainGeo& g, const ChainPart& part, uint64_t* bar, int warp, int lane) {
     constexpr int OB = O_BUFS<CP>;
-    const int j = 32 * warp + lane;
+    const int j = 32 * warp + lane, parties = part.width + 32;
     const uint32_t lanes = (uint32_t)(32 * warp) << 16;
     float* o = part.O + j;
     __half* oh = (__half*)part.O + j;
 #pragma unroll 1
     for (int b = 0; b < part.nblk; ++b) {
-        if (!wait_inline<true>(&bar[B_OD + b % OB], (b / OB) & 1, err, 331)) return;
+        named_bar(N_OD + b % OB, parties);
         tc_fence_after();
         const int Cv = min(C, g.L - (part.b0 + b) * C);
 #pragma unroll 1
         for (int c = 0; c < CP; c += 16) {
             uint32_t x[16];
-            tmem_ld16(tb + o_cols<CP>(b) + lanes + c, x);
+            tmem_ld16(o_cols<CP>(b) + lanes + c, x);
             tmem_ld_wait();
             if (c + 16 == CP) {
                 tc_fence_before();
@@ -765,10 +803,10 @@ __device__ __forceinline__ void out_role(const ChainGeo& g, const ChainPart& par
 
 // The end state, once every role is done.
 template <int DK, int R, bool SEG>
-__device__ __forceinline__ void end_state(const ChainPart& part, const ChainArgs& args, long long seq, uint32_t tb, int warp, int lane) {
+__device__ __forceinline__ void end_state(const ChainPart& part, const ChainArgs& args, long long seq, int warp, int lane) {
     constexpr int HC = DK / 2;
     const int h = warp >> 2, quarter = warp & 3, j = 32 * quarter + lane;
-    const uint32_t t_s = tb + T_S + h * HC + ((uint32_t)(32 * quarter) << 16);
+    const uint32_t t_s = T_S + h * HC + ((uint32_t)(32 * quarter) << 16);
     if (part.response) {
         __half* P = (__half*)part.S_end + (long long)j * DK + h * HC;
 #pragma unroll 1
@@ -837,13 +875,10 @@ chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __rest
         mbar_init(&bar[B_SD], 1);
         mbar_init(&bar[B_UD], 1);
         mbar_init(&bar[B_QD], 1);
-        mbar_init(&bar[B_PD], 1);
-        mbar_init(&bar[B_GFREE], 4);
-        mbar_init(&bar[B_PFREE], 4);
+        mbar_init(&bar[B_GD], 1);
         for (int x = 0; x < 2; ++x) {
             mbar_init(&bar[B_OD + x], 1);
             mbar_init(&bar[B_OFREE + x], quarters);
-            mbar_init(&bar[B_GD + x], 1);
         }
         for (int x = 0; x < NS; ++x) {
             mbar_init(&land[x], 1);
@@ -866,7 +901,11 @@ chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __rest
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tb = tmem_base;
+    if (tmem_base != 0) {                                         // (whoever holds all columns holds them from column 0 on)
+        if (tid == 0) atomicCAS(status, 0, 98);
+        if (warp == W_MMA) tmem_dealloc(tmem_base, 512);
+        return;
+    }
     // (each warpgroup sets its registers once, and no code is shared after that: its end is in its own branch)
     auto all_done = [&]() {
         __syncwarp();
@@ -877,33 +916,33 @@ chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __rest
     if (warp < W_OUT) {
         set_registers<REGS_CHAIN>();
         const bool holds_state = (warp & 3) < quarters;
-        if (holds_state) chain_role<DK>(part, status, bar, tb, warp, lane);
+        if (holds_state) chain_role<DK>(part, status, bar, warp, lane);
         all_done();                                               // (every output is written, all products are complete)
-        if (holds_state) end_state<DK, R, SEG>(part, args, seq, tb, warp, lane);
+        if (holds_state) end_state<DK, R, SEG>(part, args, seq, warp, lane);
         all_done();
     } else if (warp < W_CONV) {
         set_registers<REGS_OUT>();
-        if (warp - W_OUT < quarters) out_role<SM::C, SM::CP, DK, DV>(g, part, status, bar, tb, warp - W_OUT, lane);
+        if (warp - W_OUT < quarters) out_role<SM::C, SM::CP, DK, DV>(g, part, bar, warp - W_OUT, lane);
         all_done();
         all_done();
     } else if (warp < W_SOLVE) {
         set_registers<REGS_CONV>();
-        convert_role<DK, R, DV, NS>(part, status, smem, bar, full, tb, tid - 32 * W_CONV);
+        convert_role<DK, R, DV, NS>(part, smem, full, tid - 32 * W_CONV);
         all_done();
         all_done();
     } else if (warp < W_MMA) {
         set_registers<REGS_SOLVE>();
-        solve_role<DK, R, DV, NS>(g, part, beta, status, smem, bar, full, tb, seq, (warp - W_SOLVE) >> 2, (tid - 32 * W_SOLVE) & 127);
+        solve_role<DK, R, DV, NS>(g, part, beta, smem, full, seq, (warp - W_SOLVE) >> 2, (tid - 32 * W_SOLVE) & 127);
         all_done();
         all_done();
     } else {
         set_registers<REGS_ISSUE>();
         if (warp == W_MMA) {
-            mma_role<DK, R, DV, NS>(part, status, smem, bar, tb);
+            mma_role<DK, R, DV, NS>(part, status, smem, bar);
         } else if (warp == W_MMA_OUT) {
-            mma_out_role<DK, R, DV, NS>(part, status, smem, bar, tb);
+            mma_out_role<DK, R, DV, NS>(part, status, smem, bar);
         } else if (warp == W_GRAM) {
-            gram_role<DK, R, DV, NS>(part, status, smem, bar, land, tb);
+            gram_role<DK, R, DV, NS>(part, status, smem, bar, land);
         } else if (warp == W_LOAD) {
             bool ok = true;
 #pragma unroll 1
@@ -914,7 +953,7 @@ chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __rest
         }
         all_done();
         all_done();
-        if (warp == W_MMA) tmem_dealloc(tb, 512);
+        if (warp == W_MMA) tmem_dealloc(0, 512);
     }
 }
 
@@ -1146,8 +1185,8 @@ int launch(const Problem& p, const ChainPlan& plan, const ChainSeg& sg) {
                p.S0, p.O, p.S_final};
     const long long nseq = (long long)p.B * p.H, grid = nseq * (2 * plan.nseg - 1);
     ChainMaps maps;
-    if (!make_slab_map(&maps.k, p.k, nseq, (uint64_t)p.L * R, DK, 64, NB, DK / 64) ||
-        !make_slab_map(&maps.q, p.q, nseq, p.L, DK, 64, C, R == 3 ? 1 : DK / 64) ||
+    if (!make_slab_map(&maps.k, p.k, nseq, (uint64_t)p.L * R, DK, 64, NB, 1) ||
+        !make_slab_map(&maps.q, p.q, nseq, p.L, DK, 64, C, 1) ||
         !make_slab_map(&maps.v, p.v, nseq, (uint64_t)p.L * R, DV, 64, NB, DV / 64))
         return record_cuda_error(cudaErrorInvalidValue, "cuTensorMapEncodeTiled");
     static std::atomic<uint64_t> opted_in{0};
