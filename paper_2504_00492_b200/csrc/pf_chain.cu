@@ -959,46 +959,59 @@ chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __rest
 
 // Start states of the segments: one CTA per sequence and 16 rows j, serial over the segments; four warps with a quarter of the
 // columns i each.  start(1) = Xi_0, start(s+1) = start(s) P_s + Xi_s; the last one is S_final.  The diagonal's part of the product is
-// fp32, the rest has fp16 operands.  The next P and Xi come while the present ones are used.
+// fp32, the rest has fp16 operands.  What bounds it is the latency of a step, so P, Xi and the diagonal come through a ring of up to
+// three steps (4 sequences of 16384, r = 1, the call: 77.9 us; one step ahead, Xi and the diagonal in registers: 80.2).
+constexpr int COMPOSE_RING = 3;
+template <int DK>
+struct ComposeSmem {
+    static constexpr int LD = DK + 8, LX = 20;                    // (row pitches without bank conflicts)
+    static constexpr int p_bytes = DK * LD * 2, x_bytes = DK * LX * 4, stage = p_bytes + x_bytes + DK * 4, a_bytes = 2 * 16 * LD * 2;
+};
 template <int DK>
 __global__ void __launch_bounds__(128) chain_compose(ChainSeg sg, float* __restrict__ S_final, int nseg, int d_v) {
-    constexpr int LD = DK + 8, NT = DK / 32, PIECES = DK * DK / 8 / 128;
+    using SM = ComposeSmem<DK>;
+    constexpr int LD = SM::LD, LX = SM::LX, NT = DK / 32;
     extern __shared__ __align__(16) uint8_t smem_tail[];
-    __half* sP = (__half*)smem_tail;                                   // [2][DK][LD]
-    __half* sA = sP + 2 * DK * LD;                                // [2][16][LD]  fp16 rows of the start state
+    __half* sA = (__half*)smem_tail;                              // [2][16][LD]  fp16 rows of the start state
+    uint8_t* ring = smem_tail + SM::a_bytes;
     const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31, gq = lane >> 2, t4 = lane & 3;
-    const int groups = d_v / 16;
+    const int groups = d_v / 16, depth = min(COMPOSE_RING, nseg - 1);
     const long long seq = blockIdx.x / groups;
-    const int j = (int)(blockIdx.x % groups) * 16 + gq, i0 = w * (DK / 4) + 2 * t4;
-    auto load_p = [&](int s) {
-        const __half* src = sg.P + (seq * nseg + s) * DK * DK;
-        __half* dst = sP + (s & 1) * DK * LD;
+    const int j0 = (int)(blockIdx.x % groups) * 16, j = j0 + gq, i0 = w * (DK / 4) + 2 * t4;
+    auto copy16 = [](void* dst, const void* src) {
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+    };
+    // what step s needs (an empty group past the last: the count of groups in flight is the same in every step)
+    auto load = [&](int s, int slot) {
+        if (s < nseg) {
+            uint8_t* at = ring + slot * SM::stage;
+            const __half* P = sg.P + (seq * nseg + s) * DK * DK;
 #pragma unroll
-        for (int e = 0; e < PIECES; ++e) {
-            const int p = e * 128 + tid, row = p / (DK / 8), c = p % (DK / 8);
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst + row * LD + c * 8)), "l"(src + row * DK + c * 8) : "memory");
+            for (int e = 0; e < DK * DK / 8 / 128; ++e) {
+                const int p = e * 128 + tid, row = p / (DK / 8), c = p % (DK / 8);
+                copy16((__half*)at + row * LD + c * 8, P + row * DK + c * 8);
+            }
+            const float* Xi = sg.Xi + (seq * nseg + s) * DK * d_v + j0;
+#pragma unroll
+            for (int e = 0; e < DK * 4 / 128; ++e) {
+                const int p = e * 128 + tid, row = p / 4, c = p % 4;
+                copy16((float*)(at + SM::p_bytes) + row * LX + c * 4, Xi + (long long)row * d_v + c * 4);
+            }
+            if (tid < DK / 4) copy16((float*)(at + SM::p_bytes + SM::x_bytes) + tid * 4, sg.D + (seq * nseg + s) * DK + tid * 4);
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
     float S[NT][4];
-    auto xi = [&](int s, float (&x)[NT][4]) {
-        const float* src = sg.Xi + (seq * nseg + s) * DK * d_v;
+    wait_for_previous_kernel();
+    for (int s = 1; s <= depth; ++s) load(s, s - 1);
+    {
+        const float* src = sg.Xi + seq * nseg * DK * d_v;
 #pragma unroll
         for (int n = 0; n < NT; ++n)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) x[n][e] = src[(long long)(i0 + 8 * n + (e & 1)) * d_v + j + 8 * (e >> 1)];
-    };
-    auto diagonal = [&](int s, float2 (&x)[NT]) {
-#pragma unroll
-        for (int n = 0; n < NT; ++n) x[n] = *(const float2*)(sg.D + (seq * nseg + s) * DK + i0 + 8 * n);
-    };
-    float X[NT][4], Xn[NT][4];                                    // Xi of this step and of the next
-    float2 D[NT], Dn[NT];                                         // the diagonal of P likewise
-    wait_for_previous_kernel();
-    load_p(1);
-    xi(0, S);
-    xi(1, X);
-    diagonal(1, D);
+            for (int e = 0; e < 4; ++e) S[n][e] = src[(long long)(i0 + 8 * n + (e & 1)) * d_v + j + 8 * (e >> 1)];
+    }
+    int slot = 0;
 #pragma unroll 1
     for (int s = 1; s < nseg; ++s) {
         __half* a_s = sA + (s & 1) * 16 * LD;
@@ -1011,16 +1024,12 @@ __global__ void __launch_bounds__(128) chain_compose(ChainSeg sg, float* __restr
                 *(uint32_t*)(a_s + (gq + 8 * h) * LD + i0 + 8 * n) = x;
                 *(uint32_t*)(out + (long long)(j + 8 * h) * DK + i0 + 8 * n) = x;
             }
-        if (s + 1 < nseg) {
-            xi(s + 1, Xn);
-            diagonal(s + 1, Dn);
-            load_p(s + 1);
-            asm volatile("cp.async.wait_group 1;" ::: "memory");
-        } else {
-            asm volatile("cp.async.wait_group 0;" ::: "memory");
-        }
+        if (depth == 3) asm volatile("cp.async.wait_group 2;" ::: "memory");
+        else if (depth == 2) asm volatile("cp.async.wait_group 1;" ::: "memory");
+        else asm volatile("cp.async.wait_group 0;" ::: "memory");
         __syncthreads();
-        const __half* P = sP + (s & 1) * DK * LD;
+        const __half* P = (const __half*)(ring + slot * SM::stage);
+        const float *X = (const float*)(ring + slot * SM::stage + SM::p_bytes), *D = X + SM::x_bytes / 4;
         float M[NT][4];
 #pragma unroll
         for (int kk = 0; kk < DK / 16; ++kk) {
@@ -1034,18 +1043,17 @@ __global__ void __launch_bounds__(128) chain_compose(ChainSeg sg, float* __restr
                 mma_acc(M[2 * np + 1], a, x[2], x[3], kk > 0);
             }
         }
-        // (Xi and the diagonal last: their loads have had the whole step)
 #pragma unroll
         for (int n = 0; n < NT; ++n) {
+            const float2 d = *(const float2*)(D + i0 + 8 * n);
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                S[n][e] = fmaf(S[n][e], e & 1 ? D[n].y : D[n].x, X[n][e]) + M[n][e];
-                if (s + 1 < nseg) X[n][e] = Xn[n][e];
-            }
-            if (s + 1 < nseg) D[n] = Dn[n];
+            for (int e = 0; e < 4; ++e) S[n][e] = fmaf(S[n][e], e & 1 ? d.y : d.x, X[(i0 + 8 * n + (e & 1)) * LX + gq + 8 * (e >> 1)]) + M[n][e];
         }
-        __syncthreads();                                          // (P of this step is replaced after the next one's first barrier)
+        __syncthreads();                                          // (the slot is filled anew)
+        load(s + depth, slot);
+        slot = slot + 1 == depth ? 0 : slot + 1;
     }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
     if (S_final) {
         float* out = S_final + seq * DK * d_v;
 #pragma unroll
@@ -1220,9 +1228,10 @@ int launch_seg_tail(const Problem& p, const ChainPlan& plan, const ChainSeg& sg)
     const int nseq = p.B * p.H, dv = DV, seg_tokens = plan.seg_blk * (NB / p.r);
     constexpr int LD = DK + 8;
     {
-        constexpr int smem = (2 * DK + 2 * 16) * LD * 2;
+        using SM = ComposeSmem<DK>;
+        const int smem = SM::a_bytes + (plan.nseg - 1 < COMPOSE_RING ? plan.nseg - 1 : COMPOSE_RING) * SM::stage;
         static std::atomic<uint64_t> opted_in{0};
-        const int st = allow_smem(opted_in, (const void*)chain_compose<DK>, smem);
+        const int st = allow_smem(opted_in, (const void*)chain_compose<DK>, SM::a_bytes + COMPOSE_RING * SM::stage);
         if (st != PF_OK) return st;
         prof_begin("chain_compose", p.stream);
         void* args[] = {(void*)&sg, (void*)&p.S_final, (void*)&plan.nseg, (void*)&dv};
