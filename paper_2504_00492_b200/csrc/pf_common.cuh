@@ -124,7 +124,7 @@ size_t recur_workspace_bytes(const Problem& p);
 double recur_short_us(const Problem& p);
 int recur_forward(const Problem& p, void* workspace);
 
-// the chunk form on warp-level tensor-core products (pf_chain.cu); bf16 inputs; one kernel and no workspace, or for few long
+// the chunk form with the state in tensor memory, a CTA per sequence or segment (pf_chain.cu); bf16 inputs; one kernel and no workspace, or for few long
 // sequences three kernels
 bool chain_supported(const Problem& p);
 double chain_estimate_us(const Problem& p);

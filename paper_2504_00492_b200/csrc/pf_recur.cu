@@ -6,7 +6,7 @@
 // of the state, O is written once.  What bounds it is the serial chain of one token (dot products, two shuffle stages, the
 // update): 204 cycles at d_k = 64, r = 1 and 373 at d_k = 128, r = 2, of which the FFMA pipe is busy for 160.
 // Measured (fp32): B*H = 32, L = 2048, d = 128, r = 2: 0.389 ms against 4.9 ms for the four chunk-form kernels in
-// pf_simt.cu; one head, L = 256, d = 64, r = 1: 32 us walked as a whole, 23 in segments, against 209.
+// pf_simt.cu; one head, L = 256, d = 64, r = 1: 29 us walked as a whole, 19 in segments, against 209.
 //
 // A CTA takes one sequence and 32 columns j of the state S[j][i] (API layout X[i][j]); each of its four computing warps 8
 // columns, without any exchange between warps.  Lane (ig, j) of a warp holds S[j][i] for a quarter of the rows i, so a dot
@@ -328,10 +328,14 @@ recur_kernel(const Tin* __restrict__ q, const Tin* __restrict__ k, const Tin* __
 
 // start(1) = Xi_0, start(s+1) = start(s) P_s + Xi_s, the last one is S_final: a CTA per sequence and ROWS rows j, serial over the
 // segments.  A thread has four rows and one column i; P (stored [i][j']) comes to shared memory a step after it was requested,
-// rows padded so that 32 threads reading 16 bytes of 32 rows meet no bank twice.
-template <int DK>
-__global__ void __launch_bounds__(256) recur_compose(RecurSeg sg, float* __restrict__ S_final, int nseg, int d_v) {
-    constexpr int CG = DK / 32, ROWS = 4 * (8 / CG), LD = DK + 4, NV = DK * DK / 4 / 256;
+// rows padded so that 32 threads reading 16 bytes of 32 rows meet no bank twice.  What bounds a step is shared memory: of a CTA's warps
+// each reads its 32 rows of P once for 4 rows j.  So a CTA has 4 rows j, DK / 32 warps (the call, us, before with eight warps: one sequence of 256, d = 64,
+// r = 1: 24.1 -> 18.8; of 2000: 48.4 -> 35.7; 16 of 1000, r = 2: 62.4 -> 60.8; one of 1000, d = 128, r = 2: 63.4 -> 59.3).  At d = 128, where P is
+// four times as large and every CTA fetches its own copy, only while there is an SM for each (4 of 2000, r = 1: 86.7 -> 84.7; 8 of 1000 on 256 CTAs:
+// 92.8 -> 94.1), and otherwise 8 rows, eight warps.
+template <int DK, int WARPS>
+__global__ void __launch_bounds__(32 * WARPS) recur_compose(RecurSeg sg, float* __restrict__ S_final, int nseg, int d_v) {
+    constexpr int CG = DK / 32, THREADS = 32 * WARPS, ROWS = 4 * (WARPS / CG), LD = DK + 4, NV = DK * DK / 4 / THREADS;
     extern __shared__ __align__(16) float smf[];
     float* Ps = smf;                    // [DK i][LD]
     float* cur = smf + DK * LD;         // [ROWS][DK]
@@ -343,7 +347,7 @@ __global__ void __launch_bounds__(256) recur_compose(RecurSeg sg, float* __restr
     auto fetch_p = [&](int s) {
         const float4* p = (const float4*)(sg.P + (seq * nseg + s) * DK * DK);
 #pragma unroll
-        for (int u = 0; u < NV; ++u) pv[u] = p[u * 256 + tid];
+        for (int u = 0; u < NV; ++u) pv[u] = p[u * THREADS + tid];
     };
     auto fetch_x = [&](int s) { return *(const float4*)(sg.Xi + ((seq * nseg + s) * DK + i) * d_v + j); };
     wait_for_previous_kernel();
@@ -358,7 +362,7 @@ __global__ void __launch_bounds__(256) recur_compose(RecurSeg sg, float* __restr
         cur[(jl + 3) * DK + i] = acc.w;
 #pragma unroll
         for (int u = 0; u < NV; ++u) {
-            const int e = (u * 256 + tid) * 4;
+            const int e = (u * THREADS + tid) * 4;
             *(float4*)(Ps + (e / DK) * LD + e % DK) = pv[u];
         }
         acc = xv;
@@ -467,7 +471,7 @@ size_t seg_bytes(const Problem& p, int nseg) {
     const size_t nseq = (size_t)p.B * p.H, slots = nseq * nseg;
     return align_up(nseq * p.L * p.d_k * 4, 256) + align_up(slots * p.d_k * p.d_k * 4, 256) + 2 * align_up(slots * p.d_k * p.d_v * 4, 256);
 }
-// Segments, where they make the call shorter (one fp32 head of 256 tokens: 23 us instead of 29; of 180: 22, 21): the walk of a token costs about the same while at most one CTA
+// Segments, where they make the call shorter (one fp32 head of 256 tokens: 19 us instead of 29): the walk of a token costs about the same while at most one CTA
 // (d_k = 64: two, whose chains leave each other most of the issue slots) runs per SM; against it stand two more kernels, 1 to 2
 // us of composing per segment, and the traffic and products of the responses.
 RecurPlan make_plan(const Problem& p) {
@@ -483,7 +487,7 @@ RecurPlan make_plan(const Problem& p) {
     for (int want = 2; want <= most && want <= 64; ++want) {
         const int seg_tok = (p.L + 16 * want - 1) / (16 * want) * 16, nseg = (p.L + seg_tok - 1) / seg_tok;
         const long long ctas = nseq * (nseg * (p.d_v / RJ) + (nseg - 1) * (p.d_k / RJ));
-        const double us = extra + nseg * (big ? 1.9 : 0.8) + seg_tok * tok * (ctas > sms ? 1.2 : 1.0);
+        const double us = extra + nseg * (big ? 1.9 : 0.7) + seg_tok * tok * (ctas > sms ? 1.2 : 1.0);
         // (a caller's workspace was sized for the chunk-form kernels of pf_simt.cu)
         if (nseg > 1 && us < best && (p.own_workspace || seg_bytes(p, nseg) + 256 <= simt_workspace_bytes(p))) {
             best = us;
@@ -493,19 +497,23 @@ RecurPlan make_plan(const Problem& p) {
     return plan;
 }
 
+template <int DK, int WARPS>
+int launch_compose(const Problem& p, const RecurPlan& plan, const RecurSeg& sg, int nseq, int dv) {
+    constexpr int rows = 4 * (WARPS / (DK / 32)), smem = (DK * (DK + 4) + rows * DK) * 4;
+    static std::atomic<uint64_t> opted_in{0};
+    const int st = allow_smem(opted_in, (const void*)recur_compose<DK, WARPS>, smem);
+    if (st != PF_OK) return st;
+    prof_begin("recur_compose", p.stream);
+    void* args[] = {(void*)&sg, (void*)&p.S_final, (void*)&plan.nseg, (void*)&dv};
+    PF_CUDA_TRY(launch_early((const void*)recur_compose<DK, WARPS>, dim3((unsigned)(nseq * (dv / rows))), 32 * WARPS, args, smem, p.stream));
+    prof_end(p.stream);
+    return PF_OK;
+}
 template <int DK, int DV>
 int launch_seg_tail(const Problem& p, const RecurPlan& plan, const RecurSeg& sg) {
     const int nseq = p.B * p.H, dv = DV;
-    {
-        constexpr int rows = 4 * (8 / (DK / 32)), smem = (DK * (DK + 4) + rows * DK) * 4;
-        static std::atomic<uint64_t> opted_in{0};
-        const int st = allow_smem(opted_in, (const void*)recur_compose<DK>, smem);
-        if (st != PF_OK) return st;
-        prof_begin("recur_compose", p.stream);
-        void* args[] = {(void*)&sg, (void*)&p.S_final, (void*)&plan.nseg, (void*)&dv};
-        PF_CUDA_TRY(launch_early((const void*)recur_compose<DK>, dim3((unsigned)(nseq * (DV / rows))), 256, args, smem, p.stream));
-        prof_end(p.stream);
-    }
+    const int st0 = DK == 64 || nseq * (DV / 4) <= sm_count() ? launch_compose<DK, DK / 32>(p, plan, sg, nseq, dv) : launch_compose<DK, 8>(p, plan, sg, nseq, dv);
+    if (st0 != PF_OK) return st0;
     constexpr int smem = (DK * DV + DK * 68) * 4;
     static std::atomic<uint64_t> opted_in{0};
     const int st = allow_smem(opted_in, (const void*)recur_apply<DK, DV>, smem);

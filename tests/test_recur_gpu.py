@@ -22,7 +22,7 @@ def test_pass_and_stage_edges(dtype, mode, step, r, d_k, d_v, L):
 
 @pytest.mark.parametrize("d_k,d_v,r,H,L,mode", [
     (64, 64, 2, 2, 1000, "sum"), (64, 128, 1, 1, 2049, "sum"), (128, 64, 3, 1, 1111, "product"), (128, 128, 1, 2, 1777, "sum"),
-    (64, 64, 4, 5, 640, "product"), (64, 64, 2, 1, 200, "sum"), (128, 128, 1, 1, 300, "sum"),
+    (64, 64, 4, 5, 640, "product"), (64, 64, 2, 1, 200, "sum"), (128, 128, 1, 1, 300, "sum"), (128, 128, 1, 8, 1000, "sum"),
 ])
 def test_few_long_sequences_are_walked_in_segments(d_k, d_v, r, H, L, mode):
     """The walk, the composition of the start states, their contribution to O; step sizes to 1 and to 2."""
