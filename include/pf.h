@@ -83,7 +83,7 @@ enum { PF_MODE_SUM = 0, PF_MODE_PRODUCT = 1 };
 enum { PF_STEP_EULER = 0, PF_STEP_EXACT = 1 };
 
 /* Which kernels evaluate the operation.
- *   PF_IMPL_AUTO : bf16: whichever is expected to be faster of the chunk form on warp-level tensor-core products (one
+ *   PF_IMPL_AUTO : bf16: whichever is expected to be faster of the chunk form with the state in tensor memory (one
  *                  kernel, blocks of 64 / r tokens; few long sequences in segments side by side, three kernels), the
  *                  tcgen05 kernels, and, for a few tokens, the recurrence token by token.  fp32: the recurrence token by
  *                  token.  The result does not depend on the chunk length beyond rounding, so AUTO may evaluate with
@@ -121,8 +121,8 @@ enum { PF_IMPL_AUTO = 0, PF_IMPL_SIMT = 1, PF_IMPL_TC = 2,
  * the state S to fp16 before each product (fp32 accumulation).  fp16 has the 8 significant bits of bf16 and more, but
  * only the exponent range 6.1e-5 .. 65504: an element of v, S0 or of the running state beyond 65504 in magnitude becomes
  * infinite without an error code, and elements below 6.1e-5 lose precision gradually.  Products of the state with keys may
- * exceed 65504 (with keys of length 1, S k reaches sqrt(d_k) times the largest entry of S): they stay in fp32 in the tcgen05
- * kernels, and the warp-level kernel, where they are operands, computes the columns of O and S_final that lost them once more
+ * exceed 65504 (with keys of length 1, S k reaches sqrt(d_k) times the largest entry of S): they stay in fp32 in the single
+ * launch, and the one-kernel chunk form, where they are operands, computes the columns of O and S_final that lost them once more
  * in fp32 (slowly, 1.3 to 3 us a token; columns that are infinite or NaN for other reasons pay this too).  The stated tolerance
  * (2e-3 of max|O|) is tested for |v|, |S| up to the order of 1e3, and for states of 2e4 aligned with a key.  The operation is linear in (v, S0): scale them by a power
  * of two and O, S_final back for data outside that range, or ask for PF_IMPL_SIMT (fp32 throughout, no such limit).
@@ -245,7 +245,7 @@ int pf_select_chunk(int B, int H, int L, int d_k, int d_v, int r, int chunk, int
  * word on the current device.  pf_last_wait_code() then gives the code that was read (host thread local):
  *     1xx  flow-building role of the single-launch path (101-103 solve warps, 11x-12x bulk warps, 14x-15x MMA-issuing
  *          warps, 16x flag warp),   2xx  its scanning role (20x chain, 21x output, 22x loads, 23x MMA issue),
- *     30x  the token-by-token kernel,   31x  the warp-level chunk kernel,
+ *     30x  the token-by-token kernel,   31x - 35x  the one-kernel chunk form,
  *     1-99 the two-launch path (tc_flow, tc_scan),   99  shared memory not 1024-byte aligned,   900  pf_wait_selftest.
  * The chunk-form fp32 kernels have no such waits.
  */
