@@ -149,9 +149,9 @@ def l2_note(nbytes: int) -> str:
 # hash of those sources is stored with them; the commands are in profiles/fused_kernel_c2.md):
 #   NCU_TRAFFIC      DRAM bytes (read + write) of one full-size launch: {workload: (hash, bytes)}
 #   NCU_TENSOR_PIPE  sm__pipe_tensor_cycles_active (% of peak, elapsed), captured on the half-size case
-#                    (--batch 1 --heads 16) under the section-capture size rule: {workload: (hash, percent, case)}
-NCU_TRAFFIC = {"c2": ("b718c8d671a5a5ad", 337232640 + 122488576)}
-NCU_TENSOR_PIPE = {"c2": ("b718c8d671a5a5ad", 21.41, "half-size case B=1 H=16 of c2")}
+#                    (--path tc --batch 1 --heads 16) under the section-capture size rule: {workload: (hash, percent, case)}
+NCU_TRAFFIC = {"c2": ("940308b5ec9e5234", 336915968 + 121679616)}
+NCU_TENSOR_PIPE = {"c2": ("940308b5ec9e5234", 21.40, "half-size case B=1 H=16 of c2")}
 
 
 def kernel_source_hash() -> str:
