@@ -26,8 +26,8 @@
 // named barriers) and the instruction cache (so what is off the chain's path is written small).  148 CTAs at r = 1 move 5.5 TB/s, 84 % of
 // what a copy reaches.  Measured (us, before: the same blocks on
 // warp-level products, a warp carrying 16 rows j in registers; a shared-memory read of every tile by every such warp): 256 sequences of
-// 1024, d = 128, r = 2: 227 -> 131 (calls one after another); 128 of 4096, d = 64, r = 4: 340 -> 285; 48 of 1999, 64 x 128, r = 3: 146 -> 80 (2 segments);
-// 4 of 16384, d = 128, r = 1: 135 -> 80 (segments); 32 of 2048, d = 128, r = 1: 68 -> 54 (the tcgen05 kernel in one launch before).
+// 1024, d = 128, r = 2: 227 -> 127 (calls one after another); 128 of 4096, d = 64, r = 4: 340 -> 279; 48 of 1999, 64 x 128, r = 3: 144 -> 79 (2 segments);
+// 4 of 16384, d = 128, r = 1: 135 -> 78 (segments); 32 of 2048, d = 128, r = 1: 68 -> 54 (the tcgen05 kernel in one launch before).
 // Measured and not taken: the update's and V - K S^T's products in halves, so that one half is converted while the other is being multiplied (the
 // probe's 1.6 k cycles have it; here 412 us against 389 at 32 sequences of 8192: more instructions); the output's products issued by the chain's
 // warp (462); one election per product instead of per group (427 against 420 then, 179 against 146 with all SMs busy); products in loops on
@@ -1126,7 +1126,8 @@ __global__ void __launch_bounds__(256) chain_apply(ChainSeg sg, float* __restric
 // A sequence has one CTA, or where few sequences are long, segments walked side by side: as many as one wave of CTAs holds pay for
 // the second walk (the responses) and for two more kernels.  The time is 7 us, (waves of CTAs) x (blocks of a segment) x (time of a
 // block) and what composing segments costs.  Measured, us per block for r = 1 .. 4 with 32 CTAs (d_k = 64 and 128), and with 148, when
-// two multiprocessors share what they fetch instructions through; and 8192 tokens of 4 sequences, d = 128, r = 1, in 1, 2, 4, 8, 16
+// two multiprocessors share what they fetch instructions through (taken before G and P^T were one product; since then a block takes up to 18 % less, but so far the
+// choices come out right: with the present times 32 sequences of 16384, r = 2, would go from the single launch's 472 us to 522 in segments); and 8192 tokens of 4 sequences, d = 128, r = 1, in 1, 2, 4, 8, 16
 // segments: 259, 136, 85, 60, 55 us; of 2, d = 64, r = 2, in 2, 4, 8, 16: 163, 88, 53, 40.
 struct ChainPlan {
     int nseg, seg_blk;
