@@ -114,8 +114,9 @@ __global__ void wait_selftest_kernel(int* status, const int* flag, long long lim
         tc::flag_wait_ge_limit(flag, 1, status, 900, limit_cycles);
     }
     __syncthreads();
-    if (threadIdx.x < 32) tc::mbar_wait_tries<true>(&bar, 0, status, 901, tc::WAIT_TRIES / 64);
-    else tc::mbar_wait_tries<false>(&bar, 0, status, 902, tc::WAIT_TRIES / 64);
+    const bool lazy = threadIdx.x < 32;
+    if (!(lazy ? tc::mbar_wait_tries<true>(tc::smem_u32(&bar), 0, tc::WAIT_TRIES / 64) : tc::mbar_wait_tries<false>(tc::smem_u32(&bar), 0, tc::WAIT_TRIES / 64)))
+        atomicCAS(status, 0, lazy ? 901 : 902);
 }
 
 bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }

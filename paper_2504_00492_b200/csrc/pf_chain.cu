@@ -4,8 +4,11 @@
 //     T  = (I + Mstrict (.) (diag(beta) K K^T))^{-1} diag(beta)                      (does not depend on S)
 //     P  = (Q K^T) (.) Mincl                                                         (does not depend on S)
 //     U' = T (V - K S^T),       O = Q S^T + P U',       S <- S + U'^T K
-// i.e. W and Uh are never formed: T is applied to V - K S^T instead.  Only three products of a block depend on S one after another:
-// R = V - K S^T, U' = T R and the update.  All are tcgen05 products of 128 rows j (d_v = 64: half of them nobody's) whose A operand lies
+// evaluated in one of two forms (w_form):
+//     V - K S^T first and T applied to it: three products of a block depend on S one after another, R = V - K S^T, U' = T R and the update;
+//     with W = T K formed ahead ("W form"), U' = T V - W S^T: two, at the price of one more product, its way through tensor memory and V in fp16.
+// (Against the fp64 recurrence, 70 sequences of 400, d = 64, r = 4, beta to 2: relative L2 error of O 6.81e-4 with W and 7.12e-4 without: V - K S^T is never rounded.)
+// All are tcgen05 products of 128 rows j (d_v = 64: half of them nobody's) whose A operand lies
 // in tensor memory and whose B operand is a tile of shared memory as TMA or the preparing warps left it.  S stays in tensor memory as the
 // fp32 accumulator of its update; between two products the chain warps convert an accumulator to the next one's fp16 operand.
 //
@@ -15,9 +18,10 @@
 //                 rows, from the bf16 tiles as they land)
 //   solve (2 x 4) T of every other block: G from tensor memory, the inverse on mma.sync
 //   convert (4)   K, Q -> fp16 in place, P out of tensor memory into shared memory
-//   output (4)    O^T out of tensor memory into the rows of O;  and one warp issues the copies
-// A stage of shared memory holds what the chain needs of one block: K, Q (fp16, the rows of Q behind those of K), T, P (fp16), V (bf16 as
-// it came, added to R's accumulator as V^T times an identity).
+//   W (4)         W form: W^T = K^T T^T out of tensor memory into shared memory
+//   output (4)    O^T out of tensor memory into the rows of O; W form: V -> fp16 in place;  and one warp issues the copies
+// A stage of shared memory holds what the chain needs of one block: K, Q (fp16, the rows of Q behind those of K) and P (fp16); T, V and W have rings of their
+// own.  Without W, V is bf16 as it came and added to R's accumulator as V^T times an identity; with W, U'^T's accumulator starts as V^T T^T.
 //
 // What bounds it: the three trips of a block (issue 4 to 8 products at 30 cycles each, tensor memory to registers and back), 2.2 k cycles at
 // d = 128 with everything but the chain's own warps switched off, drawn out to 2.6 - 3 k by the others: all products go through one
@@ -26,7 +30,7 @@
 // named barriers) and the instruction cache (so what is off the chain's path is written small).  148 CTAs at r = 1 move 5.5 TB/s, 84 % of
 // what a copy reaches.  Measured (us, before: the same blocks on
 // warp-level products, a warp carrying 16 rows j in registers; a shared-memory read of every tile by every such warp): 256 sequences of
-// 1024, d = 128, r = 2: 227 -> 136 (calls on other inputs one after another; 228 -> 115 on the same); 128 of 4096, d = 64, r = 4: 340 -> 307 (336 -> 290); 48 of 1999, 64 x 128,
+// 1024, d = 128, r = 2: 227 -> 136 (calls on other inputs one after another; 228 -> 115 on the same); 128 of 4096, d = 64, r = 4: 340 -> 307 (336 -> 290; with W 264); 48 of 1999, 64 x 128,
 // r = 3: 144 -> 84 (144 -> 80; 2 segments); 4 of 16384, d = 128, r = 1: 135 -> 78 (segments); 32 of 2048, d = 128, r = 1: 68 -> 54 (the tcgen05 kernel in one launch before).
 // Measured and not taken: the update's and V - K S^T's products in halves, so that one half is converted while the other is being multiplied (the
 // probe's 1.6 k cycles have it; here 412 us against 389 at 32 sequences of 8192: more instructions); the output's products issued by the chain's
@@ -35,14 +39,20 @@
 // sequences, 290 -> 322 at d = 64, r = 4).  The chain's warps at named barriers too, one warp watching the products' ends for them (293 -> 328).
 // V in one buffer apart from the stages, which makes room for one more (142.6 -> 152.4, 128 sequences of 2048, d = 64, r = 4).  The
 // state before the last block's update in V - K S^T, with U'^T K K^T of the two blocks in its place (172 us at 256 sequences: 20 products more).
+// What counts besides the chain's latency: instructions that are fetched (what all warps execute in a block is about 40 KB; 49 KB of it, in an earlier W form, missed
+// the instruction cache in 23 % of the requests instead of 5 and took 20 % more time), so that a wait is a few instructions and its failure is reported once a
+// role; and no warps that poll mbarriers but those that watch for others.
+// Measured and not taken: the chain's warps meeting at a named barrier and the first of them issuing (128 us against 116 at 256 sequences, 314 against 264 at
+// 128 of 4096, d = 64); a predicate on every product instead of a branch around all of a step (twice the instructions); an L2 prefetch of the next tiles (128 of 4096, d = 64:
+// 359 against 338 without, at the time; level elsewhere); W's products issued by the Gram products' warp (they wait behind a later block's landing) or by the copies' (350 cycles a copy).
 //
 // Range: V - K S^T and U' are packed to fp16 like every other operand, and K S^T reaches sqrt(d_k) times the largest entry of S, so
 // that a state well inside fp16's 65504 can overflow them.  What overflows leaves its row of S infinite or NaN to the end of the walk
 // (infinity times anything is infinite or NaN), so one look at each row when the walk is over finds it and the blocks pay nothing:
 // its rows are then walked once more, token by token in fp32 (walk_fp32).
 //
-// The inverse: warp w of a team owns rows 16 w .. 16 w + 15 of G, forms A's blocks there and D_w = (I + A_ww)^{-1} by its Neumann product,
-// and after one exchange through shared memory column block w of X: X_ww = D_w, X_iw = -D_i sum_k A_ik X_kw, each X_iw^T left in
+// The inverse of I - N, N = -A: warp w of a team owns rows 16 w .. 16 w + 15 of G, forms N's blocks there and D_w = (I - N_ww)^{-1} by its Neumann product,
+// and after one exchange through shared memory column block w of X: X_ww = D_w, X_iw = D_i sum_k N_ik X_kw, each X_iw^T left in
 // registers as the operand of the next (through shared memory and in loops: 58.1 us instead of 56.5, 148 sequences of 1024, r = 2).
 #include <float.h>
 
@@ -59,6 +69,12 @@ using namespace tc;
 namespace {
 
 constexpr int NB = 64;               // rows per block
+
+// Where the W form pays (head of the file), us, W and without: 128 sequences of 4096, d = 64, r = 4: 264 and 290; 256 of 1000, d = 64, r = 2: 81 and 85; 64 of 4000,
+// r = 1: 85 and 89.  Not where the walks are short and the chain has nothing ahead at their start (4 of 8192 in segments, d = 64, r = 2: 43 and 40), not at
+// d_v = 128 (140 of 1500, 64 x 128, r = 1: 44 and 43; 48 of 1999, r = 3: level) and not at d_k = 128, where the bound is what a block moves through
+// shared memory, 2950 cycles' worth at r = 2 with W and 2350 without (256 of 1024, r = 2: 118 and 114).
+constexpr bool w_form(int d_k, int d_v, bool segments) { return d_k == 64 && d_v == 64 && !segments; }
 
 struct ChainMaps {
     CUtensorMap q, k, v;
@@ -100,25 +116,44 @@ struct ChainSmem {
     static constexpr int C = NB / R;                              // tokens per block
     static constexpr int CP = (C + 15) / 16 * 16;                 // ... in tiles of 16
     static constexpr int k_bytes = NB * DK * 2, q_bytes = CP * DK * 2;
-    static constexpr int t_bytes = NB * 128, p_bytes = CP * 128, v_bytes = NB * JS * 2;
+    static constexpr int t_bytes = NB * 128, w_bytes = DK * 128, p_bytes = CP * 128, v_bytes = NB * JS * 2;
     // slabs of 64 columns, in each the rows of K and then those of Q: one operand of NB + CP rows
-    static constexpr int rows = NB + CP, k_off = 0, q_off = NB * 128, t_off = k_bytes + q_bytes, p_off = t_off + t_bytes, v_off = p_off + p_bytes;
-    static constexpr int stage = v_off + v_bytes;
-    static constexpr int tx_bytes = k_bytes + C * DK * 2 + v_bytes;         // what the copies of a block bring
+    static constexpr int rows = NB + CP, k_off = 0, q_off = NB * 128, p_off = k_bytes + q_bytes;
+    static constexpr int stage = p_off + p_bytes;
+    static constexpr int tx_bytes = k_bytes + C * DK * 2;         // what the copies of a block's K and Q bring
 };
 
+// Barriers (mbarriers); those of the rings of shared memory follow (ChainCfg).
+enum {
+    B_SP = 0,       // chain: fp16 copy of S published
+    B_UD = 1,       // products: U' complete
+    B_UP = 2,       // chain: its fp16 copy published
+    B_SD = 3,       // products: S complete
+    B_QD = 4,       // output products: Q S^T complete
+    B_OD = 5,       // [2] output products: O^T complete
+    B_OFREE = 7,    // [2] output: O^T read
+    B_GD = 9,       // Gram products: G and P^T complete
+    B_WD = 10,      // W's products: W complete
+    B_RD = 11,      // products: V^T - S K^T complete
+    B_RP = 12,      // chain: its fp16 copy published
+    B_RINGS = 13
+};
 constexpr int TEAMS = 2;             // solve teams
-// warps: 0-7 chain, 8-11 output, 12-15 conversion, then the solve teams, then products of the chain, products of the output, Gram
-// products, copies
+// warps: 0-7 chain, 8-11 output (and V), 12-15 conversion, then the solve teams, then products of the chain, products of the output, Gram products,
+// copies, then in the W form W's
 constexpr int W_OUT = 8, W_CONV = 12, W_SOLVE = 16, W_MMA = W_SOLVE + 4 * TEAMS, W_MMA_OUT = W_MMA + 1, W_GRAM = W_MMA + 2, W_LOAD = W_MMA + 3,
-              CHAIN_THREADS = 32 * (W_MMA + 4);
+              W_W = W_MMA + 4;
+template <bool W> constexpr int CHAIN_THREADS = 32 * (W ? W_W + 4 : W_W);
 
 // Registers per thread: the launch's, and what each warpgroup makes of them (the sum is the launch's)
-constexpr int REGS = 72, REGS_CHAIN = 80, REGS_OUT = 48, REGS_CONV = 56, REGS_ISSUE = 56, REGS_SOLVE = 88;
-static_assert(2 * REGS_CHAIN + REGS_OUT + REGS_CONV + REGS_ISSUE + TEAMS * REGS_SOLVE <= REGS * CHAIN_THREADS / 128, "registers of the launch");
-template <int N>
+template <bool W> constexpr int REGS = W ? 64 : 72;
+constexpr int REGS_CHAIN = 80, REGS_OUT = 48, REGS_CONV = 48, REGS_W = 48, REGS_ISSUE = 48;
+template <bool W> constexpr int REGS_SOLVE = W ? 80 : 88;
+static_assert(2 * REGS_CHAIN + REGS_OUT + REGS_CONV + REGS_W + REGS_ISSUE + TEAMS * REGS_SOLVE<true> <= REGS<true> * CHAIN_THREADS<true> / 128 &&
+              2 * REGS_CHAIN + REGS_OUT + REGS_CONV + REGS_ISSUE + TEAMS * REGS_SOLVE<false> <= REGS<false> * CHAIN_THREADS<false> / 128, "registers of the launch");
+template <bool W, int N>
 __device__ __forceinline__ void set_registers() {
-    if (N > REGS) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
+    if (N > REGS<W>) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
     else asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N));
 }
 
@@ -136,33 +171,68 @@ struct IdStrip {
     __device__ static uint64_t desc(uint32_t base, int c) { return make_desc_ns(base + (6 - 2 * c) * 128, 7 * 128, 128); }
 };
 
-template <int DK, int R, int DV, int NS>
+// How many blocks each part of shared memory holds.  A block's K, Q and P are there from its copy to its end.  In the W form V and T until V^T T^T and W until
+// S W^T are enough; otherwise all are there to the block's end.
+struct ChainRings {
+    int kq, v, t, w;
+};
+constexpr int SMEM_MOST = 226 * 1024;
+template <int DK, bool W, int R, int DV>
+constexpr ChainRings chain_rings() {
+    using SM = ChainSmem<DK, R, DV>;
+    int left = SMEM_MOST - TEAMS * (XS_BYTES + 512) - IdStrip::bytes;
+    if (!W) {
+        const int n = left / (SM::stage + SM::v_bytes + SM::t_bytes), m = n < 6 ? n : 6;
+        return {m, m, m, 0};
+    }
+    ChainRings g{0, 2, 2, 2};
+    left -= g.v * SM::v_bytes + g.t * SM::t_bytes + g.w * SM::w_bytes;
+    g.kq = left / SM::stage;
+    if (g.kq > 6) g.kq = 6;
+    if (left - g.kq * SM::stage >= SM::t_bytes) ++g.t;
+    return g;
+}
+template <int DK, bool W, int R, int DV>
 struct ChainCfg {
     using SM = ChainSmem<DK, R, DV>;
-    static constexpr int xs_off = NS * SM::stage;                 // per team: X (unscaled) while it is being formed
+    static constexpr ChainRings ring = chain_rings<DK, W, R, DV>();
+    static constexpr int NS = ring.kq, NV = ring.v, NT = ring.t, NW = ring.w;
+    static constexpr int v_off = NS * SM::stage, t_off = v_off + NV * SM::v_bytes, w_off = t_off + NT * SM::t_bytes;
+    static constexpr int xs_off = w_off + NW * SM::w_bytes;       // per team: X (unscaled) while it is being formed
     static constexpr int beta_off = xs_off + TEAMS * XS_BYTES;    // per team: 64 step sizes, of two blocks in turn
     static constexpr int id_off = beta_off + TEAMS * 512;         // identity (IdStrip)
     static constexpr int total = id_off + IdStrip::bytes;
+    // barriers of the rings, after the others
+    static constexpr int LAND = B_RINGS, FULL = LAND + NS, EMPTY = FULL + NS, VLAND = EMPTY + NS, VFREE = VLAND + NV,
+                         TDONE = VFREE + NV, WDONE = TDONE + NT, WFREE = WDONE + NW, count = WFREE + NW;
 };
-// as many stages as fit, up to six
-template <int DK, int R, int DV>
-constexpr int chain_stages() {
-    constexpr int left = 226 * 1024 - ChainCfg<DK, R, DV, 0>::total;
-    constexpr int n = left / ChainSmem<DK, R, DV>::stage;
-    return n < 6 ? n : 6;
-}
+// a ring's slot and the parity of its present round
+template <int N>
+struct RingPos {
+    int i = 0, phase = 0;
+    __device__ __forceinline__ void next() {
+        if (++i == N) {
+            i = 0;
+            phase ^= 1;
+        }
+    }
+};
 
 // Tensor memory: columns.  All 512 are this CTA's, so that they are these very addresses: constants, where a base read from shared memory
 // would go through a register to each product.
 constexpr uint32_t T_S = 0;          // S, fp32 [j][i]
 constexpr uint32_t T_S16 = 128;      // -S, fp16 pairs
-constexpr uint32_t T_R = 192;        // V^T - S K^T, then U'^T over it, fp32 [j][m]
-constexpr uint32_t T_R16 = 256;      // V^T - S K^T and
-constexpr uint32_t T_U16 = 288;      // U'^T in fp16 pairs
-constexpr uint32_t T_G = 320;        // G, fp32 [m][m'] (16 rows in each quarter of the lanes, as products of 64 rows are laid out)
-constexpr uint32_t T_P = 384;        // P^T before its mask, fp32 [m][t], likewise: behind T_G, one product
+constexpr uint32_t T_U = 192;        // U'^T, fp32 [j][m] (without W: first V^T - S K^T)
+// In the W form with 64 tokens a block, U'^T's fp16 pairs take the place of the first half of what each chain warp has read of it; otherwise
+// they have columns of their own, so that what comes next into the accumulator need not wait for their readers.
+template <bool W, int CP> constexpr bool U_INPLACE = W && CP > 32;
+constexpr uint32_t T_R16 = 256;      // V^T - S K^T in fp16 pairs
+template <bool W, int CP> constexpr uint32_t T_U16 = U_INPLACE<W, CP> ? T_U : W ? 256 : 288;
+template <bool W, int CP> constexpr uint32_t T_W = U_INPLACE<W, CP> ? 256 : 288;       // W^T, fp32 [i][m]
+template <bool W, int CP> constexpr uint32_t T_G = W ? T_W<W, CP> + 64 : 320;   // G, fp32 [m][m'] (16 rows in each quarter of the lanes, as products of 64 rows are laid out)
+template <bool W, int CP> constexpr uint32_t T_P = T_G<W, CP> + 64;   // P^T before its mask, fp32 [m][t], likewise: behind T_G, one product
 template <int CP> constexpr int O_BUFS = CP > 32 ? 1 : 2;         // O^T, fp32 [j][t]: of two blocks in turn where there is room
-template <int CP> __device__ __forceinline__ uint32_t o_cols(int b) { return CP > 32 ? 448u : 416u + 32u * (b & 1); }
+template <int CP> __device__ __forceinline__ uint32_t o_cols(int b) { return CP > 32 ? 448u : 448u + 32u * (b & 1); }
 
 // What one CTA of the kernel works on.
 struct ChainPart {
@@ -289,21 +359,21 @@ __device__ __forceinline__ void walk_fp32(const ChainArgs& args, const ChainPart
         for (int n = 0; n < NI; ++n) part.S_end[(long long)(i0 + n) * g.d_v + j] = S[n];
 }
 
-// K, Q and V of block b (of this part) into stage b mod NS (one thread); rows past the sequence arrive as zeros
-template <int DK, int R, int JS, int NS>
-__device__ __forceinline__ void load_block(const ChainMaps& maps, uint8_t* smem, uint64_t* land, int b, int seq, const ChainPart& part) {
-    using SM = ChainSmem<DK, R, JS>;
-    const int st = b % NS;
-    uint8_t* sg = smem + st * SM::stage;
-    const int bb = part.b0 + b;
-    mbar_expect_tx(&land[st], SM::tx_bytes - (part.response ? SM::v_bytes : 0));
-#pragma unroll
-    for (int h = 0; h < DK / 64; ++h) {
-        tma_load_4d(sg + SM::k_off + h * (SM::rows * 128), &maps.k, 0, bb * SM::C * R, h, seq, &land[st]);
-        tma_load_4d(sg + SM::q_off + h * (SM::rows * 128), &maps.q, 0, bb * SM::C, h, seq, &land[st]);
+// A role's waits on mbarriers.  The first that runs out leaves its code; those after it give up at the first try, so that each CTA ends by itself.
+struct Waits {
+    uint32_t bar;           // shared address of the first barrier
+    int tries = WAIT_TRIES, code = 0;
+    __device__ __forceinline__ explicit Waits(uint32_t bar) : bar(bar) {}
+    template <bool LAZY = true>
+    __device__ __forceinline__ void wait(int which, int parity, int code_if_not) {
+        if (!mbar_wait_tries<LAZY>(bar + 8 * which, (uint32_t)parity, tries)) {
+            if (code == 0) code = code_if_not;
+            tries = 1;
+        }
     }
-    if (!part.response) tma_load_4d(sg + SM::v_off, &maps.v, 0, bb * SM::C * R, 0, seq, &land[st]);
-}
+    __device__ __forceinline__ bool ok() const { return code == 0; }
+};
+
 // byte offsets of a lane's row address for ldmatrix.x4 within a slab of 128-byte swizzled rows; the K-step kk of 16 columns
 // is at off ^ (kk << 5), everything else is added
 __device__ __forceinline__ uint32_t lane_off(int row, int half) { return (uint32_t)row * 128u + (uint32_t)((half ^ (row & 7)) << 4); }
@@ -313,12 +383,14 @@ __device__ __forceinline__ uint32_t lane_off(int row, int half) { return (uint32
 // whoever watches an mbarrier takes part in them to the end, also when it has given up (`ok`).
 enum {
     N_TEAM = 1,     // [2] solve teams
+    N_WD = 3,       // W's warps: W^T complete, and its place in shared memory free
+    N_WFREE = 4,    // W's warps: W^T read
     N_GD = 5,       // [team] Gram products -> solve: G complete
-    N_GFREE = 7,    // solve -> Gram products: G read
+    N_GFREE = 7,    // solve and conversion -> Gram products: G and P^T read
     N_PD = 8,       // Gram products -> conversion: P^T complete (and nothing reads the block's K and Q as bf16 any more)
-    N_PFREE = 9,    // conversion -> Gram products: P^T read
     N_OD = 10,      // [2] output products -> output: O^T complete
-    N_END = 12      // [4] the two chain warps of a quarter
+    N_TFREE = 12,   // [3, as many as T has slots] output products -> solve: nothing reads the T in this slot any more
+    N_END = 12      // [4] the two chain warps of a quarter (when the walk is over, and with it the use of the three before)
 };
 __device__ __forceinline__ void named_arrive(int id, int nthreads) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(nthreads) : "memory"); }
 // (after a wait for a product's mbarrier, by a whole warp)
@@ -327,54 +399,102 @@ __device__ __forceinline__ void pass_on(int id, int nthreads) {
     tc_fence_before();
     named_arrive(id, nthreads);
 }
-enum {
-    B_SP = 0,       // chain: fp16 copy of S published
-    B_RD = 1,       // products: V^T - S K^T complete
-    B_UD = 2,       // products: U' complete
-    B_UP = 3,       // chain: its fp16 copy published
-    B_SD = 4,       // products: S complete
-    B_QD = 5,       // output products: Q S^T complete
-    B_OD = 6,       // [2] output products: O^T complete
-    B_OFREE = 8,    // [2] output: O^T read
-    B_GD = 10,      // Gram products: G and P^T complete
-    B_RP = 11,      // chain: the fp16 copy of R published
-    B_LAND = 12     // then [NS] each: a block's tiles landed, a block prepared, a block's stage free
-};
-
-// Products over several K-steps, descriptors by their low words (a stage's address changes nothing else); whole warp, converged, and one
-// election for all of them (an election each is half as many instructions again).
+// Products over several K-steps, by one elected thread, descriptors by their low words (a stage's address changes nothing else).  One election for all products of
+// a step and their commits: an election each is half as many instructions again, and a predicate on each instead of a branch around all twice as many.
 // Products execute in the order of their issue only where accumulator and shape are the same.  So all products that add to one
 // accumulator without a wait between them have the same N and the same columns: the upper triangles of T and P are zeros that are multiplied (a
-// product of few columns takes 26 - 32 cycles, one of 64 columns 35), and V^T comes in products of 64 columns each.
+// product of few columns takes 26 - 32 cycles, one of 64 columns 35).
 constexpr uint32_t DESC_HI = (1024u >> 4) | (1u << 14) | (2u << 29);          // SBO 1024 bytes, version, 128-byte swizzle
 __device__ __forceinline__ uint64_t desc_lo(uint32_t lo) { return ((uint64_t)DESC_HI << 32) | lo; }
 __device__ __forceinline__ uint32_t lo_of(uint32_t saddr, uint32_t slab_bytes = 16) { return (saddr >> 4) | (slab_bytes >> 4 << 16); }
-// D [128 x N] (+)= A (tensor memory; NEG: -A) B^T: B K-major (MN false) or MN-major, KSTEPS K-steps, slabs of B_ROWS rows
-template <bool MN, int N, int KSTEPS, int B_ROWS, bool NEG = false>
+// D [128 x N] (+)= A (tensor memory; NEG: -A) B^T: B K-major (MN false) or MN-major, KSTEPS K-steps, slabs of B_ROWS rows; GAP: columns of A between its
+// second and third K-step
+template <bool MN, int N, int KSTEPS, int B_ROWS, bool NEG = false, int GAP = 0>
 __device__ __forceinline__ void products_ta(uint32_t d, uint32_t a, uint32_t b_lo, bool acc) {
-    if (elect_one())
 #pragma unroll
     for (int kk = 0; kk < KSTEPS; ++kk)
-            mma_f16_ta(d, a + 8 * kk, desc_lo(b_lo + (kstep_off<MN ? L_SWMN : L_SWK, B_ROWS>(kk) >> 4)), make_idesc(N, false, MN, NEG), acc || kk > 0);
+        mma_f16_ta(d, a + 8 * kk + (kk >= 2 ? GAP : 0), desc_lo(b_lo + (kstep_off<MN ? L_SWMN : L_SWK, B_ROWS>(kk) >> 4)), make_idesc(N, false, MN, NEG), acc || kk > 0);
+}
+// D [128 x NB] = A^T T^T: A [NB rows][128 columns] and T in shared memory, fp16
+__device__ __forceinline__ void products_tt(uint32_t d, uint32_t a_lo, uint32_t t_lo) {
+#pragma unroll
+    for (int kk = 0; kk < NB / 16; ++kk)
+        mma_f16(d, desc_lo(a_lo + (kstep_off<L_SWMN, NB>(kk) >> 4)), desc_lo(t_lo + (kstep_off<L_SWK, NB>(kk) >> 4)), make_idesc(NB, true, false, false), kk > 0);
 }
 // D [64 x N] = A B^T, B [N rows] K-major bf16 in shared memory, in slabs of ROWS rows, A its first 64 rows
 template <int N, int K, int ROWS>
 __device__ __forceinline__ void products_ss(uint32_t d, uint32_t b_base) {
     constexpr uint32_t idesc = (make_idesc(N, false, false, false) & ~(31u << 24)) | (4u << 24) | (1u << 7) | (1u << 10);     // (64 rows, bf16)
     const uint32_t b = lo_of(b_base);
-    if (elect_one())
 #pragma unroll
     for (int kk = 0; kk < K / 16; ++kk)
-            mma_f16(d, desc_lo(b + (kstep_off<L_SWK, ROWS>(kk) >> 4)), desc_lo(b + (kstep_off<L_SWK, ROWS>(kk) >> 4)), idesc, kk > 0);
+        mma_f16(d, desc_lo(b + (kstep_off<L_SWK, ROWS>(kk) >> 4)), desc_lo(b + (kstep_off<L_SWK, ROWS>(kk) >> 4)), idesc, kk > 0);
+}
+__device__ __forceinline__ void commit_at(uint32_t bar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+
+// a warp's part of an operand in shared memory is written
+__device__ __forceinline__ void publish_smem(uint32_t b, int lane) {
+    fence_async_smem();
+    mbar_arrive_at(b);
+}
+// PIECES 16-byte pieces of each of THREADS threads: bf16 -> fp16 in place (elementwise, so the swizzled layout is untouched), several per
+// round, so that their loads are in flight together
+template <int PIECES, int THREADS>
+__device__ __forceinline__ void convert_pieces(uint8_t* at, int tid) {
+    uint4* p = (uint4*)at + tid;
+    constexpr int ROUND = PIECES % 4 == 0 ? 4 : PIECES % 3 == 0 ? 3 : 5;
+    static_assert(PIECES % ROUND == 0, "pieces per round");
+#pragma unroll 1
+    for (int e0 = 0; e0 < PIECES; e0 += ROUND) {
+        uint4 y[ROUND];
+#pragma unroll
+        for (int e = 0; e < ROUND; ++e) y[e] = p[(e0 + e) * THREADS];
+#pragma unroll
+        for (int e = 0; e < ROUND; ++e) p[(e0 + e) * THREADS] = bf16_to_half8(y[e]);
+    }
+}
+
+// r = (I - N)^{-1} of a strictly lower triangular 16 x 16 block as an accumulator fragment, from the A-operand fragments of N and N^T: the product
+// (I + N)(I + N^2)(I + N^4)(I + N^8) as far as N's powers are not zero (LAST: the last of them; `deep`: up to N^8).  The diagonals of N and N^2 are +0, so that adding
+// the identity (`one`: its part of elements 0 and 3) is an OR, exact in fp16, and the first two factors need no start value.
+template <int LAST>
+__device__ __forceinline__ void neumann_product(float (&r)[2][4], const uint32_t (&n)[4], const uint32_t (&nt)[4], uint32_t one, bool deep) {
+    auto mul = [](float (&c)[2][4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1, uint32_t b2, uint32_t b3) {     // (b: fragment of the second factor transposed)
+        mma_acc(c[0], a, b0, b2, false);
+        mma_acc(c[1], a, b1, b3, false);
+    };
+    float c[2][4];
+    uint32_t p[4], pt[4], q[4];                                   // the power at hand, its transpose, what has been multiplied
+    mul(c, nt, n[0], n[1], n[2], n[3]);                           // (N^2)^T
+    frag_pack(pt, c);
+    q[0] = n[0] | one; q[1] = n[1]; q[2] = n[2]; q[3] = n[3] | one;
+    mul(r, q, pt[0] | one, pt[1], pt[2], pt[3] | one);
+    if (LAST == 2 && !deep) return;
+    mul(c, n, nt[0], nt[1], nt[2], nt[3]);                        // N^2
+    frag_pack(p, c);
+    float c4[2][4];
+    mul(c, pt, p[0], p[1], p[2], p[3]);                           // (N^4)^T
+    if (deep) mul(c4, p, pt[0], pt[1], pt[2], pt[3]);             // N^4
+    frag_pack(q, r);
+    frag_pack(pt, c);
+    frag_mul(r, q, pt);                                           // (r stays fp32: only what is added to it has passed through fp16)
+    if (!deep) return;
+    frag_pack(p, c4);
+    mul(c, pt, p[0], p[1], p[2], p[3]);                           // (N^8)^T
+    frag_pack(q, r);
+    frag_pack(pt, c);
+    frag_mul(r, q, pt);
 }
 
 // ---------------------------------------------------------------------------------------------------------------------
 // solve team: T of blocks b = team, team + TEAMS, ...
 // ---------------------------------------------------------------------------------------------------------------------
-template <int DK, int R, int JS, int NS>
+template <int DK, bool W, int R, int JS>
 __device__ __forceinline__ void solve_role(const ChainGeo& g, const ChainPart& part, const __nv_bfloat16* __restrict__ beta, uint8_t* smem,
-                                           uint64_t* full, long long seq, int team, int tid) {
-    using CFG = ChainCfg<DK, R, JS, NS>;
+                                           uint32_t bar, long long seq, int team, int tid) {
+    using CFG = ChainCfg<DK, W, R, JS>;
     using SM = ChainSmem<DK, R, JS>;
     constexpr int C = SM::C;
     const int w = tid >> 5, lane = tid & 31, gq = lane >> 2, t4 = lane & 3;
@@ -391,18 +511,29 @@ __device__ __forceinline__ void solve_role(const ChainGeo& g, const ChainPart& p
         return x;
     };
     uint16_t breg = team < part.nblk ? read_beta(team) : 0;
-    const int lim0 = (16 * w + gq) / g.rm * g.rm, lim1 = (16 * w + gq + 8) / g.rm * g.rm;      // (edges of the strict mask)
+    // the strict mask on the packed values of the diagonal tile, and of the one left of it (groups of three rows reach across the edge of a tile)
+    uint32_t keep[4], keep_left[4];
+    {
+        const int lim0 = (16 * w + gq) / g.rm * g.rm - 16 * w, lim1 = (16 * w + gq + 8) / g.rm * g.rm - 16 * w;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int c = 8 * (e / 2) + 2 * t4, lim = e % 2 ? lim1 : lim0;
+            keep[e] = (c < lim ? 0xFFFFu : 0u) | (c + 1 < lim ? 0xFFFF0000u : 0u);
+            keep_left[e] = (c < lim + 16 ? 0xFFFFu : 0u) | (c + 1 < lim + 16 ? 0xFFFF0000u : 0u);
+        }
+    }
+    const uint32_t one = gq == 2 * t4 ? 0x3C00u : gq == 2 * t4 + 1 ? 0x3C000000u : 0u;      // the identity's part of elements 0 and 3 of a fragment
 #pragma unroll 1
     for (int b = team; b < part.nblk; b += TEAMS) {
-        const int st = b % NS;
-        const uint32_t t_b = smem_u32(smem) + st * SM::stage + SM::t_off;
+        const int ts = b % CFG::NT;
+        const uint32_t t_b = smem_u32(smem) + CFG::t_off + ts * SM::t_bytes;
         // (two in turn: another warp may still be scaling T of the block before)
         float* sBeta = (float*)(smem + CFG::beta_off + team * 512 + (b / TEAMS & 1) * 256);
         if (tid < NB) sBeta[tid] = __uint_as_float((uint32_t)breg << 16);
         if (b + TEAMS < part.nblk) breg = read_beta(b + TEAMS);
         named_bar(N_GD + team, 160);                              // (and the step sizes)
         tc_fence_after();
-        const uint32_t t_g = T_G + ((uint32_t)(32 * w) << 16);
+        const uint32_t t_g = T_G<W, SM::CP> + ((uint32_t)(32 * w) << 16);
         uint32_t x[8];                                            // 16 columns of G, rows 16 w .. 16 w + 15, as mma.sync's accumulators
         const int m0 = 16 * w + gq, m1 = m0 + 8;
         if (g.exact) {
@@ -417,43 +548,32 @@ __device__ __forceinline__ void solve_role(const ChainGeo& g, const ChainPart& p
                 }
             __syncwarp();
         }
-        // ---- A = Mstrict (.) (diag(beta) G): its blocks left of the diagonal go to the other warps, the diagonal one stays as an A operand
-        const float b0 = sBeta[m0], b1 = sBeta[m1];
-        uint32_t af[4];
+        // ---- N = -A = -Mstrict (.) (diag(beta) G): its blocks left of the diagonal go to the other warps, the diagonal one stays as an A operand
+        const float b0 = -sBeta[m0], b1 = -sBeta[m1];
+        uint32_t nf[4];
 #pragma unroll 1
         for (int nb = 0;; ++nb) {
             tmem_ld_frag<16>(t_g + 16 * nb, x);
             tmem_ld_wait();
-            float v[2][4];
-            const int c0 = 16 * nb + 2 * t4;
 #pragma unroll
-            for (int h = 0; h < 2; ++h)
+            for (int e = 0; e < 4; ++e) nf[e] = pack_h2((e % 2 ? b1 : b0) * __uint_as_float(x[2 * e]), (e % 2 ? b1 : b0) * __uint_as_float(x[2 * e + 1]));
+            if (R == 3 && nb + 1 == w)
 #pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    v[h][e] = b0 * __uint_as_float(x[4 * h + e]);
-                    v[h][2 + e] = b1 * __uint_as_float(x[4 * h + 2 + e]);
-                }
-            if (nb == w || R == 3)                                // (groups of three rows reach across the edge of a tile)
-#pragma unroll
-                for (int h = 0; h < 2; ++h)
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        if (c0 + 8 * h + e >= lim0) v[h][e] = 0.f;
-                        if (c0 + 8 * h + e >= lim1) v[h][2 + e] = 0.f;
-                    }
-            frag_pack(af, v);
+                for (int e = 0; e < 4; ++e) nf[e] &= keep_left[e];
             if (nb == w) break;
-            stmatrix_x4(xs_a + nb * 512, af);
+            stmatrix_x4(xs_a + nb * 512, nf);
         }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) nf[e] &= keep[e];
         tc_fence_before();
-        if (b + 1 < part.nblk) named_arrive(N_GFREE, 160);
-        // ---- D_w = (I + A_ww)^{-1} (Neumann product, A nilpotent) for the other warps
+        if (b + 1 < part.nblk) named_arrive(N_GFREE, 288);
+        // ---- D_w = (I - N_ww)^{-1} (Neumann product, N nilpotent) for the other warps
         uint32_t y0[4];                                           // X_ww^T as an A operand
         {
-            uint32_t at[4], df[4];
+            uint32_t nt[4], df[4];
             float dd[2][4];
-            at[0] = movmatrix(af[0]); at[1] = movmatrix(af[2]); at[2] = movmatrix(af[1]); at[3] = movmatrix(af[3]);
-            neumann16(dd, af, at, lane, g.rm == 1);
+            nt[0] = movmatrix(nf[0]); nt[1] = movmatrix(nf[2]); nt[2] = movmatrix(nf[1]); nt[3] = movmatrix(nf[3]);
+            neumann_product<(R == 4 ? 2 : 4)>(dd, nf, nt, one, g.rm == 1);
             frag_pack(df, dd);
             stmatrix_x4(xs_a + w * 512, df);
             y0[0] = movmatrix(df[0]); y0[1] = movmatrix(df[2]); y0[2] = movmatrix(df[1]); y0[3] = movmatrix(df[3]);
@@ -463,10 +583,11 @@ __device__ __forceinline__ void solve_role(const ChainGeo& g, const ChainPart& p
                 dd[h][0] *= bb.x; dd[h][1] *= bb.y; dd[h][2] *= bb.x; dd[h][3] *= bb.y;
             }
             frag_pack(df, dd);
+            if (W && b >= CFG::NT) named_bar(N_TFREE + ts, 160);
             stmatrix_x4(t_b + w * 2048 + (offA ^ (uint32_t)(w << 5)), df);
         }
         named_bar(N_TEAM + team, 128);
-        // ---- down the column: X_iw = -D_i sum_k A_ik X_kw, transposed, in registers; T = X diag(beta)
+        // ---- down the column: X_iw = D_i sum_k N_ik X_kw, transposed, in registers; T = X diag(beta)
         uint32_t y[3][4];                                         // X_kw^T of k = w, w + 1, w + 2
 #pragma unroll
         for (int e = 0; e < 4; ++e) y[0][e] = y0[e];
@@ -483,30 +604,30 @@ __device__ __forceinline__ void solve_role(const ChainGeo& g, const ChainPart& p
                 mma_acc(c[1], y[k], a[2], a[3], k > 0);
             }
 #pragma unroll
-            for (int e = 0; e < 4; ++e) f[e] = pack_h2(-c[e / 2][e % 2 * 2], -c[e / 2][e % 2 * 2 + 1]);
+            for (int e = 0; e < 4; ++e) f[e] = pack_h2(c[e / 2][e % 2 * 2], c[e / 2][e % 2 * 2 + 1]);
             ldmatrix_x4(a, xs_n + xs_block(i, i));
             mma_acc(z[0], f, a[0], a[1], false);
             mma_acc(z[1], f, a[2], a[3], false);
             if (n < 3) frag_pack(y[n < 3 ? n : 0], z);
 #pragma unroll
-            for (int e = 0; e < 4; ++e) f[e] = pack_h2(z[e / 2][e % 2 * 2] * (e % 2 ? b1 : b0), z[e / 2][e % 2 * 2 + 1] * (e % 2 ? b1 : b0));
+            for (int e = 0; e < 4; ++e) f[e] = pack_h2(-z[e / 2][e % 2 * 2] * (e % 2 ? b1 : b0), -z[e / 2][e % 2 * 2 + 1] * (e % 2 ? b1 : b0));
             stmatrix_x4_trans(t_b + i * 2048 + (offN ^ (uint32_t)(w << 5)), f);
         }
-        fence_async_smem();
-        mbar_arrive(&full[st]);
+        publish_smem(bar + 8 * ((W ? CFG::TDONE : CFG::FULL) + ts), lane);
     }
 }
 
 // Conversion: K and Q of every block to fp16 in place, once the Gram products have read them as they came, and P.  Four warps.
-template <int DK, int R, int JS, int NS>
-__device__ __forceinline__ void convert_role(const ChainPart& part, uint8_t* smem, uint64_t* full, int tid) {
+template <int DK, bool W, int R, int JS>
+__device__ __forceinline__ void convert_role(const ChainPart& part, uint8_t* smem, uint32_t bar, int tid) {
     using SM = ChainSmem<DK, R, JS>;
+    using CFG = ChainCfg<DK, W, R, JS>;
     constexpr int CP = SM::CP;
     const int w = tid >> 5, lane = tid & 31, gq = lane >> 2, t4 = lane & 3;
     const uint32_t p_at = smem_u32(smem) + SM::p_off + (lane_off((lane & 7) + ((lane >> 4) << 3), (lane >> 3) & 1) ^ (uint32_t)(w << 5));
+    int st = 0;
 #pragma unroll 1
     for (int b = 0; b < part.nblk; ++b) {
-        const int st = b % NS;
         uint8_t* sg = smem + st * SM::stage;
         named_bar(N_PD, 160);
         tc_fence_after();
@@ -515,67 +636,158 @@ __device__ __forceinline__ void convert_role(const ChainPart& part, uint8_t* sme
 #pragma unroll 1
         for (int t0 = 0; t0 < CP; t0 += PC) {
             uint32_t x[PC / 2];
-            tmem_ld_frag<PC>(T_P + t0 + ((uint32_t)(32 * w) << 16), x);
+            tmem_ld_frag<PC>(T_P<W, CP> + t0 + ((uint32_t)(32 * w) << 16), x);
             tmem_ld_wait();
             if (t0 + PC == CP) {
                 tc_fence_before();
-                if (b + 1 < part.nblk) named_arrive(N_PFREE, 160);
+                if (b + 1 < part.nblk) named_arrive(N_GFREE, 288);
             }
 #pragma unroll
             for (int n = 0; n < PC / 8; n += 2) {
                 if (16 * w >= (t0 + 8 * n + 16) * R) continue;    // (nothing of the block of 16 tokens sees these rows: zeros from the start)
                 uint32_t y[4];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const int t = t0 + 8 * (n + e / 2) + 2 * t4, m = 16 * w + 8 * (e % 2) + gq, at = 4 * n + 2 * e;
-                    y[e] = pack_h2(m < (t + 1) * R ? __uint_as_float(x[at]) : 0.f, m < (t + 2) * R ? __uint_as_float(x[at + 1]) : 0.f);
-                }
+                for (int e = 0; e < 4; ++e) y[e] = pack_h2(__uint_as_float(x[4 * n + 2 * e]), __uint_as_float(x[4 * n + 2 * e + 1]));
+                if (16 * w + 15 >= (t0 + 8 * n + 1) * R)          // (not all of them are seen by all tokens of the tile)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const int t = t0 + 8 * (n + e / 2) + 2 * t4, m = 16 * w + 8 * (e % 2) + gq;
+                        y[e] &= (m < (t + 1) * R ? 0xFFFFu : 0u) | (m < (t + 2) * R ? 0xFFFF0000u : 0u);
+                    }
                 stmatrix_x4_trans(p_at + st * SM::stage + t0 * 128 + n * 1024, y);
             }
         }
-        // ---- bf16 -> fp16 (elementwise, so the swizzled layout is untouched), several pieces per round, so that their loads are in flight together
-        uint4* p = (uint4*)(sg + SM::k_off) + tid;
-        constexpr int PIECES = (SM::k_bytes + SM::q_bytes) / 2048, ROUND = PIECES % 4 == 0 ? 4 : PIECES % 3 == 0 ? 3 : 5;
-        static_assert(PIECES % ROUND == 0, "pieces per round");
-#pragma unroll 1
-        for (int e0 = 0; e0 < PIECES; e0 += ROUND) {
-            uint4 y[ROUND];
-#pragma unroll
-            for (int e = 0; e < ROUND; ++e) y[e] = p[(e0 + e) * 128];
-#pragma unroll
-            for (int e = 0; e < ROUND; ++e) p[(e0 + e) * 128] = bf16_to_half8(y[e]);
-        }
-        fence_async_smem();
-        mbar_arrive(&full[st]);
+        convert_pieces<(SM::k_bytes + SM::q_bytes) / 2048, 128>(sg + SM::k_off, tid);
+        publish_smem(bar + 8 * (CFG::FULL + st), lane);
+        if (++st == CFG::NS) st = 0;
     }
 }
 
-// Gram products (one warp): G = K K^T and K Q^T from the bf16 tiles as they landed, in products of 64 rows and NB + CP columns.
-template <int DK, int R, int JS, int NS>
-__device__ __forceinline__ void gram_role(const ChainPart& part, int* err, uint8_t* smem, uint64_t* bar, uint64_t* land) {
+// W^T = K^T T^T of every block (rows i, columns m): its products, and out of tensor memory as the fp16 operand W.  Four warps, the first of which issues; at
+// d_k = 64 the accumulator has its rows twice, and a warp takes half of the columns.
+template <int DK, bool W, int R, int JS>
+__device__ __forceinline__ void w_role(const ChainPart& part, int* err, uint8_t* smem, uint32_t bar, int tid) {
     using SM = ChainSmem<DK, R, JS>;
-    int st = 0, phase = 0;
-    bool ok = true;
+    using CFG = ChainCfg<DK, W, R, JS>;
+    const int w = tid >> 5, lane = tid & 31, i = tid & (DK - 1);
+    const int m0 = DK == 128 ? 0 : 32 * (w >> 1);
+    const uint32_t t_w = T_W<W, SM::CP> + ((uint32_t)(32 * w) << 16), smem_b = smem_u32(smem);
+    RingPos<CFG::NS> ks;
+    RingPos<CFG::NT> ts;
+    RingPos<CFG::NW> ws;
+    Waits waits(bar);
 #pragma unroll 1
     for (int b = 0; b < part.nblk; ++b) {
-        ok = ok && mbar_wait_tries<true>(&land[st], phase, err, 316);
-        if (b > 0) {
-            named_bar(N_GFREE, 160);
-            named_bar(N_PFREE, 160);
+        uint8_t* row = smem + CFG::w_off + ws.i * SM::w_bytes + i * 128;
+        if (b > 0) named_bar(N_WFREE, 128);                       // (the accumulator has been read)
+        if (w == 0) {
+            waits.wait(CFG::FULL + ks.i, ks.phase, 324);
+            waits.wait(CFG::TDONE + ts.i, ts.phase, 329);
+            tc_fence_after();
+            if (waits.ok() && elect_one()) {
+                products_tt(T_W<W, SM::CP>, lo_of(smem_b + ks.i * SM::stage + SM::k_off, DK == 128 ? SM::rows * 128 : 0), lo_of(smem_b + CFG::t_off + ts.i * SM::t_bytes));
+                commit_at(bar + 8 * B_WD);
+            }
+            __syncwarp();
+            if (b >= CFG::NW) waits.wait(CFG::WFREE + ws.i, ws.phase ^ 1, 318);
+            waits.wait(B_WD, b & 1, 330);
+            tc_fence_after();
+            tc_fence_before();
         }
+        named_bar(N_WD, 128);
         tc_fence_after();
-        if (ok) {
-            products_ss<SM::rows, DK, SM::rows>(T_G, smem_u32(smem + st * SM::stage));
-            commit_uni(&bar[B_GD]);
+#pragma unroll 1
+        for (int c = m0; c < m0 + DK / 2; c += 32) {
+            uint32_t x[32];
+            tmem_ld32(t_w + c, x);
+            tmem_ld_wait();
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                uint32_t y[4];
+#pragma unroll
+                for (int n = 0; n < 4; ++n) y[n] = pack_h2(__uint_as_float(x[8 * e + 2 * n]), __uint_as_float(x[8 * e + 2 * n + 1]));
+                *(uint4*)(row + ((((c >> 3) + e) ^ (i & 7)) << 4)) = make_uint4(y[0], y[1], y[2], y[3]);
+            }
         }
-        ok = ok && mbar_wait_tries<true>(&bar[B_GD], b & 1, err, 311);
+        tc_fence_before();
+        publish_smem(bar + 8 * (CFG::WDONE + ws.i), lane);
+        ks.next();
+        ts.next();
+        ws.next();
+    }
+    if (!waits.ok()) atomicCAS(err, 0, waits.code);
+}
+
+// Gram products (one warp): G = K K^T and K Q^T from the bf16 tiles as they landed, in products of 64 rows and NB + CP columns.
+template <int DK, bool W, int R, int JS>
+__device__ __forceinline__ void gram_role(const ChainPart& part, int* err, uint8_t* smem, uint32_t bar) {
+    using SM = ChainSmem<DK, R, JS>;
+    using CFG = ChainCfg<DK, W, R, JS>;
+    const uint32_t smem_b = smem_u32(smem);
+    RingPos<CFG::NS> ks;
+    Waits waits(bar);
+#pragma unroll 1
+    for (int b = 0; b < part.nblk; ++b) {
+        waits.wait(CFG::LAND + ks.i, ks.phase, 316);
+        if (b > 0) named_bar(N_GFREE, 288);
+        tc_fence_after();
+        if (waits.ok() && elect_one()) {
+            products_ss<SM::rows, DK, SM::rows>(T_G<W, SM::CP>, smem_b + ks.i * SM::stage);
+            commit_at(bar + 8 * B_GD);
+        }
+        __syncwarp();
+        waits.wait(B_GD, b & 1, 311);
         pass_on(N_GD + b % TEAMS, 160);
         named_arrive(N_PD, 160);
-        if (++st == NS) {
-            st = 0;
-            phase ^= 1;
+        ks.next();
+    }
+    if (!waits.ok()) atomicCAS(err, 0, waits.code);
+}
+
+// The copies (one warp).  K and Q of a block are asked for when the block before in their stage is done, and V with them, or in the W form when V^T T^T of the
+// block before it in its slot is; rows past the sequence arrive as zeros.  (Issuing a copy takes the warp some 200 cycles, five a block at d = 128.)
+template <int DK, bool W, int R, int JS>
+__device__ __forceinline__ void load_role(const ChainMaps& maps, int* err, uint8_t* smem, uint32_t bar, int seq, const ChainPart& part) {
+    using SM = ChainSmem<DK, R, JS>;
+    using CFG = ChainCfg<DK, W, R, JS>;
+    constexpr int NS = CFG::NS, NV = CFG::NV;
+    const uint32_t smem_b = smem_u32(smem);
+    Waits waits(bar);
+    RingPos<NS> ks;
+    RingPos<NV> vs;
+    // (c: the block that the chain is in, or before the first)
+#pragma unroll 1
+    for (int c = -NS; c + NV < part.nblk; ++c) {
+        if (W && c + NV >= 0) {
+            if (!part.response) {
+                if (c >= 0) waits.wait(CFG::VFREE + vs.i, vs.phase ^ 1, 342);
+                const uint32_t land = bar + 8 * (CFG::VLAND + vs.i);
+                if (waits.ok() && elect_one()) {
+                    mbar_expect_tx_at(land, SM::v_bytes);
+                    tma_load_4d(smem_b + CFG::v_off + vs.i * SM::v_bytes, &maps.v, 0, (part.b0 + c + NV) * SM::C * R, 0, seq, land);
+                }
+                __syncwarp();
+            }
+            vs.next();
+        }
+        if (c + NS < part.nblk) {
+            if (c >= 0) waits.wait(CFG::EMPTY + ks.i, ks.phase ^ 1, 341);
+            const uint32_t land = bar + 8 * (CFG::LAND + ks.i), at = smem_b + ks.i * SM::stage;
+            const int tok = (part.b0 + c + NS) * SM::C;
+            if (waits.ok() && elect_one()) {
+                mbar_expect_tx_at(land, SM::tx_bytes + (W || part.response ? 0 : SM::v_bytes));
+#pragma unroll
+                for (int h = 0; h < DK / 64; ++h) {
+                    tma_load_4d(at + SM::k_off + h * (SM::rows * 128), &maps.k, 0, tok * R, h, seq, land);
+                    tma_load_4d(at + SM::q_off + h * (SM::rows * 128), &maps.q, 0, tok, h, seq, land);
+                }
+                if (!W && !part.response) tma_load_4d(smem_b + CFG::v_off + ks.i * SM::v_bytes, &maps.v, 0, tok * R, 0, seq, land);
+            }
+            __syncwarp();
+            ks.next();
         }
     }
+    if (!waits.ok()) atomicCAS(err, 0, waits.code);
 }
 
 // ---------------------------------------------------------------------------------------------------------------------
@@ -601,12 +813,13 @@ __device__ __forceinline__ void to_operand(uint32_t src, uint32_t dst) {
 }
 
 // warp `warp` of eight: rows j = 32 (warp & 3) + lane, half warp >> 2 of the columns of everything
-template <int DK>
-__device__ __forceinline__ void chain_role(const ChainPart& part, int* err, uint64_t* bar, int warp, int lane) {
+template <int DK, bool W, int CP>
+__device__ __forceinline__ int chain_role(const ChainPart& part, uint32_t bar, int warp, int lane) {
     constexpr int HC = DK / 2;                                    // columns i of this warp
     const int h = warp >> 2, j = 32 * (warp & 3) + lane;
     const uint32_t lanes = (uint32_t)(32 * (warp & 3)) << 16;
-    const uint32_t t_s = T_S + h * HC + lanes, t_s16 = T_S16 + h * HC / 2 + lanes, t_u16 = T_U16 + 16 * h + lanes;
+    const uint32_t t_s = T_S + h * HC + lanes, t_s16 = T_S16 + h * HC / 2 + lanes;
+    const uint32_t t_u = T_U + 32 * h + lanes, t_u16 = T_U16<W, CP> + (U_INPLACE<W, CP> ? 32 : 16) * h + lanes;
 #pragma unroll 1
     for (int c = 0; c < HC; c += 16) {
         uint32_t x[16], y[8];
@@ -622,160 +835,218 @@ __device__ __forceinline__ void chain_role(const ChainPart& part, int* err, uint
         tmem_st_wait();
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&bar[b]);
+        if (lane == 0) mbar_arrive_at(bar + 8 * b);
     };
-    const uint32_t t_r = T_R + 32 * h + lanes, t_r16 = T_R16 + 16 * h + lanes;
 #pragma unroll 1
     for (int b = 0; b < part.nblk; ++b) {
         publish(B_SP);
-        if (!mbar_wait_tries<false>(&bar[B_RD], b & 1, err, 312)) return;
+        if constexpr (!W) {
+            if (!mbar_wait_tries<false>(bar + 8 * B_RD, b & 1)) return 312;
+            tc_fence_after();
+            to_operand<32, false>(t_u, T_R16 + 16 * h + lanes);
+            publish(B_RP);
+        }
+        if (!mbar_wait_tries<false>(bar + 8 * B_UD, b & 1)) return 313;
         tc_fence_after();
-        to_operand<32, false>(t_r, t_r16);
-        publish(B_RP);
-        if (!mbar_wait_tries<false>(&bar[B_UD], b & 1, err, 313)) return;
-        tc_fence_after();
-        to_operand<32, false>(t_r, t_u16);
+        to_operand<32, false>(t_u, t_u16);
         publish(B_UP);
-        if (!mbar_wait_tries<false>(&bar[B_SD], b & 1, err, 314)) return;
+        if (!mbar_wait_tries<false>(bar + 8 * B_SD, b & 1)) return 314;
         tc_fence_after();
-        if (b + 1 == part.nblk) return;
+        if (b + 1 == part.nblk) return 0;
         to_operand<HC, true>(t_s, t_s16);
     }
+    return 0;
 }
 
-// The products of the chain (one warp).
-template <int DK, int R, int DV, int NS>
-__device__ __forceinline__ void mma_role(const ChainPart& part, int* err, uint8_t* smem, uint64_t* bar) {
-    using CFG = ChainCfg<DK, R, DV, NS>;
+// The products of the chain (one warp).  Returns the code of the wait that ran out, or 0.
+template <int DK, bool W, int R, int DV>
+__device__ __forceinline__ int mma_role(const ChainPart& part, uint8_t* smem, uint32_t bar) {
+    using CFG = ChainCfg<DK, W, R, DV>;
     using SM = ChainSmem<DK, R, DV>;
-    constexpr int V_SLAB = NB * 128, K_SLAB = SM::rows * 128, OB = O_BUFS<SM::CP>;
-    uint64_t *land = bar + B_LAND, *full = land + NS, *empty = full + NS;
-    const uint32_t smem_b = smem_u32(smem), id_b = smem_b + CFG::id_off;
-    const uint32_t t_r = T_R;
-    // V^T of a block into the accumulator, as V^T times an identity, both bf16 (V as it came).  At d_v = 64 the tile's 64 columns are read
-    // twice: rows j past d_v are nobody's.
-    auto put_v = [&](int st) {
-        const uint32_t v_lo = lo_of(smem_b + st * SM::stage + SM::v_off, DV == 128 ? V_SLAB : 0);
-        constexpr uint32_t idesc = make_idesc(NB, true, false, false) | (1u << 7) | (1u << 10);
-        if (elect_one())
-#pragma unroll
-        for (int c = 0; c < 4; ++c)
-            mma_f16(t_r, desc_lo(v_lo + c * (2048 >> 4)), IdStrip::desc(id_b, c), idesc, c > 0);
-    };
-    int st = 0, phase = 0;
+    constexpr int V_SLAB = NB * 128, K_SLAB = SM::rows * 128, CP = SM::CP, OB = O_BUFS<CP>;
+    constexpr bool INPLACE = U_INPLACE<W, CP>;
+    const uint32_t smem_b = smem_u32(smem);
+    RingPos<CFG::NS> ks;
+    RingPos<CFG::NV> vs;
+    RingPos<CFG::NT> ts;
+    RingPos<CFG::NW> ws;
+    auto wait = [&](int which, int parity) { return mbar_wait_tries<false>(bar + 8 * which, (uint32_t)parity); };
 #pragma unroll 1
     for (int b = 0; b < part.nblk; ++b) {
-        const uint32_t sg = smem_b + st * SM::stage, k_lo = lo_of(sg + SM::k_off), kt_lo = lo_of(sg + SM::k_off, K_SLAB), t_lo = lo_of(sg + SM::t_off);
-        // ---- V^T (the accumulator's last reader, the chain warps' conversion of U' of the block before, is done)
-        if (!part.response) {
-            if (!mbar_wait_tries<false>(&land[st], phase, err, 327)) return;
+        const uint32_t k_at = smem_b + ks.i * SM::stage + SM::k_off, v_lo = lo_of(smem_b + CFG::v_off + vs.i * SM::v_bytes, DV == 128 ? V_SLAB : 0),
+                       t_lo = lo_of(smem_b + CFG::t_off + ts.i * SM::t_bytes);
+        // (at d_v = 64 the 64 columns of V's tile are read twice: rows j past d_v are nobody's)
+        if constexpr (W) {
+            // ---- U'^T = V^T T^T (W is there, and so T; the accumulator's last reader, the chain warps' conversion of U' of the block before, is done; its
+            //      fp16 pairs' readers are)
+            if (INPLACE && b > 0 && (!wait(B_SD, (b - 1) & 1) || !wait(B_OD + (b - 1) % OB, ((b - 1) / OB) & 1))) return 315;
+            if (!wait(CFG::WDONE + ws.i, ws.phase)) return 326;
+            if (!part.response) {
+                tc_fence_after();
+                if (elect_one()) {
+                    products_tt(T_U, v_lo, t_lo);
+                    commit_at(bar + 8 * (CFG::VFREE + vs.i));
+                }
+                __syncwarp();
+            }
+            // ---- ... - S W^T
+            // (U' completes only after the last reader of the block before's, P U', so that the chain warps need not wait for that)
+            if (!INPLACE && b > 0 && !wait(B_OD + (b - 1) % OB, ((b - 1) / OB) & 1)) return 319;
+            if (!wait(B_SP, b & 1)) return 323;
             tc_fence_after();
-            put_v(st);
+            if (elect_one()) {
+                products_ta<true, NB, DK / 16, DK>(T_U, T_S16, lo_of(smem_b + CFG::w_off + ws.i * SM::w_bytes), !part.response);
+                commit_at(bar + 8 * B_UD);
+                commit_at(bar + 8 * (CFG::WFREE + ws.i));
+            }
+            __syncwarp();
+        } else {
+            // ---- V^T into the accumulator, as V^T times an identity, both bf16 (V as it came; the accumulator's last reader is done)
+            if (!part.response) {
+                if (!wait(CFG::LAND + ks.i, ks.phase)) return 327;
+                tc_fence_after();
+                if (elect_one()) {
+                    constexpr uint32_t idesc = make_idesc(NB, true, false, false) | (1u << 7) | (1u << 10);
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) mma_f16(T_U, desc_lo(v_lo + c * (2048 >> 4)), IdStrip::desc(smem_b + CFG::id_off, c), idesc, c > 0);
+                }
+                __syncwarp();
+            }
+            // ---- R = V^T - S K^T
+            if (!wait(CFG::FULL + ks.i, ks.phase)) return 322;
+            if (!wait(B_SP, b & 1)) return 323;
+            tc_fence_after();
+            if (elect_one()) {
+                products_ta<false, NB, DK / 16, SM::rows>(T_U, T_S16, lo_of(k_at), !part.response);
+                commit_at(bar + 8 * B_RD);
+            }
+            __syncwarp();
+            // ---- U'^T = R T^T
+            // (U' completes only after the last reader of the block before's, P U', so that the chain warps need not wait for that)
+            if (b > 0 && !wait(B_OD + (b - 1) % OB, ((b - 1) / OB) & 1)) return 319;
+            if (!wait(B_RP, b & 1)) return 326;
+            tc_fence_after();
+            if (elect_one()) {
+                products_ta<false, NB, NB / 16, NB>(T_U, T_R16, t_lo, false);
+                commit_at(bar + 8 * B_UD);
+            }
+            __syncwarp();
         }
-        if (!mbar_wait_tries<false>(&full[st], phase, err, 322) || !mbar_wait_tries<false>(&bar[B_SP], b & 1, err, 323)) return;
-        tc_fence_after();
-        // ---- R = V^T - S K^T
-        products_ta<false, NB, DK / 16, SM::rows>(t_r, T_S16, k_lo, !part.response);
-        commit_uni(&bar[B_RD]);
-        // ---- U'^T = R T^T
-        // (U' completes only after the last reader of the block before's, P U', so that the chain warps need not wait for that)
-        if (b > 0 && !mbar_wait_tries<false>(&bar[B_OD + (b - 1) % OB], ((b - 1) / OB) & 1, err, 319)) return;
-        if (!mbar_wait_tries<false>(&bar[B_RP], b & 1, err, 326)) return;
-        tc_fence_after();
-        products_ta<false, NB, NB / 16, NB>(t_r, T_R16, t_lo, false);
-        commit_uni(&bar[B_UD]);
         // ---- S += U'^T K
         // (and S only after Q S^T)
-        if (!mbar_wait_tries<false>(&bar[B_QD], b & 1, err, 320) || !mbar_wait_tries<false>(&bar[B_UP], b & 1, err, 328)) return;
+        if (!wait(B_QD, b & 1)) return 320;
+        if (!wait(B_UP, b & 1)) return 328;
         tc_fence_after();
-        products_ta<true, DK, NB / 16, SM::rows>(T_S, T_U16, kt_lo, true);
-        commit_uni(&bar[B_SD]);
-        commit_uni(&empty[st]);
-        if (++st == NS) {
-            st = 0;
-            phase ^= 1;
+        if (elect_one()) {
+            products_ta<true, DK, NB / 16, SM::rows, false, INPLACE ? 16 : 0>(T_S, T_U16<W, CP>, lo_of(k_at, K_SLAB), true);
+            commit_at(bar + 8 * B_SD);
+            commit_at(bar + 8 * (CFG::EMPTY + ks.i));
         }
+        __syncwarp();
+        ks.next();
+        vs.next();
+        ts.next();
+        ws.next();
     }
+    return 0;
 }
 
 // The products of the output (one warp): O^T = S Q^T + U'^T P^T with the state before the update.
-template <int DK, int R, int DV, int NS>
-__device__ __forceinline__ void mma_out_role(const ChainPart& part, int* err, uint8_t* smem, uint64_t* bar) {
+template <int DK, bool W, int R, int DV>
+__device__ __forceinline__ void mma_out_role(const ChainPart& part, int* err, uint8_t* smem, uint32_t bar) {
     using SM = ChainSmem<DK, R, DV>;
+    using CFG = ChainCfg<DK, W, R, DV>;
     constexpr int CP = SM::CP, OB = O_BUFS<CP>;
-    uint64_t *full = bar + B_LAND + NS, *empty = full + NS;
     const uint32_t smem_b = smem_u32(smem);
     const int parties = part.width + 32;
-    int st = 0, phase = 0;
-    bool ok = true;
+    RingPos<CFG::NS> ks;
+    RingPos<CFG::NT> ts;
+    RingPos<OB> os;
+    Waits waits(bar);
 #pragma unroll 1
     for (int b = 0; b < part.nblk; ++b) {
-        const uint32_t sg = smem_b + st * SM::stage, t_o = o_cols<CP>(b);
-        ok = ok && mbar_wait_tries<true>(&full[st], phase, err, 351) && mbar_wait_tries<true>(&bar[B_SP], b & 1, err, 352);
-        if (b >= OB) ok = ok && mbar_wait_tries<true>(&bar[B_OFREE + b % OB], (b / OB - 1) & 1, err, 325);
+        const uint32_t sg = smem_b + ks.i * SM::stage, t_o = o_cols<CP>(os.i);
+        waits.wait(CFG::FULL + ks.i, ks.phase, 351);
+        if (b >= OB) waits.wait(B_OFREE + os.i, os.phase ^ 1, 325);
+        waits.wait(W ? B_SP : B_RD, b & 1, 352);
         tc_fence_after();
-        if (ok) {
+        if (waits.ok() && elect_one()) {
             products_ta<false, CP, DK / 16, SM::rows, true>(t_o, T_S16, lo_of(sg + SM::q_off), false);
-            commit_uni(&bar[B_QD]);
+            commit_at(bar + 8 * B_QD);
         }
-        ok = ok && mbar_wait_tries<true>(&bar[B_UP], b & 1, err, 354);
+        __syncwarp();
+        waits.wait(B_UP, b & 1, 354);
         tc_fence_after();
-        if (ok) {
-            products_ta<false, CP, NB / 16, CP>(t_o, T_U16, lo_of(sg + SM::p_off), true);
-            commit_uni(&bar[B_OD + b % OB]);
-            commit_uni(&empty[st]);
+        if (waits.ok() && elect_one()) {
+            products_ta<false, CP, NB / 16, CP, false, U_INPLACE<W, CP> ? 16 : 0>(t_o, T_U16<W, CP>, lo_of(sg + SM::p_off), true);
+            commit_at(bar + 8 * (B_OD + os.i));
+            commit_at(bar + 8 * (CFG::EMPTY + ks.i));
         }
-        ok = ok && mbar_wait_tries<true>(&bar[B_OD + b % OB], (b / OB) & 1, err, 331);
+        __syncwarp();
+        if (W && b + CFG::NT < part.nblk) pass_on(N_TFREE + ts.i, 160);
+        waits.wait(B_OD + os.i, os.phase, 331);
         // (also when it has given up: the output's warps must have passed this barrier before it is arrived at again)
-        if (b >= OB) ok = mbar_wait_tries<true>(&bar[B_OFREE + b % OB], (b / OB - 1) & 1, err, 332) && ok;
-        pass_on(N_OD + b % OB, parties);
-        if (++st == NS) {
-            st = 0;
-            phase ^= 1;
-        }
+        if (!waits.ok() && b >= OB) mbar_wait_tries<true>(bar + 8 * (B_OFREE + os.i), os.phase ^ 1);
+        pass_on(N_OD + os.i, parties);
+        ks.next();
+        ts.next();
+        os.next();
     }
+    if (!waits.ok()) atomicCAS(err, 0, waits.code);
 }
 
-// O of each block from tensor memory to global memory: warp `warp` of four has rows j = 32 warp + lane, and one store of a warp is
+// V of each block to fp16 in place, NV blocks ahead, and O of each block from tensor memory to global memory: warp `warp` of four has rows j = 32 warp + lane, and one store of a warp is
 // 128 contiguous bytes of a token's row (64 of a response's).
-template <int C, int CP, int DK, int DV>
-__device__ __forceinline__ void out_role(const ChainGeo& g, const ChainPart& part, uint64_t* bar, int warp, int lane) {
-    constexpr int OB = O_BUFS<CP>;
+template <int DK, bool W, int R, int DV>
+__device__ __forceinline__ void out_role(const ChainGeo& g, const ChainPart& part, int* err, uint8_t* smem, uint32_t bar, int warp, int lane) {
+    using SM = ChainSmem<DK, R, DV>;
+    using CFG = ChainCfg<DK, W, R, DV>;
+    constexpr int C = SM::C, CP = SM::CP, OB = O_BUFS<CP>;
     const int j = 32 * warp + lane, parties = part.width + 32;
+    RingPos<CFG::NV> vs;
+    RingPos<OB> os;
+    Waits waits(bar);
     const uint32_t lanes = (uint32_t)(32 * warp) << 16;
     float* o = part.O + j;
     __half* oh = (__half*)part.O + j;
 #pragma unroll 1
-    for (int b = 0; b < part.nblk; ++b) {
-        named_bar(N_OD + b % OB, parties);
-        tc_fence_after();
-        const int Cv = min(C, g.L - (part.b0 + b) * C);
+    for (int b = W ? -CFG::NV : 0; b < part.nblk; ++b) {
+        if (b >= 0) {
+            named_bar(N_OD + os.i, parties);
+            tc_fence_after();
+            const int Cv = min(C, g.L - (part.b0 + b) * C);
 #pragma unroll 1
-        for (int c = 0; c < CP; c += 16) {
-            uint32_t x[16];
-            tmem_ld16(o_cols<CP>(b) + lanes + c, x);
-            tmem_ld_wait();
-            if (c + 16 == CP) {
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&bar[B_OFREE + b % OB]);
+            for (int c = 0; c < CP; c += 16) {
+                uint32_t x[16];
+                tmem_ld16(o_cols<CP>(os.i) + lanes + c, x);
+                tmem_ld_wait();
+                if (c + 16 == CP) {
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive_at(bar + 8 * (B_OFREE + os.i));
+                }
+                if (part.response) {
+#pragma unroll
+                    for (int t = 0; t < 16; ++t)
+                        if (c + t < Cv) oh[(c + t) * DK] = __float2half_rn(__uint_as_float(x[t]));
+                } else {
+#pragma unroll
+                    for (int t = 0; t < 16; ++t)
+                        if (c + t < Cv) o[(c + t) * DV] = __uint_as_float(x[t]);
+                }
             }
-            if (part.response) {
-#pragma unroll
-                for (int t = 0; t < 16; ++t)
-                    if (c + t < Cv) oh[(c + t) * DK] = __float2half_rn(__uint_as_float(x[t]));
-            } else if (c + 16 <= Cv) {
-#pragma unroll
-                for (int t = 0; t < 16; ++t) o[(c + t) * DV] = __uint_as_float(x[t]);
-            } else {
-#pragma unroll
-                for (int t = 0; t < 16; ++t)
-                    if (c + t < Cv) o[(c + t) * DV] = __uint_as_float(x[t]);
-            }
+            o += C * DV;
+            oh += C * DK;
+            os.next();
         }
-        o += C * DV;
-        oh += C * DK;
+        if (W && b + CFG::NV < part.nblk && !part.response) {
+            waits.wait(CFG::VLAND + vs.i, vs.phase, 333);
+            convert_pieces<8, DV>(smem + CFG::v_off + vs.i * SM::v_bytes, j);
+            publish_smem(bar + 8 * (CFG::WDONE + vs.i), lane);
+            vs.next();
+        }
     }
+    if (!waits.ok()) atomicCAS(err, 0, waits.code);
 }
 
 // The end state (its last update is the chain's last product, so that this goes on beside the last block's output); lost: gets a bit for each quarter of the rows j that has to be walked again.
@@ -821,19 +1092,19 @@ __device__ __forceinline__ void end_state(const ChainPart& part, uint32_t* lost,
     }
 }
 
-template <int DK, int R, int DV, int NS, bool SEG>
-__global__ void __launch_bounds__(CHAIN_THREADS, 1)
+template <int DK, bool W, int R, int DV, bool SEG>
+__global__ void __launch_bounds__(CHAIN_THREADS<W>, 1)
 chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __restrict__ beta, const float* __restrict__ S0,
              float* __restrict__ O, float* __restrict__ S_final, int* __restrict__ status, ChainGeo g, ChainSeg sg) {
-    using CFG = ChainCfg<DK, R, DV, NS>;
+    using CFG = ChainCfg<DK, W, R, DV>;
     using SM = ChainSmem<DK, R, DV>;
     extern __shared__ __align__(1024) uint8_t smem[];
-    __shared__ uint64_t bar[B_LAND + 3 * NS];
+    __shared__ uint64_t bar[CFG::count];
     __shared__ uint32_t tmem_base;
     __shared__ ChainArgs args;
     __shared__ uint32_t lost;
-    uint64_t *land = bar + B_LAND, *full = land + NS, *empty = full + NS;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const uint32_t bar_b = smem_u32(bar);
     long long seq;
     const ChainPart part = chain_part<DK, SM::C, SEG>(g, sg, S0, O, S_final, seq);
     const int quarters = part.width / 32;                         // lane quarters that hold rows of the state
@@ -846,21 +1117,31 @@ chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __rest
     if (tid == 0) {
         lost = 0;
         mbar_init(&bar[B_SP], 2 * quarters);
-        mbar_init(&bar[B_RP], 2 * quarters);
         mbar_init(&bar[B_UP], 2 * quarters);
-        mbar_init(&bar[B_RD], 1);
         mbar_init(&bar[B_SD], 1);
         mbar_init(&bar[B_UD], 1);
         mbar_init(&bar[B_QD], 1);
         mbar_init(&bar[B_GD], 1);
+        mbar_init(&bar[B_WD], 1);
+        mbar_init(&bar[B_RD], 1);
+        mbar_init(&bar[B_RP], 2 * quarters);
         for (int x = 0; x < 2; ++x) {
             mbar_init(&bar[B_OD + x], 1);
             mbar_init(&bar[B_OFREE + x], quarters);
         }
-        for (int x = 0; x < NS; ++x) {
-            mbar_init(&land[x], 1);
-            mbar_init(&full[x], 256);
-            mbar_init(&empty[x], 2);
+        for (int x = 0; x < CFG::NS; ++x) {
+            mbar_init(&bar[CFG::LAND + x], 1);
+            mbar_init(&bar[CFG::FULL + x], 32 * (W ? 4 : 8));        // (without W also T)
+            mbar_init(&bar[CFG::EMPTY + x], 2);
+        }
+        for (int x = 0; x < CFG::NV; ++x) {
+            mbar_init(&bar[CFG::VLAND + x], 1);
+            mbar_init(&bar[CFG::VFREE + x], 1);
+        }
+        for (int x = 0; x < CFG::NT; ++x) mbar_init(&bar[CFG::TDONE + x], 32 * 4);
+        for (int x = 0; x < CFG::NW; ++x) {
+            mbar_init(&bar[CFG::WDONE + x], 32 * (part.response ? 4 : 4 + quarters));      // (W, and V of the same block: as many slots)
+            mbar_init(&bar[CFG::WFREE + x], 1);
         }
         mbar_fence_init();
         prefetch_tmap(&maps.q);
@@ -868,13 +1149,15 @@ chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __rest
         prefetch_tmap(&maps.v);
     }
     if (warp == W_MMA) tmem_alloc(&tmem_base, 512);
-    if (SM::CP > SM::C)                                           // (r = 3: query rows that no copy writes are read)
-        for (int e = tid; e < NS * SM::stage / 16; e += CHAIN_THREADS) ((uint4*)smem)[e] = make_uint4(0, 0, 0, 0);
-    else                                                          // (the upper triangles of T and P, which nothing writes)
-        for (int st = 0; st < NS && st < part.nblk; ++st)
-            for (int e = tid; e < (SM::t_bytes + SM::p_bytes) / 16; e += CHAIN_THREADS)
-                ((uint4*)(smem + st * SM::stage + SM::t_off))[e] = make_uint4(0, 0, 0, 0);
-    for (int e = tid; e < IdStrip::bytes / 2; e += CHAIN_THREADS) ((uint16_t*)(smem + CFG::id_off))[e] = IdStrip::one(e) ? 0x3F80 : 0;
+    if (SM::CP > SM::C) {                                         // (r = 3: query rows that no copy writes are read)
+        for (int e = tid; e < CFG::NS * SM::stage / 16; e += CHAIN_THREADS<W>) ((uint4*)smem)[e] = make_uint4(0, 0, 0, 0);
+    } else {                                                      // (the upper triangles of P and T, which nothing writes)
+        for (int st = 0; st < CFG::NS && st < part.nblk; ++st)
+            for (int e = tid; e < SM::p_bytes / 16; e += CHAIN_THREADS<W>) ((uint4*)(smem + st * SM::stage + SM::p_off))[e] = make_uint4(0, 0, 0, 0);
+    }
+    for (int e = tid; e < CFG::NT * SM::t_bytes / 16; e += CHAIN_THREADS<W>) ((uint4*)(smem + CFG::t_off))[e] = make_uint4(0, 0, 0, 0);
+    if (!W)
+        for (int e = tid; e < IdStrip::bytes / 2; e += CHAIN_THREADS<W>) ((uint16_t*)(smem + CFG::id_off))[e] = IdStrip::one(e) ? 0x3F80 : 0;
     fence_async_smem();
     tc_fence_before();
     __syncthreads();
@@ -895,7 +1178,7 @@ chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __rest
     auto all_done = [&]() {
         __syncwarp();
         tc_fence_before();
-        named_bar(0, CHAIN_THREADS);
+        named_bar(0, CHAIN_THREADS<W>);
         tc_fence_after();
     };
     // (the chain's and the solve teams' warps, eight rows each, us a token with every row lost and with the chain's warps alone: d = 128, r = 1, 2, 4
@@ -904,51 +1187,53 @@ chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __rest
         if (lost >> (x >> 2) & 1) walk_fp32<DK, R>(args, part, seq, 8 * x);
     };
     if (warp < W_OUT) {
-        set_registers<REGS_CHAIN>();
+        set_registers<W, REGS_CHAIN>();
         begin();
         if (tid == 0 && blockIdx.x == 0 && g.clear) *status = 0;  // (the call's status word: a wait expires a second from now at the earliest)
         const bool holds_state = (warp & 3) < quarters;
         if (holds_state) {
-            chain_role<DK>(part, status, bar, warp, lane);
+            const int code = chain_role<DK, W, SM::CP>(part, bar_b, warp, lane);
+            if (code) atomicCAS(status, 0, code);
             end_state<DK>(part, &lost, warp, lane);
         }
         all_done();                                               // (every output is written)
         walk_lost(warp);
     } else if (warp < W_CONV) {
-        set_registers<REGS_OUT>();
+        set_registers<W, REGS_OUT>();
         begin();
-        if (warp - W_OUT < quarters) out_role<SM::C, SM::CP, DK, DV>(g, part, bar, warp - W_OUT, lane);
+        if (warp - W_OUT < quarters) out_role<DK, W, R, DV>(g, part, status, smem, bar_b, warp - W_OUT, lane);
         all_done();
     } else if (warp < W_SOLVE) {
-        set_registers<REGS_CONV>();
+        set_registers<W, REGS_CONV>();
         begin();
-        convert_role<DK, R, DV, NS>(part, smem, full, tid - 32 * W_CONV);
+        convert_role<DK, W, R, DV>(part, smem, bar_b, tid - 32 * W_CONV);
         all_done();
     } else if (warp < W_MMA) {
-        set_registers<REGS_SOLVE>();
+        set_registers<W, REGS_SOLVE<W>>();
         begin();
-        solve_role<DK, R, DV, NS>(g, part, beta, smem, full, seq, (warp - W_SOLVE) >> 2, (tid - 32 * W_SOLVE) & 127);
+        solve_role<DK, W, R, DV>(g, part, beta, smem, bar_b, seq, (warp - W_SOLVE) >> 2, (tid - 32 * W_SOLVE) & 127);
         all_done();
         walk_lost(8 + warp - W_SOLVE);
-    } else {
-        set_registers<REGS_ISSUE>();
+    } else if (warp < W_W) {
+        set_registers<W, REGS_ISSUE>();
         begin();
         if (warp == W_MMA) {
-            mma_role<DK, R, DV, NS>(part, status, smem, bar);
+            const int code = mma_role<DK, W, R, DV>(part, smem, bar_b);
+            if (code) atomicCAS(status, 0, code);
         } else if (warp == W_MMA_OUT) {
-            mma_out_role<DK, R, DV, NS>(part, status, smem, bar);
+            mma_out_role<DK, W, R, DV>(part, status, smem, bar_b);
         } else if (warp == W_GRAM) {
-            gram_role<DK, R, DV, NS>(part, status, smem, bar, land);
+            gram_role<DK, W, R, DV>(part, status, smem, bar_b);
         } else if (warp == W_LOAD) {
-            bool ok = true;
-#pragma unroll 1
-            for (int b = 0; ok && b < part.nblk; ++b) {
-                if (b >= NS) ok = mbar_wait_tries<true>(&empty[b % NS], (b / NS - 1) & 1, status, 341);
-                if (ok && lane == 0) load_block<DK, R, DV, NS>(maps, smem, land, b, (int)seq, part);
-            }
+            load_role<DK, W, R, DV>(maps, status, smem, bar_b, (int)seq, part);
         }
         all_done();
         if (warp == W_MMA) tmem_dealloc(0, 512);
+    } else if constexpr (W) {
+        set_registers<W, REGS_W>();
+        begin();
+        w_role<DK, W, R, DV>(part, status, smem, bar_b, tid - 32 * W_W);
+        all_done();
     }
 }
 
@@ -1180,10 +1465,10 @@ ChainCarve carve(const Problem& p, const ChainPlan& plan) {
 
 template <int DK, int R, int DV, bool SEG>
 int launch(const Problem& p, const ChainPlan& plan, const ChainSeg& sg) {
-    constexpr int NS = chain_stages<DK, R, DV>();
-    using CFG = ChainCfg<DK, R, DV, NS>;
-    static_assert(CFG::total <= 227 * 1024 && NS >= 2, "shared memory budget");
-    const void* fn = (const void*)chain_kernel<DK, R, DV, NS, SEG>;
+    constexpr bool W = w_form(DK, DV, SEG);
+    using CFG = ChainCfg<DK, W, R, DV>;
+    static_assert(CFG::total <= SMEM_MOST && CFG::NS >= 3 && (!W || (CFG::NS >= 4 && CFG::NT <= 3 && CFG::NV == CFG::NW)), "shared memory budget");
+    const void* fn = (const void*)chain_kernel<DK, W, R, DV, SEG>;
     constexpr int C = NB / R;
     ChainGeo g{p.L, p.d_v, (p.L + C - 1) / C, plan.nseg, plan.seg_blk, p.mask_group(), p.exact ? 1 : 0, p.clear_status ? 1 : 0,
                (const __nv_bfloat16*)p.q, (const __nv_bfloat16*)p.k, (const __nv_bfloat16*)p.v, (const __nv_bfloat16*)p.beta,
@@ -1199,7 +1484,7 @@ int launch(const Problem& p, const ChainPlan& plan, const ChainSeg& sg) {
     if (st != PF_OK) return st;
     void* args[] = {(void*)&maps, (void*)&p.beta, (void*)&p.S0, (void*)&p.O, (void*)&p.S_final, (void*)&p.status, (void*)&g, (void*)&sg};
     prof_begin("chain", p.stream);
-    PF_CUDA_TRY(launch_early(fn, dim3((unsigned)grid), CHAIN_THREADS, args, (size_t)CFG::total, p.stream));
+    PF_CUDA_TRY(launch_early(fn, dim3((unsigned)grid), CHAIN_THREADS<W>, args, (size_t)CFG::total, p.stream));
     prof_end(p.stream);
     count_launch(1);
     return PF_OK;
