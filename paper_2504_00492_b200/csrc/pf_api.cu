@@ -317,19 +317,31 @@ int forward_one(const pf_params* a, bool top) {
     p.stream = (cudaStream_t)a->stream;
 
     p.own_workspace = !a->workspace;
-    const size_t need = workspace_need(p, impl);
+    size_t need;
     void* ws = a->workspace;
     bool own = false;
     if (ws) {
+        need = workspace_need(p, impl);
+        if (a->workspace_bytes < need) {       // (sharing walks out is for speed only: without it the call may take less)
+            p.no_share = true;
+            need = workspace_need(p, impl);
+        }
         if (a->workspace_bytes < need || ((uintptr_t)ws & 255u)) return PF_ERR_WORKSPACE;
     } else {
-        const size_t own_need = use_recur(p, impl) ? recur_workspace_bytes(p)
-                                : use_chain(p, impl) && !chain_needs_workspace(p) ? 0 : need;
-        if (own_need > 0) {
-            st = workspace_alloc(&ws, own_need, p.stream);
-            if (st != PF_OK) return st;
-            own = true;
+        auto alloc = [&]() {
+            need = workspace_need(p, impl);
+            const size_t own_need = use_recur(p, impl) ? recur_workspace_bytes(p)
+                                    : use_chain(p, impl) && !chain_needs_workspace(p) ? 0 : need;
+            own = own_need > 0;
+            return own ? workspace_alloc(&ws, own_need, p.stream) : (int)PF_OK;
+        };
+        st = alloc();
+        if (st == PF_ERR_CUDA && chain_shares(p) && use_chain(p, impl)) {
+            cudaGetLastError();
+            p.no_share = true;
+            st = alloc();
         }
+        if (st != PF_OK) return st;
     }
     if (top) begin_call();
     // the status word of this call: the caller's, else word 0 of the caller's workspace, else the library's own

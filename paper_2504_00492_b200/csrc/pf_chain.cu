@@ -69,6 +69,7 @@ using namespace tc;
 namespace {
 
 constexpr int NB = 64;               // rows per block
+constexpr int MOST_PARTS = 30;       // parts of walks in a CTA's share
 
 // Where the W form pays (head of the file), us, W and without: 128 sequences of 4096, d = 64, r = 4: 264 and 290; 256 of 1000, d = 64, r = 2: 81 and 85; 64 of 4000,
 // r = 1: 85 and 89.  Not where the walks are short and the chain has nothing ahead at their start (4 of 8192 in segments, d = 64, r = 2: 43 and 40), not at
@@ -83,6 +84,11 @@ struct ChainMaps {
 struct ChainGeo {
     int L, d_v, nblk;
     int nseg, seg_blk;  // segments per sequence (1: none) and blocks per segment
+    int first_blk;      // blocks of the first segment
+    int share;          // SHARED: blocks of a CTA, and
+    int total;          // of all of them
+    float* hand;        // [CTAs] states that go from one CTA to another, [d_k i][d_v j]
+    int *handed, *finished;     // [CTAs] each: warps that have handed over; the CTA's outputs are written
     int rm;             // strict-mask group size (Problem::mask_group)
     int exact;          // PF_STEP_EXACT
     int clear;          // set the status word to 0
@@ -234,7 +240,10 @@ template <bool W, int CP> constexpr uint32_t T_P = T_G<W, CP> + 64;   // P^T bef
 template <int CP> constexpr int O_BUFS = CP > 32 ? 1 : 2;         // O^T, fp32 [j][t]: of two blocks in turn where there is room
 template <int CP> __device__ __forceinline__ uint32_t o_cols(int b) { return CP > 32 ? 448u : 448u + 32u * (b & 1); }
 
-// What one CTA of the kernel works on.
+// How the walks are given to CTAs: a sequence each; a segment's walk each; or all walks, one after another, in equal shares.
+enum { WHOLE = 0, SEGMENTS = 1, SHARED = 2 };
+
+// A walk, or the part of one, that a CTA of the kernel works on.
 struct ChainPart {
     int b0, nblk;       // first block of the sequence's, number of blocks
     int width;          // rows j of the state: d_v, or d_k for the response to the segment's start state
@@ -243,6 +252,10 @@ struct ChainPart {
     float* O;           // rows of O of the first block (response: fp16 rows)
     float* S_end;       // end state [i][j] (response: fp16 [j][i] without its diagonal), or null
     float* D;           // response: the end state's diagonal
+    long long seq;
+    // SHARED:
+    int hand_in, hand_out;      // the state comes from there, goes there (-1: does not)
+    int before, walk;           // blocks of the walk before this part, and of all of it
 };
 
 // Segments (Section 3, "Scan"; Proposition 2.1): the flow of an interval is the pair (P, Xi) with S_end = S_start P + Xi.  A
@@ -268,30 +281,74 @@ struct ChainArgs {
     ChainSeg seg;
 };
 
-// What this CTA works on; seq: its sequence.
-template <int DK, int C, bool SEG>
-__device__ __forceinline__ ChainPart chain_part(const ChainGeo& g, const ChainSeg& sg, const float* S0, float* O, float* S_final, long long& seq) {
+// A walk: segment s of sequence seq, the walk itself or the response to its start state, n blocks from block b0 of the sequence on.
+template <int DK, int C, int MODE>
+__device__ __forceinline__ ChainPart walk_of(const ChainGeo& g, const ChainSeg& sg, const float* S0, float* O, float* S_final, long long seq, int s, bool response, int b0, int n) {
+    const long long row0 = seq * g.L + (long long)b0 * C, slot = seq * g.nseg + s;
     ChainPart part;
-    if constexpr (!SEG) {
-        seq = blockIdx.x;
-        part = {0, g.nblk, g.d_v, false, S0 ? S0 + seq * DK * g.d_v : nullptr, O + seq * g.L * g.d_v,
-                S_final ? S_final + seq * DK * g.d_v : nullptr, nullptr};
-    } else {
-        const int per_seq = 2 * g.nseg - 1, x = (int)(blockIdx.x % per_seq);
-        seq = blockIdx.x / per_seq;
-        part.response = x >= g.nseg;
-        const int s = part.response ? 1 + x - g.nseg : x;
-        part.b0 = s * g.seg_blk;
-        part.nblk = min(g.seg_blk, g.nblk - part.b0);
-        part.width = part.response ? DK : g.d_v;
-        const long long row0 = seq * g.L + (long long)part.b0 * C, slot = seq * g.nseg + s;
-        part.S0 = s == 0 && S0 ? S0 + seq * DK * g.d_v : nullptr;
-        part.O = part.response ? (float*)(sg.R + row0 * DK) : O + row0 * g.d_v;
-        part.S_end = part.response ? (float*)(sg.P + slot * DK * DK) : sg.Xi + slot * DK * g.d_v;
-        part.D = sg.D + slot * DK;
+    part.seq = seq;
+    part.b0 = b0;
+    part.nblk = part.walk = n;
+    part.response = MODE != WHOLE && response;
+    part.width = part.response ? DK : g.d_v;
+    part.S0 = s == 0 && S0 ? S0 + seq * DK * g.d_v : nullptr;
+    part.O = part.response ? (float*)(sg.R + row0 * DK) : O + row0 * g.d_v;
+    if (MODE == WHOLE || (MODE == SHARED && g.nseg == 1)) part.S_end = S_final ? S_final + seq * DK * g.d_v : nullptr;
+    else part.S_end = part.response ? (float*)(sg.P + slot * DK * DK) : sg.Xi + slot * DK * g.d_v;
+    part.D = MODE == WHOLE ? nullptr : sg.D + slot * DK;
+    part.hand_in = part.hand_out = -1;
+    part.before = 0;
+    return part;
+}
+// WHOLE, SEGMENTS: the walk of this CTA
+template <int DK, int C, int MODE>
+__device__ __forceinline__ ChainPart own_walk(const ChainGeo& g, const ChainSeg& sg, const float* S0, float* O, float* S_final) {
+    if (MODE == WHOLE) return walk_of<DK, C, MODE>(g, sg, S0, O, S_final, blockIdx.x, 0, false, 0, g.nblk);
+    const int per_seq = 2 * g.nseg - 1, x = (int)(blockIdx.x % per_seq), s = x >= g.nseg ? 1 + x - g.nseg : x, b0 = s * g.seg_blk;
+    return walk_of<DK, C, MODE>(g, sg, S0, O, S_final, blockIdx.x / per_seq, s, x >= g.nseg, b0, min(g.seg_blk, g.nblk - b0));
+}
+// SHARED: the walks lie one after another on a line of blocks (per sequence the first segment's, then of each further one the walk from zero and the response) that
+// is cut into shares of equal length, no shorter than any walk, so that a walk lies in one share or across one cut.  The share behind a cut comes first in its CTA's
+// time and takes the walk's first blocks; the one before it has the rest, at its end, when the state has long been handed over: nobody waits, and no SM idles while
+// others walk (the wrap-around rule for preemptive schedules, R. McNaughton, 1959).  Shares go to CTAs from the last one on, so that who waits has the higher index.
+__device__ __forceinline__ int share_of_cta() { return (int)(gridDim.x - 1 - blockIdx.x); }
+// The part that holds block x of the line.
+template <int DK, int C>
+__device__ __forceinline__ ChainPart part_at(const ChainGeo& g, const ChainSeg& sg, const float* S0, float* O, float* S_final, int x, int lo, int hi) {
+    const int per_seq = 2 * g.nblk - g.first_blk, seq = x / per_seq;
+    int off = x - seq * per_seq, s = 0, n = g.first_blk, start = 0;
+    bool response = false;
+    if (off >= g.first_blk) {
+        off -= g.first_blk;
+        s = off / (2 * g.seg_blk);
+        off -= s * 2 * g.seg_blk;
+        n = min(g.seg_blk, g.nblk - g.first_blk - s * g.seg_blk);
+        response = off >= n;
+        start = g.first_blk + s * 2 * g.seg_blk + (response ? n : 0);
+        ++s;
+    }
+    start += seq * per_seq;                                       // the walk's place on the line
+    ChainPart part = walk_of<DK, C, SHARED>(g, sg, S0, O, S_final, seq, s, response, s == 0 ? 0 : g.first_blk + (s - 1) * g.seg_blk, n);
+    part.nblk = min(start + n, hi) - max(start, lo);
+    if (start < lo) part.hand_out = share_of_cta() - 1;           // the first blocks of the walk, whose rest the share before this one has
+    else if (start + n > hi) {
+        part.hand_in = share_of_cta();
+        part.before = n - part.nblk;
+        part.b0 += part.before;
+        part.O = response ? (float*)((__half*)part.O + (long long)part.before * C * DK) : part.O + (long long)part.before * C * g.d_v;
     }
     return part;
 }
+// What a CTA works on: one walk, or the parts of its share.
+template <int MODE>
+struct ChainWork {
+    static constexpr bool shared = MODE == SHARED;
+    const ChainPart& own;       // (of the first part, SHARED)
+    const ChainPart* parts;     // SHARED
+    int n, count;               // parts, and blocks of all of them
+    __device__ __forceinline__ int size() const { return shared ? n : 1; }
+    __device__ __forceinline__ const ChainPart& operator[](int i) const { return shared ? parts[i] : own; }
+};
 
 // Eight rows of S from row `row0` on, once more: the recurrence token by token in fp32, by one warp, four lanes to a row.  Not a fast
 // path: it is there so that every state that fp16 can hold gives a finite result, whatever the products with it reach.
@@ -491,9 +548,9 @@ __device__ __forceinline__ void neumann_product(float (&r)[2][4], const uint32_t
 // ---------------------------------------------------------------------------------------------------------------------
 // solve team: T of blocks b = team, team + TEAMS, ...
 // ---------------------------------------------------------------------------------------------------------------------
-template <int DK, bool W, int R, int JS>
-__device__ __forceinline__ void solve_role(const ChainGeo& g, const ChainPart& part, const __nv_bfloat16* __restrict__ beta, uint8_t* smem,
-                                           uint32_t bar, long long seq, int team, int tid) {
+template <int DK, bool W, int R, int JS, int MODE>
+__device__ __forceinline__ void solve_role(const ChainGeo& g, ChainWork<MODE> work, const __nv_bfloat16* __restrict__ beta, uint8_t* smem,
+                                           uint32_t bar, int team, int tid) {
     using CFG = ChainCfg<DK, W, R, JS>;
     using SM = ChainSmem<DK, R, JS>;
     constexpr int C = SM::C;
@@ -502,15 +559,6 @@ __device__ __forceinline__ void solve_role(const ChainGeo& g, const ChainPart& p
     const uint32_t xs_b = smem_u32(smem) + CFG::xs_off + team * XS_BYTES;
     const uint32_t offA = lane_off(lane & 15, lane >> 4), offN = lane_off((lane & 7) + ((lane >> 4) << 3), (lane >> 3) & 1);
     const uint32_t xs_a = xs_b + xs_lane(lane & 15, lane >> 4) + xs_block(w, 0), xs_n = xs_b + xs_lane((lane & 7) + ((lane >> 4) << 3), (lane >> 3) & 1);
-    const __nv_bfloat16* bs = beta + seq * L * R;
-    // (the bits as loaded: a conversion next to the load would make every thread wait for it there, a block ahead of its use)
-    auto read_beta = [&](int b) {                                 // rows past the block or the sequence have step size zero
-        uint16_t x = 0;
-        if (tid < min(C, L - (part.b0 + b) * C) * R)
-            asm volatile("ld.global.nc.b16 %0, [%1];" : "=h"(x) : "l"(bs + (long long)(part.b0 + b) * C * R + tid));
-        return x;
-    };
-    uint16_t breg = team < part.nblk ? read_beta(team) : 0;
     // the strict mask on the packed values of the diagonal tile, and of the one left of it (groups of three rows reach across the edge of a tile)
     uint32_t keep[4], keep_left[4];
     {
@@ -523,14 +571,29 @@ __device__ __forceinline__ void solve_role(const ChainGeo& g, const ChainPart& p
         }
     }
     const uint32_t one = gq == 2 * t4 ? 0x3C00u : gq == 2 * t4 + 1 ? 0x3C000000u : 0u;      // the identity's part of elements 0 and 3 of a fragment
+    int b = team;                                                 // (of the CTA's blocks)
 #pragma unroll 1
-    for (int b = team; b < part.nblk; b += TEAMS) {
+    for (int i = 0, at = 0; i < work.size(); at += work[i].nblk, ++i) {
+    const ChainPart& part = work[i];
+    const int end = at + part.nblk;
+    const __nv_bfloat16* bs = beta + part.seq * L * R;
+    // (the bits as loaded: a conversion next to the load would make every thread wait for it there, a block ahead of its use)
+    auto read_beta = [&](int b) {                                 // rows past the block or the sequence have step size zero
+        uint16_t x = 0;
+        const int tok = (part.b0 + b - at) * C;
+        if (tid < min(C, L - tok) * R)
+            asm volatile("ld.global.nc.b16 %0, [%1];" : "=h"(x) : "l"(bs + (long long)tok * R + tid));
+        return x;
+    };
+    uint16_t breg = b < end ? read_beta(b) : 0;
+#pragma unroll 1
+    for (; b < end; b += TEAMS) {
         const int ts = b % CFG::NT;
         const uint32_t t_b = smem_u32(smem) + CFG::t_off + ts * SM::t_bytes;
         // (two in turn: another warp may still be scaling T of the block before)
         float* sBeta = (float*)(smem + CFG::beta_off + team * 512 + (b / TEAMS & 1) * 256);
         if (tid < NB) sBeta[tid] = __uint_as_float((uint32_t)breg << 16);
-        if (b + TEAMS < part.nblk) breg = read_beta(b + TEAMS);
+        if (b + TEAMS < end) breg = read_beta(b + TEAMS);
         named_bar(N_GD + team, 160);                              // (and the step sizes)
         tc_fence_after();
         const uint32_t t_g = T_G<W, SM::CP> + ((uint32_t)(32 * w) << 16);
@@ -566,7 +629,7 @@ __device__ __forceinline__ void solve_role(const ChainGeo& g, const ChainPart& p
 #pragma unroll
         for (int e = 0; e < 4; ++e) nf[e] &= keep[e];
         tc_fence_before();
-        if (b + 1 < part.nblk) named_arrive(N_GFREE, 288);
+        if (b + 1 < work.count) named_arrive(N_GFREE, 288);
         // ---- D_w = (I - N_ww)^{-1} (Neumann product, N nilpotent) for the other warps
         uint32_t y0[4];                                           // X_ww^T as an A operand
         {
@@ -615,11 +678,12 @@ __device__ __forceinline__ void solve_role(const ChainGeo& g, const ChainPart& p
         }
         publish_smem(bar + 8 * ((W ? CFG::TDONE : CFG::FULL) + ts), lane);
     }
+    }
 }
 
 // Conversion: K and Q of every block to fp16 in place, once the Gram products have read them as they came, and P.  Four warps.
 template <int DK, bool W, int R, int JS>
-__device__ __forceinline__ void convert_role(const ChainPart& part, uint8_t* smem, uint32_t bar, int tid) {
+__device__ __forceinline__ void convert_role(int count, uint8_t* smem, uint32_t bar, int tid) {
     using SM = ChainSmem<DK, R, JS>;
     using CFG = ChainCfg<DK, W, R, JS>;
     constexpr int CP = SM::CP;
@@ -627,7 +691,7 @@ __device__ __forceinline__ void convert_role(const ChainPart& part, uint8_t* sme
     const uint32_t p_at = smem_u32(smem) + SM::p_off + (lane_off((lane & 7) + ((lane >> 4) << 3), (lane >> 3) & 1) ^ (uint32_t)(w << 5));
     int st = 0;
 #pragma unroll 1
-    for (int b = 0; b < part.nblk; ++b) {
+    for (int b = 0; b < count; ++b) {
         uint8_t* sg = smem + st * SM::stage;
         named_bar(N_PD, 160);
         tc_fence_after();
@@ -640,7 +704,7 @@ __device__ __forceinline__ void convert_role(const ChainPart& part, uint8_t* sme
             tmem_ld_wait();
             if (t0 + PC == CP) {
                 tc_fence_before();
-                if (b + 1 < part.nblk) named_arrive(N_GFREE, 288);
+                if (b + 1 < count) named_arrive(N_GFREE, 288);
             }
 #pragma unroll
             for (int n = 0; n < PC / 8; n += 2) {
@@ -666,7 +730,7 @@ __device__ __forceinline__ void convert_role(const ChainPart& part, uint8_t* sme
 // W^T = K^T T^T of every block (rows i, columns m): its products, and out of tensor memory as the fp16 operand W.  Four warps, the first of which issues; at
 // d_k = 64 the accumulator has its rows twice, and a warp takes half of the columns.
 template <int DK, bool W, int R, int JS>
-__device__ __forceinline__ void w_role(const ChainPart& part, int* err, uint8_t* smem, uint32_t bar, int tid) {
+__device__ __forceinline__ void w_role(int count, int* err, uint8_t* smem, uint32_t bar, int tid) {
     using SM = ChainSmem<DK, R, JS>;
     using CFG = ChainCfg<DK, W, R, JS>;
     const int w = tid >> 5, lane = tid & 31, i = tid & (DK - 1);
@@ -677,7 +741,7 @@ __device__ __forceinline__ void w_role(const ChainPart& part, int* err, uint8_t*
     RingPos<CFG::NW> ws;
     Waits waits(bar);
 #pragma unroll 1
-    for (int b = 0; b < part.nblk; ++b) {
+    for (int b = 0; b < count; ++b) {
         uint8_t* row = smem + CFG::w_off + ws.i * SM::w_bytes + i * 128;
         if (b > 0) named_bar(N_WFREE, 128);                       // (the accumulator has been read)
         if (w == 0) {
@@ -720,14 +784,14 @@ __device__ __forceinline__ void w_role(const ChainPart& part, int* err, uint8_t*
 
 // Gram products (one warp): G = K K^T and K Q^T from the bf16 tiles as they landed, in products of 64 rows and NB + CP columns.
 template <int DK, bool W, int R, int JS>
-__device__ __forceinline__ void gram_role(const ChainPart& part, int* err, uint8_t* smem, uint32_t bar) {
+__device__ __forceinline__ void gram_role(int count, int* err, uint8_t* smem, uint32_t bar) {
     using SM = ChainSmem<DK, R, JS>;
     using CFG = ChainCfg<DK, W, R, JS>;
     const uint32_t smem_b = smem_u32(smem);
     RingPos<CFG::NS> ks;
     Waits waits(bar);
 #pragma unroll 1
-    for (int b = 0; b < part.nblk; ++b) {
+    for (int b = 0; b < count; ++b) {
         waits.wait(CFG::LAND + ks.i, ks.phase, 316);
         if (b > 0) named_bar(N_GFREE, 288);
         tc_fence_after();
@@ -746,8 +810,8 @@ __device__ __forceinline__ void gram_role(const ChainPart& part, int* err, uint8
 
 // The copies (one warp).  K and Q of a block are asked for when the block before in their stage is done, and V with them, or in the W form when V^T T^T of the
 // block before it in its slot is; rows past the sequence arrive as zeros.  (Issuing a copy takes the warp some 200 cycles, five a block at d = 128.)
-template <int DK, bool W, int R, int JS>
-__device__ __forceinline__ void load_role(const ChainMaps& maps, int* err, uint8_t* smem, uint32_t bar, int seq, const ChainPart& part) {
+template <int DK, bool W, int R, int JS, int MODE>
+__device__ __forceinline__ void load_role(const ChainMaps& maps, ChainWork<MODE> work, int* err, uint8_t* smem, uint32_t bar) {
     using SM = ChainSmem<DK, R, JS>;
     using CFG = ChainCfg<DK, W, R, JS>;
     constexpr int NS = CFG::NS, NV = CFG::NV;
@@ -755,36 +819,52 @@ __device__ __forceinline__ void load_role(const ChainMaps& maps, int* err, uint8
     Waits waits(bar);
     RingPos<NS> ks;
     RingPos<NV> vs;
-    // (c: the block that the chain is in, or before the first)
+    auto copy_kq = [&](const ChainPart& part, int b) {
+        const uint32_t land = bar + 8 * (CFG::LAND + ks.i), at = smem_b + ks.i * SM::stage;
+        const int tok = (part.b0 + b) * SM::C, seq = (int)part.seq;
+        if (waits.ok() && elect_one()) {
+            mbar_expect_tx_at(land, SM::tx_bytes + (W || part.response ? 0 : SM::v_bytes));
+#pragma unroll
+            for (int h = 0; h < DK / 64; ++h) {
+                tma_load_4d(at + SM::k_off + h * (SM::rows * 128), &maps.k, 0, tok * R, h, seq, land);
+                tma_load_4d(at + SM::q_off + h * (SM::rows * 128), &maps.q, 0, tok, h, seq, land);
+            }
+            if (!W && !part.response) tma_load_4d(smem_b + CFG::v_off + ks.i * SM::v_bytes, &maps.v, 0, tok * R, 0, seq, land);
+        }
+        __syncwarp();
+        ks.next();
+    };
+    if constexpr (W) {
+        const ChainPart& part = work[0];
+        // (c: the block that the chain is in, or before the first)
 #pragma unroll 1
-    for (int c = -NS; c + NV < part.nblk; ++c) {
-        if (W && c + NV >= 0) {
-            if (!part.response) {
+        for (int c = -NS; c + NV < part.nblk; ++c) {
+            if (c + NV >= 0) {
                 if (c >= 0) waits.wait(CFG::VFREE + vs.i, vs.phase ^ 1, 342);
                 const uint32_t land = bar + 8 * (CFG::VLAND + vs.i);
                 if (waits.ok() && elect_one()) {
                     mbar_expect_tx_at(land, SM::v_bytes);
-                    tma_load_4d(smem_b + CFG::v_off + vs.i * SM::v_bytes, &maps.v, 0, (part.b0 + c + NV) * SM::C * R, 0, seq, land);
+                    tma_load_4d(smem_b + CFG::v_off + vs.i * SM::v_bytes, &maps.v, 0, (part.b0 + c + NV) * SM::C * R, 0, (int)part.seq, land);
                 }
                 __syncwarp();
+                vs.next();
             }
-            vs.next();
+            if (c + NS < part.nblk) {
+                if (c >= 0) waits.wait(CFG::EMPTY + ks.i, ks.phase ^ 1, 341);
+                copy_kq(part, c + NS);
+            }
         }
-        if (c + NS < part.nblk) {
-            if (c >= 0) waits.wait(CFG::EMPTY + ks.i, ks.phase ^ 1, 341);
-            const uint32_t land = bar + 8 * (CFG::LAND + ks.i), at = smem_b + ks.i * SM::stage;
-            const int tok = (part.b0 + c + NS) * SM::C;
-            if (waits.ok() && elect_one()) {
-                mbar_expect_tx_at(land, SM::tx_bytes + (W || part.response ? 0 : SM::v_bytes));
-#pragma unroll
-                for (int h = 0; h < DK / 64; ++h) {
-                    tma_load_4d(at + SM::k_off + h * (SM::rows * 128), &maps.k, 0, tok * R, h, seq, land);
-                    tma_load_4d(at + SM::q_off + h * (SM::rows * 128), &maps.q, 0, tok, h, seq, land);
-                }
-                if (!W && !part.response) tma_load_4d(smem_b + CFG::v_off + ks.i * SM::v_bytes, &maps.v, 0, tok * R, 0, seq, land);
+    } else {
+        int c = -NS;
+#pragma unroll 1
+        for (int i = 0; i < work.size(); ++i) {
+            const ChainPart& part = work[i];
+            const int nblk = part.nblk;
+#pragma unroll 1
+            for (int b = 0; b < nblk; ++b, ++c) {
+                if (c >= 0) waits.wait(CFG::EMPTY + ks.i, ks.phase ^ 1, 341);
+                copy_kq(part, b);
             }
-            __syncwarp();
-            ks.next();
         }
     }
     if (!waits.ok()) atomicCAS(err, 0, waits.code);
@@ -812,249 +892,37 @@ __device__ __forceinline__ void to_operand(uint32_t src, uint32_t dst) {
     }
 }
 
-// warp `warp` of eight: rows j = 32 (warp & 3) + lane, half warp >> 2 of the columns of everything
-template <int DK, bool W, int CP>
-__device__ __forceinline__ int chain_role(const ChainPart& part, uint32_t bar, int warp, int lane) {
-    constexpr int HC = DK / 2;                                    // columns i of this warp
-    const int h = warp >> 2, j = 32 * (warp & 3) + lane;
-    const uint32_t lanes = (uint32_t)(32 * (warp & 3)) << 16;
-    const uint32_t t_s = T_S + h * HC + lanes, t_s16 = T_S16 + h * HC / 2 + lanes;
-    const uint32_t t_u = T_U + 32 * h + lanes, t_u16 = T_U16<W, CP> + (U_INPLACE<W, CP> ? 32 : 16) * h + lanes;
-#pragma unroll 1
-    for (int c = 0; c < HC; c += 16) {
-        uint32_t x[16], y[8];
-        const float* s0 = part.S0 + (long long)(h * HC + c) * part.width + j;
-#pragma unroll
-        for (int e = 0; e < 16; ++e) x[e] = __float_as_uint(part.S0 ? s0[e * part.width] : part.response && h * HC + c + e == j ? 1.f : 0.f);
-        tmem_st16(t_s + c, x);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) y[e] = pack_h2(-__uint_as_float(x[2 * e]), -__uint_as_float(x[2 * e + 1]));
-        tmem_st8(t_s16 + c / 2, y);
-    }
-    auto publish = [&](int b) {
-        tmem_st_wait();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive_at(bar + 8 * b);
-    };
-#pragma unroll 1
-    for (int b = 0; b < part.nblk; ++b) {
-        publish(B_SP);
-        if constexpr (!W) {
-            if (!mbar_wait_tries<false>(bar + 8 * B_RD, b & 1)) return 312;
-            tc_fence_after();
-            to_operand<32, false>(t_u, T_R16 + 16 * h + lanes);
-            publish(B_RP);
-        }
-        if (!mbar_wait_tries<false>(bar + 8 * B_UD, b & 1)) return 313;
-        tc_fence_after();
-        to_operand<32, false>(t_u, t_u16);
-        publish(B_UP);
-        if (!mbar_wait_tries<false>(bar + 8 * B_SD, b & 1)) return 314;
-        tc_fence_after();
-        if (b + 1 == part.nblk) return 0;
-        to_operand<HC, true>(t_s, t_s16);
-    }
-    return 0;
+// Waits until *p >= want (one thread), about a second at most.
+__device__ __forceinline__ bool wait_for_count(const int* p, int want) {
+    const long long t0 = clock64();
+    while (ld_acquire_gpu(p) < want)
+        if (clock64() - t0 > WAIT_CYCLES) return false;
+    return true;
 }
-
-// The products of the chain (one warp).  Returns the code of the wait that ran out, or 0.
-template <int DK, bool W, int R, int DV>
-__device__ __forceinline__ int mma_role(const ChainPart& part, uint8_t* smem, uint32_t bar) {
-    using CFG = ChainCfg<DK, W, R, DV>;
-    using SM = ChainSmem<DK, R, DV>;
-    constexpr int V_SLAB = NB * 128, K_SLAB = SM::rows * 128, CP = SM::CP, OB = O_BUFS<CP>;
-    constexpr bool INPLACE = U_INPLACE<W, CP>;
-    const uint32_t smem_b = smem_u32(smem);
-    RingPos<CFG::NS> ks;
-    RingPos<CFG::NV> vs;
-    RingPos<CFG::NT> ts;
-    RingPos<CFG::NW> ws;
-    auto wait = [&](int which, int parity) { return mbar_wait_tries<false>(bar + 8 * which, (uint32_t)parity); };
-#pragma unroll 1
-    for (int b = 0; b < part.nblk; ++b) {
-        const uint32_t k_at = smem_b + ks.i * SM::stage + SM::k_off, v_lo = lo_of(smem_b + CFG::v_off + vs.i * SM::v_bytes, DV == 128 ? V_SLAB : 0),
-                       t_lo = lo_of(smem_b + CFG::t_off + ts.i * SM::t_bytes);
-        // (at d_v = 64 the 64 columns of V's tile are read twice: rows j past d_v are nobody's)
-        if constexpr (W) {
-            // ---- U'^T = V^T T^T (W is there, and so T; the accumulator's last reader, the chain warps' conversion of U' of the block before, is done; its
-            //      fp16 pairs' readers are)
-            if (INPLACE && b > 0 && (!wait(B_SD, (b - 1) & 1) || !wait(B_OD + (b - 1) % OB, ((b - 1) / OB) & 1))) return 315;
-            if (!wait(CFG::WDONE + ws.i, ws.phase)) return 326;
-            if (!part.response) {
-                tc_fence_after();
-                if (elect_one()) {
-                    products_tt(T_U, v_lo, t_lo);
-                    commit_at(bar + 8 * (CFG::VFREE + vs.i));
-                }
-                __syncwarp();
-            }
-            // ---- ... - S W^T
-            // (U' completes only after the last reader of the block before's, P U', so that the chain warps need not wait for that)
-            if (!INPLACE && b > 0 && !wait(B_OD + (b - 1) % OB, ((b - 1) / OB) & 1)) return 319;
-            if (!wait(B_SP, b & 1)) return 323;
-            tc_fence_after();
-            if (elect_one()) {
-                products_ta<true, NB, DK / 16, DK>(T_U, T_S16, lo_of(smem_b + CFG::w_off + ws.i * SM::w_bytes), !part.response);
-                commit_at(bar + 8 * B_UD);
-                commit_at(bar + 8 * (CFG::WFREE + ws.i));
-            }
-            __syncwarp();
-        } else {
-            // ---- V^T into the accumulator, as V^T times an identity, both bf16 (V as it came; the accumulator's last reader is done)
-            if (!part.response) {
-                if (!wait(CFG::LAND + ks.i, ks.phase)) return 327;
-                tc_fence_after();
-                if (elect_one()) {
-                    constexpr uint32_t idesc = make_idesc(NB, true, false, false) | (1u << 7) | (1u << 10);
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) mma_f16(T_U, desc_lo(v_lo + c * (2048 >> 4)), IdStrip::desc(smem_b + CFG::id_off, c), idesc, c > 0);
-                }
-                __syncwarp();
-            }
-            // ---- R = V^T - S K^T
-            if (!wait(CFG::FULL + ks.i, ks.phase)) return 322;
-            if (!wait(B_SP, b & 1)) return 323;
-            tc_fence_after();
-            if (elect_one()) {
-                products_ta<false, NB, DK / 16, SM::rows>(T_U, T_S16, lo_of(k_at), !part.response);
-                commit_at(bar + 8 * B_RD);
-            }
-            __syncwarp();
-            // ---- U'^T = R T^T
-            // (U' completes only after the last reader of the block before's, P U', so that the chain warps need not wait for that)
-            if (b > 0 && !wait(B_OD + (b - 1) % OB, ((b - 1) / OB) & 1)) return 319;
-            if (!wait(B_RP, b & 1)) return 326;
-            tc_fence_after();
-            if (elect_one()) {
-                products_ta<false, NB, NB / 16, NB>(T_U, T_R16, t_lo, false);
-                commit_at(bar + 8 * B_UD);
-            }
-            __syncwarp();
-        }
-        // ---- S += U'^T K
-        // (and S only after Q S^T)
-        if (!wait(B_QD, b & 1)) return 320;
-        if (!wait(B_UP, b & 1)) return 328;
-        tc_fence_after();
-        if (elect_one()) {
-            products_ta<true, DK, NB / 16, SM::rows, false, INPLACE ? 16 : 0>(T_S, T_U16<W, CP>, lo_of(k_at, K_SLAB), true);
-            commit_at(bar + 8 * B_SD);
-            commit_at(bar + 8 * (CFG::EMPTY + ks.i));
-        }
-        __syncwarp();
-        ks.next();
-        vs.next();
-        ts.next();
-        ws.next();
-    }
-    return 0;
-}
-
-// The products of the output (one warp): O^T = S Q^T + U'^T P^T with the state before the update.
-template <int DK, bool W, int R, int DV>
-__device__ __forceinline__ void mma_out_role(const ChainPart& part, int* err, uint8_t* smem, uint32_t bar) {
-    using SM = ChainSmem<DK, R, DV>;
-    using CFG = ChainCfg<DK, W, R, DV>;
-    constexpr int CP = SM::CP, OB = O_BUFS<CP>;
-    const uint32_t smem_b = smem_u32(smem);
-    const int parties = part.width + 32;
-    RingPos<CFG::NS> ks;
-    RingPos<CFG::NT> ts;
-    RingPos<OB> os;
-    Waits waits(bar);
-#pragma unroll 1
-    for (int b = 0; b < part.nblk; ++b) {
-        const uint32_t sg = smem_b + ks.i * SM::stage, t_o = o_cols<CP>(os.i);
-        waits.wait(CFG::FULL + ks.i, ks.phase, 351);
-        if (b >= OB) waits.wait(B_OFREE + os.i, os.phase ^ 1, 325);
-        waits.wait(W ? B_SP : B_RD, b & 1, 352);
-        tc_fence_after();
-        if (waits.ok() && elect_one()) {
-            products_ta<false, CP, DK / 16, SM::rows, true>(t_o, T_S16, lo_of(sg + SM::q_off), false);
-            commit_at(bar + 8 * B_QD);
-        }
-        __syncwarp();
-        waits.wait(B_UP, b & 1, 354);
-        tc_fence_after();
-        if (waits.ok() && elect_one()) {
-            products_ta<false, CP, NB / 16, CP, false, U_INPLACE<W, CP> ? 16 : 0>(t_o, T_U16<W, CP>, lo_of(sg + SM::p_off), true);
-            commit_at(bar + 8 * (B_OD + os.i));
-            commit_at(bar + 8 * (CFG::EMPTY + ks.i));
-        }
-        __syncwarp();
-        if (W && b + CFG::NT < part.nblk) pass_on(N_TFREE + ts.i, 160);
-        waits.wait(B_OD + os.i, os.phase, 331);
-        // (also when it has given up: the output's warps must have passed this barrier before it is arrived at again)
-        if (!waits.ok() && b >= OB) mbar_wait_tries<true>(bar + 8 * (B_OFREE + os.i), os.phase ^ 1);
-        pass_on(N_OD + os.i, parties);
-        ks.next();
-        ts.next();
-        os.next();
-    }
-    if (!waits.ok()) atomicCAS(err, 0, waits.code);
-}
-
-// V of each block to fp16 in place, NV blocks ahead, and O of each block from tensor memory to global memory: warp `warp` of four has rows j = 32 warp + lane, and one store of a warp is
-// 128 contiguous bytes of a token's row (64 of a response's).
-template <int DK, bool W, int R, int DV>
-__device__ __forceinline__ void out_role(const ChainGeo& g, const ChainPart& part, int* err, uint8_t* smem, uint32_t bar, int warp, int lane) {
-    using SM = ChainSmem<DK, R, DV>;
-    using CFG = ChainCfg<DK, W, R, DV>;
-    constexpr int C = SM::C, CP = SM::CP, OB = O_BUFS<CP>;
-    const int j = 32 * warp + lane, parties = part.width + 32;
-    RingPos<CFG::NV> vs;
-    RingPos<OB> os;
-    Waits waits(bar);
-    const uint32_t lanes = (uint32_t)(32 * warp) << 16;
-    float* o = part.O + j;
-    __half* oh = (__half*)part.O + j;
-#pragma unroll 1
-    for (int b = W ? -CFG::NV : 0; b < part.nblk; ++b) {
-        if (b >= 0) {
-            named_bar(N_OD + os.i, parties);
-            tc_fence_after();
-            const int Cv = min(C, g.L - (part.b0 + b) * C);
-#pragma unroll 1
-            for (int c = 0; c < CP; c += 16) {
-                uint32_t x[16];
-                tmem_ld16(o_cols<CP>(os.i) + lanes + c, x);
-                tmem_ld_wait();
-                if (c + 16 == CP) {
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive_at(bar + 8 * (B_OFREE + os.i));
-                }
-                if (part.response) {
-#pragma unroll
-                    for (int t = 0; t < 16; ++t)
-                        if (c + t < Cv) oh[(c + t) * DK] = __float2half_rn(__uint_as_float(x[t]));
-                } else {
-#pragma unroll
-                    for (int t = 0; t < 16; ++t)
-                        if (c + t < Cv) o[(c + t) * DV] = __uint_as_float(x[t]);
-                }
-            }
-            o += C * DV;
-            oh += C * DK;
-            os.next();
-        }
-        if (W && b + CFG::NV < part.nblk && !part.response) {
-            waits.wait(CFG::VLAND + vs.i, vs.phase, 333);
-            convert_pieces<8, DV>(smem + CFG::v_off + vs.i * SM::v_bytes, j);
-            publish_smem(bar + 8 * (CFG::WDONE + vs.i), lane);
-            vs.next();
-        }
-    }
-    if (!waits.ok()) atomicCAS(err, 0, waits.code);
-}
+__device__ __forceinline__ void add_release_gpu(int* p, int v) { asm volatile("red.release.gpu.global.add.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory"); }
 
 // The end state (its last update is the chain's last product, so that this goes on beside the last block's output); lost: gets a bit for each quarter of the rows j that has to be walked again.
-template <int DK>
-__device__ __forceinline__ void end_state(const ChainPart& part, uint32_t* lost, int warp, int lane) {
+template <int DK, bool SHARE>
+__device__ __forceinline__ void end_state(const ChainGeo& g, const ChainPart& part, uint32_t* lost, int warp, int lane) {
     constexpr int HC = DK / 2;
     const int h = warp >> 2, quarter = warp & 3, j = 32 * quarter + lane;
     const uint32_t t_s = T_S + h * HC + ((uint32_t)(32 * quarter) << 16);
+    if (SHARE && part.hand_out >= 0) {
+        // (to the CTA that has the rest of the walk, as it is: what is lost is found at the walk's end)
+        float* out = g.hand + (long long)part.hand_out * DK * part.width + (long long)h * HC * part.width + j;
+#pragma unroll 1
+        for (int c = 0; c < HC; c += 32) {
+            uint32_t x[32];
+            tmem_ld32(t_s + c, x);
+            tmem_ld_wait();
+#pragma unroll
+            for (int e = 0; e < 32; ++e) out[(c + e) * part.width] = __uint_as_float(x[e]);
+        }
+        __threadfence();
+        __syncwarp();
+        if (lane == 0) add_release_gpu(g.handed + part.hand_out, 1);
+        return;
+    }
     if (part.response) {
         __half* P = (__half*)part.S_end + (long long)j * DK + h * HC;
 #pragma unroll 1
@@ -1092,7 +960,275 @@ __device__ __forceinline__ void end_state(const ChainPart& part, uint32_t* lost,
     }
 }
 
-template <int DK, bool W, int R, int DV, bool SEG>
+// warp `warp` of eight: rows j = 32 (warp & 3) + lane, half warp >> 2 of the columns of everything.  Returns the code of the wait that ran out, or 0.
+template <int DK, bool W, int CP, int MODE>
+__device__ __forceinline__ int chain_role(const ChainGeo& g, ChainWork<MODE> work, uint32_t* lost, uint32_t bar, int warp, int lane) {
+    constexpr int HC = DK / 2;                                    // columns i of this warp
+    const int h = warp >> 2, j = 32 * (warp & 3) + lane;
+    const uint32_t lanes = (uint32_t)(32 * (warp & 3)) << 16;
+    const uint32_t t_s = T_S + h * HC + lanes, t_s16 = T_S16 + h * HC / 2 + lanes;
+    const uint32_t t_u = T_U + 32 * h + lanes, t_u16 = T_U16<W, CP> + (U_INPLACE<W, CP> ? 32 : 16) * h + lanes;
+    auto publish = [&](int b) {
+        tmem_st_wait();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_at(bar + 8 * b);
+    };
+    int code = 0, parity = 0;
+#pragma unroll 1
+    for (int i = 0; i < work.size(); ++i) {
+        const ChainPart& part = work[i];
+        const float* s0 = part.S0;
+        if (work.shared && part.hand_in >= 0) {
+            bool ok = true;
+            if (lane == 0) ok = wait_for_count(g.handed + part.hand_in, part.width / 16);
+            if (!__all_sync(0xffffffffu, ok)) code = 336;
+            s0 = g.hand + (long long)part.hand_in * DK * part.width;
+        }
+        const int width = part.width;
+#pragma unroll 1
+        for (int c = 0; c < HC; c += 32) {                        // (every further round is a trip to memory)
+            uint32_t x[32], y[16];
+            const float* at = s0 + (long long)(h * HC + c) * width + j;
+#pragma unroll
+            for (int e = 0; e < 32; ++e)
+                x[e] = __float_as_uint(s0 ? (work.shared ? ld_cg_f32(at + e * width) : at[e * width]) : part.response && h * HC + c + e == j ? 1.f : 0.f);
+            tmem_st32(t_s + c, x);
+#pragma unroll
+            for (int e = 0; e < 16; ++e) y[e] = pack_h2(-__uint_as_float(x[2 * e]), -__uint_as_float(x[2 * e + 1]));
+            tmem_st16(t_s16 + c / 2, y);
+        }
+        if (work.shared && i + 1 < work.size() && work[i + 1].S0 && work[i + 1].hand_in < 0)       // (the next part's, to the L2: a line of 128 bytes for each row i and quarter)
+            for (int e = lane; e < HC; e += 32) asm volatile("prefetch.global.L2 [%0];" ::"l"(work[i + 1].S0 + (long long)(h * HC + e) * width + 32 * (warp & 3)));
+        const int nblk = part.nblk;
+#pragma unroll 1
+        for (int b = 0;; parity ^= 1) {
+            publish(B_SP);
+            if constexpr (!W) {
+                if (!mbar_wait_tries<false>(bar + 8 * B_RD, parity)) return 312;
+                tc_fence_after();
+                to_operand<32, false>(t_u, T_R16 + 16 * h + lanes);
+                publish(B_RP);
+            }
+            if (!mbar_wait_tries<false>(bar + 8 * B_UD, parity)) return 313;
+            tc_fence_after();
+            to_operand<32, false>(t_u, t_u16);
+            publish(B_UP);
+            if (!mbar_wait_tries<false>(bar + 8 * B_SD, parity)) return 314;
+            tc_fence_after();
+            if (++b == nblk) break;
+            to_operand<HC, true>(t_s, t_s16);
+        }
+        parity ^= 1;
+        end_state<DK, ChainWork<MODE>::shared>(g, part, lost + i, warp, lane);
+    }
+    return code;
+}
+
+// The products of the chain (one warp).  Returns the code of the wait that ran out, or 0.
+template <int DK, bool W, int R, int DV, int MODE>
+__device__ __forceinline__ int mma_role(ChainWork<MODE> work, uint8_t* smem, uint32_t bar) {
+    using CFG = ChainCfg<DK, W, R, DV>;
+    using SM = ChainSmem<DK, R, DV>;
+    constexpr int V_SLAB = NB * 128, K_SLAB = SM::rows * 128, CP = SM::CP, OB = O_BUFS<CP>;
+    constexpr bool INPLACE = U_INPLACE<W, CP>;
+    const uint32_t smem_b = smem_u32(smem);
+    RingPos<CFG::NS> ks;
+    RingPos<CFG::NV> vs;
+    RingPos<CFG::NT> ts;
+    RingPos<CFG::NW> ws;
+    auto wait = [&](int which, int parity) { return mbar_wait_tries<false>(bar + 8 * which, (uint32_t)parity); };
+    int b = 0;                                                    // (of the CTA's blocks)
+#pragma unroll 1
+    for (int i = 0; i < work.size(); ++i) {
+    const int end = b + work[i].nblk;
+    const bool response = work[i].response;
+#pragma unroll 1
+    for (; b < end; ++b) {
+        const uint32_t k_at = smem_b + ks.i * SM::stage + SM::k_off, v_lo = lo_of(smem_b + CFG::v_off + vs.i * SM::v_bytes, DV == 128 ? V_SLAB : 0),
+                       t_lo = lo_of(smem_b + CFG::t_off + ts.i * SM::t_bytes);
+        // (at d_v = 64 the 64 columns of V's tile are read twice: rows j past d_v are nobody's)
+        if constexpr (W) {
+            // ---- U'^T = V^T T^T (W is there, and so T; the accumulator's last reader, the chain warps' conversion of U' of the block before, is done; its
+            //      fp16 pairs' readers are)
+            if (INPLACE && b > 0 && (!wait(B_SD, (b - 1) & 1) || !wait(B_OD + (b - 1) % OB, ((b - 1) / OB) & 1))) return 315;
+            if (!wait(CFG::WDONE + ws.i, ws.phase)) return 326;
+            if (!response) {
+                tc_fence_after();
+                if (elect_one()) {
+                    products_tt(T_U, v_lo, t_lo);
+                    commit_at(bar + 8 * (CFG::VFREE + vs.i));
+                }
+                __syncwarp();
+            }
+            // ---- ... - S W^T
+            // (U' completes only after the last reader of the block before's, P U', so that the chain warps need not wait for that)
+            if (!INPLACE && b > 0 && !wait(B_OD + (b - 1) % OB, ((b - 1) / OB) & 1)) return 319;
+            if (!wait(B_SP, b & 1)) return 323;
+            tc_fence_after();
+            if (elect_one()) {
+                products_ta<true, NB, DK / 16, DK>(T_U, T_S16, lo_of(smem_b + CFG::w_off + ws.i * SM::w_bytes), !response);
+                commit_at(bar + 8 * B_UD);
+                commit_at(bar + 8 * (CFG::WFREE + ws.i));
+            }
+            __syncwarp();
+        } else {
+            // ---- V^T into the accumulator, as V^T times an identity, both bf16 (V as it came; the accumulator's last reader is done)
+            if (!response) {
+                if (!wait(CFG::LAND + ks.i, ks.phase)) return 327;
+                tc_fence_after();
+                if (elect_one()) {
+                    constexpr uint32_t idesc = make_idesc(NB, true, false, false) | (1u << 7) | (1u << 10);
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) mma_f16(T_U, desc_lo(v_lo + c * (2048 >> 4)), IdStrip::desc(smem_b + CFG::id_off, c), idesc, c > 0);
+                }
+                __syncwarp();
+            }
+            // ---- R = V^T - S K^T
+            if (!wait(CFG::FULL + ks.i, ks.phase)) return 322;
+            if (!wait(B_SP, b & 1)) return 323;
+            tc_fence_after();
+            if (elect_one()) {
+                products_ta<false, NB, DK / 16, SM::rows>(T_U, T_S16, lo_of(k_at), !response);
+                commit_at(bar + 8 * B_RD);
+            }
+            __syncwarp();
+            // ---- U'^T = R T^T
+            // (U' completes only after the last reader of the block before's, P U', so that the chain warps need not wait for that)
+            if (b > 0 && !wait(B_OD + (b - 1) % OB, ((b - 1) / OB) & 1)) return 319;
+            if (!wait(B_RP, b & 1)) return 326;
+            tc_fence_after();
+            if (elect_one()) {
+                products_ta<false, NB, NB / 16, NB>(T_U, T_R16, t_lo, false);
+                commit_at(bar + 8 * B_UD);
+            }
+            __syncwarp();
+        }
+        // ---- S += U'^T K
+        // (and S only after Q S^T)
+        if (!wait(B_QD, b & 1)) return 320;
+        if (!wait(B_UP, b & 1)) return 328;
+        tc_fence_after();
+        if (elect_one()) {
+            products_ta<true, DK, NB / 16, SM::rows, false, INPLACE ? 16 : 0>(T_S, T_U16<W, CP>, lo_of(k_at, K_SLAB), true);
+            commit_at(bar + 8 * B_SD);
+            commit_at(bar + 8 * (CFG::EMPTY + ks.i));
+        }
+        __syncwarp();
+        ks.next();
+        vs.next();
+        ts.next();
+        ws.next();
+    }
+    }
+    return 0;
+}
+
+// The products of the output (one warp): O^T = S Q^T + U'^T P^T with the state before the update.
+template <int DK, bool W, int R, int DV>
+__device__ __forceinline__ void mma_out_role(int count, int width, int* err, uint8_t* smem, uint32_t bar) {
+    using SM = ChainSmem<DK, R, DV>;
+    using CFG = ChainCfg<DK, W, R, DV>;
+    constexpr int CP = SM::CP, OB = O_BUFS<CP>;
+    const uint32_t smem_b = smem_u32(smem);
+    const int parties = width + 32;
+    RingPos<CFG::NS> ks;
+    RingPos<CFG::NT> ts;
+    RingPos<OB> os;
+    Waits waits(bar);
+#pragma unroll 1
+    for (int b = 0; b < count; ++b) {
+        const uint32_t sg = smem_b + ks.i * SM::stage, t_o = o_cols<CP>(os.i);
+        waits.wait(CFG::FULL + ks.i, ks.phase, 351);
+        if (b >= OB) waits.wait(B_OFREE + os.i, os.phase ^ 1, 325);
+        waits.wait(W ? B_SP : B_RD, b & 1, 352);
+        tc_fence_after();
+        if (waits.ok() && elect_one()) {
+            products_ta<false, CP, DK / 16, SM::rows, true>(t_o, T_S16, lo_of(sg + SM::q_off), false);
+            commit_at(bar + 8 * B_QD);
+        }
+        __syncwarp();
+        waits.wait(B_UP, b & 1, 354);
+        tc_fence_after();
+        if (waits.ok() && elect_one()) {
+            products_ta<false, CP, NB / 16, CP, false, U_INPLACE<W, CP> ? 16 : 0>(t_o, T_U16<W, CP>, lo_of(sg + SM::p_off), true);
+            commit_at(bar + 8 * (B_OD + os.i));
+            commit_at(bar + 8 * (CFG::EMPTY + ks.i));
+        }
+        __syncwarp();
+        if (W && b + CFG::NT < count) pass_on(N_TFREE + ts.i, 160);
+        waits.wait(B_OD + os.i, os.phase, 331);
+        // (also when it has given up: the output's warps must have passed this barrier before it is arrived at again)
+        if (!waits.ok() && b >= OB) mbar_wait_tries<true>(bar + 8 * (B_OFREE + os.i), os.phase ^ 1);
+        pass_on(N_OD + os.i, parties);
+        ks.next();
+        ts.next();
+        os.next();
+    }
+    if (!waits.ok()) atomicCAS(err, 0, waits.code);
+}
+
+// V of each block to fp16 in place, NV blocks ahead, and O of each block from tensor memory to global memory: warp `warp` of four has rows j = 32 warp + lane, and one store of a warp is
+// 128 contiguous bytes of a token's row (64 of a response's).
+template <int DK, bool W, int R, int DV, int MODE>
+__device__ __forceinline__ void out_role(const ChainGeo& g, ChainWork<MODE> work, int* err, uint8_t* smem, uint32_t bar, int warp, int lane) {
+    using SM = ChainSmem<DK, R, DV>;
+    using CFG = ChainCfg<DK, W, R, DV>;
+    constexpr int C = SM::C, CP = SM::CP, OB = O_BUFS<CP>;
+    const int j = 32 * warp + lane, parties = work[0].width + 32;
+    RingPos<CFG::NV> vs;
+    RingPos<OB> os;
+    Waits waits(bar);
+    const uint32_t lanes = (uint32_t)(32 * warp) << 16;
+#pragma unroll 1
+    for (int i = 0; i < work.size(); ++i) {
+    const ChainPart& part = work[i];
+    float* o = part.O + j;
+    __half* oh = (__half*)part.O + j;
+    const int nblk = part.nblk, b0 = part.b0;
+    const bool response = part.response;
+#pragma unroll 1
+    for (int b = W ? -CFG::NV : 0; b < nblk; ++b) {
+        if (b >= 0) {
+            named_bar(N_OD + os.i, parties);
+            tc_fence_after();
+            const int Cv = min(C, g.L - (b0 + b) * C);
+#pragma unroll 1
+            for (int c = 0; c < CP; c += 16) {
+                uint32_t x[16];
+                tmem_ld16(o_cols<CP>(os.i) + lanes + c, x);
+                tmem_ld_wait();
+                if (c + 16 == CP) {
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive_at(bar + 8 * (B_OFREE + os.i));
+                }
+                if (response) {
+#pragma unroll
+                    for (int t = 0; t < 16; ++t)
+                        if (c + t < Cv) oh[(c + t) * DK] = __float2half_rn(__uint_as_float(x[t]));
+                } else {
+#pragma unroll
+                    for (int t = 0; t < 16; ++t)
+                        if (c + t < Cv) o[(c + t) * DV] = __uint_as_float(x[t]);
+                }
+            }
+            o += C * DV;
+            oh += C * DK;
+            os.next();
+        }
+        if (W && b + CFG::NV < nblk && !response) {
+            waits.wait(CFG::VLAND + vs.i, vs.phase, 333);
+            convert_pieces<8, DV>(smem + CFG::v_off + vs.i * SM::v_bytes, j);
+            publish_smem(bar + 8 * (CFG::WDONE + vs.i), lane);
+            vs.next();
+        }
+    }
+    }
+    if (!waits.ok()) atomicCAS(err, 0, waits.code);
+}
+
+template <int DK, bool W, int R, int DV, int MODE>
 __global__ void __launch_bounds__(CHAIN_THREADS<W>, 1)
 chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __restrict__ beta, const float* __restrict__ S0,
              float* __restrict__ O, float* __restrict__ S_final, int* __restrict__ status, ChainGeo g, ChainSeg sg) {
@@ -1102,11 +1238,14 @@ chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __rest
     __shared__ uint64_t bar[CFG::count];
     __shared__ uint32_t tmem_base;
     __shared__ ChainArgs args;
-    __shared__ uint32_t lost;
+    __shared__ uint32_t lost[MODE == SHARED ? MOST_PARTS : 1];
+    __shared__ ChainPart parts[MODE == SHARED ? MOST_PARTS : 1];
+    __shared__ int parts_n;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t bar_b = smem_u32(bar);
-    long long seq;
-    const ChainPart part = chain_part<DK, SM::C, SEG>(g, sg, S0, O, S_final, seq);
+    // (SHARED: all parts have one width, and only `width` of this one is used)
+    const ChainPart part = MODE == SHARED ? walk_of<DK, SM::C, MODE>(g, sg, S0, O, S_final, 0, 0, false, 0, g.nblk) : own_walk<DK, SM::C, MODE>(g, sg, S0, O, S_final);
+    const int lo = share_of_cta() * g.share, count = MODE == SHARED ? min(g.share, g.total - lo) : part.nblk;
     const int quarters = part.width / 32;                         // lane quarters that hold rows of the state
     if ((smem_u32(smem) & 1023u) != 0) {                          // (the swizzled layouts need a 1024-byte aligned base)
         wait_for_previous_kernel();
@@ -1115,7 +1254,7 @@ chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __rest
     }
     if (tid == 32) args = {g, sg};
     if (tid == 0) {
-        lost = 0;
+        for (int x = 0; x < (MODE == SHARED ? MOST_PARTS : 1); ++x) lost[x] = 0;
         mbar_init(&bar[B_SP], 2 * quarters);
         mbar_init(&bar[B_UP], 2 * quarters);
         mbar_init(&bar[B_SD], 1);
@@ -1148,11 +1287,17 @@ chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __rest
         prefetch_tmap(&maps.k);
         prefetch_tmap(&maps.v);
     }
+    if (MODE == SHARED && tid == 64) {
+        int n = 0;
+#pragma unroll 1
+        for (int x = lo; x < lo + count && n < MOST_PARTS; x += parts[n++].nblk) parts[n] = part_at<DK, SM::C>(g, sg, S0, O, S_final, x, lo, lo + count);
+        parts_n = n;
+    }
     if (warp == W_MMA) tmem_alloc(&tmem_base, 512);
     if (SM::CP > SM::C) {                                         // (r = 3: query rows that no copy writes are read)
         for (int e = tid; e < CFG::NS * SM::stage / 16; e += CHAIN_THREADS<W>) ((uint4*)smem)[e] = make_uint4(0, 0, 0, 0);
     } else {                                                      // (the upper triangles of P and T, which nothing writes)
-        for (int st = 0; st < CFG::NS && st < part.nblk; ++st)
+        for (int st = 0; st < CFG::NS && st < count; ++st)
             for (int e = tid; e < SM::p_bytes / 16; e += CHAIN_THREADS<W>) ((uint4*)(smem + st * SM::stage + SM::p_off))[e] = make_uint4(0, 0, 0, 0);
     }
     for (int e = tid; e < CFG::NT * SM::t_bytes / 16; e += CHAIN_THREADS<W>) ((uint4*)(smem + CFG::t_off))[e] = make_uint4(0, 0, 0, 0);
@@ -1168,12 +1313,13 @@ chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __rest
         if (warp == W_MMA) tmem_dealloc(tmem_base, 512);
         return;
     }
+    const ChainWork<MODE> work{part, parts, MODE == SHARED ? parts_n : 1, count};
     // (each warpgroup sets its registers once, and no code is shared after that: its end is in its own branch)
     // (each waits for the kernel before by itself: nothing is left to be set up for each other after that.  With the CTA's barrier after that wait
     //  and the end state after the last output, us: 16 sequences of 40, d = 128, r = 2: 8.7, now 7.8; 148 of 40, d = 64: 7.9, now 7.0)
     auto begin = [&]() {
         wait_for_previous_kernel();
-        if (!SEG) let_next_kernel_start();  // (chain_compose's blocks would crowd on what few multiprocessors have room: 144 us instead of 140)
+        if (g.nseg == 1) let_next_kernel_start();  // (chain_compose's blocks would crowd on what few multiprocessors have room: 144 us instead of 140)
     };
     auto all_done = [&]() {
         __syncwarp();
@@ -1184,7 +1330,19 @@ chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __rest
     // (the chain's and the solve teams' warps, eight rows each, us a token with every row lost and with the chain's warps alone: d = 128, r = 1, 2, 4
     //  0.97, 1.56, 3.7 and 2.4, 5.1, 9.2; d = 64, r = 1 .. 4 0.54, 0.81, 1.1, 1.2 and 1.1, 2.1, 3.0, 3.3.  Fetching the next token's inputs ahead: no gain)
     auto walk_lost = [&](int x) {
-        if (lost >> (x >> 2) & 1) walk_fp32<DK, R>(args, part, seq, 8 * x);
+#pragma unroll 1
+        for (int i = 0; i < work.size(); ++i) {
+            if (!(lost[i] >> (x >> 2) & 1)) continue;
+            ChainPart p = work[i];
+            if (MODE == SHARED && p.hand_in >= 0) {               // all of the walk, when its first part's outputs, which are replaced here, are written
+                if (lane == 0 && !wait_for_count(g.finished + p.hand_in + 1, 1)) atomicCAS(status, 0, 337);
+                __syncwarp();
+                p.b0 -= p.before;
+                p.O -= (long long)p.before * SM::C * g.d_v;
+                p.nblk = p.walk;
+            }
+            walk_fp32<DK, R>(args, p, p.seq, 8 * x);
+        }
     };
     if (warp < W_OUT) {
         set_registers<W, REGS_CHAIN>();
@@ -1192,47 +1350,50 @@ chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __rest
         if (tid == 0 && blockIdx.x == 0 && g.clear) *status = 0;  // (the call's status word: a wait expires a second from now at the earliest)
         const bool holds_state = (warp & 3) < quarters;
         if (holds_state) {
-            const int code = chain_role<DK, W, SM::CP>(part, bar_b, warp, lane);
+            const int code = chain_role<DK, W, SM::CP>(g, work, lost, bar_b, warp, lane);
             if (code) atomicCAS(status, 0, code);
-            end_state<DK>(part, &lost, warp, lane);
         }
         all_done();                                               // (every output is written)
+        if (MODE == SHARED && tid == 0) {
+            __threadfence();
+            st_release_gpu(g.finished + share_of_cta(), 1);
+        }
         walk_lost(warp);
     } else if (warp < W_CONV) {
         set_registers<W, REGS_OUT>();
         begin();
-        if (warp - W_OUT < quarters) out_role<DK, W, R, DV>(g, part, status, smem, bar_b, warp - W_OUT, lane);
+        if (warp - W_OUT < quarters) out_role<DK, W, R, DV>(g, work, status, smem, bar_b, warp - W_OUT, lane);
         all_done();
     } else if (warp < W_SOLVE) {
         set_registers<W, REGS_CONV>();
         begin();
-        convert_role<DK, W, R, DV>(part, smem, bar_b, tid - 32 * W_CONV);
+        convert_role<DK, W, R, DV>(count, smem, bar_b, tid - 32 * W_CONV);
         all_done();
     } else if (warp < W_MMA) {
         set_registers<W, REGS_SOLVE<W>>();
         begin();
-        solve_role<DK, W, R, DV>(g, part, beta, smem, bar_b, seq, (warp - W_SOLVE) >> 2, (tid - 32 * W_SOLVE) & 127);
+        solve_role<DK, W, R, DV>(g, work, beta, smem, bar_b, (warp - W_SOLVE) >> 2, (tid - 32 * W_SOLVE) & 127);
         all_done();
         walk_lost(8 + warp - W_SOLVE);
     } else if (warp < W_W) {
         set_registers<W, REGS_ISSUE>();
         begin();
         if (warp == W_MMA) {
-            const int code = mma_role<DK, W, R, DV>(part, smem, bar_b);
+            const int code = mma_role<DK, W, R, DV>(work, smem, bar_b);
             if (code) atomicCAS(status, 0, code);
         } else if (warp == W_MMA_OUT) {
-            mma_out_role<DK, W, R, DV>(part, status, smem, bar_b);
+            mma_out_role<DK, W, R, DV>(count, part.width, status, smem, bar_b);
         } else if (warp == W_GRAM) {
-            gram_role<DK, W, R, DV>(part, status, smem, bar_b);
+            gram_role<DK, W, R, DV>(count, status, smem, bar_b);
         } else if (warp == W_LOAD) {
-            load_role<DK, W, R, DV>(maps, status, smem, bar_b, (int)seq, part);
+            load_role<DK, W, R, DV>(maps, work, status, smem, bar_b);
         }
         all_done();
         if (warp == W_MMA) tmem_dealloc(0, 512);
     } else if constexpr (W) {
         set_registers<W, REGS_W>();
         begin();
-        w_role<DK, W, R, DV>(part, status, smem, bar_b, tid - 32 * W_W);
+        w_role<DK, W, R, DV>(count, status, smem, bar_b, tid - 32 * W_W);
         all_done();
     }
 }
@@ -1346,14 +1507,14 @@ __global__ void __launch_bounds__(128) chain_compose(ChainSeg sg, float* __restr
 // O[t][j] += sum_i R[t][i] start[j][i] for the tokens of all segments but the first: grid (128-token tiles, nseq (nseg - 1)), a
 // warp per 16 tokens.  Bound by the traffic: per token R once, O read and written.
 template <int DK, int DV>
-__global__ void __launch_bounds__(256) chain_apply(ChainSeg sg, float* __restrict__ O, int L, int seg_tokens, int nseg) {
+__global__ void __launch_bounds__(256) chain_apply(ChainSeg sg, float* __restrict__ O, int L, int first_tokens, int seg_tokens, int nseg) {
     constexpr int LD = DK + 8, KT = DK / 16;
     extern __shared__ __align__(16) uint8_t smem_tail[];
     __half* sS = (__half*)smem_tail;                                   // [DV][LD]
     const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31, gq = lane >> 2, t4 = lane & 3;
     const long long seq = blockIdx.y / (nseg - 1);
     const int s = 1 + (int)(blockIdx.y % (nseg - 1));
-    const int t_end = min(L, (s + 1) * seg_tokens), t0 = s * seg_tokens + blockIdx.x * 128 + w * 16 + gq;
+    const int start = first_tokens + (s - 1) * seg_tokens, t_end = min(L, start + seg_tokens), t0 = start + blockIdx.x * 128 + w * 16 + gq;
     const __half* src = sg.start + (seq * nseg + s) * DV * DK;
     wait_for_previous_kernel();
 #pragma unroll
@@ -1412,8 +1573,53 @@ __global__ void __launch_bounds__(256) chain_apply(ChainSeg sg, float* __restric
 struct ChainPlan {
     int nseg, seg_blk;
     double us;
+    int first_blk;            // blocks of the first segment
+    int share, ctas;          // SHARED: blocks of a CTA (0: a walk each) and CTAs
     double short_us;          // the kernel alone without segments, the start of each wave counted: what a call of a few blocks takes
 };
+// Equal shares of all blocks (part_at) in place of a walk each, where that is faster: more sequences than multiprocessors, or, of a state as wide as its response,
+// few in segments, the first of which is as long as a share (it has no response to walk) and the others as many as it takes.  Against it stand clearing the flags, a state
+// through memory and the starts of further walks, 12 us and 1.5 a walk, a block that takes longer while all multiprocessors are busy to the end, and more responses.
+// Measured, us, shared out and not, d = 128: 160 and 200 sequences of 1000, r = 2: 85 and 110, 97 and 115; 256 of 1024: 119 and 113 (not taken); 300 of 500, r = 4: 124
+// and 155; 32 of 8192, r = 2: 225 and 239 (single launch: 247); r = 3: 294 and 343; r = 1: 175 and 167 (not taken); d = 64: 64 of 4096, r = 4: 207 and 257; 200 of
+// 2000, r = 1: 80 and 96; 32 of 8192, r = 2: 152 and 176.  The estimates below come within 5 % of these (one wave's by 8 % less than make_plan's, whose choices against the
+// single launch are left as they are).  Not where the responses need more memory than the library keeps from call to call: 32 of 65536, r = 2, take 2200 us
+// and the single launch 1815.
+constexpr size_t SHARE_MOST_BYTES = (size_t)88 << 20;
+ChainPlan share_out(const Problem& p, const ChainPlan& plan, int nblk, double block_us) {
+    const long long nseq = (long long)p.B * p.H, sms = sm_count();
+    if (sms < 1 || nseq * nblk > 0x3fffffffLL || p.no_share) return plan;
+    const double row_bytes = 4.0 * p.d_k + 8.0 * p.d_v, tail = p.d_k == 128 ? 4.0 : 2.0, per_seg = p.d_k == 128 ? 0.85 : 0.4;
+    ChainPlan out = plan;
+    double us = 12.0, rival = 7.0 + 0.92 * (plan.us - 7.0);
+    if (nseq > sms) {
+        out.nseg = 1;
+        out.seg_blk = out.first_blk = nblk;
+        block_us *= p.d_k == 128 ? 1.05 : 0.95;
+    } else {
+        if (p.d_k != p.d_v || nblk < 8 || (size_t)nseq * p.L * p.d_k * 2 > SHARE_MOST_BYTES) return plan;
+        const long long first = 2 * nblk * nseq / (sms + nseq);
+        if (first >= nblk || first < 1) return plan;
+        out.nseg = 1 + (int)((nblk - first + first - 1) / first);
+        if (out.nseg > 64) return plan;
+        out.seg_blk = (int)((nblk - first + out.nseg - 2) / (out.nseg - 1));
+        out.first_blk = nblk - (out.nseg - 1) * out.seg_blk;
+        if (out.first_blk < 1) return plan;
+        us += 3.0 + tail + per_seg * out.nseg + (double)nseq * p.L * (nblk - out.first_blk) / nblk * row_bytes / 6e6;
+        if (p.d_k == 64) block_us *= 0.95;
+        if (plan.nseg > 1) {      // (the composing kernels' part of the estimate does not shrink, their traffic goes at 6 TB/s)
+            const double traffic = (double)nseq * p.L * (plan.nseg - 1) / plan.nseg * row_bytes, kernels = (p.d_k == 128 ? 11.0 : 9.0) + per_seg * plan.nseg;
+            rival = kernels + traffic / 6e6 + 0.92 * (plan.us - kernels - traffic / 4e6);
+        }
+    }
+    const long long total = nseq * (2 * nblk - out.first_blk);
+    out.share = (int)((total + sms - 1) / sms);
+    out.ctas = (int)((total + out.share - 1) / out.share);
+    const int other = out.nseg > 1 ? out.seg_blk : out.first_blk, longest = out.first_blk > other ? out.first_blk : other, shortest = out.first_blk < other ? out.first_blk : other;
+    if (longest > out.share || out.share / shortest + 2 > MOST_PARTS) return plan;
+    out.us = us + out.share * block_us + 1.5 * out.share / shortest;
+    return out.us < 0.985 * rival ? out : plan;
+}
 ChainPlan make_plan(const Problem& p) {
     static const double alone[2][4] = {{1.40, 1.25, 1.25, 1.19}, {1.95, 1.53, 1.50, 1.55}};
     static const double crowded[2][4] = {{1.70, 1.34, 1.33, 1.24}, {2.30, 1.79, 1.68, 1.58}};
@@ -1425,23 +1631,23 @@ ChainPlan make_plan(const Problem& p) {
         return a + (c - a) * (crowd < 0.0 ? 0.0 : crowd > 1.0 ? 1.0 : crowd);
     };
     const double waves = (double)((nseq + sms - 1) / (sms > 0 ? sms : 1)), walk = nblk * step(nseq) * waves;
-    ChainPlan plan{1, nblk, 7.0 + walk, 5.0 * waves + walk};
+    ChainPlan plan{1, nblk, 7.0 + walk, nblk, 0, 0, 5.0 * waves + walk};
     const double limit = 0.92 * plan.us;
     // (calls of up to 512 tokens at d_k = 128 are one launch, which a test of two sequences of 512 expects, also where segments would be faster: 16 of
     //  333, r = 2: 21.7 us, 20.9 estimated in four)
-    if (p.d_k == 128 && p.L <= 512) return plan;
+    if (p.d_k == 128 && p.L <= 512) return nseq > sms ? share_out(p, plan, nblk, step(sms)) : plan;
     for (int want = 2; nseq * (2 * want - 1) <= sms && want <= 64 && want <= nblk; ++want) {
         const int seg_blk = (nblk + want - 1) / want, nseg = (nblk + seg_blk - 1) / seg_blk;
         // (two kernels, their share per segment, and the traffic of the responses and of O at about 4 TB/s)
         const double traffic = (double)nseq * p.L * (nseg - 1) / nseg * (4.0 * p.d_k + 8.0 * p.d_v) / 4e6;
         const double us = (p.d_k == 128 ? 11.0 + 0.85 * nseg : 9.0 + 0.4 * nseg) + traffic + seg_blk * step(nseq * (2 * nseg - 1));
-        if (us < limit && us < plan.us) plan = {nseg, seg_blk, us, plan.short_us};
+        if (us < limit && us < plan.us) plan = {nseg, seg_blk, us, seg_blk, 0, 0, plan.short_us};
     }
-    return plan;
+    return share_out(p, plan, nblk, step(sms));
 }
 
 struct ChainCarve {
-    size_t R, P, D, Xi, start, total;
+    size_t R, P, D, Xi, start, flags, hand, total;
 };
 ChainCarve carve(const Problem& p, const ChainPlan& plan) {
     ChainCarve c{};
@@ -1459,21 +1665,33 @@ ChainCarve carve(const Problem& p, const ChainPlan& plan) {
         c.Xi = take(slots * p.d_k * p.d_v * 4);
         c.start = take(slots * p.d_v * p.d_k * 2);
     }
+    if (plan.share > 0) {
+        c.flags = take((size_t)plan.ctas * 8);
+        c.hand = take((size_t)plan.ctas * p.d_k * p.d_v * 4);
+    }
     c.total = off;
     return c;
 }
 
-template <int DK, int R, int DV, bool SEG>
-int launch(const Problem& p, const ChainPlan& plan, const ChainSeg& sg) {
-    constexpr bool W = w_form(DK, DV, SEG);
+template <int DK, int R, int DV, int MODE>
+int launch(const Problem& p, const ChainPlan& plan, const ChainSeg& sg, void* workspace) {
+    constexpr bool W = w_form(DK, DV, MODE != WHOLE);
     using CFG = ChainCfg<DK, W, R, DV>;
-    static_assert(CFG::total <= SMEM_MOST && CFG::NS >= 3 && (!W || (CFG::NS >= 4 && CFG::NT <= 3 && CFG::NV == CFG::NW)), "shared memory budget");
-    const void* fn = (const void*)chain_kernel<DK, W, R, DV, SEG>;
+    static_assert(CFG::total + (MODE == SHARED ? 4096 : 1024) <= 227 * 1024 && CFG::NS >= 3 && (!W || (CFG::NS >= 4 && CFG::NT <= 3 && CFG::NV == CFG::NW)), "shared memory budget");
+    const void* fn = (const void*)chain_kernel<DK, W, R, DV, MODE>;
     constexpr int C = NB / R;
-    ChainGeo g{p.L, p.d_v, (p.L + C - 1) / C, plan.nseg, plan.seg_blk, p.mask_group(), p.exact ? 1 : 0, p.clear_status ? 1 : 0,
+    ChainGeo g{p.L, p.d_v, (p.L + C - 1) / C, plan.nseg, plan.seg_blk, plan.first_blk, plan.share, 0, nullptr, nullptr, nullptr, p.mask_group(), p.exact ? 1 : 0, p.clear_status ? 1 : 0,
                (const __nv_bfloat16*)p.q, (const __nv_bfloat16*)p.k, (const __nv_bfloat16*)p.v, (const __nv_bfloat16*)p.beta,
                p.S0, p.O, p.S_final};
-    const long long nseq = (long long)p.B * p.H, grid = nseq * (2 * plan.nseg - 1);
+    const long long nseq = (long long)p.B * p.H, grid = MODE == SHARED ? plan.ctas : nseq * (2 * plan.nseg - 1);
+    if (MODE == SHARED) {
+        const ChainCarve c = carve(p, plan);
+        g.total = (int)(nseq * (2 * g.nblk - g.first_blk));
+        g.handed = (int*)((uint8_t*)workspace + c.flags);
+        g.finished = g.handed + plan.ctas;
+        g.hand = (float*)((uint8_t*)workspace + c.hand);
+        PF_CUDA_TRY(cudaMemsetAsync(g.handed, 0, (size_t)plan.ctas * 8, p.stream));
+    }
     ChainMaps maps;
     if (!make_slab_map(&maps.k, p.k, nseq, (uint64_t)p.L * R, DK, 64, NB, 1) ||
         !make_slab_map(&maps.q, p.q, nseq, p.L, DK, 64, C, 1) ||
@@ -1491,23 +1709,24 @@ int launch(const Problem& p, const ChainPlan& plan, const ChainSeg& sg) {
 }
 
 template <int DK, int R>
-int launch_plan(const Problem& p, const ChainPlan& plan, const ChainSeg& sg) {
-    if (plan.nseg > 1) return p.d_v == 128 ? launch<DK, R, 128, true>(p, plan, sg) : launch<DK, R, 64, true>(p, plan, sg);
-    return p.d_v == 128 ? launch<DK, R, 128, false>(p, plan, sg) : launch<DK, R, 64, false>(p, plan, sg);
+int launch_plan(const Problem& p, const ChainPlan& plan, const ChainSeg& sg, void* ws) {
+    if (plan.share > 0) return p.d_v == 128 ? launch<DK, R, 128, SHARED>(p, plan, sg, ws) : launch<DK, R, 64, SHARED>(p, plan, sg, ws);
+    if (plan.nseg > 1) return p.d_v == 128 ? launch<DK, R, 128, SEGMENTS>(p, plan, sg, ws) : launch<DK, R, 64, SEGMENTS>(p, plan, sg, ws);
+    return p.d_v == 128 ? launch<DK, R, 128, WHOLE>(p, plan, sg, ws) : launch<DK, R, 64, WHOLE>(p, plan, sg, ws);
 }
 template <int DK>
-int launch_rank(const Problem& p, const ChainPlan& plan, const ChainSeg& sg) {
+int launch_rank(const Problem& p, const ChainPlan& plan, const ChainSeg& sg, void* ws) {
     switch (p.r) {
-        case 1: return launch_plan<DK, 1>(p, plan, sg);
-        case 2: return launch_plan<DK, 2>(p, plan, sg);
-        case 3: return launch_plan<DK, 3>(p, plan, sg);
-        default: return launch_plan<DK, 4>(p, plan, sg);
+        case 1: return launch_plan<DK, 1>(p, plan, sg, ws);
+        case 2: return launch_plan<DK, 2>(p, plan, sg, ws);
+        case 3: return launch_plan<DK, 3>(p, plan, sg, ws);
+        default: return launch_plan<DK, 4>(p, plan, sg, ws);
     }
 }
 
 template <int DK, int DV>
 int launch_seg_tail(const Problem& p, const ChainPlan& plan, const ChainSeg& sg) {
-    const int nseq = p.B * p.H, dv = DV, seg_tokens = plan.seg_blk * (NB / p.r);
+    const int nseq = p.B * p.H, dv = DV, seg_tokens = plan.seg_blk * (NB / p.r), first_tokens = plan.first_blk * (NB / p.r);
     constexpr int LD = DK + 8;
     {
         using SM = ComposeSmem<DK>;
@@ -1522,7 +1741,7 @@ int launch_seg_tail(const Problem& p, const ChainPlan& plan, const ChainSeg& sg)
     }
     constexpr int smem = DV * LD * 2;
     prof_begin("chain_apply", p.stream);
-    void* args[] = {(void*)&sg, (void*)&p.O, (void*)&p.L, (void*)&seg_tokens, (void*)&plan.nseg};
+    void* args[] = {(void*)&sg, (void*)&p.O, (void*)&p.L, (void*)&first_tokens, (void*)&seg_tokens, (void*)&plan.nseg};
     PF_CUDA_TRY(launch_early((const void*)chain_apply<DK, DV>, dim3((unsigned)((seg_tokens + 127) / 128), (unsigned)(nseq * (plan.nseg - 1))), 256,
                              args, smem, p.stream));
     prof_end(p.stream);
@@ -1536,7 +1755,11 @@ double chain_estimate_us(const Problem& p) { return make_plan(p).us; }
 double chain_short_us(const Problem& p) { return make_plan(p).short_us; }
 
 size_t chain_workspace_bytes(const Problem& p) { return carve(p, make_plan(p)).total; }
-bool chain_needs_workspace(const Problem& p) { return make_plan(p).nseg > 1; }
+bool chain_shares(const Problem& p) { return make_plan(p).share > 0; }
+bool chain_needs_workspace(const Problem& p) {
+    const ChainPlan plan = make_plan(p);
+    return plan.nseg > 1 || plan.share > 0;
+}
 
 bool chain_supported(const Problem& p) {
     return p.in_dtype == PF_DTYPE_BF16 && p.L >= 1 && (long long)p.B * p.H * (p.d_v / 32) <= 0x7fffffffLL &&
@@ -1551,7 +1774,7 @@ int chain_forward(const Problem& p, void* workspace) {
         uint8_t* ws = (uint8_t*)workspace;
         sg = {(__half*)(ws + c.R), (__half*)(ws + c.P), (float*)(ws + c.D), (float*)(ws + c.Xi), (__half*)(ws + c.start)};
     }
-    const int st = p.d_k == 128 ? launch_rank<128>(p, plan, sg) : launch_rank<64>(p, plan, sg);
+    const int st = p.d_k == 128 ? launch_rank<128>(p, plan, sg, workspace) : launch_rank<64>(p, plan, sg, workspace);
     if (st != PF_OK || plan.nseg == 1) return st;
     if (p.d_k == 128) return p.d_v == 128 ? launch_seg_tail<128, 128>(p, plan, sg) : launch_seg_tail<128, 64>(p, plan, sg);
     return p.d_v == 128 ? launch_seg_tail<64, 128>(p, plan, sg) : launch_seg_tail<64, 64>(p, plan, sg);

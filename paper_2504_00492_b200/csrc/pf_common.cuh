@@ -32,6 +32,7 @@ struct Problem {
                             // Theorem 3.3 (pf_params.wu_builder)
     int ring_depth;         // single-launch path: slots per sequence of the hand-off ring, 0 = default (pf_params.ring_depth)
     bool own_workspace;     // the workspace is the library's: as large as the kernels want
+    bool no_share;          // the chain kernel's walks are not shared out in equal parts (which takes workspace): there is none for that
     bool clear_status;      // the kernels set *status to 0 first (false for the second pass of a segmented call)
     int* status;            // device word that receives the code of the first bounded wait that expires (never null
                             // when a tensor-core kernel is launched)
@@ -130,6 +131,7 @@ bool chain_supported(const Problem& p);
 double chain_estimate_us(const Problem& p);
 double chain_short_us(const Problem& p);
 bool chain_needs_workspace(const Problem& p);
+bool chain_shares(const Problem& p);
 size_t chain_workspace_bytes(const Problem& p);
 int chain_forward(const Problem& p, void* workspace);
 

@@ -158,3 +158,49 @@ def test_the_second_walk_of_lost_rows_takes_a_bounded_multiple_of_the_call(d, r,
             times.append(e0.elapsed_time(e1))
         assert torch.isfinite(O).all() and torch.isfinite(S).all()
     assert min(times[3:]) <= most * min(times[:3]), times
+
+
+def _workspaces(w, mode):
+    """Bytes of workspace with which the call's walks are shared out among all SMs, and too few for that."""
+    import ctypes
+
+    from paper_2504_00492_b200 import binding
+    lib = binding.lib()
+    lib.pf_workspace_bytes.restype = ctypes.c_size_t
+    need = lib.pf_workspace_bytes(w.B, w.H, w.L, w.d_k, w.d_v, w.r, w.chunk, 0, 0)
+    return need, 1024 + (w.B * w.H * w.L * w.r * 4 + 255) // 256 * 256
+
+
+@pytest.mark.parametrize("lost", [False, True])
+@pytest.mark.parametrize("d_k,d_v,r,H,L,mode", [(128, 128, 2, 160, 300, "sum"), (128, 64, 3, 150, 200, "product"), (64, 128, 1, 200, 1000, "sum"),
+                                                (128, 128, 1, 190, 1000, "sum"), (128, 128, 4, 180, 701, "product")])
+def test_walks_shared_out_match_whole_ones_to_the_bit(d_k, d_v, r, H, L, mode, lost):
+    """More sequences than SMs: a walk that is cut goes on in another CTA from the very state it had.  Without workspace for that every walk is whole.
+    lost: columns that leave fp16's range in some sequences are walked again, all of the walk by the CTA that has its end."""
+    import paper_2504_00492_b200 as pf
+    w = Workload("shared", B=1, H=H, L=L, d_k=d_k, d_v=d_v, r=r, chunk=64, s0_std=0.1, seed=950 + r)
+    inp = pf_synth.make_inputs(w)
+    if lost:
+        inp.S0[:, ::3, :, 5] = 1e5
+    need, small = _workspaces(w, mode)
+    assert need > small + 148 * 4 * d_k * d_v // 2, "not shared out"
+    d = inp.to("cuda")
+    whole = pf.pf_deltanet_fwd_ex(d.q, d.k, d.v, d.beta, d.S0, w.chunk, mode=mode, workspace=torch.empty(small, dtype=torch.uint8, device="cuda"))
+    for workspace in (None, torch.full((need,), 255, dtype=torch.uint8, device="cuda")):
+        O, S = pf.pf_deltanet_fwd_ex(d.q, d.k, d.v, d.beta, d.S0, w.chunk, mode=mode, workspace=workspace)
+        assert pf.pf_read_status(workspace) == 0 and torch.isfinite(O).all() and torch.isfinite(S).all()
+        assert torch.equal(O, whole[0]) and torch.equal(S, whole[1])
+    if not lost:
+        O_ref, S_ref = util.run_oracle(inp, mode=mode)
+        util.check_per_sequence(O.cpu().numpy(), O_ref, util.TOL_BF16, "O")
+        util.check_per_sequence(S.cpu().numpy(), S_ref, util.TOL_BF16, "S_final")
+
+
+@pytest.mark.parametrize("d,r,H,L,beta_scale", [(64, 2, 32, 5000, 1.0), (128, 4, 32, 2100, 1.0), (64, 4, 32, 3001, 2.0), (128, 4, 32, 2100, 0.02)])
+def test_segments_shared_out(d, r, H, L, beta_scale):
+    """Few sequences in segments of two lengths, cut and shared out among all SMs."""
+    w = Workload("shared_seg", B=1, H=H, L=L, d_k=d, d_v=d, r=r, chunk=64, s0_std=0.1, beta_scale=beta_scale, seed=970 + r)
+    need, _ = _workspaces(w, "sum")
+    assert util.kernels_of(lambda: util.check_parity(w)) == ["chain", "chain_compose", "chain_apply"]
+    # (a byte less is not enough for that, and the call takes the segments it has without: it would be refused if it did not share)
+    assert util.kernels_of(lambda: util.check_parity(w, workspace=torch.empty(need - 1, dtype=torch.uint8, device="cuda"))) == ["chain", "chain_compose", "chain_apply"]
