@@ -4,7 +4,7 @@
 //     T  = (I + Mstrict (.) (diag(beta) K K^T))^{-1} diag(beta)                      (does not depend on S)
 //     P  = (Q K^T) (.) Mincl                                                         (does not depend on S)
 //     U' = T (V - K S^T),       O = Q S^T + P U',       S <- S + U'^T K
-// evaluated in one of two forms (w_form):
+// evaluated in one of two forms (W_FORM_BLOCKS):
 //     V - K S^T first and T applied to it: three products of a block depend on S one after another, R = V - K S^T, U' = T R and the update;
 //     with W = T K formed ahead ("W form"), U' = T V - W S^T: two, at the price of one more product, its way through tensor memory and V in fp16.
 // (Against the fp64 recurrence, 70 sequences of 400, d = 64, r = 4, beta to 2: relative L2 error of O 6.81e-4 with W and 7.12e-4 without: V - K S^T is never rounded.)
@@ -71,11 +71,12 @@ namespace {
 constexpr int NB = 64;               // rows per block
 constexpr int MOST_PARTS = 30;       // parts of walks in a CTA's share
 
-// Where the W form pays (head of the file), us, W and without: 128 sequences of 4096, d = 64, r = 4: 264 and 290; 256 of 1000, d = 64, r = 2: 81 and 85; 64 of 4000,
-// r = 1: 85 and 89.  Not where the walks are short and the chain has nothing ahead at their start (4 of 8192 in segments, d = 64, r = 2: 43 and 40), not at
-// d_v = 128 (140 of 1500, 64 x 128, r = 1: 44 and 43; 48 of 1999, r = 3: level) and not at d_k = 128, where the bound is what a block moves through
-// shared memory, 2950 cycles' worth at r = 2 with W and 2350 without (256 of 1024, r = 2: 118 and 114).
-constexpr bool w_form(int d_k, int d_v, bool segments) { return d_k == 64 && d_v == 64 && !segments; }
+// Where the W form pays (head of the file), us, with W and without, d_k = d_v = 64, a walk to each CTA: 128 sequences of 4096, r = 4: 264 and 290; 256 of 1000, r = 2: 81 and
+// 85; 64 of 4000, r = 1: 85 and 89.  Not where the walks are short and the chain has nothing ahead at their start: 8 of 400, r = 4 (25 blocks): 16.4 and 15.3; 100 of 200,
+// r = 3 (10): 16.5 and 15.9; 140 of 900, r = 1 (15): 26.3 and 26.0; 4 of 8192 in segments, r = 2: 43 and 40.  Not at d_v = 128 (140 of 1500, 64 x 128, r = 1: 44 and 43; 48 of
+// 1999, r = 3: level) and not at d_k = 128, where the bound is what a block moves through shared memory, 2950 cycles' worth at r = 2 with W and 2350 without (256 of 1024,
+// r = 2: 118 and 114).
+constexpr int W_FORM_BLOCKS = 32;
 
 struct ChainMaps {
     CUtensorMap q, k, v;
@@ -1141,7 +1142,7 @@ __device__ __forceinline__ void mma_out_role(int count, int width, int* err, uin
         const uint32_t sg = smem_b + ks.i * SM::stage, t_o = o_cols<CP>(os.i);
         waits.wait(CFG::FULL + ks.i, ks.phase, 351);
         if (b >= OB) waits.wait(B_OFREE + os.i, os.phase ^ 1, 325);
-        waits.wait(W ? B_SP : B_RD, b & 1, 352);
+        waits.wait(W || DK == 64 ? B_SP : B_RD, b & 1, 352);
         tc_fence_after();
         if (waits.ok() && elect_one()) {
             products_ta<false, CP, DK / 16, SM::rows, true>(t_o, T_S16, lo_of(sg + SM::q_off), false);
@@ -1295,12 +1296,12 @@ chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __rest
     }
     if (warp == W_MMA) tmem_alloc(&tmem_base, 512);
     if (SM::CP > SM::C) {                                         // (r = 3: query rows that no copy writes are read)
-        for (int e = tid; e < CFG::NS * SM::stage / 16; e += CHAIN_THREADS<W>) ((uint4*)smem)[e] = make_uint4(0, 0, 0, 0);
+        for (int e = tid; e < min(CFG::NS, count) * (SM::stage / 16); e += CHAIN_THREADS<W>) ((uint4*)smem)[e] = make_uint4(0, 0, 0, 0);
     } else {                                                      // (the upper triangles of P and T, which nothing writes)
         for (int st = 0; st < CFG::NS && st < count; ++st)
             for (int e = tid; e < SM::p_bytes / 16; e += CHAIN_THREADS<W>) ((uint4*)(smem + st * SM::stage + SM::p_off))[e] = make_uint4(0, 0, 0, 0);
     }
-    for (int e = tid; e < CFG::NT * SM::t_bytes / 16; e += CHAIN_THREADS<W>) ((uint4*)(smem + CFG::t_off))[e] = make_uint4(0, 0, 0, 0);
+    for (int e = tid; e < min(CFG::NT, count) * (SM::t_bytes / 16); e += CHAIN_THREADS<W>) ((uint4*)(smem + CFG::t_off))[e] = make_uint4(0, 0, 0, 0);
     if (!W)
         for (int e = tid; e < IdStrip::bytes / 2; e += CHAIN_THREADS<W>) ((uint16_t*)(smem + CFG::id_off))[e] = IdStrip::one(e) ? 0x3F80 : 0;
     fence_async_smem();
@@ -1673,9 +1674,8 @@ ChainCarve carve(const Problem& p, const ChainPlan& plan) {
     return c;
 }
 
-template <int DK, int R, int DV, int MODE>
+template <int DK, int R, int DV, int MODE, bool W = false>
 int launch(const Problem& p, const ChainPlan& plan, const ChainSeg& sg, void* workspace) {
-    constexpr bool W = w_form(DK, DV, MODE != WHOLE);
     using CFG = ChainCfg<DK, W, R, DV>;
     static_assert(CFG::total + (MODE == SHARED ? 4096 : 1024) <= 227 * 1024 && CFG::NS >= 3 && (!W || (CFG::NS >= 4 && CFG::NT <= 3 && CFG::NV == CFG::NW)), "shared memory budget");
     const void* fn = (const void*)chain_kernel<DK, W, R, DV, MODE>;
@@ -1712,6 +1712,8 @@ template <int DK, int R>
 int launch_plan(const Problem& p, const ChainPlan& plan, const ChainSeg& sg, void* ws) {
     if (plan.share > 0) return p.d_v == 128 ? launch<DK, R, 128, SHARED>(p, plan, sg, ws) : launch<DK, R, 64, SHARED>(p, plan, sg, ws);
     if (plan.nseg > 1) return p.d_v == 128 ? launch<DK, R, 128, SEGMENTS>(p, plan, sg, ws) : launch<DK, R, 64, SEGMENTS>(p, plan, sg, ws);
+    if constexpr (DK == 64)
+        if (p.d_v == 64 && plan.seg_blk >= W_FORM_BLOCKS) return launch<DK, R, 64, WHOLE, true>(p, plan, sg, ws);
     return p.d_v == 128 ? launch<DK, R, 128, WHOLE>(p, plan, sg, ws) : launch<DK, R, 64, WHOLE>(p, plan, sg, ws);
 }
 template <int DK>
