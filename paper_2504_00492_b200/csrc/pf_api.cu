@@ -317,11 +317,10 @@ int forward_one(const pf_params* a, bool top) {
     p.stream = (cudaStream_t)a->stream;
 
     p.own_workspace = !a->workspace;
-    size_t need;
     void* ws = a->workspace;
     bool own = false;
     if (ws) {
-        need = workspace_need(p, impl);
+        size_t need = workspace_need(p, impl);
         if (a->workspace_bytes < need) {       // (sharing walks out is for speed only: without it the call may take less)
             p.no_share = true;
             need = workspace_need(p, impl);
@@ -329,9 +328,8 @@ int forward_one(const pf_params* a, bool top) {
         if (a->workspace_bytes < need || ((uintptr_t)ws & 255u)) return PF_ERR_WORKSPACE;
     } else {
         auto alloc = [&]() {
-            need = workspace_need(p, impl);
             const size_t own_need = use_recur(p, impl) ? recur_workspace_bytes(p)
-                                    : use_chain(p, impl) && !chain_needs_workspace(p) ? 0 : need;
+                                    : use_chain(p, impl) && !chain_needs_workspace(p) ? 0 : workspace_need(p, impl);
             own = own_need > 0;
             return own ? workspace_alloc(&ws, own_need, p.stream) : (int)PF_OK;
         };

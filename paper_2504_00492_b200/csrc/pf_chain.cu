@@ -1142,7 +1142,7 @@ __device__ __forceinline__ void mma_out_role(int count, int width, int* err, uin
         const uint32_t sg = smem_b + ks.i * SM::stage, t_o = o_cols<CP>(os.i);
         waits.wait(CFG::FULL + ks.i, ks.phase, 351);
         if (b >= OB) waits.wait(B_OFREE + os.i, os.phase ^ 1, 325);
-        waits.wait(W || DK == 64 ? B_SP : B_RD, b & 1, 352);
+        waits.wait(W ? B_SP : B_RD, b & 1, 352);
         tc_fence_after();
         if (waits.ok() && elect_one()) {
             products_ta<false, CP, DK / 16, SM::rows, true>(t_o, T_S16, lo_of(sg + SM::q_off), false);
@@ -1296,12 +1296,12 @@ chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __rest
     }
     if (warp == W_MMA) tmem_alloc(&tmem_base, 512);
     if (SM::CP > SM::C) {                                         // (r = 3: query rows that no copy writes are read)
-        for (int e = tid; e < min(CFG::NS, count) * (SM::stage / 16); e += CHAIN_THREADS<W>) ((uint4*)smem)[e] = make_uint4(0, 0, 0, 0);
+        for (int e = tid; e < CFG::NS * SM::stage / 16; e += CHAIN_THREADS<W>) ((uint4*)smem)[e] = make_uint4(0, 0, 0, 0);
     } else {                                                      // (the upper triangles of P and T, which nothing writes)
         for (int st = 0; st < CFG::NS && st < count; ++st)
             for (int e = tid; e < SM::p_bytes / 16; e += CHAIN_THREADS<W>) ((uint4*)(smem + st * SM::stage + SM::p_off))[e] = make_uint4(0, 0, 0, 0);
     }
-    for (int e = tid; e < min(CFG::NT, count) * (SM::t_bytes / 16); e += CHAIN_THREADS<W>) ((uint4*)(smem + CFG::t_off))[e] = make_uint4(0, 0, 0, 0);
+    for (int e = tid; e < CFG::NT * SM::t_bytes / 16; e += CHAIN_THREADS<W>) ((uint4*)(smem + CFG::t_off))[e] = make_uint4(0, 0, 0, 0);
     if (!W)
         for (int e = tid; e < IdStrip::bytes / 2; e += CHAIN_THREADS<W>) ((uint16_t*)(smem + CFG::id_off))[e] = IdStrip::one(e) ? 0x3F80 : 0;
     fence_async_smem();
