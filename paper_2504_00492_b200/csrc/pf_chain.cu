@@ -4,10 +4,8 @@
 //     T  = (I + Mstrict (.) (diag(beta) K K^T))^{-1} diag(beta)                      (does not depend on S)
 //     P  = (Q K^T) (.) Mincl                                                         (does not depend on S)
 //     U' = T (V - K S^T),       O = Q S^T + P U',       S <- S + U'^T K
-// evaluated in one of two forms (W_FORM_BLOCKS):
-//     V - K S^T first and T applied to it: three products of a block depend on S one after another, R = V - K S^T, U' = T R and the update;
-//     with W = T K formed ahead ("W form"), U' = T V - W S^T: two, at the price of one more product, its way through tensor memory and V in fp16.
-// (Against the fp64 recurrence, 70 sequences of 400, d = 64, r = 4, beta to 2: relative L2 error of O 6.81e-4 with W and 7.12e-4 without: V - K S^T is never rounded.)
+// with W = T K and Uh = T V never formed: T is applied to V - K S^T, in which what the state predicts of V is taken away before anything is rounded.  Only three
+// products of a block depend on S one after another: R = V - K S^T, U' = T R and the update.
 // All are tcgen05 products of 128 rows j (d_v = 64: half of them nobody's) whose A operand lies
 // in tensor memory and whose B operand is a tile of shared memory as TMA or the preparing warps left it.  S stays in tensor memory as the
 // fp32 accumulator of its update; between two products the chain warps convert an accumulator to the next one's fp16 operand.
@@ -18,10 +16,9 @@
 //                 rows, from the bf16 tiles as they land)
 //   solve (2 x 4) T of every other block: G from tensor memory, the inverse on mma.sync
 //   convert (4)   K, Q -> fp16 in place, P out of tensor memory into shared memory
-//   W (4)         W form: W^T = K^T T^T out of tensor memory into shared memory
-//   output (4)    O^T out of tensor memory into the rows of O; W form: V -> fp16 in place;  and one warp issues the copies
-// A stage of shared memory holds what the chain needs of one block: K, Q (fp16, the rows of Q behind those of K) and P (fp16); T, V and W have rings of their
-// own.  Without W, V is bf16 as it came and added to R's accumulator as V^T times an identity; with W, U'^T's accumulator starts as V^T T^T.
+//   output (4)    O^T out of tensor memory into the rows of O;  and one warp issues the copies
+// A stage of shared memory holds what the chain needs of one block: K, Q (fp16, the rows of Q behind those of K), P, T (fp16), V (bf16 as
+// it came, added to R's accumulator as V^T times an identity).
 //
 // What bounds it: the three trips of a block (issue 4 to 8 products at 30 cycles each, tensor memory to registers and back), 2.2 k cycles at
 // d = 128 with everything but the chain's own warps switched off, drawn out to 2.6 - 3 k by the others: all products go through one
@@ -30,7 +27,7 @@
 // named barriers) and the instruction cache (so what is off the chain's path is written small).  148 CTAs at r = 1 move 5.5 TB/s, 84 % of
 // what a copy reaches.  Measured (us, before: the same blocks on
 // warp-level products, a warp carrying 16 rows j in registers; a shared-memory read of every tile by every such warp): 256 sequences of
-// 1024, d = 128, r = 2: 227 -> 136 (calls on other inputs one after another; 228 -> 115 on the same); 128 of 4096, d = 64, r = 4: 340 -> 307 (336 -> 290; with W 264); 48 of 1999, 64 x 128,
+// 1024, d = 128, r = 2: 227 -> 136 (calls on other inputs one after another; 228 -> 115 on the same); 128 of 4096, d = 64, r = 4: 340 -> 307 (336 -> 290); 48 of 1999, 64 x 128,
 // r = 3: 144 -> 84 (144 -> 80; 2 segments); 4 of 16384, d = 128, r = 1: 135 -> 78 (segments); 32 of 2048, d = 128, r = 1: 68 -> 54 (the tcgen05 kernel in one launch before).
 // Measured and not taken: the update's and V - K S^T's products in halves, so that one half is converted while the other is being multiplied (the
 // probe's 1.6 k cycles have it; here 412 us against 389 at 32 sequences of 8192: more instructions); the output's products issued by the chain's
@@ -39,12 +36,14 @@
 // sequences, 290 -> 322 at d = 64, r = 4).  The chain's warps at named barriers too, one warp watching the products' ends for them (293 -> 328).
 // V in one buffer apart from the stages, which makes room for one more (142.6 -> 152.4, 128 sequences of 2048, d = 64, r = 4).  The
 // state before the last block's update in V - K S^T, with U'^T K K^T of the two blocks in its place (172 us at 256 sequences: 20 products more).
-// What counts besides the chain's latency: instructions that are fetched (what all warps execute in a block is about 40 KB; 49 KB of it, in an earlier W form, missed
+// What counts besides the chain's latency: instructions that are fetched (what all warps execute in a block is about 40 KB; 49 KB of it, in a form with one more role, missed
 // the instruction cache in 23 % of the requests instead of 5 and took 20 % more time), so that a wait is a few instructions and its failure is reported once a
 // role; and no warps that poll mbarriers but those that watch for others.
 // Measured and not taken: the chain's warps meeting at a named barrier and the first of them issuing (128 us against 116 at 256 sequences, 314 against 264 at
 // 128 of 4096, d = 64); a predicate on every product instead of a branch around all of a step (twice the instructions); an L2 prefetch of the next tiles (128 of 4096, d = 64:
-// 359 against 338 without, at the time; level elsewhere); W's products issued by the Gram products' warp (they wait behind a later block's landing) or by the copies' (350 cycles a copy).
+// 359 against 338 without, at the time; level elsewhere); W = T K formed ahead, U' = T V - W S^T, two dependent products instead of three (128 of 4096, d = 64, r = 4: 298, 291 without; slower at d = 128): T is then
+// applied to all of V and not to what the state leaves of it, and W is rounded, which costs up to 1.4 times the error where the state predicts V
+// (d = 64, r = 4, beta to 2, V = S* K, relative L2 error of O: 3.7e-4, 2.7e-4 without).
 //
 // Range: V - K S^T and U' are packed to fp16 like every other operand, and K S^T reaches sqrt(d_k) times the largest entry of S, so
 // that a state well inside fp16's 65504 can overflow them.  What overflows leaves its row of S infinite or NaN to the end of the walk
@@ -70,13 +69,6 @@ namespace {
 
 constexpr int NB = 64;               // rows per block
 constexpr int MOST_PARTS = 30;       // parts of walks in a CTA's share
-
-// Where the W form pays (head of the file), us, with W and without, d_k = d_v = 64, a walk to each CTA: 128 sequences of 4096, r = 4: 264 and 290; 256 of 1000, r = 2: 81 and
-// 85; 64 of 4000, r = 1: 85 and 89.  Not where the walks are short and the chain has nothing ahead at their start: 8 of 400, r = 4 (25 blocks): 16.4 and 15.3; 100 of 200,
-// r = 3 (10): 16.5 and 15.9; 140 of 900, r = 1 (15): 26.3 and 26.0; 4 of 8192 in segments, r = 2: 43 and 40.  Not at d_v = 128 (140 of 1500, 64 x 128, r = 1: 44 and 43; 48 of
-// 1999, r = 3: level) and not at d_k = 128, where the bound is what a block moves through shared memory, 2950 cycles' worth at r = 2 with W and 2350 without (256 of 1024,
-// r = 2: 118 and 114).
-constexpr int W_FORM_BLOCKS = 32;
 
 struct ChainMaps {
     CUtensorMap q, k, v;
@@ -123,7 +115,7 @@ struct ChainSmem {
     static constexpr int C = NB / R;                              // tokens per block
     static constexpr int CP = (C + 15) / 16 * 16;                 // ... in tiles of 16
     static constexpr int k_bytes = NB * DK * 2, q_bytes = CP * DK * 2;
-    static constexpr int t_bytes = NB * 128, w_bytes = DK * 128, p_bytes = CP * 128, v_bytes = NB * JS * 2;
+    static constexpr int t_bytes = NB * 128, p_bytes = CP * 128, v_bytes = NB * JS * 2;
     // slabs of 64 columns, in each the rows of K and then those of Q: one operand of NB + CP rows
     static constexpr int rows = NB + CP, k_off = 0, q_off = NB * 128, p_off = k_bytes + q_bytes;
     static constexpr int stage = p_off + p_bytes;
@@ -140,27 +132,22 @@ enum {
     B_OD = 5,       // [2] output products: O^T complete
     B_OFREE = 7,    // [2] output: O^T read
     B_GD = 9,       // Gram products: G and P^T complete
-    B_WD = 10,      // W's products: W complete
-    B_RD = 11,      // products: V^T - S K^T complete
-    B_RP = 12,      // chain: its fp16 copy published
-    B_RINGS = 13
+    B_RD = 10,      // products: V^T - S K^T complete
+    B_RP = 11,      // chain: its fp16 copy published
+    B_RINGS = 12
 };
 constexpr int TEAMS = 2;             // solve teams
-// warps: 0-7 chain, 8-11 output (and V), 12-15 conversion, then the solve teams, then products of the chain, products of the output, Gram products,
-// copies, then in the W form W's
+// warps: 0-7 chain, 8-11 output, 12-15 conversion, then the solve teams, then products of the chain, products of the output, Gram products,
+// copies
 constexpr int W_OUT = 8, W_CONV = 12, W_SOLVE = 16, W_MMA = W_SOLVE + 4 * TEAMS, W_MMA_OUT = W_MMA + 1, W_GRAM = W_MMA + 2, W_LOAD = W_MMA + 3,
-              W_W = W_MMA + 4;
-template <bool W> constexpr int CHAIN_THREADS = 32 * (W ? W_W + 4 : W_W);
+              CHAIN_THREADS = 32 * (W_MMA + 4);
 
 // Registers per thread: the launch's, and what each warpgroup makes of them (the sum is the launch's)
-template <bool W> constexpr int REGS = W ? 64 : 72;
-constexpr int REGS_CHAIN = 80, REGS_OUT = 48, REGS_CONV = 48, REGS_W = 48, REGS_ISSUE = 48;
-template <bool W> constexpr int REGS_SOLVE = W ? 80 : 88;
-static_assert(2 * REGS_CHAIN + REGS_OUT + REGS_CONV + REGS_W + REGS_ISSUE + TEAMS * REGS_SOLVE<true> <= REGS<true> * CHAIN_THREADS<true> / 128 &&
-              2 * REGS_CHAIN + REGS_OUT + REGS_CONV + REGS_ISSUE + TEAMS * REGS_SOLVE<false> <= REGS<false> * CHAIN_THREADS<false> / 128, "registers of the launch");
-template <bool W, int N>
+constexpr int REGS = 72, REGS_CHAIN = 80, REGS_OUT = 48, REGS_CONV = 48, REGS_ISSUE = 48, REGS_SOLVE = 88;
+static_assert(2 * REGS_CHAIN + REGS_OUT + REGS_CONV + REGS_ISSUE + TEAMS * REGS_SOLVE <= REGS * CHAIN_THREADS / 128, "registers of the launch");
+template <int N>
 __device__ __forceinline__ void set_registers() {
-    if (N > REGS<W>) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
+    if (N > REGS) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
     else asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N));
 }
 
@@ -178,40 +165,19 @@ struct IdStrip {
     __device__ static uint64_t desc(uint32_t base, int c) { return make_desc_ns(base + (6 - 2 * c) * 128, 7 * 128, 128); }
 };
 
-// How many blocks each part of shared memory holds.  A block's K, Q and P are there from its copy to its end.  In the W form V and T until V^T T^T and W until
-// S W^T are enough; otherwise all are there to the block's end.
-struct ChainRings {
-    int kq, v, t, w;
-};
 constexpr int SMEM_MOST = 226 * 1024;
-template <int DK, bool W, int R, int DV>
-constexpr ChainRings chain_rings() {
-    using SM = ChainSmem<DK, R, DV>;
-    int left = SMEM_MOST - TEAMS * (XS_BYTES + 512) - IdStrip::bytes;
-    if (!W) {
-        const int n = left / (SM::stage + SM::v_bytes + SM::t_bytes), m = n < 6 ? n : 6;
-        return {m, m, m, 0};
-    }
-    ChainRings g{0, 2, 2, 2};
-    left -= g.v * SM::v_bytes + g.t * SM::t_bytes + g.w * SM::w_bytes;
-    g.kq = left / SM::stage;
-    if (g.kq > 6) g.kq = 6;
-    if (left - g.kq * SM::stage >= SM::t_bytes) ++g.t;
-    return g;
-}
-template <int DK, bool W, int R, int DV>
+template <int DK, int R, int DV>
 struct ChainCfg {
     using SM = ChainSmem<DK, R, DV>;
-    static constexpr ChainRings ring = chain_rings<DK, W, R, DV>();
-    static constexpr int NS = ring.kq, NV = ring.v, NT = ring.t, NW = ring.w;
-    static constexpr int v_off = NS * SM::stage, t_off = v_off + NV * SM::v_bytes, w_off = t_off + NT * SM::t_bytes;
-    static constexpr int xs_off = w_off + NW * SM::w_bytes;       // per team: X (unscaled) while it is being formed
+    // as many stages as fit, up to six; their V and T behind all of the rest
+    static constexpr int fit = (SMEM_MOST - TEAMS * (XS_BYTES + 512) - IdStrip::bytes) / (SM::stage + SM::v_bytes + SM::t_bytes), NS = fit < 6 ? fit : 6;
+    static constexpr int v_off = NS * SM::stage, t_off = v_off + NS * SM::v_bytes;
+    static constexpr int xs_off = t_off + NS * SM::t_bytes;       // per team: X (unscaled) while it is being formed
     static constexpr int beta_off = xs_off + TEAMS * XS_BYTES;    // per team: 64 step sizes, of two blocks in turn
     static constexpr int id_off = beta_off + TEAMS * 512;         // identity (IdStrip)
     static constexpr int total = id_off + IdStrip::bytes;
-    // barriers of the rings, after the others
-    static constexpr int LAND = B_RINGS, FULL = LAND + NS, EMPTY = FULL + NS, VLAND = EMPTY + NS, VFREE = VLAND + NV,
-                         TDONE = VFREE + NV, WDONE = TDONE + NT, WFREE = WDONE + NW, count = WFREE + NW;
+    // barriers of the stages, after the others: a block's tiles landed, a block prepared, a block's stage free
+    static constexpr int LAND = B_RINGS, FULL = LAND + NS, EMPTY = FULL + NS, count = EMPTY + NS;
 };
 // a ring's slot and the parity of its present round
 template <int N>
@@ -229,15 +195,11 @@ struct RingPos {
 // would go through a register to each product.
 constexpr uint32_t T_S = 0;          // S, fp32 [j][i]
 constexpr uint32_t T_S16 = 128;      // -S, fp16 pairs
-constexpr uint32_t T_U = 192;        // U'^T, fp32 [j][m] (without W: first V^T - S K^T)
-// In the W form with 64 tokens a block, U'^T's fp16 pairs take the place of the first half of what each chain warp has read of it; otherwise
-// they have columns of their own, so that what comes next into the accumulator need not wait for their readers.
-template <bool W, int CP> constexpr bool U_INPLACE = W && CP > 32;
-constexpr uint32_t T_R16 = 256;      // V^T - S K^T in fp16 pairs
-template <bool W, int CP> constexpr uint32_t T_U16 = U_INPLACE<W, CP> ? T_U : W ? 256 : 288;
-template <bool W, int CP> constexpr uint32_t T_W = U_INPLACE<W, CP> ? 256 : 288;       // W^T, fp32 [i][m]
-template <bool W, int CP> constexpr uint32_t T_G = W ? T_W<W, CP> + 64 : 320;   // G, fp32 [m][m'] (16 rows in each quarter of the lanes, as products of 64 rows are laid out)
-template <bool W, int CP> constexpr uint32_t T_P = T_G<W, CP> + 64;   // P^T before its mask, fp32 [m][t], likewise: behind T_G, one product
+constexpr uint32_t T_R = 192;        // V^T - S K^T, then U'^T over it, fp32 [j][m]
+constexpr uint32_t T_R16 = 256;      // V^T - S K^T and
+constexpr uint32_t T_U16 = 288;      // U'^T in fp16 pairs
+constexpr uint32_t T_G = 320;        // G, fp32 [m][m'] (16 rows in each quarter of the lanes, as products of 64 rows are laid out)
+constexpr uint32_t T_P = 384;        // P^T before its mask, fp32 [m][t], likewise: behind T_G, one product
 template <int CP> constexpr int O_BUFS = CP > 32 ? 1 : 2;         // O^T, fp32 [j][t]: of two blocks in turn where there is room
 template <int CP> __device__ __forceinline__ uint32_t o_cols(int b) { return CP > 32 ? 448u : 448u + 32u * (b & 1); }
 
@@ -441,14 +403,11 @@ __device__ __forceinline__ uint32_t lane_off(int row, int half) { return (uint32
 // whoever watches an mbarrier takes part in them to the end, also when it has given up (`ok`).
 enum {
     N_TEAM = 1,     // [2] solve teams
-    N_WD = 3,       // W's warps: W^T complete, and its place in shared memory free
-    N_WFREE = 4,    // W's warps: W^T read
     N_GD = 5,       // [team] Gram products -> solve: G complete
     N_GFREE = 7,    // solve and conversion -> Gram products: G and P^T read
     N_PD = 8,       // Gram products -> conversion: P^T complete (and nothing reads the block's K and Q as bf16 any more)
     N_OD = 10,      // [2] output products -> output: O^T complete
-    N_TFREE = 12,   // [3, as many as T has slots] output products -> solve: nothing reads the T in this slot any more
-    N_END = 12      // [4] the two chain warps of a quarter (when the walk is over, and with it the use of the three before)
+    N_END = 12      // [4] the two chain warps of a quarter, when a walk is over
 };
 __device__ __forceinline__ void named_arrive(int id, int nthreads) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(nthreads) : "memory"); }
 // (after a wait for a product's mbarrier, by a whole warp)
@@ -465,19 +424,12 @@ __device__ __forceinline__ void pass_on(int id, int nthreads) {
 constexpr uint32_t DESC_HI = (1024u >> 4) | (1u << 14) | (2u << 29);          // SBO 1024 bytes, version, 128-byte swizzle
 __device__ __forceinline__ uint64_t desc_lo(uint32_t lo) { return ((uint64_t)DESC_HI << 32) | lo; }
 __device__ __forceinline__ uint32_t lo_of(uint32_t saddr, uint32_t slab_bytes = 16) { return (saddr >> 4) | (slab_bytes >> 4 << 16); }
-// D [128 x N] (+)= A (tensor memory; NEG: -A) B^T: B K-major (MN false) or MN-major, KSTEPS K-steps, slabs of B_ROWS rows; GAP: columns of A between its
-// second and third K-step
-template <bool MN, int N, int KSTEPS, int B_ROWS, bool NEG = false, int GAP = 0>
+// D [128 x N] (+)= A (tensor memory; NEG: -A) B^T: B K-major (MN false) or MN-major, KSTEPS K-steps, slabs of B_ROWS rows
+template <bool MN, int N, int KSTEPS, int B_ROWS, bool NEG = false>
 __device__ __forceinline__ void products_ta(uint32_t d, uint32_t a, uint32_t b_lo, bool acc) {
 #pragma unroll
     for (int kk = 0; kk < KSTEPS; ++kk)
-        mma_f16_ta(d, a + 8 * kk + (kk >= 2 ? GAP : 0), desc_lo(b_lo + (kstep_off<MN ? L_SWMN : L_SWK, B_ROWS>(kk) >> 4)), make_idesc(N, false, MN, NEG), acc || kk > 0);
-}
-// D [128 x NB] = A^T T^T: A [NB rows][128 columns] and T in shared memory, fp16
-__device__ __forceinline__ void products_tt(uint32_t d, uint32_t a_lo, uint32_t t_lo) {
-#pragma unroll
-    for (int kk = 0; kk < NB / 16; ++kk)
-        mma_f16(d, desc_lo(a_lo + (kstep_off<L_SWMN, NB>(kk) >> 4)), desc_lo(t_lo + (kstep_off<L_SWK, NB>(kk) >> 4)), make_idesc(NB, true, false, false), kk > 0);
+        mma_f16_ta(d, a + 8 * kk, desc_lo(b_lo + (kstep_off<MN ? L_SWMN : L_SWK, B_ROWS>(kk) >> 4)), make_idesc(N, false, MN, NEG), acc || kk > 0);
 }
 // D [64 x N] = A B^T, B [N rows] K-major bf16 in shared memory, in slabs of ROWS rows, A its first 64 rows
 template <int N, int K, int ROWS>
@@ -493,7 +445,7 @@ __device__ __forceinline__ void commit_at(uint32_t bar) {
 }
 
 // a warp's part of an operand in shared memory is written
-__device__ __forceinline__ void publish_smem(uint32_t b, int lane) {
+__device__ __forceinline__ void publish_smem(uint32_t b) {
     fence_async_smem();
     mbar_arrive_at(b);
 }
@@ -549,10 +501,10 @@ __device__ __forceinline__ void neumann_product(float (&r)[2][4], const uint32_t
 // ---------------------------------------------------------------------------------------------------------------------
 // solve team: T of blocks b = team, team + TEAMS, ...
 // ---------------------------------------------------------------------------------------------------------------------
-template <int DK, bool W, int R, int JS, int MODE>
+template <int DK, int R, int JS, int MODE>
 __device__ __forceinline__ void solve_role(const ChainGeo& g, ChainWork<MODE> work, const __nv_bfloat16* __restrict__ beta, uint8_t* smem,
                                            uint32_t bar, int team, int tid) {
-    using CFG = ChainCfg<DK, W, R, JS>;
+    using CFG = ChainCfg<DK, R, JS>;
     using SM = ChainSmem<DK, R, JS>;
     constexpr int C = SM::C;
     const int w = tid >> 5, lane = tid & 31, gq = lane >> 2, t4 = lane & 3;
@@ -589,15 +541,15 @@ __device__ __forceinline__ void solve_role(const ChainGeo& g, ChainWork<MODE> wo
     uint16_t breg = b < end ? read_beta(b) : 0;
 #pragma unroll 1
     for (; b < end; b += TEAMS) {
-        const int ts = b % CFG::NT;
-        const uint32_t t_b = smem_u32(smem) + CFG::t_off + ts * SM::t_bytes;
+        const int st = b % CFG::NS;
+        const uint32_t t_b = smem_u32(smem) + CFG::t_off + st * SM::t_bytes;
         // (two in turn: another warp may still be scaling T of the block before)
         float* sBeta = (float*)(smem + CFG::beta_off + team * 512 + (b / TEAMS & 1) * 256);
         if (tid < NB) sBeta[tid] = __uint_as_float((uint32_t)breg << 16);
         if (b + TEAMS < end) breg = read_beta(b + TEAMS);
         named_bar(N_GD + team, 160);                              // (and the step sizes)
         tc_fence_after();
-        const uint32_t t_g = T_G<W, SM::CP> + ((uint32_t)(32 * w) << 16);
+        const uint32_t t_g = T_G + ((uint32_t)(32 * w) << 16);
         uint32_t x[8];                                            // 16 columns of G, rows 16 w .. 16 w + 15, as mma.sync's accumulators
         const int m0 = 16 * w + gq, m1 = m0 + 8;
         if (g.exact) {
@@ -647,7 +599,6 @@ __device__ __forceinline__ void solve_role(const ChainGeo& g, ChainWork<MODE> wo
                 dd[h][0] *= bb.x; dd[h][1] *= bb.y; dd[h][2] *= bb.x; dd[h][3] *= bb.y;
             }
             frag_pack(df, dd);
-            if (W && b >= CFG::NT) named_bar(N_TFREE + ts, 160);
             stmatrix_x4(t_b + w * 2048 + (offA ^ (uint32_t)(w << 5)), df);
         }
         named_bar(N_TEAM + team, 128);
@@ -677,16 +628,16 @@ __device__ __forceinline__ void solve_role(const ChainGeo& g, ChainWork<MODE> wo
             for (int e = 0; e < 4; ++e) f[e] = pack_h2(-z[e / 2][e % 2 * 2] * (e % 2 ? b1 : b0), -z[e / 2][e % 2 * 2 + 1] * (e % 2 ? b1 : b0));
             stmatrix_x4_trans(t_b + i * 2048 + (offN ^ (uint32_t)(w << 5)), f);
         }
-        publish_smem(bar + 8 * ((W ? CFG::TDONE : CFG::FULL) + ts), lane);
+        publish_smem(bar + 8 * (CFG::FULL + st));
     }
     }
 }
 
 // Conversion: K and Q of every block to fp16 in place, once the Gram products have read them as they came, and P.  Four warps.
-template <int DK, bool W, int R, int JS>
+template <int DK, int R, int JS>
 __device__ __forceinline__ void convert_role(int count, uint8_t* smem, uint32_t bar, int tid) {
     using SM = ChainSmem<DK, R, JS>;
-    using CFG = ChainCfg<DK, W, R, JS>;
+    using CFG = ChainCfg<DK, R, JS>;
     constexpr int CP = SM::CP;
     const int w = tid >> 5, lane = tid & 31, gq = lane >> 2, t4 = lane & 3;
     const uint32_t p_at = smem_u32(smem) + SM::p_off + (lane_off((lane & 7) + ((lane >> 4) << 3), (lane >> 3) & 1) ^ (uint32_t)(w << 5));
@@ -701,7 +652,7 @@ __device__ __forceinline__ void convert_role(int count, uint8_t* smem, uint32_t 
 #pragma unroll 1
         for (int t0 = 0; t0 < CP; t0 += PC) {
             uint32_t x[PC / 2];
-            tmem_ld_frag<PC>(T_P<W, CP> + t0 + ((uint32_t)(32 * w) << 16), x);
+            tmem_ld_frag<PC>(T_P + t0 + ((uint32_t)(32 * w) << 16), x);
             tmem_ld_wait();
             if (t0 + PC == CP) {
                 tc_fence_before();
@@ -723,71 +674,16 @@ __device__ __forceinline__ void convert_role(int count, uint8_t* smem, uint32_t 
             }
         }
         convert_pieces<(SM::k_bytes + SM::q_bytes) / 2048, 128>(sg + SM::k_off, tid);
-        publish_smem(bar + 8 * (CFG::FULL + st), lane);
+        publish_smem(bar + 8 * (CFG::FULL + st));
         if (++st == CFG::NS) st = 0;
     }
 }
 
-// W^T = K^T T^T of every block (rows i, columns m): its products, and out of tensor memory as the fp16 operand W.  Four warps, the first of which issues; at
-// d_k = 64 the accumulator has its rows twice, and a warp takes half of the columns.
-template <int DK, bool W, int R, int JS>
-__device__ __forceinline__ void w_role(int count, int* err, uint8_t* smem, uint32_t bar, int tid) {
-    using SM = ChainSmem<DK, R, JS>;
-    using CFG = ChainCfg<DK, W, R, JS>;
-    const int w = tid >> 5, lane = tid & 31, i = tid & (DK - 1);
-    const int m0 = DK == 128 ? 0 : 32 * (w >> 1);
-    const uint32_t t_w = T_W<W, SM::CP> + ((uint32_t)(32 * w) << 16), smem_b = smem_u32(smem);
-    RingPos<CFG::NS> ks;
-    RingPos<CFG::NT> ts;
-    RingPos<CFG::NW> ws;
-    Waits waits(bar);
-#pragma unroll 1
-    for (int b = 0; b < count; ++b) {
-        uint8_t* row = smem + CFG::w_off + ws.i * SM::w_bytes + i * 128;
-        if (b > 0) named_bar(N_WFREE, 128);                       // (the accumulator has been read)
-        if (w == 0) {
-            waits.wait(CFG::FULL + ks.i, ks.phase, 324);
-            waits.wait(CFG::TDONE + ts.i, ts.phase, 329);
-            tc_fence_after();
-            if (waits.ok() && elect_one()) {
-                products_tt(T_W<W, SM::CP>, lo_of(smem_b + ks.i * SM::stage + SM::k_off, DK == 128 ? SM::rows * 128 : 0), lo_of(smem_b + CFG::t_off + ts.i * SM::t_bytes));
-                commit_at(bar + 8 * B_WD);
-            }
-            __syncwarp();
-            if (b >= CFG::NW) waits.wait(CFG::WFREE + ws.i, ws.phase ^ 1, 318);
-            waits.wait(B_WD, b & 1, 330);
-            tc_fence_after();
-            tc_fence_before();
-        }
-        named_bar(N_WD, 128);
-        tc_fence_after();
-#pragma unroll 1
-        for (int c = m0; c < m0 + DK / 2; c += 32) {
-            uint32_t x[32];
-            tmem_ld32(t_w + c, x);
-            tmem_ld_wait();
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                uint32_t y[4];
-#pragma unroll
-                for (int n = 0; n < 4; ++n) y[n] = pack_h2(__uint_as_float(x[8 * e + 2 * n]), __uint_as_float(x[8 * e + 2 * n + 1]));
-                *(uint4*)(row + ((((c >> 3) + e) ^ (i & 7)) << 4)) = make_uint4(y[0], y[1], y[2], y[3]);
-            }
-        }
-        tc_fence_before();
-        publish_smem(bar + 8 * (CFG::WDONE + ws.i), lane);
-        ks.next();
-        ts.next();
-        ws.next();
-    }
-    if (!waits.ok()) atomicCAS(err, 0, waits.code);
-}
-
 // Gram products (one warp): G = K K^T and K Q^T from the bf16 tiles as they landed, in products of 64 rows and NB + CP columns.
-template <int DK, bool W, int R, int JS>
+template <int DK, int R, int JS>
 __device__ __forceinline__ void gram_role(int count, int* err, uint8_t* smem, uint32_t bar) {
     using SM = ChainSmem<DK, R, JS>;
-    using CFG = ChainCfg<DK, W, R, JS>;
+    using CFG = ChainCfg<DK, R, JS>;
     const uint32_t smem_b = smem_u32(smem);
     RingPos<CFG::NS> ks;
     Waits waits(bar);
@@ -797,7 +693,7 @@ __device__ __forceinline__ void gram_role(int count, int* err, uint8_t* smem, ui
         if (b > 0) named_bar(N_GFREE, 288);
         tc_fence_after();
         if (waits.ok() && elect_one()) {
-            products_ss<SM::rows, DK, SM::rows>(T_G<W, SM::CP>, smem_b + ks.i * SM::stage);
+            products_ss<SM::rows, DK, SM::rows>(T_G, smem_b + ks.i * SM::stage);
             commit_at(bar + 8 * B_GD);
         }
         __syncwarp();
@@ -809,63 +705,39 @@ __device__ __forceinline__ void gram_role(int count, int* err, uint8_t* smem, ui
     if (!waits.ok()) atomicCAS(err, 0, waits.code);
 }
 
-// The copies (one warp).  K and Q of a block are asked for when the block before in their stage is done, and V with them, or in the W form when V^T T^T of the
-// block before it in its slot is; rows past the sequence arrive as zeros.  (Issuing a copy takes the warp some 200 cycles, five a block at d = 128.)
-template <int DK, bool W, int R, int JS, int MODE>
+// The copies (one warp).  K and Q of a block are asked for when the block before in their stage is done, V with them; rows past the sequence arrive as zeros.  (Issuing a copy takes the warp some 200 cycles, five a block at d = 128.)
+template <int DK, int R, int JS, int MODE>
 __device__ __forceinline__ void load_role(const ChainMaps& maps, ChainWork<MODE> work, int* err, uint8_t* smem, uint32_t bar) {
     using SM = ChainSmem<DK, R, JS>;
-    using CFG = ChainCfg<DK, W, R, JS>;
-    constexpr int NS = CFG::NS, NV = CFG::NV;
+    using CFG = ChainCfg<DK, R, JS>;
+    constexpr int NS = CFG::NS;
     const uint32_t smem_b = smem_u32(smem);
     Waits waits(bar);
     RingPos<NS> ks;
-    RingPos<NV> vs;
     auto copy_kq = [&](const ChainPart& part, int b) {
         const uint32_t land = bar + 8 * (CFG::LAND + ks.i), at = smem_b + ks.i * SM::stage;
         const int tok = (part.b0 + b) * SM::C, seq = (int)part.seq;
         if (waits.ok() && elect_one()) {
-            mbar_expect_tx_at(land, SM::tx_bytes + (W || part.response ? 0 : SM::v_bytes));
+            mbar_expect_tx_at(land, SM::tx_bytes + (part.response ? 0 : SM::v_bytes));
 #pragma unroll
             for (int h = 0; h < DK / 64; ++h) {
                 tma_load_4d(at + SM::k_off + h * (SM::rows * 128), &maps.k, 0, tok * R, h, seq, land);
                 tma_load_4d(at + SM::q_off + h * (SM::rows * 128), &maps.q, 0, tok, h, seq, land);
             }
-            if (!W && !part.response) tma_load_4d(smem_b + CFG::v_off + ks.i * SM::v_bytes, &maps.v, 0, tok * R, 0, seq, land);
+            if (!part.response) tma_load_4d(smem_b + CFG::v_off + ks.i * SM::v_bytes, &maps.v, 0, tok * R, 0, seq, land);
         }
         __syncwarp();
         ks.next();
     };
-    if constexpr (W) {
-        const ChainPart& part = work[0];
-        // (c: the block that the chain is in, or before the first)
+    int c = -NS;
 #pragma unroll 1
-        for (int c = -NS; c + NV < part.nblk; ++c) {
-            if (c + NV >= 0) {
-                if (c >= 0) waits.wait(CFG::VFREE + vs.i, vs.phase ^ 1, 342);
-                const uint32_t land = bar + 8 * (CFG::VLAND + vs.i);
-                if (waits.ok() && elect_one()) {
-                    mbar_expect_tx_at(land, SM::v_bytes);
-                    tma_load_4d(smem_b + CFG::v_off + vs.i * SM::v_bytes, &maps.v, 0, (part.b0 + c + NV) * SM::C * R, 0, (int)part.seq, land);
-                }
-                __syncwarp();
-                vs.next();
-            }
-            if (c + NS < part.nblk) {
-                if (c >= 0) waits.wait(CFG::EMPTY + ks.i, ks.phase ^ 1, 341);
-                copy_kq(part, c + NS);
-            }
-        }
-    } else {
-        int c = -NS;
+    for (int i = 0; i < work.size(); ++i) {
+        const ChainPart& part = work[i];
+        const int nblk = part.nblk;
 #pragma unroll 1
-        for (int i = 0; i < work.size(); ++i) {
-            const ChainPart& part = work[i];
-            const int nblk = part.nblk;
-#pragma unroll 1
-            for (int b = 0; b < nblk; ++b, ++c) {
-                if (c >= 0) waits.wait(CFG::EMPTY + ks.i, ks.phase ^ 1, 341);
-                copy_kq(part, b);
-            }
+        for (int b = 0; b < nblk; ++b, ++c) {
+            if (c >= 0) waits.wait(CFG::EMPTY + ks.i, ks.phase ^ 1, 341);
+            copy_kq(part, b);
         }
     }
     if (!waits.ok()) atomicCAS(err, 0, waits.code);
@@ -962,13 +834,13 @@ __device__ __forceinline__ void end_state(const ChainGeo& g, const ChainPart& pa
 }
 
 // warp `warp` of eight: rows j = 32 (warp & 3) + lane, half warp >> 2 of the columns of everything.  Returns the code of the wait that ran out, or 0.
-template <int DK, bool W, int CP, int MODE>
+template <int DK, int MODE>
 __device__ __forceinline__ int chain_role(const ChainGeo& g, ChainWork<MODE> work, uint32_t* lost, uint32_t bar, int warp, int lane) {
     constexpr int HC = DK / 2;                                    // columns i of this warp
     const int h = warp >> 2, j = 32 * (warp & 3) + lane;
     const uint32_t lanes = (uint32_t)(32 * (warp & 3)) << 16;
     const uint32_t t_s = T_S + h * HC + lanes, t_s16 = T_S16 + h * HC / 2 + lanes;
-    const uint32_t t_u = T_U + 32 * h + lanes, t_u16 = T_U16<W, CP> + (U_INPLACE<W, CP> ? 32 : 16) * h + lanes;
+    const uint32_t t_r = T_R + 32 * h + lanes, t_r16 = T_R16 + 16 * h + lanes, t_u16 = T_U16 + 16 * h + lanes;
     auto publish = [&](int b) {
         tmem_st_wait();
         tc_fence_before();
@@ -1005,15 +877,13 @@ __device__ __forceinline__ int chain_role(const ChainGeo& g, ChainWork<MODE> wor
 #pragma unroll 1
         for (int b = 0;; parity ^= 1) {
             publish(B_SP);
-            if constexpr (!W) {
-                if (!mbar_wait_tries<false>(bar + 8 * B_RD, parity)) return 312;
-                tc_fence_after();
-                to_operand<32, false>(t_u, T_R16 + 16 * h + lanes);
-                publish(B_RP);
-            }
+            if (!mbar_wait_tries<false>(bar + 8 * B_RD, parity)) return 312;
+            tc_fence_after();
+            to_operand<32, false>(t_r, t_r16);
+            publish(B_RP);
             if (!mbar_wait_tries<false>(bar + 8 * B_UD, parity)) return 313;
             tc_fence_after();
-            to_operand<32, false>(t_u, t_u16);
+            to_operand<32, false>(t_r, t_u16);
             publish(B_UP);
             if (!mbar_wait_tries<false>(bar + 8 * B_SD, parity)) return 314;
             tc_fence_after();
@@ -1027,17 +897,13 @@ __device__ __forceinline__ int chain_role(const ChainGeo& g, ChainWork<MODE> wor
 }
 
 // The products of the chain (one warp).  Returns the code of the wait that ran out, or 0.
-template <int DK, bool W, int R, int DV, int MODE>
+template <int DK, int R, int DV, int MODE>
 __device__ __forceinline__ int mma_role(ChainWork<MODE> work, uint8_t* smem, uint32_t bar) {
-    using CFG = ChainCfg<DK, W, R, DV>;
+    using CFG = ChainCfg<DK, R, DV>;
     using SM = ChainSmem<DK, R, DV>;
     constexpr int V_SLAB = NB * 128, K_SLAB = SM::rows * 128, CP = SM::CP, OB = O_BUFS<CP>;
-    constexpr bool INPLACE = U_INPLACE<W, CP>;
     const uint32_t smem_b = smem_u32(smem);
     RingPos<CFG::NS> ks;
-    RingPos<CFG::NV> vs;
-    RingPos<CFG::NT> ts;
-    RingPos<CFG::NW> ws;
     auto wait = [&](int which, int parity) { return mbar_wait_tries<false>(bar + 8 * which, (uint32_t)parity); };
     int b = 0;                                                    // (of the CTA's blocks)
 #pragma unroll 1
@@ -1046,95 +912,65 @@ __device__ __forceinline__ int mma_role(ChainWork<MODE> work, uint8_t* smem, uin
     const bool response = work[i].response;
 #pragma unroll 1
     for (; b < end; ++b) {
-        const uint32_t k_at = smem_b + ks.i * SM::stage + SM::k_off, v_lo = lo_of(smem_b + CFG::v_off + vs.i * SM::v_bytes, DV == 128 ? V_SLAB : 0),
-                       t_lo = lo_of(smem_b + CFG::t_off + ts.i * SM::t_bytes);
+        const uint32_t k_at = smem_b + ks.i * SM::stage + SM::k_off, v_lo = lo_of(smem_b + CFG::v_off + ks.i * SM::v_bytes, DV == 128 ? V_SLAB : 0),
+                       t_lo = lo_of(smem_b + CFG::t_off + ks.i * SM::t_bytes);
         // (at d_v = 64 the 64 columns of V's tile are read twice: rows j past d_v are nobody's)
-        if constexpr (W) {
-            // ---- U'^T = V^T T^T (W is there, and so T; the accumulator's last reader, the chain warps' conversion of U' of the block before, is done; its
-            //      fp16 pairs' readers are)
-            if (INPLACE && b > 0 && (!wait(B_SD, (b - 1) & 1) || !wait(B_OD + (b - 1) % OB, ((b - 1) / OB) & 1))) return 315;
-            if (!wait(CFG::WDONE + ws.i, ws.phase)) return 326;
-            if (!response) {
-                tc_fence_after();
-                if (elect_one()) {
-                    products_tt(T_U, v_lo, t_lo);
-                    commit_at(bar + 8 * (CFG::VFREE + vs.i));
-                }
-                __syncwarp();
-            }
-            // ---- ... - S W^T
-            // (U' completes only after the last reader of the block before's, P U', so that the chain warps need not wait for that)
-            if (!INPLACE && b > 0 && !wait(B_OD + (b - 1) % OB, ((b - 1) / OB) & 1)) return 319;
-            if (!wait(B_SP, b & 1)) return 323;
+        // ---- V^T into the accumulator, as V^T times an identity, both bf16 (V as it came; the accumulator's last reader is done)
+        if (!response) {
+            if (!wait(CFG::LAND + ks.i, ks.phase)) return 327;
             tc_fence_after();
             if (elect_one()) {
-                products_ta<true, NB, DK / 16, DK>(T_U, T_S16, lo_of(smem_b + CFG::w_off + ws.i * SM::w_bytes), !response);
-                commit_at(bar + 8 * B_UD);
-                commit_at(bar + 8 * (CFG::WFREE + ws.i));
-            }
-            __syncwarp();
-        } else {
-            // ---- V^T into the accumulator, as V^T times an identity, both bf16 (V as it came; the accumulator's last reader is done)
-            if (!response) {
-                if (!wait(CFG::LAND + ks.i, ks.phase)) return 327;
-                tc_fence_after();
-                if (elect_one()) {
-                    constexpr uint32_t idesc = make_idesc(NB, true, false, false) | (1u << 7) | (1u << 10);
+                constexpr uint32_t idesc = make_idesc(NB, true, false, false) | (1u << 7) | (1u << 10);
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) mma_f16(T_U, desc_lo(v_lo + c * (2048 >> 4)), IdStrip::desc(smem_b + CFG::id_off, c), idesc, c > 0);
-                }
-                __syncwarp();
-            }
-            // ---- R = V^T - S K^T
-            if (!wait(CFG::FULL + ks.i, ks.phase)) return 322;
-            if (!wait(B_SP, b & 1)) return 323;
-            tc_fence_after();
-            if (elect_one()) {
-                products_ta<false, NB, DK / 16, SM::rows>(T_U, T_S16, lo_of(k_at), !response);
-                commit_at(bar + 8 * B_RD);
-            }
-            __syncwarp();
-            // ---- U'^T = R T^T
-            // (U' completes only after the last reader of the block before's, P U', so that the chain warps need not wait for that)
-            if (b > 0 && !wait(B_OD + (b - 1) % OB, ((b - 1) / OB) & 1)) return 319;
-            if (!wait(B_RP, b & 1)) return 326;
-            tc_fence_after();
-            if (elect_one()) {
-                products_ta<false, NB, NB / 16, NB>(T_U, T_R16, t_lo, false);
-                commit_at(bar + 8 * B_UD);
+                for (int c = 0; c < 4; ++c) mma_f16(T_R, desc_lo(v_lo + c * (2048 >> 4)), IdStrip::desc(smem_b + CFG::id_off, c), idesc, c > 0);
             }
             __syncwarp();
         }
+        // ---- R = V^T - S K^T
+        if (!wait(CFG::FULL + ks.i, ks.phase)) return 322;
+        if (!wait(B_SP, b & 1)) return 323;
+        tc_fence_after();
+        if (elect_one()) {
+            products_ta<false, NB, DK / 16, SM::rows>(T_R, T_S16, lo_of(k_at), !response);
+            commit_at(bar + 8 * B_RD);
+        }
+        __syncwarp();
+        // ---- U'^T = R T^T
+        // (U' completes only after the last reader of the block before's, P U', so that the chain warps need not wait for that)
+        if (b > 0 && !wait(B_OD + (b - 1) % OB, ((b - 1) / OB) & 1)) return 319;
+        if (!wait(B_RP, b & 1)) return 326;
+        tc_fence_after();
+        if (elect_one()) {
+            products_ta<false, NB, NB / 16, NB>(T_R, T_R16, t_lo, false);
+            commit_at(bar + 8 * B_UD);
+        }
+        __syncwarp();
         // ---- S += U'^T K
         // (and S only after Q S^T)
         if (!wait(B_QD, b & 1)) return 320;
         if (!wait(B_UP, b & 1)) return 328;
         tc_fence_after();
         if (elect_one()) {
-            products_ta<true, DK, NB / 16, SM::rows, false, INPLACE ? 16 : 0>(T_S, T_U16<W, CP>, lo_of(k_at, K_SLAB), true);
+            products_ta<true, DK, NB / 16, SM::rows>(T_S, T_U16, lo_of(k_at, K_SLAB), true);
             commit_at(bar + 8 * B_SD);
             commit_at(bar + 8 * (CFG::EMPTY + ks.i));
         }
         __syncwarp();
         ks.next();
-        vs.next();
-        ts.next();
-        ws.next();
     }
     }
     return 0;
 }
 
 // The products of the output (one warp): O^T = S Q^T + U'^T P^T with the state before the update.
-template <int DK, bool W, int R, int DV>
+template <int DK, int R, int DV>
 __device__ __forceinline__ void mma_out_role(int count, int width, int* err, uint8_t* smem, uint32_t bar) {
     using SM = ChainSmem<DK, R, DV>;
-    using CFG = ChainCfg<DK, W, R, DV>;
+    using CFG = ChainCfg<DK, R, DV>;
     constexpr int CP = SM::CP, OB = O_BUFS<CP>;
     const uint32_t smem_b = smem_u32(smem);
     const int parties = width + 32;
     RingPos<CFG::NS> ks;
-    RingPos<CFG::NT> ts;
     RingPos<OB> os;
     Waits waits(bar);
 #pragma unroll 1
@@ -1142,7 +978,7 @@ __device__ __forceinline__ void mma_out_role(int count, int width, int* err, uin
         const uint32_t sg = smem_b + ks.i * SM::stage, t_o = o_cols<CP>(os.i);
         waits.wait(CFG::FULL + ks.i, ks.phase, 351);
         if (b >= OB) waits.wait(B_OFREE + os.i, os.phase ^ 1, 325);
-        waits.wait(W ? B_SP : B_RD, b & 1, 352);
+        waits.wait(B_RD, b & 1, 352);
         tc_fence_after();
         if (waits.ok() && elect_one()) {
             products_ta<false, CP, DK / 16, SM::rows, true>(t_o, T_S16, lo_of(sg + SM::q_off), false);
@@ -1152,34 +988,29 @@ __device__ __forceinline__ void mma_out_role(int count, int width, int* err, uin
         waits.wait(B_UP, b & 1, 354);
         tc_fence_after();
         if (waits.ok() && elect_one()) {
-            products_ta<false, CP, NB / 16, CP, false, U_INPLACE<W, CP> ? 16 : 0>(t_o, T_U16<W, CP>, lo_of(sg + SM::p_off), true);
+            products_ta<false, CP, NB / 16, CP>(t_o, T_U16, lo_of(sg + SM::p_off), true);
             commit_at(bar + 8 * (B_OD + os.i));
             commit_at(bar + 8 * (CFG::EMPTY + ks.i));
         }
         __syncwarp();
-        if (W && b + CFG::NT < count) pass_on(N_TFREE + ts.i, 160);
         waits.wait(B_OD + os.i, os.phase, 331);
         // (also when it has given up: the output's warps must have passed this barrier before it is arrived at again)
         if (!waits.ok() && b >= OB) mbar_wait_tries<true>(bar + 8 * (B_OFREE + os.i), os.phase ^ 1);
         pass_on(N_OD + os.i, parties);
         ks.next();
-        ts.next();
         os.next();
     }
     if (!waits.ok()) atomicCAS(err, 0, waits.code);
 }
 
-// V of each block to fp16 in place, NV blocks ahead, and O of each block from tensor memory to global memory: warp `warp` of four has rows j = 32 warp + lane, and one store of a warp is
+// O of each block from tensor memory to global memory: warp `warp` of four has rows j = 32 warp + lane, and one store of a warp is
 // 128 contiguous bytes of a token's row (64 of a response's).
-template <int DK, bool W, int R, int DV, int MODE>
-__device__ __forceinline__ void out_role(const ChainGeo& g, ChainWork<MODE> work, int* err, uint8_t* smem, uint32_t bar, int warp, int lane) {
+template <int DK, int R, int DV, int MODE>
+__device__ __forceinline__ void out_role(const ChainGeo& g, ChainWork<MODE> work, uint32_t bar, int warp, int lane) {
     using SM = ChainSmem<DK, R, DV>;
-    using CFG = ChainCfg<DK, W, R, DV>;
     constexpr int C = SM::C, CP = SM::CP, OB = O_BUFS<CP>;
     const int j = 32 * warp + lane, parties = work[0].width + 32;
-    RingPos<CFG::NV> vs;
     RingPos<OB> os;
-    Waits waits(bar);
     const uint32_t lanes = (uint32_t)(32 * warp) << 16;
 #pragma unroll 1
     for (int i = 0; i < work.size(); ++i) {
@@ -1189,51 +1020,42 @@ __device__ __forceinline__ void out_role(const ChainGeo& g, ChainWork<MODE> work
     const int nblk = part.nblk, b0 = part.b0;
     const bool response = part.response;
 #pragma unroll 1
-    for (int b = W ? -CFG::NV : 0; b < nblk; ++b) {
-        if (b >= 0) {
-            named_bar(N_OD + os.i, parties);
-            tc_fence_after();
-            const int Cv = min(C, g.L - (b0 + b) * C);
+    for (int b = 0; b < nblk; ++b) {
+        named_bar(N_OD + os.i, parties);
+        tc_fence_after();
+        const int Cv = min(C, g.L - (b0 + b) * C);
 #pragma unroll 1
-            for (int c = 0; c < CP; c += 16) {
-                uint32_t x[16];
-                tmem_ld16(o_cols<CP>(os.i) + lanes + c, x);
-                tmem_ld_wait();
-                if (c + 16 == CP) {
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive_at(bar + 8 * (B_OFREE + os.i));
-                }
-                if (response) {
-#pragma unroll
-                    for (int t = 0; t < 16; ++t)
-                        if (c + t < Cv) oh[(c + t) * DK] = __float2half_rn(__uint_as_float(x[t]));
-                } else {
-#pragma unroll
-                    for (int t = 0; t < 16; ++t)
-                        if (c + t < Cv) o[(c + t) * DV] = __uint_as_float(x[t]);
-                }
+        for (int c = 0; c < CP; c += 16) {
+            uint32_t x[16];
+            tmem_ld16(o_cols<CP>(os.i) + lanes + c, x);
+            tmem_ld_wait();
+            if (c + 16 == CP) {
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_at(bar + 8 * (B_OFREE + os.i));
             }
-            o += C * DV;
-            oh += C * DK;
-            os.next();
+            if (response) {
+#pragma unroll
+                for (int t = 0; t < 16; ++t)
+                    if (c + t < Cv) oh[(c + t) * DK] = __float2half_rn(__uint_as_float(x[t]));
+            } else {
+#pragma unroll
+                for (int t = 0; t < 16; ++t)
+                    if (c + t < Cv) o[(c + t) * DV] = __uint_as_float(x[t]);
+            }
         }
-        if (W && b + CFG::NV < nblk && !response) {
-            waits.wait(CFG::VLAND + vs.i, vs.phase, 333);
-            convert_pieces<8, DV>(smem + CFG::v_off + vs.i * SM::v_bytes, j);
-            publish_smem(bar + 8 * (CFG::WDONE + vs.i), lane);
-            vs.next();
-        }
+        o += C * DV;
+        oh += C * DK;
+        os.next();
     }
     }
-    if (!waits.ok()) atomicCAS(err, 0, waits.code);
 }
 
-template <int DK, bool W, int R, int DV, int MODE>
-__global__ void __launch_bounds__(CHAIN_THREADS<W>, 1)
+template <int DK, int R, int DV, int MODE>
+__global__ void __launch_bounds__(CHAIN_THREADS, 1)
 chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __restrict__ beta, const float* __restrict__ S0,
              float* __restrict__ O, float* __restrict__ S_final, int* __restrict__ status, ChainGeo g, ChainSeg sg) {
-    using CFG = ChainCfg<DK, W, R, DV>;
+    using CFG = ChainCfg<DK, R, DV>;
     using SM = ChainSmem<DK, R, DV>;
     extern __shared__ __align__(1024) uint8_t smem[];
     __shared__ uint64_t bar[CFG::count];
@@ -1262,7 +1084,6 @@ chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __rest
         mbar_init(&bar[B_UD], 1);
         mbar_init(&bar[B_QD], 1);
         mbar_init(&bar[B_GD], 1);
-        mbar_init(&bar[B_WD], 1);
         mbar_init(&bar[B_RD], 1);
         mbar_init(&bar[B_RP], 2 * quarters);
         for (int x = 0; x < 2; ++x) {
@@ -1271,17 +1092,8 @@ chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __rest
         }
         for (int x = 0; x < CFG::NS; ++x) {
             mbar_init(&bar[CFG::LAND + x], 1);
-            mbar_init(&bar[CFG::FULL + x], 32 * (W ? 4 : 8));        // (without W also T)
+            mbar_init(&bar[CFG::FULL + x], 32 * 8);
             mbar_init(&bar[CFG::EMPTY + x], 2);
-        }
-        for (int x = 0; x < CFG::NV; ++x) {
-            mbar_init(&bar[CFG::VLAND + x], 1);
-            mbar_init(&bar[CFG::VFREE + x], 1);
-        }
-        for (int x = 0; x < CFG::NT; ++x) mbar_init(&bar[CFG::TDONE + x], 32 * 4);
-        for (int x = 0; x < CFG::NW; ++x) {
-            mbar_init(&bar[CFG::WDONE + x], 32 * (part.response ? 4 : 4 + quarters));      // (W, and V of the same block: as many slots)
-            mbar_init(&bar[CFG::WFREE + x], 1);
         }
         mbar_fence_init();
         prefetch_tmap(&maps.q);
@@ -1296,14 +1108,13 @@ chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __rest
     }
     if (warp == W_MMA) tmem_alloc(&tmem_base, 512);
     if (SM::CP > SM::C) {                                         // (r = 3: query rows that no copy writes are read)
-        for (int e = tid; e < CFG::NS * SM::stage / 16; e += CHAIN_THREADS<W>) ((uint4*)smem)[e] = make_uint4(0, 0, 0, 0);
+        for (int e = tid; e < CFG::NS * SM::stage / 16; e += CHAIN_THREADS) ((uint4*)smem)[e] = make_uint4(0, 0, 0, 0);
     } else {                                                      // (the upper triangles of P and T, which nothing writes)
         for (int st = 0; st < CFG::NS && st < count; ++st)
-            for (int e = tid; e < SM::p_bytes / 16; e += CHAIN_THREADS<W>) ((uint4*)(smem + st * SM::stage + SM::p_off))[e] = make_uint4(0, 0, 0, 0);
+            for (int e = tid; e < SM::p_bytes / 16; e += CHAIN_THREADS) ((uint4*)(smem + st * SM::stage + SM::p_off))[e] = make_uint4(0, 0, 0, 0);
     }
-    for (int e = tid; e < CFG::NT * SM::t_bytes / 16; e += CHAIN_THREADS<W>) ((uint4*)(smem + CFG::t_off))[e] = make_uint4(0, 0, 0, 0);
-    if (!W)
-        for (int e = tid; e < IdStrip::bytes / 2; e += CHAIN_THREADS<W>) ((uint16_t*)(smem + CFG::id_off))[e] = IdStrip::one(e) ? 0x3F80 : 0;
+    for (int e = tid; e < CFG::NS * SM::t_bytes / 16; e += CHAIN_THREADS) ((uint4*)(smem + CFG::t_off))[e] = make_uint4(0, 0, 0, 0);
+    for (int e = tid; e < IdStrip::bytes / 2; e += CHAIN_THREADS) ((uint16_t*)(smem + CFG::id_off))[e] = IdStrip::one(e) ? 0x3F80 : 0;
     fence_async_smem();
     tc_fence_before();
     __syncthreads();
@@ -1325,7 +1136,7 @@ chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __rest
     auto all_done = [&]() {
         __syncwarp();
         tc_fence_before();
-        named_bar(0, CHAIN_THREADS<W>);
+        named_bar(0, CHAIN_THREADS);
         tc_fence_after();
     };
     // (the chain's and the solve teams' warps, eight rows each, us a token with every row lost and with the chain's warps alone: d = 128, r = 1, 2, 4
@@ -1346,12 +1157,12 @@ chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __rest
         }
     };
     if (warp < W_OUT) {
-        set_registers<W, REGS_CHAIN>();
+        set_registers<REGS_CHAIN>();
         begin();
         if (tid == 0 && blockIdx.x == 0 && g.clear) *status = 0;  // (the call's status word: a wait expires a second from now at the earliest)
         const bool holds_state = (warp & 3) < quarters;
         if (holds_state) {
-            const int code = chain_role<DK, W, SM::CP>(g, work, lost, bar_b, warp, lane);
+            const int code = chain_role<DK>(g, work, lost, bar_b, warp, lane);
             if (code) atomicCAS(status, 0, code);
         }
         all_done();                                               // (every output is written)
@@ -1361,41 +1172,36 @@ chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __rest
         }
         walk_lost(warp);
     } else if (warp < W_CONV) {
-        set_registers<W, REGS_OUT>();
+        set_registers<REGS_OUT>();
         begin();
-        if (warp - W_OUT < quarters) out_role<DK, W, R, DV>(g, work, status, smem, bar_b, warp - W_OUT, lane);
+        if (warp - W_OUT < quarters) out_role<DK, R, DV>(g, work, bar_b, warp - W_OUT, lane);
         all_done();
     } else if (warp < W_SOLVE) {
-        set_registers<W, REGS_CONV>();
+        set_registers<REGS_CONV>();
         begin();
-        convert_role<DK, W, R, DV>(count, smem, bar_b, tid - 32 * W_CONV);
+        convert_role<DK, R, DV>(count, smem, bar_b, tid - 32 * W_CONV);
         all_done();
     } else if (warp < W_MMA) {
-        set_registers<W, REGS_SOLVE<W>>();
+        set_registers<REGS_SOLVE>();
         begin();
-        solve_role<DK, W, R, DV>(g, work, beta, smem, bar_b, (warp - W_SOLVE) >> 2, (tid - 32 * W_SOLVE) & 127);
+        solve_role<DK, R, DV>(g, work, beta, smem, bar_b, (warp - W_SOLVE) >> 2, (tid - 32 * W_SOLVE) & 127);
         all_done();
         walk_lost(8 + warp - W_SOLVE);
-    } else if (warp < W_W) {
-        set_registers<W, REGS_ISSUE>();
+    } else {
+        set_registers<REGS_ISSUE>();
         begin();
         if (warp == W_MMA) {
-            const int code = mma_role<DK, W, R, DV>(work, smem, bar_b);
+            const int code = mma_role<DK, R, DV>(work, smem, bar_b);
             if (code) atomicCAS(status, 0, code);
         } else if (warp == W_MMA_OUT) {
-            mma_out_role<DK, W, R, DV>(count, part.width, status, smem, bar_b);
+            mma_out_role<DK, R, DV>(count, part.width, status, smem, bar_b);
         } else if (warp == W_GRAM) {
-            gram_role<DK, W, R, DV>(count, status, smem, bar_b);
+            gram_role<DK, R, DV>(count, status, smem, bar_b);
         } else if (warp == W_LOAD) {
-            load_role<DK, W, R, DV>(maps, work, status, smem, bar_b);
+            load_role<DK, R, DV>(maps, work, status, smem, bar_b);
         }
         all_done();
         if (warp == W_MMA) tmem_dealloc(0, 512);
-    } else if constexpr (W) {
-        set_registers<W, REGS_W>();
-        begin();
-        w_role<DK, W, R, DV>(count, status, smem, bar_b, tid - 32 * W_W);
-        all_done();
     }
 }
 
@@ -1674,11 +1480,11 @@ ChainCarve carve(const Problem& p, const ChainPlan& plan) {
     return c;
 }
 
-template <int DK, int R, int DV, int MODE, bool W = false>
+template <int DK, int R, int DV, int MODE>
 int launch(const Problem& p, const ChainPlan& plan, const ChainSeg& sg, void* workspace) {
-    using CFG = ChainCfg<DK, W, R, DV>;
-    static_assert(CFG::total + (MODE == SHARED ? 4096 : 1024) <= 227 * 1024 && CFG::NS >= 3 && (!W || (CFG::NS >= 4 && CFG::NT <= 3 && CFG::NV == CFG::NW)), "shared memory budget");
-    const void* fn = (const void*)chain_kernel<DK, W, R, DV, MODE>;
+    using CFG = ChainCfg<DK, R, DV>;
+    static_assert(CFG::total + (MODE == SHARED ? 4096 : 1024) <= 227 * 1024 && CFG::NS >= 3, "shared memory budget");
+    const void* fn = (const void*)chain_kernel<DK, R, DV, MODE>;
     constexpr int C = NB / R;
     ChainGeo g{p.L, p.d_v, (p.L + C - 1) / C, plan.nseg, plan.seg_blk, plan.first_blk, plan.share, 0, nullptr, nullptr, nullptr, p.mask_group(), p.exact ? 1 : 0, p.clear_status ? 1 : 0,
                (const __nv_bfloat16*)p.q, (const __nv_bfloat16*)p.k, (const __nv_bfloat16*)p.v, (const __nv_bfloat16*)p.beta,
@@ -1702,7 +1508,7 @@ int launch(const Problem& p, const ChainPlan& plan, const ChainSeg& sg, void* wo
     if (st != PF_OK) return st;
     void* args[] = {(void*)&maps, (void*)&p.beta, (void*)&p.S0, (void*)&p.O, (void*)&p.S_final, (void*)&p.status, (void*)&g, (void*)&sg};
     prof_begin("chain", p.stream);
-    PF_CUDA_TRY(launch_early(fn, dim3((unsigned)grid), CHAIN_THREADS<W>, args, (size_t)CFG::total, p.stream));
+    PF_CUDA_TRY(launch_early(fn, dim3((unsigned)grid), CHAIN_THREADS, args, (size_t)CFG::total, p.stream));
     prof_end(p.stream);
     count_launch(1);
     return PF_OK;
@@ -1712,8 +1518,6 @@ template <int DK, int R>
 int launch_plan(const Problem& p, const ChainPlan& plan, const ChainSeg& sg, void* ws) {
     if (plan.share > 0) return p.d_v == 128 ? launch<DK, R, 128, SHARED>(p, plan, sg, ws) : launch<DK, R, 64, SHARED>(p, plan, sg, ws);
     if (plan.nseg > 1) return p.d_v == 128 ? launch<DK, R, 128, SEGMENTS>(p, plan, sg, ws) : launch<DK, R, 64, SEGMENTS>(p, plan, sg, ws);
-    if constexpr (DK == 64)
-        if (p.d_v == 64 && plan.seg_blk >= W_FORM_BLOCKS) return launch<DK, R, 64, WHOLE, true>(p, plan, sg, ws);
     return p.d_v == 128 ? launch<DK, R, 128, WHOLE>(p, plan, sg, ws) : launch<DK, R, 64, WHOLE>(p, plan, sg, ws);
 }
 template <int DK>
