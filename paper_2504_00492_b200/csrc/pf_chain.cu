@@ -134,7 +134,8 @@ enum {
     B_GD = 9,       // Gram products: G and P^T complete
     B_RD = 10,      // products: V^T - S K^T complete
     B_RP = 11,      // chain: its fp16 copy published
-    B_RINGS = 12
+    B_END = 12,     // [4] the two chain warps of a quarter, when a walk is over
+    B_RINGS = 16
 };
 constexpr int TEAMS = 2;             // solve teams
 // warps: 0-7 chain, 8-11 output, 12-15 conversion, then the solve teams, then products of the chain, products of the output, Gram products,
@@ -406,8 +407,7 @@ enum {
     N_GD = 5,       // [team] Gram products -> solve: G complete
     N_GFREE = 7,    // solve and conversion -> Gram products: G and P^T read
     N_PD = 8,       // Gram products -> conversion: P^T complete (and nothing reads the block's K and Q as bf16 any more)
-    N_OD = 10,      // [2] output products -> output: O^T complete
-    N_END = 12      // [4] the two chain warps of a quarter, when a walk is over
+    N_OD = 10       // [2] output products -> output: O^T complete
 };
 __device__ __forceinline__ void named_arrive(int id, int nthreads) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(nthreads) : "memory"); }
 // (after a wait for a product's mbarrier, by a whole warp)
@@ -775,8 +775,9 @@ __device__ __forceinline__ bool wait_for_count(const int* p, int want) {
 __device__ __forceinline__ void add_release_gpu(int* p, int v) { asm volatile("red.release.gpu.global.add.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory"); }
 
 // The end state (its last update is the chain's last product, so that this goes on beside the last block's output); lost: gets a bit for each quarter of the rows j that has to be walked again.
+// end_bar, met: where the two warps of a quarter meet, and its parity.  Returns false if the other one does not come.
 template <int DK, bool SHARE>
-__device__ __forceinline__ void end_state(const ChainGeo& g, const ChainPart& part, uint32_t* lost, int warp, int lane) {
+__device__ __forceinline__ bool end_state(const ChainGeo& g, const ChainPart& part, uint32_t* lost, uint32_t end_bar, int& met, int warp, int lane) {
     constexpr int HC = DK / 2;
     const int h = warp >> 2, quarter = warp & 3, j = 32 * quarter + lane;
     const uint32_t t_s = T_S + h * HC + ((uint32_t)(32 * quarter) << 16);
@@ -794,7 +795,7 @@ __device__ __forceinline__ void end_state(const ChainGeo& g, const ChainPart& pa
         __threadfence();
         __syncwarp();
         if (lane == 0) add_release_gpu(g.handed + part.hand_out, 1);
-        return;
+        return true;
     }
     if (part.response) {
         __half* P = (__half*)part.S_end + (long long)j * DK + h * HC;
@@ -814,15 +815,21 @@ __device__ __forceinline__ void end_state(const ChainGeo& g, const ChainPart& pa
                 *(uint4*)(P + c + e) = make_uint4(pack_h2(__uint_as_float(x[e]), __uint_as_float(x[e + 1])), pack_h2(__uint_as_float(x[e + 2]), __uint_as_float(x[e + 3])),
                                                   pack_h2(__uint_as_float(x[e + 4]), __uint_as_float(x[e + 5])), pack_h2(__uint_as_float(x[e + 6]), __uint_as_float(x[e + 7])));
         }
-        return;
+        return true;
     }
-    // (one entry tells for its row.  The end state may replace the start state, which is still needed where rows are lost)
+    // (one entry tells for its row.  The end state may replace the start state, which is still needed where rows are lost, so that both warps have to know before
+    //  either writes.  They meet at an mbarrier, whose wait has a limit: one of them may have given up)
     uint32_t x[32];
     tmem_ld32(t_s, x);
     tmem_ld_wait();
-    if (!named_bar_and(N_END + quarter, 64, fabsf(__uint_as_float(x[0])) <= FLT_MAX)) {
-        if (h == 0 && lane == 0) atomicOr(lost, 1u << quarter);
-    } else if (part.S_end) {
+    const bool finite = __all_sync(0xffffffffu, fabsf(__uint_as_float(x[0])) <= FLT_MAX);
+    if (lane == 0) {
+        if (!finite) atomicOr(lost, 1u << quarter);
+        mbar_arrive_at(end_bar);
+    }
+    if (!mbar_wait_tries<false>(end_bar, met)) return false;
+    met ^= 1;
+    if (part.S_end && !(*(volatile uint32_t*)lost >> quarter & 1)) {
 #pragma unroll 1
         for (int c = 0; c < HC; c += 32) {
             tmem_ld32(t_s + c, x);
@@ -831,6 +838,7 @@ __device__ __forceinline__ void end_state(const ChainGeo& g, const ChainPart& pa
             for (int e = 0; e < 32; ++e) part.S_end[(long long)(h * HC + c + e) * part.width + j] = __uint_as_float(x[e]);
         }
     }
+    return true;
 }
 
 // warp `warp` of eight: rows j = 32 (warp & 3) + lane, half warp >> 2 of the columns of everything.  Returns the code of the wait that ran out, or 0.
@@ -847,7 +855,7 @@ __device__ __forceinline__ int chain_role(const ChainGeo& g, ChainWork<MODE> wor
         __syncwarp();
         if (lane == 0) mbar_arrive_at(bar + 8 * b);
     };
-    int code = 0, parity = 0;
+    int code = 0, parity = 0, met = 0;
 #pragma unroll 1
     for (int i = 0; i < work.size(); ++i) {
         const ChainPart& part = work[i];
@@ -891,7 +899,7 @@ __device__ __forceinline__ int chain_role(const ChainGeo& g, ChainWork<MODE> wor
             to_operand<HC, true>(t_s, t_s16);
         }
         parity ^= 1;
-        end_state<DK, ChainWork<MODE>::shared>(g, part, lost + i, warp, lane);
+        if (!end_state<DK, ChainWork<MODE>::shared>(g, part, lost + i, bar + 8 * (B_END + (warp & 3)), met, warp, lane)) return 315;
     }
     return code;
 }
@@ -1086,6 +1094,7 @@ chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __rest
         mbar_init(&bar[B_GD], 1);
         mbar_init(&bar[B_RD], 1);
         mbar_init(&bar[B_RP], 2 * quarters);
+        for (int x = 0; x < 4; ++x) mbar_init(&bar[B_END + x], 2);
         for (int x = 0; x < 2; ++x) {
             mbar_init(&bar[B_OD + x], 1);
             mbar_init(&bar[B_OFREE + x], quarters);
