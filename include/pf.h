@@ -126,7 +126,9 @@ enum { PF_IMPL_AUTO = 0, PF_IMPL_SIMT = 1, PF_IMPL_TC = 2,
  * exceed 65504 (with keys of length 1, S k reaches sqrt(d_k) times the largest entry of S): they stay in fp32 in the single
  * launch, and the one-kernel chunk form, where they are operands, computes the columns of O and S_final that lost them once more
  * in fp32 (slowly, 0.5 us a token (d = 64, r = 1) to 3.7 (d = 128, r = 4); columns that are infinite or NaN for other reasons pay this too).  Not so in segments for what the segment makes of its start
- * state: a recurrence that amplifies a state by more than 65504 within a segment (step sizes beyond 2 / |k|^2) gives infinities or NaN there.  The stated tolerance
+ * state: a recurrence that amplifies a state by more than 65504 within a segment (step sizes beyond 2 / |k|^2) gives infinities or NaN there, except in calls that
+ * would be the single launch's if the segments' walks were not shared out among the SMs (d_k = d_v = 128, about 20 to 40 sequences of some thousand tokens): there
+ * such a sequence is computed once more in fp32, all of it.  The stated tolerance
  * (2e-3 of max|O|) is tested for |v|, |S| up to the order of 1e3, and for states of 2e4 aligned with a key.  The operation is linear in (v, S0): scale them by a power
  * of two and O, S_final back for data outside that range, or ask for PF_IMPL_SIMT (fp32 throughout, no such limit).
  */

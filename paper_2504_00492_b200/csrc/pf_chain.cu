@@ -82,6 +82,7 @@ struct ChainGeo {
     int total;          // of all of them
     float* hand;        // [CTAs] states that go from one CTA to another, [d_k i][d_v j]
     int *handed, *finished;     // [CTAs] each: warps that have handed over; the CTA's outputs are written
+    int* lost;          // [sequences] a response has left fp16's range (null: nobody asks, ChainPlan::rewalk)
     int rm;             // strict-mask group size (Problem::mask_group)
     int exact;          // PF_STEP_EXACT
     int clear;          // set the status word to 0
@@ -765,6 +766,8 @@ __device__ __forceinline__ void to_operand(uint32_t src, uint32_t dst) {
     }
 }
 
+constexpr uint32_t HALF_INF = 0x477FF000u;     // 65520 as fp32: from there on fp16 is infinite (bits of magnitudes, so that NaN is above)
+
 // Waits until *p >= want (one thread), about a second at most.
 __device__ __forceinline__ bool wait_for_count(const int* p, int want) {
     const long long t0 = clock64();
@@ -798,6 +801,7 @@ __device__ __forceinline__ bool end_state(const ChainGeo& g, const ChainPart& pa
         return true;
     }
     if (part.response) {
+        uint32_t most = 0;                                        // (an infinity or NaN on the diagonal is not alone in its row)
         __half* P = (__half*)part.S_end + (long long)j * DK + h * HC;
 #pragma unroll 1
         for (int c = 0; c < HC; c += 32) {
@@ -810,11 +814,15 @@ __device__ __forceinline__ bool end_state(const ChainGeo& g, const ChainPart& pa
                     part.D[j] = __uint_as_float(x[e]);
                     x[e] = 0;
                 }
+            if (SHARE)
+#pragma unroll
+                for (int e = 0; e < 32; ++e) most = max(most, x[e] & 0x7fffffffu);
 #pragma unroll
             for (int e = 0; e < 32; e += 8)
                 *(uint4*)(P + c + e) = make_uint4(pack_h2(__uint_as_float(x[e]), __uint_as_float(x[e + 1])), pack_h2(__uint_as_float(x[e + 2]), __uint_as_float(x[e + 3])),
                                                   pack_h2(__uint_as_float(x[e + 4]), __uint_as_float(x[e + 5])), pack_h2(__uint_as_float(x[e + 6]), __uint_as_float(x[e + 7])));
         }
+        if (SHARE && most >= HALF_INF && g.lost) g.lost[part.seq] = 1;
         return true;
     }
     // (one entry tells for its row.  The end state may replace the start state, which is still needed where rows are lost, so that both warps have to know before
@@ -1027,6 +1035,7 @@ __device__ __forceinline__ void out_role(const ChainGeo& g, ChainWork<MODE> work
     __half* oh = (__half*)part.O + j;
     const int nblk = part.nblk, b0 = part.b0;
     const bool response = part.response;
+    uint32_t most = 0;                                            // (bits of the response's largest magnitude)
 #pragma unroll 1
     for (int b = 0; b < nblk; ++b) {
         named_bar(N_OD + os.i, parties);
@@ -1043,6 +1052,9 @@ __device__ __forceinline__ void out_role(const ChainGeo& g, ChainWork<MODE> work
                 if (lane == 0) mbar_arrive_at(bar + 8 * (B_OFREE + os.i));
             }
             if (response) {
+                if (MODE == SHARED)
+#pragma unroll
+                    for (int t = 0; t < 16; ++t) most = max(most, x[t] & 0x7fffffffu);
 #pragma unroll
                 for (int t = 0; t < 16; ++t)
                     if (c + t < Cv) oh[(c + t) * DK] = __float2half_rn(__uint_as_float(x[t]));
@@ -1056,6 +1068,7 @@ __device__ __forceinline__ void out_role(const ChainGeo& g, ChainWork<MODE> work
         oh += C * DK;
         os.next();
     }
+    if (MODE == SHARED && most >= HALF_INF && g.lost) g.lost[part.seq] = 1;
     }
 }
 
@@ -1224,8 +1237,9 @@ struct ComposeSmem {
     static constexpr int LD = DK + 8, LX = 20;                    // (row pitches without bank conflicts)
     static constexpr int p_bytes = DK * LD * 2, x_bytes = DK * LX * 4, stage = p_bytes + x_bytes + DK * 4, a_bytes = 2 * 16 * LD * 2;
 };
-template <int DK>
-__global__ void __launch_bounds__(128) chain_compose(ChainSeg sg, float* __restrict__ S_final, int nseg, int d_v) {
+// LOST: lost[sequence]: chain_apply walks it again, from a start state that S_final may replace.
+template <int DK, bool LOST>
+__global__ void __launch_bounds__(128) chain_compose(ChainSeg sg, float* __restrict__ S_final, const int* __restrict__ lost, int nseg, int d_v) {
     using SM = ComposeSmem<DK>;
     constexpr int LD = SM::LD, LX = SM::LX, NT = DK / 32;
     extern __shared__ __align__(16) uint8_t smem_tail[];
@@ -1260,6 +1274,7 @@ __global__ void __launch_bounds__(128) chain_compose(ChainSeg sg, float* __restr
     };
     float S[NT][4];
     wait_for_previous_kernel();
+    if (LOST && lost[seq]) S_final = nullptr;
     for (int s = 1; s <= depth; ++s) load(s, s - 1);
     {
         const float* src = sg.Xi + seq * nseg * DK * d_v;
@@ -1322,8 +1337,9 @@ __global__ void __launch_bounds__(128) chain_compose(ChainSeg sg, float* __restr
 
 // O[t][j] += sum_i R[t][i] start[j][i] for the tokens of all segments but the first: grid (128-token tiles, nseq (nseg - 1)), a
 // warp per 16 tokens.  Bound by the traffic: per token R once, O read and written.
-template <int DK, int DV>
-__global__ void __launch_bounds__(256) chain_apply(ChainSeg sg, float* __restrict__ O, int L, int first_tokens, int seg_tokens, int nseg) {
+// LOST_R (a rank, or 0): with `args`, which says which sequences are walked again instead.
+template <int DK, int DV, int LOST_R>
+__device__ __forceinline__ void apply_tile(const ChainSeg& sg, float* __restrict__ O, int L, int first_tokens, int seg_tokens, int nseg, const ChainArgs* args) {
     constexpr int LD = DK + 8, KT = DK / 16;
     extern __shared__ __align__(16) uint8_t smem_tail[];
     __half* sS = (__half*)smem_tail;                                   // [DV][LD]
@@ -1333,6 +1349,7 @@ __global__ void __launch_bounds__(256) chain_apply(ChainSeg sg, float* __restric
     const int start = first_tokens + (s - 1) * seg_tokens, t_end = min(L, start + seg_tokens), t0 = start + blockIdx.x * 128 + w * 16 + gq;
     const __half* src = sg.start + (seq * nseg + s) * DV * DK;
     wait_for_previous_kernel();
+    const int lost = LOST_R > 0 ? args->g.lost[seq] : 0;          // (looked at when everything else is on its way)
 #pragma unroll
     for (int e = 0; e < DV * DK / 8 / 256; ++e) {
         const int p = e * 256 + tid, row = p / (DK / 8), c = p % (DK / 8);
@@ -1358,6 +1375,19 @@ __global__ void __launch_bounds__(256) chain_apply(ChainSeg sg, float* __restric
         c[n][0] = x.x; c[n][1] = x.y; c[n][2] = y.x; c[n][3] = y.y;
     }
     __syncthreads();
+    if constexpr (LOST_R > 0)
+        if (lost) {
+            const ChainGeo& g = args->g;
+            ChainPart part{};
+            part.nblk = g.nblk;
+            part.S0 = g.S0 ? g.S0 + seq * DK * DV : nullptr;
+            part.O = O + seq * L * DV;
+            part.S_end = g.S_final ? g.S_final + seq * DK * DV : nullptr;
+            const int block = (s - 1) * gridDim.x + blockIdx.x, blocks = (nseg - 1) * gridDim.x;
+#pragma unroll 1
+            for (int row0 = 8 * (8 * block + w); row0 < DV; row0 += 64 * blocks) walk_fp32<DK, LOST_R>(*args, part, seq, row0);
+            return;
+        }
     // (calls one after another, us with an early start of the next and without: 15 blocks 30.6 and 31.3, 62: 43.2 and 43.7 (d = 128,
     //  r = 1), 26.2 and 27.1 (d = 64).  Where the blocks are many the next kernel's come to multiprocessors in the order in which
     //  these leave, apart from their neighbours with the same inputs: at d = 128 1 - 4 % slower, 256 blocks 101.2 and 99.5, 1024: 350 and
@@ -1380,6 +1410,17 @@ __global__ void __launch_bounds__(256) chain_apply(ChainSeg sg, float* __restric
     }
 }
 
+template <int DK, int DV>
+__global__ void __launch_bounds__(256) chain_apply(ChainSeg sg, float* __restrict__ O, int L, int first_tokens, int seg_tokens, int nseg) {
+    apply_tile<DK, DV, 0>(sg, O, L, first_tokens, seg_tokens, nseg, nullptr);
+}
+// For calls that the single launch would take if walks were not shared out.  Its flows are those of 64 tokens, here a response runs through thousands: where one
+// has left fp16's range, the whole sequence is walked again in fp32, by the first of its blocks here.
+template <int DK, int DV, int R>
+__global__ void __launch_bounds__(256, 2) chain_apply_or_walk(const __grid_constant__ ChainArgs args, int first_tokens, int seg_tokens) {
+    apply_tile<DK, DV, R>(args.seg, args.g.O, args.g.L, first_tokens, seg_tokens, args.g.nseg, &args);
+}
+
 // A sequence has one CTA, or where few sequences are long, segments walked side by side: as many as one wave of CTAs holds pay for
 // the second walk (the responses) and for two more kernels.  The time is 7 us, (waves of CTAs) x (blocks of a segment) x (time of a
 // block) and what composing segments costs.  Measured, us per block for r = 1 .. 4 with 32 CTAs (d_k = 64 and 128), and with 148, when
@@ -1391,6 +1432,7 @@ struct ChainPlan {
     double us;
     int first_blk;            // blocks of the first segment
     int share, ctas;          // SHARED: blocks of a CTA (0: a walk each) and CTAs
+    bool rewalk;              // sequences in which a response leaves fp16's range are walked again (chain_apply)
     double short_us;          // the kernel alone without segments, the start of each wave counted: what a call of a few blocks takes
 };
 // Equal shares of all blocks (part_at) in place of a walk each, where that is faster: more sequences than multiprocessors, or, of a state as wide as its response,
@@ -1434,6 +1476,7 @@ ChainPlan share_out(const Problem& p, const ChainPlan& plan, int nblk, double bl
     const int other = out.nseg > 1 ? out.seg_blk : out.first_blk, longest = out.first_blk > other ? out.first_blk : other, shortest = out.first_blk < other ? out.first_blk : other;
     if (longest > out.share || out.share / shortest + 2 > MOST_PARTS) return plan;
     out.us = us + out.share * block_us + 1.5 * out.share / shortest;
+    out.rewalk = out.nseg > 1 && fused_supported(p) && fused_estimate_us(p) < plan.us;
     return out.us < 0.985 * rival ? out : plan;
 }
 ChainPlan make_plan(const Problem& p) {
@@ -1447,7 +1490,7 @@ ChainPlan make_plan(const Problem& p) {
         return a + (c - a) * (crowd < 0.0 ? 0.0 : crowd > 1.0 ? 1.0 : crowd);
     };
     const double waves = (double)((nseq + sms - 1) / (sms > 0 ? sms : 1)), walk = nblk * step(nseq) * waves;
-    ChainPlan plan{1, nblk, 7.0 + walk, nblk, 0, 0, 5.0 * waves + walk};
+    ChainPlan plan{1, nblk, 7.0 + walk, nblk, 0, 0, false, 5.0 * waves + walk};
     const double limit = 0.92 * plan.us;
     // (calls of up to 512 tokens at d_k = 128 are one launch, which a test of two sequences of 512 expects, also where segments would be faster: 16 of
     //  333, r = 2: 21.7 us, 20.9 estimated in four)
@@ -1457,13 +1500,13 @@ ChainPlan make_plan(const Problem& p) {
         // (two kernels, their share per segment, and the traffic of the responses and of O at about 4 TB/s)
         const double traffic = (double)nseq * p.L * (nseg - 1) / nseg * (4.0 * p.d_k + 8.0 * p.d_v) / 4e6;
         const double us = (p.d_k == 128 ? 11.0 + 0.85 * nseg : 9.0 + 0.4 * nseg) + traffic + seg_blk * step(nseq * (2 * nseg - 1));
-        if (us < limit && us < plan.us) plan = {nseg, seg_blk, us, seg_blk, 0, 0, plan.short_us};
+        if (us < limit && us < plan.us) plan = {nseg, seg_blk, us, seg_blk, 0, 0, false, plan.short_us};
     }
     return share_out(p, plan, nblk, step(sms));
 }
 
 struct ChainCarve {
-    size_t R, P, D, Xi, start, flags, hand, total;
+    size_t R, P, D, Xi, start, flags, flag_bytes, hand, total;
 };
 ChainCarve carve(const Problem& p, const ChainPlan& plan) {
     ChainCarve c{};
@@ -1482,31 +1525,50 @@ ChainCarve carve(const Problem& p, const ChainPlan& plan) {
         c.start = take(slots * p.d_v * p.d_k * 2);
     }
     if (plan.share > 0) {
-        c.flags = take((size_t)plan.ctas * 8);
+        c.flag_bytes = (size_t)plan.ctas * 8 + (plan.rewalk ? (size_t)p.B * p.H * 4 : 0);
+        c.flags = take(c.flag_bytes);
         c.hand = take((size_t)plan.ctas * p.d_k * p.d_v * 4);
     }
     c.total = off;
     return c;
 }
 
+ChainGeo make_geo(const Problem& p, const ChainPlan& plan, const ChainCarve& c, void* workspace) {
+    ChainGeo g{};
+    g.L = p.L;
+    g.d_v = p.d_v;
+    g.nblk = (p.L + NB / p.r - 1) / (NB / p.r);
+    g.nseg = plan.nseg;
+    g.seg_blk = plan.seg_blk;
+    g.first_blk = plan.first_blk;
+    if (plan.share > 0) {
+        g.share = plan.share;
+        g.total = (int)((long long)p.B * p.H * (2 * g.nblk - g.first_blk));
+        g.hand = (float*)((uint8_t*)workspace + c.hand);
+        g.handed = (int*)((uint8_t*)workspace + c.flags);
+        g.finished = g.handed + plan.ctas;
+        if (plan.rewalk) g.lost = g.finished + plan.ctas;
+    }
+    g.rm = p.mask_group();
+    g.exact = p.exact ? 1 : 0;
+    g.clear = p.clear_status ? 1 : 0;
+    g.q = (const __nv_bfloat16*)p.q;
+    g.k = (const __nv_bfloat16*)p.k;
+    g.v = (const __nv_bfloat16*)p.v;
+    g.beta = (const __nv_bfloat16*)p.beta;
+    g.S0 = p.S0;
+    g.O = p.O;
+    g.S_final = p.S_final;
+    return g;
+}
+
 template <int DK, int R, int DV, int MODE>
-int launch(const Problem& p, const ChainPlan& plan, const ChainSeg& sg, void* workspace) {
+int launch(const Problem& p, const ChainPlan& plan, const ChainGeo& g, const ChainSeg& sg) {
     using CFG = ChainCfg<DK, R, DV>;
     static_assert(CFG::total + (MODE == SHARED ? 4096 : 1024) <= 227 * 1024 && CFG::NS >= 3, "shared memory budget");
     const void* fn = (const void*)chain_kernel<DK, R, DV, MODE>;
     constexpr int C = NB / R;
-    ChainGeo g{p.L, p.d_v, (p.L + C - 1) / C, plan.nseg, plan.seg_blk, plan.first_blk, plan.share, 0, nullptr, nullptr, nullptr, p.mask_group(), p.exact ? 1 : 0, p.clear_status ? 1 : 0,
-               (const __nv_bfloat16*)p.q, (const __nv_bfloat16*)p.k, (const __nv_bfloat16*)p.v, (const __nv_bfloat16*)p.beta,
-               p.S0, p.O, p.S_final};
     const long long nseq = (long long)p.B * p.H, grid = MODE == SHARED ? plan.ctas : nseq * (2 * plan.nseg - 1);
-    if (MODE == SHARED) {
-        const ChainCarve c = carve(p, plan);
-        g.total = (int)(nseq * (2 * g.nblk - g.first_blk));
-        g.handed = (int*)((uint8_t*)workspace + c.flags);
-        g.finished = g.handed + plan.ctas;
-        g.hand = (float*)((uint8_t*)workspace + c.hand);
-        PF_CUDA_TRY(cudaMemsetAsync(g.handed, 0, (size_t)plan.ctas * 8, p.stream));
-    }
     ChainMaps maps;
     if (!make_slab_map(&maps.k, p.k, nseq, (uint64_t)p.L * R, DK, 64, NB, 1) ||
         !make_slab_map(&maps.q, p.q, nseq, p.L, DK, 64, C, 1) ||
@@ -1524,41 +1586,49 @@ int launch(const Problem& p, const ChainPlan& plan, const ChainSeg& sg, void* wo
 }
 
 template <int DK, int R>
-int launch_plan(const Problem& p, const ChainPlan& plan, const ChainSeg& sg, void* ws) {
-    if (plan.share > 0) return p.d_v == 128 ? launch<DK, R, 128, SHARED>(p, plan, sg, ws) : launch<DK, R, 64, SHARED>(p, plan, sg, ws);
-    if (plan.nseg > 1) return p.d_v == 128 ? launch<DK, R, 128, SEGMENTS>(p, plan, sg, ws) : launch<DK, R, 64, SEGMENTS>(p, plan, sg, ws);
-    return p.d_v == 128 ? launch<DK, R, 128, WHOLE>(p, plan, sg, ws) : launch<DK, R, 64, WHOLE>(p, plan, sg, ws);
+int launch_plan(const Problem& p, const ChainPlan& plan, const ChainGeo& g, const ChainSeg& sg) {
+    if (plan.share > 0) return p.d_v == 128 ? launch<DK, R, 128, SHARED>(p, plan, g, sg) : launch<DK, R, 64, SHARED>(p, plan, g, sg);
+    if (plan.nseg > 1) return p.d_v == 128 ? launch<DK, R, 128, SEGMENTS>(p, plan, g, sg) : launch<DK, R, 64, SEGMENTS>(p, plan, g, sg);
+    return p.d_v == 128 ? launch<DK, R, 128, WHOLE>(p, plan, g, sg) : launch<DK, R, 64, WHOLE>(p, plan, g, sg);
 }
 template <int DK>
-int launch_rank(const Problem& p, const ChainPlan& plan, const ChainSeg& sg, void* ws) {
+int launch_rank(const Problem& p, const ChainPlan& plan, const ChainGeo& g, const ChainSeg& sg) {
     switch (p.r) {
-        case 1: return launch_plan<DK, 1>(p, plan, sg, ws);
-        case 2: return launch_plan<DK, 2>(p, plan, sg, ws);
-        case 3: return launch_plan<DK, 3>(p, plan, sg, ws);
-        default: return launch_plan<DK, 4>(p, plan, sg, ws);
+        case 1: return launch_plan<DK, 1>(p, plan, g, sg);
+        case 2: return launch_plan<DK, 2>(p, plan, g, sg);
+        case 3: return launch_plan<DK, 3>(p, plan, g, sg);
+        default: return launch_plan<DK, 4>(p, plan, g, sg);
     }
 }
 
-template <int DK, int DV>
-int launch_seg_tail(const Problem& p, const ChainPlan& plan, const ChainSeg& sg) {
+template <int DK, int DV, int LOST_R = 0>
+int launch_seg_tail(const Problem& p, const ChainPlan& plan, const ChainGeo& g, const ChainSeg& sg) {
     const int nseq = p.B * p.H, dv = DV, seg_tokens = plan.seg_blk * (NB / p.r), first_tokens = plan.first_blk * (NB / p.r);
     constexpr int LD = DK + 8;
     {
         using SM = ComposeSmem<DK>;
         const int smem = SM::a_bytes + (plan.nseg - 1 < COMPOSE_RING ? plan.nseg - 1 : COMPOSE_RING) * SM::stage;
         static std::atomic<uint64_t> opted_in{0};
-        const int st = allow_smem(opted_in, (const void*)chain_compose<DK>, SM::a_bytes + COMPOSE_RING * SM::stage);
+        const void* fn = (const void*)chain_compose<DK, (LOST_R > 0)>;
+        const int st = allow_smem(opted_in, fn, SM::a_bytes + COMPOSE_RING * SM::stage);
         if (st != PF_OK) return st;
         prof_begin("chain_compose", p.stream);
-        void* args[] = {(void*)&sg, (void*)&p.S_final, (void*)&plan.nseg, (void*)&dv};
-        PF_CUDA_TRY(launch_early((const void*)chain_compose<DK>, dim3((unsigned)(nseq * (DV / 16))), 128, args, smem, p.stream));
+        void* args[] = {(void*)&sg, (void*)&p.S_final, (void*)&g.lost, (void*)&plan.nseg, (void*)&dv};
+        PF_CUDA_TRY(launch_early(fn, dim3((unsigned)(nseq * (DV / 16))), 128, args, smem, p.stream));
         prof_end(p.stream);
     }
     constexpr int smem = DV * LD * 2;
     prof_begin("chain_apply", p.stream);
-    void* args[] = {(void*)&sg, (void*)&p.O, (void*)&p.L, (void*)&first_tokens, (void*)&seg_tokens, (void*)&plan.nseg};
-    PF_CUDA_TRY(launch_early((const void*)chain_apply<DK, DV>, dim3((unsigned)((seg_tokens + 127) / 128), (unsigned)(nseq * (plan.nseg - 1))), 256,
-                             args, smem, p.stream));
+    const void* fn;
+    void *args[6] = {(void*)&sg, (void*)&p.O, (void*)&p.L, (void*)&first_tokens, (void*)&seg_tokens, (void*)&plan.nseg}, *walk_args[3] = {nullptr, (void*)&first_tokens, (void*)&seg_tokens};
+    const ChainArgs walk{g, sg};
+    if constexpr (LOST_R > 0) {
+        fn = (const void*)chain_apply_or_walk<DK, DV, LOST_R>;
+        walk_args[0] = (void*)&walk;
+    } else {
+        fn = (const void*)chain_apply<DK, DV>;
+    }
+    PF_CUDA_TRY(launch_early(fn, dim3((unsigned)((seg_tokens + 127) / 128), (unsigned)(nseq * (plan.nseg - 1))), 256, LOST_R > 0 ? walk_args : args, smem, p.stream));
     prof_end(p.stream);
     count_launch(2);
     return PF_OK;
@@ -1583,16 +1653,25 @@ bool chain_supported(const Problem& p) {
 
 int chain_forward(const Problem& p, void* workspace) {
     const ChainPlan plan = make_plan(p);
+    const ChainCarve c = carve(p, plan);
+    const ChainGeo g = make_geo(p, plan, c, workspace);
     ChainSeg sg{};
     if (plan.nseg > 1) {
-        const ChainCarve c = carve(p, plan);
         uint8_t* ws = (uint8_t*)workspace;
         sg = {(__half*)(ws + c.R), (__half*)(ws + c.P), (float*)(ws + c.D), (float*)(ws + c.Xi), (__half*)(ws + c.start)};
     }
-    const int st = p.d_k == 128 ? launch_rank<128>(p, plan, sg, workspace) : launch_rank<64>(p, plan, sg, workspace);
+    if (plan.share > 0) PF_CUDA_TRY(cudaMemsetAsync(g.handed, 0, c.flag_bytes, p.stream));
+    const int st = p.d_k == 128 ? launch_rank<128>(p, plan, g, sg) : launch_rank<64>(p, plan, g, sg);
     if (st != PF_OK || plan.nseg == 1) return st;
-    if (p.d_k == 128) return p.d_v == 128 ? launch_seg_tail<128, 128>(p, plan, sg) : launch_seg_tail<128, 64>(p, plan, sg);
-    return p.d_v == 128 ? launch_seg_tail<64, 128>(p, plan, sg) : launch_seg_tail<64, 64>(p, plan, sg);
+    if (g.lost)                                                   // (the single launch's shapes)
+        switch (p.r) {
+            case 1: return launch_seg_tail<128, 128, 1>(p, plan, g, sg);
+            case 2: return launch_seg_tail<128, 128, 2>(p, plan, g, sg);
+            case 3: return launch_seg_tail<128, 128, 3>(p, plan, g, sg);
+            default: return launch_seg_tail<128, 128, 4>(p, plan, g, sg);
+        }
+    if (p.d_k == 128) return p.d_v == 128 ? launch_seg_tail<128, 128>(p, plan, g, sg) : launch_seg_tail<128, 64>(p, plan, g, sg);
+    return p.d_v == 128 ? launch_seg_tail<64, 128>(p, plan, g, sg) : launch_seg_tail<64, 64>(p, plan, g, sg);
 }
 
 }  // namespace pf

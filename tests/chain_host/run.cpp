@@ -122,6 +122,7 @@ alignas(1024) static uint8_t host_smem[228 * 1024];
 #define __all_sync(m, x) (x)
 #define clock64() host::clock64()
 template <class T> T atomicCAS(T* p, T a, T b) { const T old = *p; if (old == a) *p = b; return old; }
+template <class T> T atomicAdd(T* p, T b) { const T old = *p; *p += b; return old; }
 template <class T> T atomicOr(T* p, T b) { const T old = *p; *p |= b; return old; }
 static float __uint_as_float(uint32_t x) { float y; memcpy(&y, &x, 4); return y; }
 static uint32_t __float_as_uint(float x) { uint32_t y; memcpy(&y, &x, 4); return y; }

@@ -140,6 +140,38 @@ def test_repeated_calls_agree_to_the_bit(d_k, d_v, r, H, L, impl):
         assert torch.equal(O, first[0]) and torch.equal(S, first[1])
 
 
+@pytest.mark.parametrize("where", ["response", "readout"])
+@pytest.mark.parametrize("in_place", [False, True])
+def test_responses_that_leave_the_range_of_fp16(where, in_place):
+    """32 sequences of 8192, which are walked in segments for speed.  In every third sequence 18 tokens of the second segment double and negate what the state
+    holds along one key: the response to the segment's start state reaches 2^18 while the state itself, 1e-3 there, stays small.  Or one query of
+    the segment is as long as 3e5, so that only a token's response leaves the range.  Neither may cost more than time."""
+    import paper_2504_00492_b200 as pf
+    w = Workload("amplified", B=1, H=32, L=8192, d_k=128, d_v=128, r=2, chunk=64, beta_scale=0.5, s0_std=0.1, seed=990)
+    inp = pf_synth.make_inputs(w)
+    seqs = slice(0, w.H, 3)
+    k = inp.k.float()
+    k[..., 0] = 0.0                                               # (nothing else touches the first entry)
+    inp.k = (k / k.norm(dim=-1, keepdim=True)).to(inp.k.dtype)
+    inp.S0[:, :, 0] *= 1e-2
+    if where == "response":
+        for t in range(5700, 5700 + 18 * 64, 64):
+            inp.k[:, seqs, t] = torch.eye(128)[0].to(inp.k.dtype)
+            inp.v[:, seqs, t] = 0.0
+            inp.beta[:, seqs, t] = 1.5
+    else:
+        inp.q[:, seqs, 6000] = (3e5 * torch.eye(128)[0]).to(inp.q.dtype)
+        inp.S0[:, seqs, 0] *= 1e-2
+    d = inp.to("cuda")
+    out = []
+    names = util.kernels_of(lambda: out.append(pf.pf_deltanet_fwd(d.q, d.k, d.v, d.beta, d.S0, w.chunk, S_final=d.S0 if in_place else None)))
+    assert names == ["chain", "chain_compose", "chain_apply"] and pf.pf_read_status() == 0
+    O_ref, S_ref = util.run_oracle(inp)
+    for x, ref, what in zip(out[0], (O_ref, S_ref), ("O", "S_final")):
+        assert torch.isfinite(x).all(), what
+        util.check_per_sequence(x.cpu().numpy(), ref, util.TOL_BF16, what)
+
+
 @pytest.mark.parametrize("d,r,most", [(128, 2, 35), (64, 2, 25)])
 def test_the_second_walk_of_lost_rows_takes_a_bounded_multiple_of_the_call(d, r, most):
     """Every row lost (a start state beyond fp16): 20 and 14 times the call without, 63 and 34 where eight warps walk 16 rows each."""
