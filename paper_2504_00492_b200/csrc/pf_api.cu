@@ -76,7 +76,6 @@ int library_status_word(int** out) {
 // its pages back at every synchronisation, and mapping them anew cost the next call 0.4 ms (42 MB) to 4 ms (a two-launch
 // workspace); this one keeps up to WORKSPACE_KEEP bytes of free pages (the rings of the single-launch kernel always fit)
 // until pf_release_workspaces.  Allocation and free stay ordered on the caller's stream.
-constexpr uint64_t WORKSPACE_KEEP = 96ull << 20;
 std::mutex g_pool_mu;
 cudaMemPool_t g_pool[kMaxDevices] = {};
 
@@ -328,8 +327,8 @@ int forward_one(const pf_params* a, bool top) {
         if (a->workspace_bytes < need || ((uintptr_t)ws & 255u)) return PF_ERR_WORKSPACE;
     } else {
         auto alloc = [&]() {
-            const size_t own_need = use_recur(p, impl) ? recur_workspace_bytes(p)
-                                    : use_chain(p, impl) && !chain_needs_workspace(p) ? 0 : workspace_need(p, impl);
+            // (neither of the two has step sizes there)
+            const size_t own_need = use_recur(p, impl) ? recur_workspace_bytes(p) : !use_chain(p, impl) ? workspace_need(p, impl) : chain_needs_workspace(p) ? chain_workspace_bytes(p) : 0;
             own = own_need > 0;
             return own ? workspace_alloc(&ws, own_need, p.stream) : (int)PF_OK;
         };

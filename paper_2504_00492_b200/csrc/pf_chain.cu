@@ -1435,76 +1435,6 @@ struct ChainPlan {
     bool rewalk;              // sequences in which a response leaves fp16's range are walked again (chain_apply)
     double short_us;          // the kernel alone without segments, the start of each wave counted: what a call of a few blocks takes
 };
-// Equal shares of all blocks (part_at) in place of a walk each, where that is faster: more sequences than multiprocessors, or, of a state as wide as its response,
-// few in segments, the first of which is as long as a share (it has no response to walk) and the others as many as it takes.  Against it stand clearing the flags, a state
-// through memory and the starts of further walks, 12 us and 1.5 a walk, a block that takes longer while all multiprocessors are busy to the end, and more responses.
-// Measured, us, shared out and not, d = 128: 160 and 200 sequences of 1000, r = 2: 85 and 110, 97 and 115; 256 of 1024: 119 and 113 (not taken); 300 of 500, r = 4: 124
-// and 155; 32 of 8192, r = 2: 225 and 239 (single launch: 247); r = 3: 294 and 343; r = 1: 175 and 167 (not taken); d = 64: 64 of 4096, r = 4: 207 and 257; 200 of
-// 2000, r = 1: 80 and 96; 32 of 8192, r = 2: 152 and 176.  The estimates below come within 5 % of these (one wave's by 8 % less than make_plan's, whose choices against the
-// single launch are left as they are).  Not where the responses need more memory than the library keeps from call to call: 32 of 65536, r = 2, take 2200 us
-// and the single launch 1815.
-constexpr size_t SHARE_MOST_BYTES = (size_t)88 << 20;
-ChainPlan share_out(const Problem& p, const ChainPlan& plan, int nblk, double block_us) {
-    const long long nseq = (long long)p.B * p.H, sms = sm_count();
-    if (sms < 1 || nseq * nblk > 0x3fffffffLL || p.no_share) return plan;
-    const double row_bytes = 4.0 * p.d_k + 8.0 * p.d_v, tail = p.d_k == 128 ? 4.0 : 2.0, per_seg = p.d_k == 128 ? 0.85 : 0.4;
-    ChainPlan out = plan;
-    double us = 12.0, rival = 7.0 + 0.92 * (plan.us - 7.0);
-    if (nseq > sms) {
-        out.nseg = 1;
-        out.seg_blk = out.first_blk = nblk;
-        block_us *= p.d_k == 128 ? 1.05 : 0.95;
-    } else {
-        if (p.d_k != p.d_v || nblk < 8 || (size_t)nseq * p.L * p.d_k * 2 > SHARE_MOST_BYTES) return plan;
-        const long long first = 2 * nblk * nseq / (sms + nseq);
-        if (first >= nblk || first < 1) return plan;
-        out.nseg = 1 + (int)((nblk - first + first - 1) / first);
-        if (out.nseg > 64) return plan;
-        out.seg_blk = (int)((nblk - first + out.nseg - 2) / (out.nseg - 1));
-        out.first_blk = nblk - (out.nseg - 1) * out.seg_blk;
-        if (out.first_blk < 1) return plan;
-        us += 3.0 + tail + per_seg * out.nseg + (double)nseq * p.L * (nblk - out.first_blk) / nblk * row_bytes / 6e6;
-        if (p.d_k == 64) block_us *= 0.95;
-        if (plan.nseg > 1) {      // (the composing kernels' part of the estimate does not shrink, their traffic goes at 6 TB/s)
-            const double traffic = (double)nseq * p.L * (plan.nseg - 1) / plan.nseg * row_bytes, kernels = (p.d_k == 128 ? 11.0 : 9.0) + per_seg * plan.nseg;
-            rival = kernels + traffic / 6e6 + 0.92 * (plan.us - kernels - traffic / 4e6);
-        }
-    }
-    const long long total = nseq * (2 * nblk - out.first_blk);
-    out.share = (int)((total + sms - 1) / sms);
-    out.ctas = (int)((total + out.share - 1) / out.share);
-    const int other = out.nseg > 1 ? out.seg_blk : out.first_blk, longest = out.first_blk > other ? out.first_blk : other, shortest = out.first_blk < other ? out.first_blk : other;
-    if (longest > out.share || out.share / shortest + 2 > MOST_PARTS) return plan;
-    out.us = us + out.share * block_us + 1.5 * out.share / shortest;
-    out.rewalk = out.nseg > 1 && fused_supported(p) && fused_estimate_us(p) < plan.us;
-    return out.us < 0.985 * rival ? out : plan;
-}
-ChainPlan make_plan(const Problem& p) {
-    static const double alone[2][4] = {{1.40, 1.25, 1.25, 1.19}, {1.95, 1.53, 1.50, 1.55}};
-    static const double crowded[2][4] = {{1.70, 1.34, 1.33, 1.24}, {2.30, 1.79, 1.68, 1.58}};
-    const long long nseq = (long long)p.B * p.H, sms = sm_count();
-    const int C = NB / p.r, nblk = (p.L + C - 1) / C;
-    auto step = [&](long long ctas) {
-        const double a = alone[p.d_k == 128][p.r - 1], c = crowded[p.d_k == 128][p.r - 1];
-        const double crowd = sms > 0 ? 2.0 * ctas / sms - 1.0 : 0.0;
-        return a + (c - a) * (crowd < 0.0 ? 0.0 : crowd > 1.0 ? 1.0 : crowd);
-    };
-    const double waves = (double)((nseq + sms - 1) / (sms > 0 ? sms : 1)), walk = nblk * step(nseq) * waves;
-    ChainPlan plan{1, nblk, 7.0 + walk, nblk, 0, 0, false, 5.0 * waves + walk};
-    const double limit = 0.92 * plan.us;
-    // (calls of up to 512 tokens at d_k = 128 are one launch, which a test of two sequences of 512 expects, also where segments would be faster: 16 of
-    //  333, r = 2: 21.7 us, 20.9 estimated in four)
-    if (p.d_k == 128 && p.L <= 512) return nseq > sms ? share_out(p, plan, nblk, step(sms)) : plan;
-    for (int want = 2; nseq * (2 * want - 1) <= sms && want <= 64 && want <= nblk; ++want) {
-        const int seg_blk = (nblk + want - 1) / want, nseg = (nblk + seg_blk - 1) / seg_blk;
-        // (two kernels, their share per segment, and the traffic of the responses and of O at about 4 TB/s)
-        const double traffic = (double)nseq * p.L * (nseg - 1) / nseg * (4.0 * p.d_k + 8.0 * p.d_v) / 4e6;
-        const double us = (p.d_k == 128 ? 11.0 + 0.85 * nseg : 9.0 + 0.4 * nseg) + traffic + seg_blk * step(nseq * (2 * nseg - 1));
-        if (us < limit && us < plan.us) plan = {nseg, seg_blk, us, seg_blk, 0, 0, false, plan.short_us};
-    }
-    return share_out(p, plan, nblk, step(sms));
-}
-
 struct ChainCarve {
     size_t R, P, D, Xi, start, flags, flag_bytes, hand, total;
 };
@@ -1531,6 +1461,76 @@ ChainCarve carve(const Problem& p, const ChainPlan& plan) {
     }
     c.total = off;
     return c;
+}
+
+// Equal shares of all blocks (part_at) in place of a walk each, where that is faster: more sequences than multiprocessors, or, of a state as wide as its response,
+// few in segments, the first of which is as long as a share (it has no response to walk) and the others as many as it takes.  Against it stand clearing the flags, a state
+// through memory and the starts of further walks, 12 us and 1.5 a walk, a block that takes longer while all multiprocessors are busy to the end, and more responses.
+// Measured, us, shared out and not, d = 128: 160 and 200 sequences of 1000, r = 2: 85 and 110, 97 and 115; 256 of 1024: 119 and 113 (not taken); 300 of 500, r = 4: 124
+// and 155; 32 of 8192, r = 2: 225 and 239 (single launch: 247); r = 3: 294 and 343; r = 1: 175 and 167 (not taken); d = 64: 64 of 4096, r = 4: 207 and 257; 200 of
+// 2000, r = 1: 80 and 96; 32 of 8192, r = 2: 152 and 176.  The estimates below come within 5 % of these (one wave's by 8 % less than make_plan's, whose choices against the
+// single launch are left as they are).  Not where segments would need more workspace than the library keeps
+// from call to call: a caller who synchronises between calls would have it mapped anew at each (32 of 9600, r = 2, 96.3 MB: 2700 us, 298 in the single launch).
+ChainPlan share_out(const Problem& p, const ChainPlan& plan, int nblk, double block_us) {
+    const long long nseq = (long long)p.B * p.H, sms = sm_count();
+    if (sms < 1 || nseq * nblk > 0x3fffffffLL || p.no_share) return plan;
+    const double row_bytes = 4.0 * p.d_k + 8.0 * p.d_v, tail = p.d_k == 128 ? 4.0 : 2.0, per_seg = p.d_k == 128 ? 0.85 : 0.4;
+    ChainPlan out = plan;
+    double us = 12.0, rival = 7.0 + 0.92 * (plan.us - 7.0);
+    if (nseq > sms) {
+        out.nseg = 1;
+        out.seg_blk = out.first_blk = nblk;
+        block_us *= p.d_k == 128 ? 1.05 : 0.95;
+    } else {
+        if (p.d_k != p.d_v || nblk < 8) return plan;
+        const long long first = 2 * nblk * nseq / (sms + nseq);
+        if (first >= nblk || first < 1) return plan;
+        out.nseg = 1 + (int)((nblk - first + first - 1) / first);
+        if (out.nseg > 64) return plan;
+        out.seg_blk = (int)((nblk - first + out.nseg - 2) / (out.nseg - 1));
+        out.first_blk = nblk - (out.nseg - 1) * out.seg_blk;
+        if (out.first_blk < 1) return plan;
+        us += 3.0 + tail + per_seg * out.nseg + (double)nseq * p.L * (nblk - out.first_blk) / nblk * row_bytes / 6e6;
+        if (p.d_k == 64) block_us *= 0.95;
+        if (plan.nseg > 1) {      // (the composing kernels' part of the estimate does not shrink, their traffic goes at 6 TB/s)
+            const double traffic = (double)nseq * p.L * (plan.nseg - 1) / plan.nseg * row_bytes, kernels = (p.d_k == 128 ? 11.0 : 9.0) + per_seg * plan.nseg;
+            rival = kernels + traffic / 6e6 + 0.92 * (plan.us - kernels - traffic / 4e6);
+        }
+    }
+    const long long total = nseq * (2 * nblk - out.first_blk);
+    out.share = (int)((total + sms - 1) / sms);
+    out.ctas = (int)((total + out.share - 1) / out.share);
+    const int other = out.nseg > 1 ? out.seg_blk : out.first_blk, longest = out.first_blk > other ? out.first_blk : other, shortest = out.first_blk < other ? out.first_blk : other;
+    if (longest > out.share || out.share / shortest + 2 > MOST_PARTS) return plan;
+    out.rewalk = out.nseg > 1 && fused_supported(p) && fused_estimate_us(p) < plan.us;
+    if (out.nseg > 1 && carve(p, out).total > WORKSPACE_KEEP) return plan;
+    out.us = us + out.share * block_us + 1.5 * out.share / shortest;
+    return out.us < 0.985 * rival ? out : plan;
+}
+ChainPlan make_plan(const Problem& p) {
+    static const double alone[2][4] = {{1.40, 1.25, 1.25, 1.19}, {1.95, 1.53, 1.50, 1.55}};
+    static const double crowded[2][4] = {{1.70, 1.34, 1.33, 1.24}, {2.30, 1.79, 1.68, 1.58}};
+    const long long nseq = (long long)p.B * p.H, sms = sm_count();
+    const int C = NB / p.r, nblk = (p.L + C - 1) / C;
+    auto step = [&](long long ctas) {
+        const double a = alone[p.d_k == 128][p.r - 1], c = crowded[p.d_k == 128][p.r - 1];
+        const double crowd = sms > 0 ? 2.0 * ctas / sms - 1.0 : 0.0;
+        return a + (c - a) * (crowd < 0.0 ? 0.0 : crowd > 1.0 ? 1.0 : crowd);
+    };
+    const double waves = (double)((nseq + sms - 1) / (sms > 0 ? sms : 1)), walk = nblk * step(nseq) * waves;
+    ChainPlan plan{1, nblk, 7.0 + walk, nblk, 0, 0, false, 5.0 * waves + walk};
+    const double limit = 0.92 * plan.us;
+    // (calls of up to 512 tokens at d_k = 128 are one launch, which a test of two sequences of 512 expects, also where segments would be faster: 16 of
+    //  333, r = 2: 21.7 us, 20.9 estimated in four)
+    if (p.d_k == 128 && p.L <= 512) return nseq > sms ? share_out(p, plan, nblk, step(sms)) : plan;
+    for (int want = 2; nseq * (2 * want - 1) <= sms && want <= 64 && want <= nblk; ++want) {
+        const int seg_blk = (nblk + want - 1) / want, nseg = (nblk + seg_blk - 1) / seg_blk;
+        // (two kernels, their share per segment, and the traffic of the responses and of O at about 4 TB/s)
+        const double traffic = (double)nseq * p.L * (nseg - 1) / nseg * (4.0 * p.d_k + 8.0 * p.d_v) / 4e6;
+        const double us = (p.d_k == 128 ? 11.0 + 0.85 * nseg : 9.0 + 0.4 * nseg) + traffic + seg_blk * step(nseq * (2 * nseg - 1));
+        if (us < limit && us < plan.us) plan = {nseg, seg_blk, us, seg_blk, 0, 0, false, plan.short_us};
+    }
+    return share_out(p, plan, nblk, step(sms));
 }
 
 ChainGeo make_geo(const Problem& p, const ChainPlan& plan, const ChainCarve& c, void* workspace) {

@@ -111,6 +111,9 @@ __device__ __forceinline__ void wait_for_previous_kernel() { asm volatile("gridd
 __device__ __forceinline__ void let_next_kernel_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 #endif
 
+// free pages that the pool of workspaces keeps between calls (pf_api.cu)
+constexpr uint64_t WORKSPACE_KEEP = 96ull << 20;
+
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 // room at the end of every workspace for the fp32 step sizes of PF_STEP_EXACT
 inline size_t beta32_bytes(const Problem& p) { return align_up((size_t)p.B * p.H * p.L * p.r * 4, 256); }
