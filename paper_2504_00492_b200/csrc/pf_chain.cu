@@ -1129,13 +1129,14 @@ chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __rest
         parts_n = n;
     }
     if (warp == W_MMA) tmem_alloc(&tmem_base, 512);
+    // (as many slots as there are blocks, also of T at its end: with NS of them, 81.8 us instead of 80.5 at 48 sequences of 1999, r = 3)
     if (SM::CP > SM::C) {                                         // (r = 3: query rows that no copy writes are read)
         for (int e = tid; e < CFG::NS * SM::stage / 16; e += CHAIN_THREADS) ((uint4*)smem)[e] = make_uint4(0, 0, 0, 0);
     } else {                                                      // (the upper triangles of P and T, which nothing writes)
         for (int st = 0; st < CFG::NS && st < count; ++st)
             for (int e = tid; e < SM::p_bytes / 16; e += CHAIN_THREADS) ((uint4*)(smem + st * SM::stage + SM::p_off))[e] = make_uint4(0, 0, 0, 0);
     }
-    for (int e = tid; e < CFG::NS * SM::t_bytes / 16; e += CHAIN_THREADS) ((uint4*)(smem + CFG::t_off))[e] = make_uint4(0, 0, 0, 0);
+    for (int e = tid; e < min(CFG::NS, count) * SM::t_bytes / 16; e += CHAIN_THREADS) ((uint4*)(smem + CFG::t_off))[e] = make_uint4(0, 0, 0, 0);
     for (int e = tid; e < IdStrip::bytes / 2; e += CHAIN_THREADS) ((uint16_t*)(smem + CFG::id_off))[e] = IdStrip::one(e) ? 0x3F80 : 0;
     fence_async_smem();
     tc_fence_before();
