@@ -641,9 +641,10 @@ pf_params seg_subproblem(const pf_params* a, int S) {
 size_t seg_tail_bytes(const pf_params* a, int S) {
     return 4 * seg_array_bytes(a, S) + seg_response_bytes(a) + seg_zero_v_bytes(a);
 }
-size_t seg_workspace_need(const pf_params* a, int S) {
+size_t seg_workspace_need(const pf_params* a, int S, bool no_share = false) {
     const pf_params b = seg_subproblem(a, S);
     Problem p = as_problem(&b);
+    p.no_share = no_share;
     const int impl = select_impl(p, b.impl);
     if (impl < 0) return 0;
     return align_up(workspace_need(p, impl), 256) + seg_tail_bytes(a, S);
@@ -654,15 +655,22 @@ int forward_segmented(const pf_params* a, int S) {
     if (st != PF_OK) return st;
     if (!seg_applicable(a, S)) return PF_ERR_UNSUPPORTED;
     pf_params sub = seg_subproblem(a, S);
-    const size_t need = seg_workspace_need(a, S);
+    size_t need = seg_workspace_need(a, S);
     if (need == 0) return PF_ERR_UNSUPPORTED;
     cudaStream_t stream = (cudaStream_t)a->stream;
     void* ws = a->workspace;
     bool own = false;
     if (ws) {
+        if (a->workspace_bytes < need) need = seg_workspace_need(a, S, true);      // (as in forward_one, which sees what its passes have)
         if (a->workspace_bytes < need || ((uintptr_t)ws & 255u)) return PF_ERR_WORKSPACE;
     } else {
         st = workspace_alloc(&ws, need, stream);
+        const size_t less = seg_workspace_need(a, S, true);
+        if (st == PF_ERR_CUDA && less < need) {
+            cudaGetLastError();
+            need = less;
+            st = workspace_alloc(&ws, need, stream);
+        }
         if (st != PF_OK) return st;
         own = true;
     }

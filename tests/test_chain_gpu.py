@@ -260,3 +260,13 @@ def test_shared_out_segments_need_no_more_workspace_than_the_library_keeps():
         assert need - (small - 1024) <= 96 << 20, (L, need)
         shared = max(shared, need)
     assert shared > 90 << 20, "not shared out"
+
+
+def test_segments_of_an_option_take_less_workspace_than_sharing_walks_out_would():
+    """160 walks of the option `segments` are shared out for speed where there is workspace for that, and are a CTA's each where not."""
+    import paper_2504_00492_b200 as pf
+    w = Workload("option", B=1, H=20, L=8000, d_k=128, d_v=128, r=2, chunk=64, s0_std=0.1, seed=995)
+    need = pf.pf_workspace_bytes_ex(w.B, w.H, w.L, w.d_k, w.d_v, w.r, w.chunk, segments=8)
+    states = torch.cuda.get_device_properties(0).multi_processor_count // 2 * 4 * w.d_k * w.d_v
+    for workspace in (None, need, need - states):
+        util.check_parity(w, segments=8, workspace=workspace and torch.empty(workspace, dtype=torch.uint8, device="cuda"))
