@@ -126,11 +126,12 @@ def kernel_roofline(prof: dict, w, chunk_selected: int, peaks: dict, peak_kind: 
         achieved = fl / seconds / 1e12
         return {"bound": kind, "achieved": achieved, "peak": rate, "unit": "TFLOP/s", "frac": achieved / rate, "traffic": None,
                 "flops_per_launch": fl, "flop_count": "triangular-aware", **common}
-    # The kernel does everything: its algorithmic traffic is one read of q, k, v, beta and one write of O.  What binds is
-    # the longer of that and the arithmetic of its own form (dense FLOPs), each at the measured peak; both are printed.
+    # The kernel does everything: the pass's algorithmic traffic is one read of q, k, v, beta and one write of O, in the time of this kernel and of
+    # those that follow it in segments, which are part of the pass.  What binds is the longer of that and the arithmetic of its own form (dense
+    # FLOPs, in its own time), each at the measured peak; both are printed.
     nbytes = w.token_heads * alg_bytes_per_token_head(w)
     fl = pass_flops(top, w, chunk_selected, tri=False, solve=False)
-    gbs, tflops = nbytes / seconds / 1e9, fl / seconds / 1e12
+    gbs, tflops = nbytes / (sum(prof.values()) * 1e-3) / 1e9, fl / seconds / 1e12
     math = {"tflops_dense": tflops, "peak": rate, "frac": tflops / rate}
     if kind == "tensor":
         math["pipe_active_pct"], math["pipe_active_from"] = ncu_tensor_pipe(w) if top == "fused" else (None, None)

@@ -31,6 +31,14 @@ def test_chain_kernel_is_counted_in_its_own_blocks():
     assert r["tensor"]["pipe_active_pct"] is None            # (no capture of this kernel at this size)
 
 
+def test_kernels_that_follow_in_segments_are_part_of_the_pass():
+    w = pf_synth.CONFIGS["c2"]
+    r = bench.kernel_roofline({"chain": 0.18, "chain_compose": 0.01, "chain_apply": 0.06}, w, 64, PEAKS, "measured")
+    nbytes = w.token_heads * bench.alg_bytes_per_token_head(w)
+    assert r["kernel"] == "chain" and r["bound"] == "hbm" and r["achieved"] == pytest.approx(nbytes / 0.25e-3 / 1e9)
+    assert r["frac"] == pytest.approx(r["achieved"] / PEAKS["hbm_gbs"])
+
+
 def test_single_launch_keeps_the_chunk_form():
     w = pf_synth.CONFIGS["c2"]
     assert bench.chunk_of("fused", w, 64) == 64
