@@ -4,9 +4,8 @@
 //     T  = (I + Mstrict (.) (diag(beta) K K^T))^{-1} diag(beta)                      (does not depend on S)
 //     P  = (Q K^T) (.) Mincl                                                         (does not depend on S)
 //     U' = T (V - K S^T),       O = Q S^T + P U',       S <- S + U'^T K
-// with W = T K and Uh = T V never formed: T is applied to V - K S^T, in which what the state predicts of V is taken away before anything is rounded.  Only three
-// products of a block depend on S one after another: R = V - K S^T, U' = T R and the update.
-// All are tcgen05 products of 128 rows j (d_v = 64: half of them nobody's) whose A operand lies
+// W = T K and Uh = T V are never formed: T is applied to V - K S^T, which is rounded when what the state predicts of V is out of it.  Three products of a
+// block depend on S one after another: R = V - K S^T, U' = T R and the update.  All are tcgen05 products of 128 rows j (d_v = 64: half of them nobody's) whose A operand lies
 // in tensor memory and whose B operand is a tile of shared memory as TMA or the preparing warps left it.  S stays in tensor memory as the
 // fp32 accumulator of its update; between two products the chain warps convert an accumulator to the next one's fp16 operand.
 //
@@ -1129,14 +1128,15 @@ chain_kernel(const __grid_constant__ ChainMaps maps, const __nv_bfloat16* __rest
         parts_n = n;
     }
     if (warp == W_MMA) tmem_alloc(&tmem_base, 512);
-    // (as many slots as there are blocks, also of T at its end: with NS of them, 81.8 us instead of 80.5 at 48 sequences of 1999, r = 3)
     if (SM::CP > SM::C) {                                         // (r = 3: query rows that no copy writes are read)
         for (int e = tid; e < CFG::NS * SM::stage / 16; e += CHAIN_THREADS) ((uint4*)smem)[e] = make_uint4(0, 0, 0, 0);
     } else {                                                      // (the upper triangles of P and T, which nothing writes)
         for (int st = 0; st < CFG::NS && st < count; ++st)
             for (int e = tid; e < SM::p_bytes / 16; e += CHAIN_THREADS) ((uint4*)(smem + st * SM::stage + SM::p_off))[e] = make_uint4(0, 0, 0, 0);
     }
-    for (int e = tid; e < min(CFG::NS, count) * SM::t_bytes / 16; e += CHAIN_THREADS) ((uint4*)(smem + CFG::t_off))[e] = make_uint4(0, 0, 0, 0);
+    // (r = 3: as many slots as there are blocks, 80.5 us instead of 81.8 at 48 sequences of 1999; elsewhere all, 20.9 instead of 21.1 at 16 of 333, r = 2)
+    const int t_slots = SM::CP > SM::C ? min(CFG::NS, count) : CFG::NS;
+    for (int e = tid; e < t_slots * SM::t_bytes / 16; e += CHAIN_THREADS) ((uint4*)(smem + CFG::t_off))[e] = make_uint4(0, 0, 0, 0);
     for (int e = tid; e < IdStrip::bytes / 2; e += CHAIN_THREADS) ((uint16_t*)(smem + CFG::id_off))[e] = IdStrip::one(e) ? 0x3F80 : 0;
     fence_async_smem();
     tc_fence_before();
@@ -1467,10 +1467,11 @@ ChainCarve carve(const Problem& p, const ChainPlan& plan) {
 // Equal shares of all blocks (part_at) in place of a walk each, where that is faster: more sequences than multiprocessors, or, of a state as wide as its response,
 // few in segments, the first of which is as long as a share (it has no response to walk) and the others as many as it takes.  Against it stand clearing the flags, a state
 // through memory and the starts of further walks, 12 us and 1.5 a walk, a block that takes longer while all multiprocessors are busy to the end, and more responses.
-// Measured, us, shared out and not, d = 128: 160 and 200 sequences of 1000, r = 2: 85 and 110, 97 and 115; 256 of 1024: 119 and 113 (not taken); 300 of 500, r = 4: 124
-// and 155; 32 of 8192, r = 2: 225 and 239 (single launch: 247); r = 3: 294 and 343; r = 1: 175 and 167 (not taken); d = 64: 64 of 4096, r = 4: 207 and 257; 200 of
-// 2000, r = 1: 80 and 96; 32 of 8192, r = 2: 152 and 176.  The estimates below come within 5 % of these (one wave's by 8 % less than make_plan's, whose choices against the
-// single launch are left as they are).  Not where segments would need more workspace than the library keeps
+// Measured, us, shared out and not, inputs that change from call to call, d = 128: 160 and 200 sequences of 1000, r = 2: 82 and 110, 100 and 112; 300 of 500, r = 4: 123
+// and 156; 150 of 2000, r = 3, d_v = 64: 171 and 297; 32 of 8192, r = 2: 243, and 250 in the single launch; r = 3: 302 and 344; 32 of 4096, r = 4: 187 and 214; d = 64: 64 of
+// 4096, r = 4: 208 and 276; 200 of 2000, r = 1: 79 and 92; 32 of 8192, r = 2: 153 and 176; 200 of 1000, 64 x 128, r = 1: 54 and 57.  Not taken, and measured when they were (same
+// inputs): 256 of 1024, r = 2: 119 and 113; 32 of 8192, r = 1: 175 and 167.  The estimates below are within 10 % of these, but 15 % low at 32 of 8192, r = 2 (207), and 16 % high
+// for 200 of 2000 without sharing (107); one wave's without sharing is 8 % below make_plan's, whose choices against the single launch are left as they are.  Not where segments would need more workspace than the library keeps
 // from call to call: a caller who synchronises between calls would have it mapped anew at each (32 of 9600, r = 2, 96.3 MB: 2700 us, 298 in the single launch).
 ChainPlan share_out(const Problem& p, const ChainPlan& plan, int nblk, double block_us) {
     const long long nseq = (long long)p.B * p.H, sms = sm_count();
