@@ -216,8 +216,9 @@ typedef struct pf_params {
 
 /* Same operation with explicit options.  The workspace holds per-chunk intermediates (T', W, Uh, P
  * of Theorem 3.2 in the forms the selected kernels exchange) and, at its end, the fp32 step sizes of
- * PF_STEP_EXACT; its content after the call is unspecified.  Same passages as pf_deltanet_fwd, plus those
- * named at PF_MODE_* and PF_STEP_*. */
+ * PF_STEP_EXACT; its content after the call is unspecified.  Where PF_IMPL_AUTO would share the walks of the one-kernel chunk form out
+ * among all SMs, a workspace of less than pf_workspace_bytes is taken too if it is enough without that (none where each walk is a whole sequence): the call is
+ * then slower, and in segments its results differ in rounding.  Same passages as pf_deltanet_fwd, plus those named at PF_MODE_* and PF_STEP_*. */
 int pf_deltanet_fwd_ex(const pf_params* p);
 
 /* Bytes of scratch pf_deltanet_fwd_ex needs for this problem with this in_dtype/impl and every option at its
@@ -239,7 +240,8 @@ int pf_select_chunk(int B, int H, int L, int d_k, int d_v, int r, int chunk, int
  * The tensor-core kernels synchronise their warps, and the single-launch path its CTAs, with waits on barriers and
  * flags.  Every such wait is bounded (about a second).  A wait that runs out writes its code into a
  * 4-byte STATUS WORD and the kernels give up: they return, every other wait that sees the word set returns too (those of the
- * one-kernel chunk form do not look at it and count tries, about a second's worth: each of its CTAs ends by itself), and
+ * one-kernel chunk form do not look at it: within a CTA they count tries, about a second's worth, and those for another CTA's state or outputs go by
+ * the clock, so that each of its CTAs ends by itself), and
  * O / S_final of that call are undefined.  Nothing traps, hangs or faults, and the context stays usable.
  *
  * Where the word lives, in this order: pf_params.status if given; else word 0 of pf_params.workspace if the caller
@@ -251,7 +253,8 @@ int pf_select_chunk(int B, int H, int L, int d_k, int d_v, int r, int chunk, int
  * word on the current device.  pf_last_wait_code() then gives the code that was read (host thread local):
  *     1xx  flow-building role of the single-launch path (101-103 solve warps, 11x-12x bulk warps, 14x-15x MMA-issuing
  *          warps, 16x flag warp),   2xx  its scanning role (20x chain, 21x output, 22x loads, 23x MMA issue),
- *     30x  the token-by-token kernel,   31x - 35x  the one-kernel chunk form (350: its tensor memory is not at column 0),
+ *     30x  the token-by-token kernel,   31x - 35x  the one-kernel chunk form (336, 337: another CTA's state, outputs; 350: its tensor memory is not
+ *          at column 0),
  *     1-99 the two-launch path (tc_flow, tc_scan),   99  shared memory not 1024-byte aligned,   900  pf_wait_selftest.
  * The chunk-form fp32 kernels have no such waits.
  */
