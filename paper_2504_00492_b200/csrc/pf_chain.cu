@@ -874,17 +874,25 @@ __device__ __forceinline__ int chain_role(const ChainGeo& g, ChainWork<MODE> wor
             s0 = g.hand + (long long)part.hand_in * DK * part.width;
         }
         const int width = part.width;
+        // (Every further round is a trip to memory, but at d_k = 64, where there are one or two, the shorter code of two is the faster one, us with one and two: 48 sequences of
+        //  1999, 64 x 64, r = 4: 88.1 and 85.2, 140 of 1000: 72.9 and 71.1; of 300, r = 2, in segments: 17.1 and 16.4.  At d_k = 128 with two and four: 16 of 333, r = 2: 21.0 and 21.2)
+        constexpr int SC = DK == 64 && MODE != SHARED ? 16 : 32;  // columns a round
 #pragma unroll 1
-        for (int c = 0; c < HC; c += 32) {                        // (every further round is a trip to memory)
-            uint32_t x[32], y[16];
+        for (int c = 0; c < HC; c += SC) {
+            uint32_t x[SC], y[SC / 2];
             const float* at = s0 + (long long)(h * HC + c) * width + j;
 #pragma unroll
-            for (int e = 0; e < 32; ++e)
+            for (int e = 0; e < SC; ++e)
                 x[e] = __float_as_uint(s0 ? (work.shared ? ld_cg_f32(at + e * width) : at[e * width]) : part.response && h * HC + c + e == j ? 1.f : 0.f);
-            tmem_st32(t_s + c, x);
 #pragma unroll
-            for (int e = 0; e < 16; ++e) y[e] = pack_h2(-__uint_as_float(x[2 * e]), -__uint_as_float(x[2 * e + 1]));
-            tmem_st16(t_s16 + c / 2, y);
+            for (int e = 0; e < SC / 2; ++e) y[e] = pack_h2(-__uint_as_float(x[2 * e]), -__uint_as_float(x[2 * e + 1]));
+            if constexpr (SC == 32) {
+                tmem_st32(t_s + c, x);
+                tmem_st16(t_s16 + c / 2, y);
+            } else {
+                tmem_st16(t_s + c, x);
+                tmem_st8(t_s16 + c / 2, y);
+            }
         }
         if (work.shared && i + 1 < work.size() && work[i + 1].S0 && work[i + 1].hand_in < 0)       // (the next part's, to the L2: a line of 128 bytes for each row i and quarter)
             for (int e = lane; e < HC; e += 32) asm volatile("prefetch.global.L2 [%0];" ::"l"(work[i + 1].S0 + (long long)(h * HC + e) * width + 32 * (warp & 3)));

@@ -39,6 +39,7 @@ template <int N> inline void tmem_ld_frag(uint32_t, uint32_t (&r)[N / 2]) { zero
 inline void tmem_ld_wait() {}
 template <int N> inline void tmem_st32(uint32_t, const uint32_t (&)[N]) {}
 template <int N> inline void tmem_st16(uint32_t, const uint32_t (&)[N]) {}
+template <int N> inline void tmem_st8(uint32_t, const uint32_t (&)[N]) {}
 inline void tmem_st_wait() {}
 inline uint64_t make_desc_ns(uint32_t, uint32_t, uint32_t) { return 0; }
 constexpr uint32_t make_idesc(int, bool, bool, bool) { return 0; }
