@@ -26,8 +26,8 @@
 // named barriers) and the instruction cache (so what is off the chain's path is written small).  148 CTAs at r = 1 move 5.5 TB/s, 84 % of
 // what a copy reaches.  Measured (us, before: the same blocks on
 // warp-level products, a warp carrying 16 rows j in registers; a shared-memory read of every tile by every such warp): 256 sequences of
-// 1024, d = 128, r = 2: 227 -> 136 (calls on other inputs one after another; 228 -> 115 on the same); 128 of 4096, d = 64, r = 4: 340 -> 307 (336 -> 290); 48 of 1999, 64 x 128,
-// r = 3: 144 -> 84 (144 -> 80; 2 segments); 4 of 16384, d = 128, r = 1: 135 -> 78 (segments); 32 of 2048, d = 128, r = 1: 68 -> 54 (the tcgen05 kernel in one launch before).
+// 1024, d = 128, r = 2: 227 -> 130 (calls on other inputs one after another; 228 -> 113 on the same); 128 of 4096, d = 64, r = 4: 340 -> 282 (336 -> 275); 48 of 1999, 64 x 128,
+// r = 3: 144 -> 81 (2 segments); 4 of 16384, d = 128, r = 1: 135 -> 76 (segments); 32 of 2048, d = 128, r = 1: 68 -> 53 (the tcgen05 kernel in one launch before).
 // Measured and not taken: the update's and V - K S^T's products in halves, so that one half is converted while the other is being multiplied (the
 // probe's 1.6 k cycles have it; here 412 us against 389 at 32 sequences of 8192: more instructions); the output's products issued by the chain's
 // warp (462); one election per product instead of per group (427 against 420 then, 179 against 146 with all SMs busy); products in loops on
@@ -40,7 +40,7 @@
 // role; and no warps that poll mbarriers but those that watch for others.
 // Measured and not taken: the chain's warps meeting at a named barrier and the first of them issuing (128 us against 116 at 256 sequences, 314 against 264 at
 // 128 of 4096, d = 64); a predicate on every product instead of a branch around all of a step (twice the instructions); an L2 prefetch of the next tiles (128 of 4096, d = 64:
-// 359 against 338 without, at the time; level elsewhere); W = T K formed ahead, U' = T V - W S^T, two dependent products instead of three (128 of 4096, d = 64, r = 4: 298, 291 without; slower at d = 128): T is then
+// 359 against 338 without, at the time; level elsewhere); W = T K formed ahead, U' = T V - W S^T, two dependent products instead of three (128 of 4096, d = 64, r = 4: 298, 291 without on the same day; slower at d = 128): T is then
 // applied to all of V and not to what the state leaves of it, and W is rounded, which costs up to 1.4 times the error where the state predicts V
 // (d = 64, r = 4, beta to 2, V = S* K, relative L2 error of O: 3.7e-4, 2.7e-4 without).
 //
@@ -1248,7 +1248,7 @@ struct ComposeSmem {
 };
 // LOST: lost[sequence]: chain_apply walks it again, from a start state that S_final may replace.
 template <int DK, bool LOST>
-__global__ void __launch_bounds__(128) chain_compose(ChainSeg sg, float* __restrict__ S_final, const int* __restrict__ lost, int nseg, int d_v) {
+__global__ void __launch_bounds__(128) chain_compose(ChainSeg sg, float* __restrict__ S_final, const int* lost, int nseg, int d_v) {
     using SM = ComposeSmem<DK>;
     constexpr int LD = SM::LD, LX = SM::LX, NT = DK / 32;
     extern __shared__ __align__(16) uint8_t smem_tail[];
@@ -1283,7 +1283,7 @@ __global__ void __launch_bounds__(128) chain_compose(ChainSeg sg, float* __restr
     };
     float S[NT][4];
     wait_for_previous_kernel();
-    if (LOST && lost[seq]) S_final = nullptr;
+    if (LOST && lost[seq]) S_final = nullptr;                     // (not __restrict__: what may not change could be read ahead of the wait)
     for (int s = 1; s <= depth; ++s) load(s, s - 1);
     {
         const float* src = sg.Xi + seq * nseg * DK * d_v;
