@@ -40,7 +40,7 @@
 // role; and no warps that poll mbarriers but those that watch for others.
 // Measured and not taken: the chain's warps meeting at a named barrier and the first of them issuing (128 us against 116 at 256 sequences, 314 against 264 at
 // 128 of 4096, d = 64); a predicate on every product instead of a branch around all of a step (twice the instructions); an L2 prefetch of the next tiles (128 of 4096, d = 64:
-// 359 against 338 without, at the time; level elsewhere); W = T K formed ahead, U' = T V - W S^T, two dependent products instead of three (128 of 4096, d = 64, r = 4: 298, 291 without on the same day; slower at d = 128): T is then
+// 359 against 338 without, at the time; level elsewhere); W = T K formed ahead, U' = T V - W S^T, two dependent products instead of three (128 of 4096, d = 64, r = 4: 298, in turn with 291 without; slower at d = 128): T is then
 // applied to all of V and not to what the state leaves of it, and W is rounded, which costs up to 1.4 times the error where the state predicts V
 // (d = 64, r = 4, beta to 2, V = S* K, relative L2 error of O: 3.7e-4, 2.7e-4 without).
 //
